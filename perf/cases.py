@@ -156,6 +156,79 @@ def work(case):
     return {"bytes": forward + backward + grads, "flops": flops + 12 * R * d * f}
 
 
+def exact(case, seed):
+    """What run() returns for these inputs, by the layer's definition in float64 (plain torch, one expert at a time)."""
+    s = prepare(case, seed)
+    mode, T, E, k = (case[n] for n in ("mode", "T", "E", "k"))
+    x, W_r = s["x"].double(), s["W_r"].double()
+    logits = x @ W_r if s["b_r"] is None else x @ W_r + s["b_r"].double()
+    p = logits.softmax(dim=1)
+    idx = logits.topk(k, dim=1).indices  # no ties: _tokens keeps the logits apart
+    gates = p.gather(1, idx)
+    gates = gates / gates.sum(dim=1, keepdim=True)
+    counts = torch.bincount(idx.reshape(-1), minlength=E)
+    perm = torch.sort(idx.reshape(-1), stable=True).indices
+    share = counts.double() / (T * k)
+    aux = (E * (share * p.mean(dim=0)).sum()).reshape(1)
+    dy = s["dy"].double() if mode != "score" else None
+    y, dx = torch.zeros_like(x), torch.zeros_like(x)
+    dg = torch.zeros_like(gates)
+    grads = {}
+
+    def add(name, e, value):  # gradients of expert e
+        if name not in grads:
+            grads[name] = torch.zeros((E, *value.shape), dtype=torch.float64, device="cuda")
+        grads[name][e] = value
+
+    first = 0
+    for e, n in enumerate(counts.tolist()):
+        rows = perm[first:first + n]
+        first += n
+        tok, slot = rows // k, rows % k
+        Wg, Wu, Wd = (s[w][e].double() for w in ("W_gate", "W_up", "W_down"))
+        if mode == "lora":
+            c = s["scale"]
+            A1, B1g, B1u, A2, B2 = (s["adapters"][w][e].double() for w in ("A1", "B1_gate", "B1_up", "A2", "B2"))
+            Wg, Wu, Wd = Wg + c * A1 @ B1g, Wu + c * A1 @ B1u, Wd + c * A2 @ B2
+        xe, g = x[tok], gates[tok, slot][:, None]
+        hg, hu = xe @ Wg, xe @ Wu
+        sig = torch.sigmoid(hg)
+        act = hg * sig * hu
+        o = act @ Wd
+        y.index_add_(0, tok, g * o)
+        if mode == "score":
+            continue
+        dye = dy[tok]
+        dg[tok, slot] = (dye * o).sum(dim=1)
+        da = g * (dye @ Wd.T)
+        dhg, dhu = da * hu * sig * (1.0 + hg * (1.0 - sig)), da * hg * sig
+        dx.index_add_(0, tok, dhg @ Wg.T + dhu @ Wu.T)
+        dWg, dWu, dWd = xe.T @ dhg, xe.T @ dhu, act.T @ (g * dye)
+        if mode == "lora":
+            for name, v in (("dA1", dWg @ B1g.T + dWu @ B1u.T), ("dB1_gate", A1.T @ dWg), ("dB1_up", A1.T @ dWu), ("dA2", dWd @ B2.T), ("dB2", A2.T @ dWd)):
+                add(name, e, c * v)
+        else:
+            for name, v in (("dW_gate", dWg), ("dW_up", dWu), ("dW_down", dWd)):
+                add(name, e, v)
+    out = {"y": y, "idx": idx.int(), "gates": gates, "counts": counts.int(), "aux": aux}
+    if mode != "lora":
+        out.update(perm=perm.int(), logits=None)
+    if mode == "score":
+        return out
+    # gates are a softmax over the selected logits; the loss term reaches the logits through the mean probabilities
+    dl = torch.zeros_like(p).scatter_(1, idx, gates * (dg - (gates * dg).sum(dim=1, keepdim=True)))
+    dp = (D_AUX * E / T) * share
+    dl += p * (dp - (p * dp).sum(dim=1, keepdim=True))
+    dx += dl @ W_r.T
+    dW_r = x.T @ dl
+    if mode == "accumulate":
+        return [out, dx, {n: s["acc"][n].double() + (dW_r if n == "dW_r" else grads[n]) for n in s["acc"]}]
+    grads.update(dx=dx, dW_r=dW_r)
+    if mode == "train":
+        grads["db_r"] = None
+    return [out, grads]
+
+
 def tolerance(case):
     # bf16 intermediates (pre-activations, activation, expert outputs, their gradients) and bf16 results.  Measured
     # against the same layer in float64: 2.3e-3 to 3.5e-3 (adapters, whose products are rounded once more: 3.3e-3 to
