@@ -21,6 +21,8 @@
 // Warp roles: warp 0 TMA producer, warp 1 MMA issuer (owns the TMEM allocation), warps 2..9 epilogue (2..5 for the
 // routing kind).  The expert-LoRA variant runs on the same template (launch_lora_gemm at the end of this file).
 // Every mbarrier wait is bounded; on a timeout the kernel records it in the status word and leaves.
+#include <math.h>
+
 #include "gemm_common.cuh"
 
 namespace moe {
@@ -188,7 +190,6 @@ __global__ void __launch_bounds__(KIND == GEMM_RT ? 192 : GEMM_THREADS, 1)
     // lane quadrant, each draining half of the tile's columns - the routing epilogue needs whole rows and uses one)
     const int ew = warp & 3;           // TMEM lane quadrant this warp may read
     const int half = (warp - 2) >> 2;  // which half of the columns
-    constexpr int NHALF = EPI_WARPS / 4;
     EpiStage es{smem_base + STAGES * STAGE_BYTES + (warp - 2) * (EPI_UNITS * EPI_UNIT_BYTES), 0u};
     uint32_t tc = 0;
     bool ok = true;
@@ -225,11 +226,11 @@ __global__ void __launch_bounds__(KIND == GEMM_RT ? 192 : GEMM_THREADS, 1)
       tc_fence_after();
       const uint32_t taddr = tmem_base + (static_cast<uint32_t>(ew * 32) << 16) + acc * ACC_COLS;
       const int64_t row = static_cast<int64_t>(tl.row0) + rin;
-      if (KIND == GEMM_F3 || KIND == GEMM_B2) {
-        expert_epilogue<KIND>(p, tl.e, row, (TR::WGRAD ? tl.m0 : tl.row0) + ew * 32, tl.n0, taddr, true,
-                              TR::WGRAD ? p.M_total - (tl.m0 + ew * 32) : (KIND == GEMM_DX ? static_cast<int>(p.T - tl.row0 - ew * 32) : 32),
-                              es, lane, half, NHALF);
-      } else if (KIND == GEMM_RT) {
+      auto release = [&]() {
+        tc_fence_before();
+        mbar_arrive(tempty_bar(acc));
+      };
+      if (KIND == GEMM_RT) {
         if (p.N_total <= 128 && p.top_k <= ROUTE_SMEM_MAX_K)
           routing_epilogue_smem(p, s_bias, s_hist, smem_base + STAGES * RT_STAGE_BYTES,
                                 smem_base + STAGES * RT_STAGE_BYTES + ROUTE_SCRATCH_BYTES, row, tl.row0 / BM, ew, taddr,
@@ -261,10 +262,9 @@ __global__ void __launch_bounds__(KIND == GEMM_RT ? 192 : GEMM_THREADS, 1)
       } else {
         expert_epilogue<KIND>(p, tl.e, row, (TR::WGRAD ? tl.m0 : tl.row0) + ew * 32, tl.n0, taddr, true,
                               TR::WGRAD ? p.M_total - (tl.m0 + ew * 32) : (KIND == GEMM_DX ? static_cast<int>(p.T - tl.row0 - ew * 32) : 32),
-                              es, lane, half, NHALF);
+                              es, lane, half, release);
       }
-      tc_fence_before();
-      mbar_arrive(tempty_bar(acc));
+      if (KIND == GEMM_RT || KIND == GEMM_DWR) release();
     }
     if (p.timers && lane == 0 && ew == 0 && half == 0) {
       atomicAdd(p.timers + 5, static_cast<unsigned long long>(clock64() - t_begin));  // epilogue warp: total
@@ -537,37 +537,55 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
   return MOE_ERR_INVALID_ARG;
 }
 
+// Expected number of `size`-row tiles of an expert when the loads scatter around `mean` like independent picks
+// (variance = mean): sum over j of P(load > j size).
+static double expected_tiles(double mean, double size) {
+  const double sd = sqrt(mean > 1.0 ? mean : 1.0);
+  double n = 0.0;
+  for (int j = 0; j < 4096; ++j) {
+    const double above = 0.5 * erfc((j * size - mean) / (sd * 1.4142135623730951));
+    n += j == 0 ? 1.0 : above;
+    if (j > 0 && above < 1e-3) break;
+  }
+  return n;
+}
+
 // Tile shape per GEMM.  A CTA pair (256 x 256 tile, each CTA staging its rows of A and half of B) moves a third
 // less operand data from L2 per flop than a one-CTA 128 x 256 tile, and the L2 -> SM feed is what limits these
-// kernels: at the Qwen3-30B-A3B shape the pair kernel needs 14 - 18 % fewer cycles per useful flop.  In the
-// power-capped steady state the step is bound by energy rather than cycles and the gain shrinks to 1 - 3 %.
-// Row GEMMs pair two 128-row blocks of ONE expert, so an expert with an odd block count has a block left over.
-// Two ways to deal with it were built and measured in steady state (Qwen shape, ms per step): half-empty pairs
-// (the empty half loads no A rows) 4.17; complete pairs on the pair kernel plus the leftover blocks on one-CTA tiles
-// in a second launch (MOE_FLAG_HYBRID_TILES) 4.22 - the second launch's ramp and ragged last round cost what the
-// empty halves cost; one-CTA tiles throughout 4.39.  Default: half-empty pairs from 512 rows per expert upwards; below
-// that there are few complete pairs and the layer is bound by streaming the weights from HBM anyway.
-// Weight gradients pair along the weight dimension without leftovers, but their K loop is the expert's row count:
-// below ~768 rows per expert the two coupled epilogues bound them and one-CTA tiles are faster.
+// kernels: a 128-row block costs 0.87 of its one-CTA time on the pair kernel.  Row GEMMs pair two 128-row blocks of ONE
+// expert, so an expert with an odd block count pays for a block it does not have.  Whether pairs win therefore
+// oscillates with the rows per expert, and the rule compares the two expected costs.  Measured (d 2048, f 768, 128
+// experts, one-CTA -> pair, us; gate/up, down, dgrad gate/up): 62 rows per expert 164 -> 168, 81 -> 84, 161 -> 161;
+// 200: 200 -> 188, 106 -> 97, 193 -> 175; 312: 261 -> 276, 152 -> 157, 272 -> 296; 437: 331 -> 294, 197 -> 169,
+// 355 -> 320; 512: 372 -> 361, 217 -> 196, 393 -> 389; 1024: 696 -> 659, 407 -> 354, 741 -> 719.  The rule misses by at
+// most 1 % at 62 rows and 375 rows (equal there).
+// The dgrad-down GEMM is held by its epilogue (it reads hg and hu) rather than by the feed and gains less: 151 -> 152 at
+// 200 rows, 242 -> 252 at 512, 284 -> 295 at 625, 455 -> 439 at 1024: pairs from 768 rows on.
+// Half-empty pairs are better than complete pairs plus the leftover blocks in a second, one-CTA launch
+// (MOE_FLAG_HYBRID_TILES: 4.22 ms a step against 4.17 at 1024 rows per expert).
+// Weight gradients pair along the weight dimension without leftovers, but their K loop is the expert's row count, and
+// with few K blocks the output leaves as fast as HBM takes it (a plain fill runs at 3.9 TB/s here) only from one-CTA
+// tiles, whose two CTAs do not have to meet: wgrad-down / wgrad-gate/up 162 -> 172 / 322 -> 330 at 312 rows, equal at
+// 375, 200 -> 187 / 399 -> 374 at 437, 222 -> 195 / 430 -> 392 at 512.
 moe_status launch_grouped_gemm(moe_ctx_impl* ctx, GemmKind kind, int64_t T, const WsLayout& L, char* ws,
                                const GemmIO& io, cudaStream_t st) {
   const bool row_kind = kind == GEMM_F3 || kind == GEMM_F4 || kind == GEMM_B2 || kind == GEMM_B4;
   const bool wgrad_kind = kind == GEMM_B3 || kind == GEMM_B5;
   const double rows_per_expert = static_cast<double>(T) * ctx->s.k / ctx->s.E;
   if (wgrad_kind) {
-    const bool pair = ctx->tile_mode == 1 || ctx->tile_mode == 3 || (ctx->tile_mode == 0 && rows_per_expert >= 768.0);
+    const bool pair = ctx->tile_mode == 1 || ctx->tile_mode == 3 || (ctx->tile_mode == 0 && rows_per_expert >= 384.0);
     return launch_gemm_variant(ctx, kind, T, L, ws, io, st, pair, 0);
   }
   if (!row_kind) return launch_gemm_variant(ctx, kind, T, L, ws, io, st, false, 0);
-  if (ctx->tile_mode == 1) return launch_gemm_variant(ctx, kind, T, L, ws, io, st, true, 0);
-  // dgrad gate/up at short K (2 f / 64 < 64 K blocks per tile) gains from pairs only from 768 rows per expert on
-  // (Qwen3-30B-A3B shape, steady state under the power cap: 453 vs 443 us at 512 rows per expert, 838 vs 875 us at
-  // 1024, 1590 vs 1709 us at 2048)
-  bool long_k = kind != GEMM_B4 || 2 * ctx->s.f / BK >= 64 || rows_per_expert >= 768.0;
-  if (kind == GEMM_B4 && ctx->b4_pair_override >= 0) long_k = ctx->b4_pair_override != 0;
-  if (ctx->tile_mode == 0 && rows_per_expert >= 512.0 && long_k)
-    return launch_gemm_variant(ctx, kind, T, L, ws, io, st, true, 0);
-  if (ctx->tile_mode != 3) return launch_gemm_variant(ctx, kind, T, L, ws, io, st, false, 0);
+  bool pair = ctx->tile_mode == 1;
+  if (ctx->tile_mode == 0) {
+    if (kind == GEMM_B2)
+      pair = rows_per_expert >= 768.0;
+    else
+      pair = 0.87 * 2.0 * expected_tiles(rows_per_expert, 2 * BM) < expected_tiles(rows_per_expert, BM);
+    if (kind == GEMM_B4 && ctx->b4_pair_override >= 0) pair = ctx->b4_pair_override != 0;
+  }
+  if (ctx->tile_mode != 3) return launch_gemm_variant(ctx, kind, T, L, ws, io, st, pair, 0);
   const moe_status rc = launch_gemm_variant(ctx, kind, T, L, ws, io, st, true, 1);
   if (rc != MOE_OK) return rc;
   return launch_gemm_variant(ctx, kind, T, L, ws, io, st, false, 2);

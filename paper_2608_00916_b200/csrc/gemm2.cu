@@ -296,10 +296,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
       tc_fence_after();
       const uint32_t taddr = tmem_base + (static_cast<uint32_t>(ew * 32) << 16) + acc * ACC_COLS;
       expert_epilogue<KIND>(p, tl.e, static_cast<int64_t>(tl.row0) + rin, (TR::WGRAD ? tl.m0 : tl.row0) + ew * 32, tl.n0, taddr,
-                            tl.write, TR::WGRAD ? p.M_total - (tl.m0 + ew * 32) : 32, es, lane, half, 2);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(mapa_shared(tempty_bar(acc), 0));
+                            tl.write, TR::WGRAD ? p.M_total - (tl.m0 + ew * 32) : 32, es, lane, half, [&]() {
+                              tc_fence_before();
+                              __syncwarp();
+                              if (lane == 0) mbar_arrive_cluster(mapa_shared(tempty_bar(acc), 0));
+                            });
     }
     if (p.timers && lane == 0 && ew == 0 && half == 0 && leader) {
       atomicAdd(p.timers + 5, static_cast<unsigned long long>(clock64() - t_begin));
