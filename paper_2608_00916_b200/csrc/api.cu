@@ -9,6 +9,8 @@
 
 namespace moe {
 
+thread_local Chain* Chain::current_ = nullptr;
+
 static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 static std::atomic<long long> g_kernel_launches{0};
@@ -379,6 +381,7 @@ static moe_status forward_impl(bool training, moe_ctx* ctx, int64_t T, const uin
   io.idx_out = topk_idx; io.gates_out = topk_w; io.logits_out = logits_out;
   const bool tc_router = router_on_tensor_cores(s) && logits_in == nullptr;
   if (c->router_fp32 && (lora || !training)) return MOE_ERR_UNSUPPORTED;  // fp32 router weight: moe_forward / moe_backward
+  Chain chain;
   launch_prepare(L, ws, st);  // before any kernel that may record a status
   if (c->router_fp32 && W_r) {
     // W_r points at fp32 values: split them into three exact bf16 terms, kept in the workspace for the backward pass
@@ -510,6 +513,7 @@ static moe_status backward_impl(moe_ctx* ctx, int64_t T, const uint16_t* dy, flo
   io.dW_gate_acc = acc_gate; io.dW_up_acc = acc_up; io.dW_down_acc = acc_down;
   const bool tc_router = router_on_tensor_cores(s);
   if (T > 0) {
+  Chain chain;
     StageTimer tm(c, st, 5);
     launch_gather_rows(s, T, L, ws, dy, reinterpret_cast<uint16_t*>(ws + L.o), st, c->debug_checks != 0);
   }
@@ -525,6 +529,7 @@ static moe_status backward_impl(moe_ctx* ctx, int64_t T, const uint16_t* dy, flo
         return MOE_ERR_CUDA;
       rs = c->s_side;
       forked = true;
+      chain.waits(rs);
     }
     {
       StageTimer tm(c, rs, 10);
@@ -560,6 +565,7 @@ static moe_status backward_impl(moe_ctx* ctx, int64_t T, const uint16_t* dy, flo
         return MOE_ERR_CUDA;
       xs = c->s_side;
     }
+      chain.waits(xs);
     {
       StageTimer tm(c, xs, 12);
       if (tc_router && T > 0) {

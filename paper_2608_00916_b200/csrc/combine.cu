@@ -11,6 +11,8 @@ namespace moe {
 __global__ void __launch_bounds__(256) combine_kernel(int d, int k, const uint16_t* __restrict__ o,
                                                       const float* __restrict__ gates, const int32_t* __restrict__ inv,
                                                       uint16_t* __restrict__ y, int32_t* dbg_status, int64_t rows_max) {
+  chain_wait();
+  chain_next();
   const int64_t t = blockIdx.x;
   __shared__ int sr[MAX_K];
   (void)gates;
@@ -48,8 +50,7 @@ __global__ void __launch_bounds__(256) combine_kernel(int d, int k, const uint16
 void launch_combine(const Shape& s, int64_t T, const uint16_t* o, const float* gates, const int32_t* inv,
                     uint16_t* y, cudaStream_t st, int32_t* dbg_status, int64_t rows_max) {
   if (T == 0) return;
-  combine_kernel<<<static_cast<unsigned>(T), 256, 0, st>>>(s.d, s.k, o, gates, inv, y, dbg_status, rows_max);
-  note_launch();
+  launch_kernel(combine_kernel, static_cast<unsigned>(T), 256, 0, st, s.d, s.k, o, gates, inv, y, dbg_status, rows_max);
 }
 
 // ------------------------------------------------------------------------------------------ router backward
@@ -66,6 +67,8 @@ __global__ void __launch_bounds__(256) router_bwd_kernel(int64_t T, int E, int k
                                                          const int32_t* __restrict__ counts, float d_aux,
                                                          float* __restrict__ dl, uint16_t* __restrict__ dl_hi,
                                                          uint16_t* __restrict__ dl_lo, int32_t* dbg_status) {
+  chain_wait();
+  chain_next();
   const int lane = threadIdx.x & 31;
   const int64_t t = static_cast<int64_t>(blockIdx.x) * 8 + (threadIdx.x >> 5);
   if (t >= T) return;
@@ -157,10 +160,8 @@ void launch_router_bwd(const Shape& s, int64_t T, const float* logits, const int
                        const int32_t* counts, float d_aux, float* dl, uint16_t* dl_hi, uint16_t* dl_lo,
                        cudaStream_t st, int32_t* dbg_status) {
   if (T == 0) return;
-  router_bwd_kernel<<<static_cast<unsigned>((T + 7) / 8), 256, 0, st>>>(T, s.E, s.k, logits, idx, gates, dg_part,
-                                                                        dg_tiles, rows_max, inv, dg, counts, d_aux, dl,
-                                                                        dl_hi, dl_lo, dbg_status);
-  note_launch();
+  launch_kernel(router_bwd_kernel, static_cast<unsigned>((T + 7) / 8), 256, 0, st, T, s.E, s.k, logits, idx, gates,
+                dg_part, dg_tiles, rows_max, inv, dg, counts, d_aux, dl, dl_hi, dl_lo, dbg_status);
 }
 
 // ------------------------------------------------------------------------------------------ dW_r, db_r
@@ -171,6 +172,8 @@ constexpr int DW_BM = 64, DW_BK = 32;
 
 __global__ void __launch_bounds__(256) dwr_partial_kernel(int64_t T, int d, int E, const uint16_t* __restrict__ x,
                                                           const float* __restrict__ dl, float* __restrict__ part) {
+  chain_wait();
+  chain_next();
   // thread layout: 16 (row groups of 4) x 16 (column groups); columns handled: cg + 16*i for i < E/16 (<= 16)
   __shared__ float xs[DW_BK][DW_BM];        // x^T tile
   extern __shared__ float dls[];            // [DW_BK][E]
@@ -229,6 +232,8 @@ __global__ void __launch_bounds__(256) dwr_partial_kernel(int64_t T, int d, int 
 
 __global__ void dwr_reduce_kernel(int64_t n, const float* __restrict__ part, float* __restrict__ dW_r,
                                   int accumulate) {
+  chain_wait();
+  chain_next();
   const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i >= n) return;
   float s = 0.f;
@@ -240,6 +245,8 @@ __global__ void dwr_reduce_kernel(int64_t n, const float* __restrict__ part, flo
 // db_r[e] = sum_t dl[t,e]: one block per 32 experts, 8 warps stride over the tokens, fixed-order final sum.
 __global__ void __launch_bounds__(256) dbr_kernel(int64_t T, int E, const float* __restrict__ dl,
                                                   float* __restrict__ db_r, int accumulate) {
+  chain_wait();
+  chain_next();
   __shared__ float part[8][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int e = blockIdx.x * 32 + lane;
@@ -261,14 +268,12 @@ void launch_dwr(const Shape& s, int64_t T, const uint16_t* x, const float* dl, f
   const int64_t n = static_cast<int64_t>(s.d) * s.E;
   if (!partials_ready) {
     dim3 grid(s.d / DW_BM, DWR_SPLIT);
-    dwr_partial_kernel<<<grid, 256, sizeof(float) * DW_BK * s.E, st>>>(T, s.d, s.E, x, dl, part);
-    note_launch();
+    launch_kernel(dwr_partial_kernel, grid, 256, sizeof(float) * DW_BK * s.E, st, T, s.d, s.E, x, dl, part);
   }
-  dwr_reduce_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, st>>>(n, part, dW_r, accumulate ? 1 : 0);
-  note_launch();
+  launch_kernel(dwr_reduce_kernel, static_cast<unsigned>((n + 255) / 256), 256, 0, st, n, part, dW_r,
+                accumulate ? 1 : 0);
   if (db_r) {
-    dbr_kernel<<<(s.E + 31) / 32, 256, 0, st>>>(T, s.E, dl, db_r, accumulate ? 1 : 0);
-    note_launch();
+    launch_kernel(dbr_kernel, (s.E + 31) / 32, 256, 0, st, T, s.E, dl, db_r, accumulate ? 1 : 0);
   }
 }
 
@@ -283,6 +288,8 @@ __global__ void __launch_bounds__(256) unpermute_bwd_kernel(int64_t T, int d, in
                                                             const float* __restrict__ dl,
                                                             const uint16_t* __restrict__ W_r,
                                                             uint16_t* __restrict__ dx) {
+  chain_wait();
+  chain_next();
   extern __shared__ float ub_dl[];  // [UB_TOK][E]
   __shared__ int s_inv[UB_TOK][MAX_K];
   const int64_t t0 = static_cast<int64_t>(blockIdx.x) * UB_TOK;
@@ -370,6 +377,8 @@ __global__ void __launch_bounds__(256) unpermute_sum_kernel(int d, int k, const 
                                                             const uint16_t* __restrict__ dxr,
                                                             uint16_t* __restrict__ dx, int32_t* dbg_status,
                                                             int64_t rows_max) {
+  chain_wait();
+  chain_next();
   const int64_t t = blockIdx.x;
   __shared__ int sr[MAX_K];
   if (threadIdx.x < k) {
@@ -411,16 +420,15 @@ __global__ void __launch_bounds__(256) unpermute_sum_kernel(int d, int k, const 
 void launch_unpermute_sum(const Shape& s, int64_t T, const uint16_t* dxp, const int32_t* inv, const uint16_t* dxr,
                           uint16_t* dx, cudaStream_t st, int32_t* dbg_status, int64_t rows_max) {
   if (T == 0) return;
-  unpermute_sum_kernel<<<static_cast<unsigned>(T), 256, 0, st>>>(s.d, s.k, dxp, inv, dxr, dx, dbg_status, rows_max);
-  note_launch();
+  launch_kernel(unpermute_sum_kernel, static_cast<unsigned>(T), 256, 0, st, s.d, s.k, dxp, inv, dxr, dx, dbg_status,
+                rows_max);
 }
 
 void launch_unpermute_bwd(const Shape& s, int64_t T, const uint16_t* dxp, const int32_t* inv, const float* dl,
                           const uint16_t* W_r, uint16_t* dx, cudaStream_t st) {
   if (T == 0) return;
-  unpermute_bwd_kernel<<<static_cast<unsigned>((T + UB_TOK - 1) / UB_TOK), 256, sizeof(float) * UB_TOK * s.E, st>>>(
-      T, s.d, s.E, s.k, dxp, inv, dl, W_r, dx);
-  note_launch();
+  launch_kernel(unpermute_bwd_kernel, static_cast<unsigned>((T + UB_TOK - 1) / UB_TOK), 256,
+                sizeof(float) * UB_TOK * s.E, st, T, s.d, s.E, s.k, dxp, inv, dl, W_r, dx);
 }
 
 }  // namespace moe

@@ -43,12 +43,6 @@ __global__ void __launch_bounds__(KIND == GEMM_RT ? 192 : GEMM_THREADS, 1)
   __shared__ uint32_t tmem_base_slot;
   __shared__ float s_bias[KIND == GEMM_RT ? MAX_E : 1];  // router bias (zero beyond E)
   __shared__ int s_hist[KIND == GEMM_RT ? 128 : 1];      // picks per expert of the tile (routing epilogue for E <= 128)
-  if (KIND == GEMM_RT)
-    for (int i = threadIdx.x; i < MAX_E; i += blockDim.x) {
-      s_bias[i] = (p.bias && i < p.N_total) ? p.bias[i] : 0.f;
-      if (i < 128) s_hist[i] = 0;
-    }
-
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t smem_base = (smem_u32(gemm_smem_raw) + 1023u) & ~1023u;
   const uint32_t stage_stride = (KIND == GEMM_RT && p.b_chunks <= 2) ? RT_STAGE_BYTES : STAGE_BYTES;
@@ -76,6 +70,12 @@ __global__ void __launch_bounds__(KIND == GEMM_RT ? 192 : GEMM_THREADS, 1)
     tmem_alloc(smem_u32(&tmem_base_slot), TMEM_COLS);
     tmem_relinquish();
   }
+  chain_wait();  // everything above touches only this CTA's own state
+  if (KIND == GEMM_RT)
+    for (int i = threadIdx.x; i < MAX_E; i += blockDim.x) {
+      s_bias[i] = (p.bias && i < p.N_total) ? p.bias[i] : 0.f;
+      if (i < 128) s_hist[i] = 0;
+    }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -108,6 +108,7 @@ __global__ void __launch_bounds__(KIND == GEMM_RT ? 192 : GEMM_THREADS, 1)
         __syncwarp();
       }
     }
+    chain_next();  // not earlier: blocks of the next kernel that only wait would sit beside the main loop
     if (p.timers && lane == 0) {
       atomicAdd(p.timers + 0, static_cast<unsigned long long>(clock64() - t_begin));  // producer: total
       atomicAdd(p.timers + 1, static_cast<unsigned long long>(t_wait));               // producer: waiting for a free stage
@@ -321,9 +322,10 @@ static moe_status launch_kind(moe_ctx_impl* ctx, const GemmParams& p, cudaStream
       return MOE_ERR_CUDA;
     ctx->attr_done[0][KIND] = 1;
   }
-  grouped_gemm_kernel<KIND><<<ctx->sm_count, KIND == GEMM_RT ? 192 : GEMM_THREADS, GEMM_SMEM, st>>>(p);
-  note_launch();
-  return cudaGetLastError() == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
+  return launch_kernel(grouped_gemm_kernel<KIND>, ctx->sm_count, KIND == GEMM_RT ? 192 : GEMM_THREADS, GEMM_SMEM, st,
+                       p) == cudaSuccess
+             ? MOE_OK
+             : MOE_ERR_CUDA;
 }
 
 // Row tiles (or pairs) walked together inside a column tile: 1 while the expert's weights are few column tiles wide (they

@@ -150,6 +150,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
   tc_fence_before();
   cluster_sync_all();  // barriers of both CTAs are initialised before anyone signals across the pair
   tc_fence_after();
+  chain_wait();  // everything above touches only this CTA's own state
   const uint32_t tmem_base = tmem_base_slot;
   const int ntiles = total_tiles2<KIND>(p);
   const int cid = blockIdx.x >> 1, nclusters = gridDim.x >> 1;
@@ -183,6 +184,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
     if (p.timers && lane == 0 && leader) {
       atomicAdd(p.timers + 0, static_cast<unsigned long long>(clock64() - t_begin));
       atomicAdd(p.timers + 1, static_cast<unsigned long long>(t_wait));
+    chain_next();
     }
     if (!ok) {
       // gave up: the leader waits (bounded) for the copies of BOTH CTAs that were already issued - they are all credited
@@ -329,9 +331,9 @@ static moe_status launch_pair_kind(moe_ctx_impl* ctx, const GemmParams& p, cudaS
     ctx->attr_done[1][KIND] = 1;
   }
   const int grid = ctx->sm_count & ~1;  // whole pairs
-  grouped_gemm_pair_kernel<KIND><<<grid, GEMM2_THREADS, GEMM2_SMEM, st>>>(p);
-  note_launch();
-  return cudaGetLastError() == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
+  return launch_kernel(grouped_gemm_pair_kernel<KIND>, grid, GEMM2_THREADS, GEMM2_SMEM, st, p) == cudaSuccess
+             ? MOE_OK
+             : MOE_ERR_CUDA;
 }
 
 moe_status launch_pair_gemm(moe_ctx_impl* ctx, GemmKind kind, const GemmParams& p, cudaStream_t st) {

@@ -23,6 +23,8 @@ __global__ void __launch_bounds__(256) router_kernel(int64_t T, int d, int E, in
                                                      int32_t* __restrict__ idx, float* __restrict__ gates,
                                                      int32_t* __restrict__ idx_out, float* __restrict__ gates_out,
                                                      float* __restrict__ logits_out, float* __restrict__ psum_part) {
+  chain_wait();
+  chain_next();
   extern __shared__ __align__(16) unsigned char rt_smem[];
   float* xs = reinterpret_cast<float*>(rt_smem);           // [RT_CH][ROUTER_TOK]
   float* ls = xs + RT_CH * ROUTER_TOK;                     // [ROUTER_TOK][E]
@@ -194,9 +196,8 @@ void launch_router(const Shape& s, int64_t T, const uint16_t* x, const uint16_t*
   if (T == 0) return;
   const int blocks = static_cast<int>((T + ROUTER_TOK - 1) / ROUTER_TOK);
   const size_t smem = sizeof(float) * (RT_CH * ROUTER_TOK + ROUTER_TOK * s.E + 8 * s.E);
-  router_kernel<<<blocks, 256, smem, st>>>(T, s.d, s.E, s.k, x, W_r, b_r, logits_in, logits, idx, gates, idx_out,
-                                           gates_out, logits_out, psum_part);
-  note_launch();
+  launch_kernel(router_kernel, blocks, 256, smem, st, T, s.d, s.E, s.k, x, W_r, b_r, logits_in, logits, idx, gates,
+                idx_out, gates_out, logits_out, psum_part);
 }
 
 // ------------------------------------------------------------------------------------------ permutation
@@ -221,6 +222,8 @@ __device__ __forceinline__ void build_masks(uint32_t* masks /* [TOK_WARPS][E] */
 
 __global__ void __launch_bounds__(TOK_TILE) hist_kernel(int64_t T, int E, int k, const int32_t* __restrict__ idx,
                                                         int32_t* __restrict__ tile_counts) {
+  chain_wait();
+  chain_next();
   extern __shared__ uint32_t hist_masks[];
   build_masks(hist_masks, idx, T, E, k, static_cast<int64_t>(blockIdx.x) * TOK_TILE);
   for (int e = threadIdx.x; e < E; e += TOK_TILE) {
@@ -240,6 +243,8 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_kernel(int64_t T, int E, in
                                                             const float* __restrict__ psum_part,
                                                             float* __restrict__ psum, int32_t* __restrict__ counts_out,
                                                             float* __restrict__ aux_out) {
+  chain_wait();
+  chain_next();
   __shared__ int s_cnt[MAX_E];
   __shared__ TableScratch s_tab;
   __shared__ float s_term[MAX_E];
@@ -338,6 +343,8 @@ __global__ void __launch_bounds__(TOK_TILE) scatter_kernel(int64_t T, int E, int
                                                            float* __restrict__ row_gate,
                                                            int32_t* __restrict__ perm_out, int32_t* dbg_status,
                                                            int64_t rows_max) {
+  chain_wait();
+  chain_next();
   extern __shared__ uint32_t sc_masks[];
   const int64_t tile_t0 = static_cast<int64_t>(blockIdx.x) * TOK_TILE;
   build_masks(sc_masks, idx, T, E, k, tile_t0);
@@ -376,6 +383,8 @@ __global__ void __launch_bounds__(256) scatter_rows_kernel(int64_t T, int d, int
                                                            const int32_t* __restrict__ pad_offsets,
                                                            uint16_t* __restrict__ rows, int32_t* dbg_status,
                                                            int64_t rows_max) {
+  chain_wait();
+  chain_next();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int n16 = d / 8;
   if (static_cast<int>(blockIdx.x) >= tok_blocks) {
@@ -411,11 +420,10 @@ __global__ void __launch_bounds__(256) scatter_rows_kernel(int64_t T, int d, int
 void launch_gather_rows(const Shape& s, int64_t T, const WsLayout& L, const char* ws, const uint16_t* src,
                         uint16_t* rows, cudaStream_t st, bool debug) {
   const int tok_blocks = static_cast<int>((T + 7) / 8);
-  scatter_rows_kernel<<<tok_blocks + s.E, 256, 0, st>>>(
-      T, s.d, s.k, s.E, tok_blocks, src, reinterpret_cast<const int32_t*>(ws + L.inv),
+  launch_kernel(
+      scatter_rows_kernel, tok_blocks + s.E, 256, 0, st, T, s.d, s.k, s.E, tok_blocks, src, reinterpret_cast<const int32_t*>(ws + L.inv),
       reinterpret_cast<const int32_t*>(ws + L.counts), reinterpret_cast<const int32_t*>(ws + L.pad_offsets), rows,
       debug ? reinterpret_cast<int32_t*>(const_cast<char*>(ws) + L.status) : nullptr, L.rows_max);
-  note_launch();
 }
 
 // First kernel of every forward call: clears the row gates (pad rows must read 0) and makes sure the workspace's status
@@ -423,6 +431,8 @@ void launch_gather_rows(const Shape& s, int64_t T, const WsLayout& L, const char
 // earlier call stays visible until the host has reported it; memory seen for the first time gets a clean block.
 __global__ void __launch_bounds__(256) prepare_kernel(int32_t* __restrict__ status, float* __restrict__ row_gate,
                                                       int64_t rows) {
+  chain_wait();
+  chain_next();
   if (blockIdx.x == 0 && threadIdx.x == 0 && (status[2] != STATUS_COOKIE0 || status[3] != STATUS_COOKIE1)) {
     status[0] = DEV_OK;
     status[1] = 0;
@@ -435,9 +445,8 @@ __global__ void __launch_bounds__(256) prepare_kernel(int32_t* __restrict__ stat
 
 void launch_prepare(const WsLayout& L, char* ws, cudaStream_t st) {
   const int blocks = static_cast<int>(std::min<int64_t>(296, std::max<int64_t>(1, (L.rows_alloc + 255) / 256)));
-  prepare_kernel<<<blocks, 256, 0, st>>>(reinterpret_cast<int32_t*>(ws + L.status),
-                                         reinterpret_cast<float*>(ws + L.row_gate), L.rows_alloc);
-  note_launch();
+  launch_kernel(prepare_kernel, blocks, 256, 0, st, reinterpret_cast<int32_t*>(ws + L.status),
+                reinterpret_cast<float*>(ws + L.row_gate), L.rows_alloc);
 }
 
 // tables_only: stop after the histogram and the scan (per-tile prefixes, counts, tables, aux loss); the expert-parallel
@@ -447,6 +456,8 @@ void launch_prepare(const WsLayout& L, char* ws, cudaStream_t st) {
 __global__ void __launch_bounds__(256) split_fp32_kernel(const float* __restrict__ w, uint16_t* __restrict__ hi,
                                                          uint16_t* __restrict__ mid, uint16_t* __restrict__ lo,
                                                          int64_t n) {
+  chain_wait();
+  chain_next();
   const int64_t i = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x;
   if (i >= n) return;
   const float v = w[i];
@@ -461,8 +472,7 @@ __global__ void __launch_bounds__(256) split_fp32_kernel(const float* __restrict
 
 void launch_split_fp32(const float* w, uint16_t* hi, uint16_t* mid, uint16_t* lo, int64_t n, cudaStream_t st) {
   if (n == 0) return;
-  split_fp32_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, st>>>(w, hi, mid, lo, n);
-  note_launch();
+  launch_kernel(split_fp32_kernel, static_cast<unsigned>((n + 255) / 256), 256, 0, st, w, hi, mid, lo, n);
 }
 
 void launch_permute(const Shape& s, int64_t T, const WsLayout& L, char* ws, const uint16_t* x, int32_t* counts_out,
@@ -473,20 +483,17 @@ void launch_permute(const Shape& s, int64_t T, const WsLayout& L, char* ws, cons
   const int tiles = static_cast<int>(L.tok_tiles);
   const size_t msm = sizeof(uint32_t) * TOK_WARPS * s.E;
   if (tiles > 0 && !histogram_done) {
-    hist_kernel<<<tiles, TOK_TILE, msm, st>>>(T, s.E, s.k, idx, tile_counts);
-    note_launch();
+    launch_kernel(hist_kernel, tiles, TOK_TILE, msm, st, T, s.E, s.k, idx, tile_counts);
   }
-  scan_kernel<<<1, SCAN_THREADS, 0, st>>>(T, s.E, s.k, tiles, psum_rows, tile_counts, table_pointers(L, ws),
-                                 reinterpret_cast<const float*>(ws + L.psum_part),
-                                 reinterpret_cast<float*>(ws + L.psum), counts_out, aux_out);
-  note_launch();
+  launch_kernel(scan_kernel, 1, SCAN_THREADS, 0, st, T, s.E, s.k, tiles, psum_rows, tile_counts,
+                table_pointers(L, ws), reinterpret_cast<const float*>(ws + L.psum_part),
+                reinterpret_cast<float*>(ws + L.psum), counts_out, aux_out);
   if (tiles > 0 && !tables_only) {
-    scatter_kernel<<<tiles, TOK_TILE, msm, st>>>(
-        T, s.E, s.k, idx, tile_counts, reinterpret_cast<const int32_t*>(ws + L.offsets),
+    launch_kernel(
+        scatter_kernel, tiles, TOK_TILE, msm, st, T, s.E, s.k, idx, tile_counts, reinterpret_cast<const int32_t*>(ws + L.offsets),
         reinterpret_cast<const int32_t*>(ws + L.pad_offsets), reinterpret_cast<const float*>(ws + L.gates),
         reinterpret_cast<int32_t*>(ws + L.inv), reinterpret_cast<float*>(ws + L.row_gate), perm_out,
         debug ? reinterpret_cast<int32_t*>(ws + L.status) : nullptr, L.rows_max);
-    note_launch();
     launch_gather_rows(s, T, L, ws, x, reinterpret_cast<uint16_t*>(ws + L.xp), st, debug);
   }
 }
