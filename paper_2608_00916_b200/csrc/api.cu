@@ -512,8 +512,8 @@ static moe_status backward_impl(moe_ctx* ctx, int64_t T, const uint16_t* dy, flo
   io.dW_gate = dW_gate; io.dW_up = dW_up; io.dW_down = dW_down; io.dx = dx;
   io.dW_gate_acc = acc_gate; io.dW_up_acc = acc_up; io.dW_down_acc = acc_down;
   const bool tc_router = router_on_tensor_cores(s);
-  if (T > 0) {
   Chain chain;
+  if (T > 0) {
     StageTimer tm(c, st, 5);
     launch_gather_rows(s, T, L, ws, dy, reinterpret_cast<uint16_t*>(ws + L.o), st, c->debug_checks != 0);
   }
@@ -528,8 +528,8 @@ static moe_status backward_impl(moe_ctx* ctx, int64_t T, const uint16_t* dy, flo
       if (cudaEventRecord(c->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(c->s_side, c->ev_fork, 0) != cudaSuccess)
         return MOE_ERR_CUDA;
       rs = c->s_side;
-      forked = true;
       chain.waits(rs);
+      forked = true;
     }
     {
       StageTimer tm(c, rs, 10);
@@ -564,8 +564,8 @@ static moe_status backward_impl(moe_ctx* ctx, int64_t T, const uint16_t* dy, flo
       if (cudaEventRecord(c->ev_b4, st) != cudaSuccess || cudaStreamWaitEvent(c->s_side, c->ev_b4, 0) != cudaSuccess)
         return MOE_ERR_CUDA;
       xs = c->s_side;
-    }
       chain.waits(xs);
+    }
     {
       StageTimer tm(c, xs, 12);
       if (tc_router && T > 0) {

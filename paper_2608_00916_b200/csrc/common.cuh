@@ -251,7 +251,6 @@ inline int64_t router_psum_rows(const Shape& s, int64_t T, bool logits_given) {
 // counts kernel launches of the library (process-wide; read through moe_kernel_launches)
 void note_launch(int n = 1);
 
-// ---- device helpers
 // The kernels of one call, in order, on the caller's stream and on the context's second one.  A kernel that directly
 // follows another one of the same call on its stream is launched chained (programmatic stream serialization): it is set
 // up while its predecessor drains, and chain_wait(), called by every such kernel before its first access to global
@@ -312,11 +311,12 @@ inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, si
   return rc;
 }
 
-// Records a device-side failure.  The first failure sticks: later ones do not overwrite it, and no kernel ever resets
+// ---- device helpers
 // Waits for the previous kernel of the chain (a no-op in a kernel launched plainly).
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Lets the next kernel of the chain be set up once every block of this one has got here or ended.
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Records a device-side failure.  The first failure sticks: later ones do not overwrite it, and no kernel ever resets
 // the word (the host acknowledges it after reporting it, see moe_poll_status).
 __device__ __forceinline__ void record_status(int32_t* status, int code, int where) {
   if (atomicCAS(status, DEV_OK, code) == DEV_OK) status[1] = where;

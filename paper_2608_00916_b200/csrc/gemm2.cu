@@ -147,10 +147,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
     tmem_alloc_pair(smem_u32(&tmem_base_slot), TMEM_COLS);
     tmem_relinquish_pair();
   }
+  chain_wait();  // everything above touches only this CTA's own state
   tc_fence_before();
   cluster_sync_all();  // barriers of both CTAs are initialised before anyone signals across the pair
   tc_fence_after();
-  chain_wait();  // everything above touches only this CTA's own state
   const uint32_t tmem_base = tmem_base_slot;
   const int ntiles = total_tiles2<KIND>(p);
   const int cid = blockIdx.x >> 1, nclusters = gridDim.x >> 1;
@@ -181,10 +181,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
         __syncwarp();
       }
     }
+    chain_next();
     if (p.timers && lane == 0 && leader) {
       atomicAdd(p.timers + 0, static_cast<unsigned long long>(clock64() - t_begin));
       atomicAdd(p.timers + 1, static_cast<unsigned long long>(t_wait));
-    chain_next();
     }
     if (!ok) {
       // gave up: the leader waits (bounded) for the copies of BOTH CTAs that were already issued - they are all credited
