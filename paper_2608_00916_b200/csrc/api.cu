@@ -407,7 +407,8 @@ static moe_status forward_impl(bool training, moe_ctx* ctx, int64_t T, const uin
     StageTimer tm(c, st, 1);
     launch_permute(s, T, L, ws, x, expert_counts, perm, aux_loss,
                    static_cast<int>(router_psum_rows(s, T, logits_in != nullptr)), st, /*tables_only=*/false,
-                   /*histogram_done=*/tc_router && T > 0 && router_writes_histogram(s), c->debug_checks != 0);
+                   /*histogram_done=*/tc_router && T > 0 && router_writes_histogram(s), c->debug_checks != 0,
+                   /*clear_pads=*/training);
   }
   if (T > 0) {
     {

@@ -160,7 +160,7 @@ void launch_router(const Shape& s, int64_t T, const uint16_t* x, const uint16_t*
                    float* gates_out, float* logits_out, float* psum_part, cudaStream_t st);
 void launch_permute(const Shape& s, int64_t T, const WsLayout& L, char* ws, const uint16_t* x, int32_t* counts_out,
                     int32_t* perm_out, float* aux_out, int psum_rows, cudaStream_t st, bool tables_only = false,
-                    bool histogram_done = false, bool debug = false);
+                    bool histogram_done = false, bool debug = false, bool clear_pads = true);
 // fp32 [n] -> three bf16 terms hi, mid, lo with hi + mid + lo == w exactly (route.cu)
 void launch_split_fp32(const float* w, uint16_t* hi, uint16_t* mid, uint16_t* lo, int64_t n, cudaStream_t st);
 // ---- launchers (combine.cu)
@@ -168,9 +168,10 @@ void launch_split_fp32(const float* w, uint16_t* hi, uint16_t* mid, uint16_t* lo
 // it is about to use, records DEV_BOUNDS and skips or redirects the access instead of touching memory out of range
 void launch_combine(const Shape& s, int64_t T, const uint16_t* o, const float* gates, const int32_t* inv,
                     uint16_t* y, cudaStream_t st, int32_t* dbg_status = nullptr, int64_t rows_max = 0);
-// rows[inv[t,j],:] = src[t,:] for every (token, slot), pad rows zeroed: xp from x, and the dy rows of backward
+// rows[inv[t,j],:] = src[t,:] for every (token, slot): xp from x, and the dy rows of backward.  clear_pads: pad rows are
+// zeroed (the weight gradients read them; a forward-only call never does)
 void launch_gather_rows(const Shape& s, int64_t T, const WsLayout& L, const char* ws, const uint16_t* src,
-                        uint16_t* rows, cudaStream_t st, bool debug = false);
+                        uint16_t* rows, cudaStream_t st, bool debug = false, bool clear_pads = true);
 // dg[t,j] = sum over column tiles of dg_part[tile][inv[t,j]], then dl (fp32 and the two-term bf16 split)
 void launch_router_bwd(const Shape& s, int64_t T, const float* logits, const int32_t* idx, const float* gates,
                        const float* dg_part, int dg_tiles, int64_t rows_max, const int32_t* inv, float* dg,

@@ -262,7 +262,10 @@ __global__ void __launch_bounds__(KIND == GEMM_RT ? 192 : GEMM_THREADS, 1)
         }
       } else {
         expert_epilogue<KIND>(p, tl.e, row, (TR::WGRAD ? tl.m0 : tl.row0) + ew * 32, tl.n0, taddr, true,
-                              TR::WGRAD ? p.M_total - (tl.m0 + ew * 32) : (KIND == GEMM_DX ? static_cast<int>(p.T - tl.row0 - ew * 32) : 32),
+                              TR::WGRAD          ? p.M_total - (tl.m0 + ew * 32)
+                              : KIND == GEMM_DX ? static_cast<int>(p.T - tl.row0 - ew * 32)
+                              : p.clip_rows     ? tl.valid - ew * 32
+                                                : 32,
                               es, lane, half, release);
       }
       if (KIND == GEMM_RT || KIND == GEMM_DWR) release();
@@ -336,6 +339,16 @@ static int row_group_for(int n_tiles, const moe_ctx_impl* ctx) {
   return n_tiles > 12 ? 16 : 1;
 }
 
+// Forward-only calls leave pad rows alone (nothing reads them afterwards), which at few rows per expert is most of what
+// the activations move: scoring 241 tokens (15 rows per expert) 296 -> 268 us, 2048 tokens 367 -> 356 us.  Below 192
+// rows per expert most tiles are partial as well, and A comes in groups of 32 rows of which the empty ones are not read:
+// 268 -> 263 us and 356 -> 354 us.  Above, the extra copy instructions cost more than the reads they save (with them at
+// 1024 rows per expert 1437 -> 1557 us).
+static void clip_pads(GemmParams* p, bool forward_only, double rows_per_expert) {
+  p->clip_rows = forward_only ? 1 : 0;
+  p->part_rows = forward_only && rows_per_expert < 192.0 ? 1 : 0;
+}
+
 // One launch of an expert / router contraction.  `pair`: CTA-pair kernel.  `part`: 0 = the whole tile list; row GEMMs
 // of the mixed schedule: 1 = the pair kernel over complete pairs of row blocks only, 2 = the one-CTA kernel over the
 // leftover blocks.
@@ -346,6 +359,7 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
   const Shape& s = ctx->s;
   const int d = s.d, f = s.f, E = s.E;
   const int64_t R = L.rows_max;
+  const double rows_per_expert = static_cast<double>(T) * s.k / E;
   void* fn = ctx->encode_fn;
   uint16_t* xp = reinterpret_cast<uint16_t*>(ws + L.xp);
   uint16_t* hg = reinterpret_cast<uint16_t*>(ws + L.hg);
@@ -388,9 +402,10 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
   bool ok = true;
   switch (kind) {
     case GEMM_F3:
-      ok = map_2d(fn, &p.mapA0, xp, R, d, 128) && map_3d(fn, &p.mapB0, W_gate, E, d, f, 64) &&
-           map_3d(fn, &p.mapB1, W_up, E, d, f, 64);
+      ok = map_2d(fn, &p.mapA0, xp, R, d, 128) && map_2d(fn, &p.mapS0, xp, R, d, 32) &&
+           map_3d(fn, &p.mapB0, W_gate, E, d, f, 64) && map_3d(fn, &p.mapB1, W_up, E, d, f, 64);
       p.mapA1 = p.mapA0;
+      clip_pads(&p, !io.save_preactivations, rows_per_expert);
       p.n_tiles = (f + 127) / 128;
       p.k_blocks = d / BK;
       p.N_total = f;
@@ -402,8 +417,10 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
       p.row_group = row_group_for(p.n_tiles, ctx);
       return pair ? launch_pair_gemm(ctx, kind, p, st) : launch_kind<GEMM_F3>(ctx, p, st);
     case GEMM_F4:
-      ok = map_2d(fn, &p.mapA0, act, R, f, 128) && map_3d(fn, &p.mapB0, W_down, E, f, d, 64);
+      ok = map_2d(fn, &p.mapA0, act, R, f, 128) && map_2d(fn, &p.mapS0, act, R, f, 32) &&
+           map_3d(fn, &p.mapB0, W_down, E, f, d, 64);
       p.mapA1 = p.mapA0; p.mapB1 = p.mapB0;
+      clip_pads(&p, !io.save_preactivations, rows_per_expert);
       p.n_tiles = (d + 255) / 256;
       p.k_blocks = f / BK;
       p.N_total = d;

@@ -31,6 +31,7 @@ constexpr size_t GEMM2_SMEM = static_cast<size_t>(STAGES2) * STAGE2_BYTES + EPI_
 struct Tile2 {
   int e, row0, m0, n0, nkb;
   int klast;    // K = 16 steps issued in the last K block
+  int valid;    // row GEMMs: rows of this CTA's 128 that exist (clip_rows: that are routed rows)
   bool write;   // this CTA's 128 rows exist (false: the empty half of an odd expert's last pair)
   bool full;    // both halves of the pair exist
 };
@@ -55,6 +56,7 @@ __device__ __forceinline__ Tile2 get_tile2(const GemmParams& p, int t, int rank)
     tl.row0 = p.pad_offsets[tl.e];
     tl.nkb = (p.counts[tl.e] + BK - 1) / BK;  // the rest of the 128-row padding is zeros
     tl.klast = last_k_steps(p.counts[tl.e]);
+    tl.valid = BM;
     tl.write = true;
     tl.full = true;
   } else {
@@ -64,6 +66,7 @@ __device__ __forceinline__ Tile2 get_tile2(const GemmParams& p, int t, int rank)
     tl.e = info.x;
     tl.row0 = info.y + rank * BM;
     tl.write = rank < info.z;
+    tl.valid = !tl.write ? 0 : p.clip_rows ? rows_in_tile(p, tl.e, tl.row0) : BM;
     tl.full = info.z == 2;
     tl.m0 = 0;
     tl.n0 = nt * Traits<KIND>::N_SPAN;
@@ -77,12 +80,12 @@ template <int KIND>
 __device__ __forceinline__ void issue_loads2(const GemmParams& p, const Tile2& tl, int kb, int rank, uint32_t sA,
                                              uint32_t sB, uint32_t bar) {
   if (KIND == GEMM_F3) {
-    tma_load_2d_pair(sA, &p.mapA0, bar, kb * BK, tl.write ? tl.row0 : p.oob_row);
+    load_a_rows<true>(p, sA, bar, kb * BK, tl.row0, tl.valid);
     const CUtensorMap* mb = rank ? &p.mapB1 : &p.mapB0;  // leader: gate columns, partner: the matching up columns
 #pragma unroll
     for (int c = 0; c < 2; ++c) tma_load_3d_pair(sB + c * CHUNK_BYTES, mb, bar, tl.n0 + c * 64, kb * BK, tl.e);
   } else if (KIND == GEMM_F4) {
-    tma_load_2d_pair(sA, &p.mapA0, bar, kb * BK, tl.write ? tl.row0 : p.oob_row);
+    load_a_rows<true>(p, sA, bar, kb * BK, tl.row0, tl.valid);
 #pragma unroll
     for (int c = 0; c < 2; ++c)
       tma_load_3d_pair(sB + c * CHUNK_BYTES, &p.mapB0, bar, tl.n0 + rank * 128 + c * 64, kb * BK, tl.e);
@@ -298,7 +301,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
       tc_fence_after();
       const uint32_t taddr = tmem_base + (static_cast<uint32_t>(ew * 32) << 16) + acc * ACC_COLS;
       expert_epilogue<KIND>(p, tl.e, static_cast<int64_t>(tl.row0) + rin, (TR::WGRAD ? tl.m0 : tl.row0) + ew * 32, tl.n0, taddr,
-                            tl.write, TR::WGRAD ? p.M_total - (tl.m0 + ew * 32) : 32, es, lane, half, [&]() {
+                            tl.write, TR::WGRAD ? p.M_total - (tl.m0 + ew * 32) : p.clip_rows ? tl.valid - ew * 32 : 32, es,
+                            lane, half, [&]() {
                               tc_fence_before();
                               __syncwarp();
                               if (lane == 0) mbar_arrive_cluster(mapa_shared(tempty_bar(acc), 0));

@@ -418,10 +418,10 @@ __global__ void __launch_bounds__(256) scatter_rows_kernel(int64_t T, int d, int
 }
 
 void launch_gather_rows(const Shape& s, int64_t T, const WsLayout& L, const char* ws, const uint16_t* src,
-                        uint16_t* rows, cudaStream_t st, bool debug) {
+                        uint16_t* rows, cudaStream_t st, bool debug, bool clear_pads) {
   const int tok_blocks = static_cast<int>((T + 7) / 8);
   launch_kernel(
-      scatter_rows_kernel, tok_blocks + s.E, 256, 0, st, T, s.d, s.k, s.E, tok_blocks, src, reinterpret_cast<const int32_t*>(ws + L.inv),
+      scatter_rows_kernel, tok_blocks + (clear_pads ? s.E : 0), 256, 0, st, T, s.d, s.k, s.E, tok_blocks, src, reinterpret_cast<const int32_t*>(ws + L.inv),
       reinterpret_cast<const int32_t*>(ws + L.counts), reinterpret_cast<const int32_t*>(ws + L.pad_offsets), rows,
       debug ? reinterpret_cast<int32_t*>(const_cast<char*>(ws) + L.status) : nullptr, L.rows_max);
 }
@@ -477,7 +477,7 @@ void launch_split_fp32(const float* w, uint16_t* hi, uint16_t* mid, uint16_t* lo
 
 void launch_permute(const Shape& s, int64_t T, const WsLayout& L, char* ws, const uint16_t* x, int32_t* counts_out,
                     int32_t* perm_out, float* aux_out, int psum_rows, cudaStream_t st, bool tables_only,
-                    bool histogram_done, bool debug) {
+                    bool histogram_done, bool debug, bool clear_pads) {
   int32_t* idx = reinterpret_cast<int32_t*>(ws + L.idx);
   int32_t* tile_counts = reinterpret_cast<int32_t*>(ws + L.tile_counts);
   const int tiles = static_cast<int>(L.tok_tiles);
@@ -494,7 +494,7 @@ void launch_permute(const Shape& s, int64_t T, const WsLayout& L, char* ws, cons
         reinterpret_cast<const int32_t*>(ws + L.pad_offsets), reinterpret_cast<const float*>(ws + L.gates),
         reinterpret_cast<int32_t*>(ws + L.inv), reinterpret_cast<float*>(ws + L.row_gate), perm_out,
         debug ? reinterpret_cast<int32_t*>(ws + L.status) : nullptr, L.rows_max);
-    launch_gather_rows(s, T, L, ws, x, reinterpret_cast<uint16_t*>(ws + L.xp), st, debug);
+    launch_gather_rows(s, T, L, ws, x, reinterpret_cast<uint16_t*>(ws + L.xp), st, debug, clear_pads);
   }
 }
 

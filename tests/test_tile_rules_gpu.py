@@ -1,6 +1,7 @@
 """Stage-by-stage parity at the sizes where the choice of tile shape changes and where a staging unit of the GEMM
 epilogues (32 rows x 64 columns) is only partly inside the output."""
 import pytest
+import torch
 
 from paper_2608_00916_b200 import synth
 from gpu_util import Run, oracle_run
@@ -21,3 +22,25 @@ def test_tile_shape_boundaries(T, d, E, k, f, seed):
     inp = synth.make_inputs(synth.MoEShape(T, d, E, k, f), seed, x_std=1.0)
     ofw, obw = oracle_run(inp, k, 0.05)
     check_all(Run(inp, k), ofw, obw, 0.05)
+
+
+@pytest.mark.parametrize("T,d,E,k,f,seed,flags", [
+    (5, 64, 16, 2, 64, 81, 0),       # experts with one row or none
+    (150, 192, 16, 2, 320, 82, 0),   # about 19 rows: one group of 32 per tile
+    (1030, 128, 16, 2, 192, 83, 1),  # about 129 rows on pairs: the second half empty or nearly so
+    (770, 256, 16, 2, 256, 84, 2),   # about 96 rows: the last group of 32 just used or just not
+    (2000, 128, 8, 2, 128, 85, 0),   # about 500 rows
+])
+def test_scoring_never_uses_pad_rows(T, d, E, k, f, seed, flags):
+    """A forward-only call neither clears nor stores the pad rows of its buffers: with a workspace full of NaN bit
+    patterns its result is bitwise that of the training forward, which does."""
+    inp = synth.make_inputs(synth.MoEShape(T, d, E, k, f), seed, x_std=1.0)
+    train = Run(inp, k, flags=flags).forward()
+    r = Run(inp, k, flags=flags)
+    v = r.dev
+    r.layer._ensure_ws(T, inference=True)
+    r.layer.ws.fill_(0xFF)
+    got = r.layer.forward(v["x"], v["W_r"], v["W_gate"], v["W_up"], v["W_down"], inference=True)
+    r.layer.poll()
+    assert torch.equal(got["y"], train["y"])
+    assert torch.isfinite(got["y"].float()).all()
