@@ -82,109 +82,100 @@ __global__ void __launch_bounds__(KIND == GEMM_RT ? 192 : GEMM_THREADS, 1)
   const uint32_t tmem_base = tmem_base_slot;
   const int ntiles = total_tiles<KIND>(p);
 
+  // The producer and the MMA issuer are one thread each.  What they do per K block (a wait, a few copies or four MMAs, a
+  // commit) has to fit well inside the 512 cycles that the tensor core needs for it; run by a whole warp with one lane
+  // enabled, with a division for the stage index, it took 400 - 700 cycles and set the pace of every kernel here.
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    uint32_t it = 0;
-    bool ok = true;
-    long long t_wait = 0, t_begin = clock64();
-    for (int rd = 0; rd * static_cast<int>(gridDim.x) < ntiles && ok; ++rd) {
-      const int t = tile_of_round<KIND>(rd, blockIdx.x, gridDim.x);
-      if (t >= ntiles) continue;
-      const Tile tl = get_tile<KIND>(p, t);
-      for (int kb = 0; kb < tl.nkb; ++kb, ++it) {
-        const int s = it % NST;
-        const uint32_t ph = (it / NST) & 1u;
-        const long long w0 = clock64();
-        if (!mbar_wait(empty_bar(s), ph ^ 1u)) {
-          ok = false;
-          break;
+    if (elect_one()) {
+      RingPos pos;
+      uint32_t it = 0;
+      bool ok = true;
+      RoleClock clk(p.timers);
+      for (int rd = 0; rd * static_cast<int>(gridDim.x) < ntiles && ok; ++rd) {
+        const int t = tile_of_round<KIND>(rd, blockIdx.x, gridDim.x);
+        if (t >= ntiles) continue;
+        const Tile tl = get_tile<KIND>(p, t);
+        for (int kb = 0; kb < tl.nkb; ++kb, ++it) {
+          clk.start();
+          if (!mbar_wait(empty_bar(pos.s), pos.phase ^ 1u)) {
+            ok = false;
+            break;
+          }
+          clk.add(0);
+          const uint32_t sA = smem_base + pos.s * stage_stride;
+          mbar_expect_tx(full_bar(pos.s), p.stage_tx);
+          issue_loads<KIND>(p, tl, kb, sA, sA + A_BYTES, full_bar(pos.s));
+          pos.next(NST);
         }
-        t_wait += clock64() - w0;
-        const uint32_t sA = smem_base + s * stage_stride;
-        if (lane == 0) {
-          mbar_expect_tx(full_bar(s), p.stage_tx);
-          issue_loads<KIND>(p, tl, kb, sA, sA + A_BYTES, full_bar(s));
-        }
-        __syncwarp();
       }
-    }
-    chain_next();  // not earlier: blocks of the next kernel that only wait would sit beside the main loop
-    if (p.timers && lane == 0) {
-      atomicAdd(p.timers + 0, static_cast<unsigned long long>(clock64() - t_begin));  // producer: total
-      atomicAdd(p.timers + 1, static_cast<unsigned long long>(t_wait));               // producer: waiting for a free stage
-    }
-    if (!ok) {
-      // gave up: the copies already issued still land in this CTA's shared memory - wait for them (bounded again)
-      // before the CTA may exit
-      if (lane == 0) record_status(p.status, DEV_TIMEOUT, 100 + KIND);
-      for (uint32_t i = it > static_cast<uint32_t>(NST) ? it - NST : 0; i < it; ++i) mbar_wait(full_bar(i % NST), (i / NST) & 1u);
+      chain_next();  // not earlier: blocks of the next kernel that only wait would sit beside the main loop
+      clk.report(0, 1);  // total; waiting for a free stage
+      if (!ok) {
+        // gave up: the copies already issued still land in this CTA's shared memory - wait for them (bounded again)
+        // before the CTA may exit
+        record_status(p.status, DEV_TIMEOUT, 100 + KIND);
+        for (uint32_t i = it > static_cast<uint32_t>(NST) ? it - NST : 0; i < it; ++i)
+          mbar_wait(full_bar(i % NST), (i / NST) & 1u);
+      }
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    const uint32_t idesc = umma_idesc(BM, p.mma_n, TR::A_MN, TR::B_MN);
-    constexpr uint32_t A_LBO = TR::A_MN ? CHUNK_BYTES : 0, B_LBO = TR::B_MN ? CHUNK_BYTES : 0;
-    constexpr uint32_t A_KSTEP = TR::A_MN ? 2048 : 32, B_KSTEP = TR::B_MN ? 2048 : 32;  // bytes per K = 16
-    uint32_t it = 0, tc = 0;
-    bool ok = true;
-    long long t_acc = 0, t_full = 0, t_begin = clock64();
-    for (int rd = 0; rd * static_cast<int>(gridDim.x) < ntiles && ok; ++rd) {
-      const int t = tile_of_round<KIND>(rd, blockIdx.x, gridDim.x);
-      if (t >= ntiles) continue;
-      const Tile tl = get_tile<KIND>(p, t);
-      if (tl.nkb == 0) continue;
-      const int acc = tc & 1;
-      const uint32_t aph = (tc >> 1) & 1u;
-      ++tc;
-      const long long w0 = clock64();
-      if (!mbar_wait(tempty_bar(acc), aph ^ 1u)) {
-        ok = false;
-        break;
-      }
-      t_acc += clock64() - w0;
-      tc_fence_after();
-      const uint32_t d_tmem = tmem_base + acc * ACC_COLS;
-      for (int kb = 0; kb < tl.nkb; ++kb, ++it) {
-        const int s = it % NST;
-        const uint32_t ph = (it / NST) & 1u;
-        const long long w1 = clock64();
-        if (!mbar_wait(full_bar(s), ph)) {
+    if (elect_one()) {
+      const uint32_t idesc = umma_idesc(BM, p.mma_n, TR::A_MN, TR::B_MN);
+      constexpr uint32_t A_KSTEP = TR::A_MN ? 2048 : 32, B_KSTEP = TR::B_MN ? 2048 : 32;  // bytes per K = 16
+      const uint64_t descA = smem_desc(smem_base, TR::A_MN ? CHUNK_BYTES : 0, 1024);
+      const uint64_t descB = smem_desc(smem_base + A_BYTES, TR::B_MN ? CHUNK_BYTES : 0, 1024);
+      RingPos pos;
+      uint32_t tc = 0;
+      bool ok = true;
+      RoleClock clk(p.timers);
+      for (int rd = 0; rd * static_cast<int>(gridDim.x) < ntiles && ok; ++rd) {
+        const int t = tile_of_round<KIND>(rd, blockIdx.x, gridDim.x);
+        if (t >= ntiles) continue;
+        const Tile tl = get_tile<KIND>(p, t);
+        if (tl.nkb == 0) continue;
+        const int acc = tc & 1;
+        const uint32_t aph = (tc >> 1) & 1u;
+        ++tc;
+        clk.start();
+        if (!mbar_wait(tempty_bar(acc), aph ^ 1u)) {
           ok = false;
           break;
         }
-        t_full += clock64() - w1;
+        clk.add(0);
         tc_fence_after();
-        if (lane == 0) {
-          const uint32_t sA = smem_base + s * stage_stride;
-          const uint32_t sB = sA + A_BYTES;
+        const uint32_t d_tmem = tmem_base + acc * ACC_COLS;
+        bool ready = false;  // the stage about to be used was already seen full
+        for (int kb = 0; kb < tl.nkb; ++kb) {
+          clk.start();
+          if (!ready && !mbar_wait(full_bar(pos.s), pos.phase)) {
+            ok = false;
+            break;
+          }
+          clk.add(1);
+          tc_fence_after();
+          const uint64_t off = (pos.s * stage_stride) >> 4;
+          const uint32_t done = empty_bar(pos.s);
+          pos.next(NST);
+          ready = kb + 1 < tl.nkb && mbar_try_wait(full_bar(pos.s), pos.phase);  // its latency passes under the MMAs
           const int nks = kb == tl.nkb - 1 ? tl.klast : BK / 16;
 #pragma unroll
-          for (int ks = 0; ks < BK / 16; ++ks) {
-            if (ks < nks) {
-              const uint64_t da = smem_desc(sA + ks * A_KSTEP, A_LBO, 1024);
-              const uint64_t db = smem_desc(sB + ks * B_KSTEP, B_LBO, 1024);
-              umma_bf16(d_tmem, da, db, idesc, (kb | ks) != 0 ? 1u : 0u);
-            }
-          }
-          umma_commit(empty_bar(s));
+          for (int ks = 0; ks < BK / 16; ++ks)
+            if (ks < nks)
+              umma_bf16(d_tmem, descA + off + (ks * A_KSTEP >> 4), descB + off + (ks * B_KSTEP >> 4), idesc,
+                        (kb | ks) != 0 ? 1u : 0u);
+          umma_commit(done);
         }
-        __syncwarp();
+        if (ok) umma_commit(tfull_bar(acc));
       }
-      if (ok && lane == 0) umma_commit(tfull_bar(acc));
-      __syncwarp();
-    }
-    if (p.timers && lane == 0) {
-      atomicAdd(p.timers + 2, static_cast<unsigned long long>(clock64() - t_begin));  // MMA issuer: total
-      atomicAdd(p.timers + 3, static_cast<unsigned long long>(t_acc));                // waiting for a drained accumulator
-      atomicAdd(p.timers + 4, static_cast<unsigned long long>(t_full));               // waiting for operands
-    }
-    if (!ok) {
-      // gave up: let every MMA issued so far finish (bounded) before the tensor memory is freed
-      if (lane == 0) {
+      clk.report(2, 3, 4);  // total; waiting for a drained accumulator; waiting for operands
+      if (!ok) {
+        // gave up: let every MMA issued so far finish (bounded) before the tensor memory is freed
         record_status(p.status, DEV_TIMEOUT, 200 + KIND);
         umma_commit(bar0 + 8u * (2 * STAGES + 4));
+        mbar_wait(bar0 + 8u * (2 * STAGES + 4), 0u);
       }
-      __syncwarp();
-      mbar_wait(bar0 + 8u * (2 * STAGES + 4), 0u);
     }
   } else if (warp < 2 + EPI_WARPS) {
     // ------------------------------------------------------------------ epilogue (128 TMEM lanes; two warps per
@@ -194,7 +185,7 @@ __global__ void __launch_bounds__(KIND == GEMM_RT ? 192 : GEMM_THREADS, 1)
     EpiStage es{smem_base + STAGES * STAGE_BYTES + (warp - 2) * (EPI_UNITS * EPI_UNIT_BYTES), 0u};
     uint32_t tc = 0;
     bool ok = true;
-    long long t_idle = 0, t_begin = clock64();
+    RoleClock clk(p.timers);
     for (int rd = 0; rd * static_cast<int>(gridDim.x) < ntiles && ok; ++rd) {
       const int t = tile_of_round<KIND>(rd, blockIdx.x, gridDim.x);
       if (t >= ntiles) continue;
@@ -218,12 +209,12 @@ __global__ void __launch_bounds__(KIND == GEMM_RT ? 192 : GEMM_THREADS, 1)
       const uint32_t aph = (tc >> 1) & 1u;
       ++tc;
       epilogue_prefetch<KIND>(p, static_cast<int64_t>(tl.row0) + rin, tl.n0, half == 0, tl.e, tl.m0 + rin);
-      const long long w0 = clock64();
+      clk.start();
       if (!mbar_wait(tfull_bar(acc), aph)) {
         ok = false;
         break;
       }
-      t_idle += clock64() - w0;
+      clk.add(0);
       tc_fence_after();
       const uint32_t taddr = tmem_base + (static_cast<uint32_t>(ew * 32) << 16) + acc * ACC_COLS;
       const int64_t row = static_cast<int64_t>(tl.row0) + rin;
@@ -270,10 +261,9 @@ __global__ void __launch_bounds__(KIND == GEMM_RT ? 192 : GEMM_THREADS, 1)
       }
       if (KIND == GEMM_RT || KIND == GEMM_DWR) release();
     }
-    if (p.timers && lane == 0 && ew == 0 && half == 0) {
-      atomicAdd(p.timers + 5, static_cast<unsigned long long>(clock64() - t_begin));  // epilogue warp: total
-      atomicAdd(p.timers + 6, static_cast<unsigned long long>(t_idle));               // waiting for a finished accumulator
-      atomicAdd(p.timers + 7, 1ull);                                                  // CTAs counted
+    if (lane == 0 && ew == 0 && half == 0) {
+      clk.report(5, 6);  // total; waiting for a finished accumulator
+      if (p.timers) atomicAdd(p.timers + 7, 1ull);  // CTAs counted
     }
     if (!ok && lane == 0) {
       record_status(p.status, DEV_TIMEOUT, 300 + KIND);
@@ -315,6 +305,30 @@ static bool map_3d(void* fn, CUtensorMap* m, const void* base, int64_t E, int64_
                                              strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
                                              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// MN-major operands, `chunks` 64-column chunks of 64 K rows in one box that lands in shared memory chunk by chunk.  The
+// chunk is a dimension of the map (64 columns apart), so the width has to be a multiple of 64, or at most 64 with one
+// chunk in use (columns beyond the width read as zeros).
+static bool map_chunks(void* fn, CUtensorMap* m, const void* base, int64_t E, int64_t rows, int64_t width, int chunks,
+                       int rank) {
+  cuuint64_t dims[4] = {static_cast<cuuint64_t>(width < 64 ? width : 64), static_cast<cuuint64_t>(rows),
+                        static_cast<cuuint64_t>((width + 63) / 64), static_cast<cuuint64_t>(E)};
+  cuuint64_t strides[3] = {static_cast<cuuint64_t>(width) * 2, 128, static_cast<cuuint64_t>(width) * rows * 2};
+  cuuint32_t box[4] = {64, 64, static_cast<cuuint32_t>(chunks), 1};
+  cuuint32_t es[4] = {1, 1, 1, 1};
+  return reinterpret_cast<EncodeTiledFn>(fn)(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void*>(base), dims,
+                                             strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                                             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                                             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+// bf16 weights [E, rows, width]: coordinates (0, row, chunk, expert)
+static bool map_mn(void* fn, CUtensorMap* m, const void* base, int64_t E, int64_t rows, int64_t width, int chunks) {
+  return map_chunks(fn, m, base, E, rows, width, chunks, 4);
+}
+// bf16 rows [rows, width]: coordinates (0, row, chunk)
+static bool map_mn_rows(void* fn, CUtensorMap* m, const void* base, int64_t rows, int64_t width, int chunks) {
+  return map_chunks(fn, m, base, 1, rows, width, chunks, 3);
 }
 
 template <int KIND>
@@ -393,7 +407,6 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
     p.e_first = io.e_first;
     p.expert_grouped = 1;
   }
-  p.b_chunks = 4;
   p.mma_n = BN;
   p.stage_tx = STAGE_BYTES;
   p.nseg = (kind == GEMM_B4 || kind == GEMM_DX) ? 2 : 1;
@@ -403,7 +416,7 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
   switch (kind) {
     case GEMM_F3:
       ok = map_2d(fn, &p.mapA0, xp, R, d, 128) && map_2d(fn, &p.mapS0, xp, R, d, 32) &&
-           map_3d(fn, &p.mapB0, W_gate, E, d, f, 64) && map_3d(fn, &p.mapB1, W_up, E, d, f, 64);
+           map_mn(fn, &p.mapB0, W_gate, E, d, f, 2) && map_mn(fn, &p.mapB1, W_up, E, d, f, 2);
       p.mapA1 = p.mapA0;
       clip_pads(&p, !io.save_preactivations, rows_per_expert);
       p.n_tiles = (f + 127) / 128;
@@ -418,7 +431,7 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
       return pair ? launch_pair_gemm(ctx, kind, p, st) : launch_kind<GEMM_F3>(ctx, p, st);
     case GEMM_F4:
       ok = map_2d(fn, &p.mapA0, act, R, f, 128) && map_2d(fn, &p.mapS0, act, R, f, 32) &&
-           map_3d(fn, &p.mapB0, W_down, E, f, d, 64);
+           map_mn(fn, &p.mapB0, W_down, E, f, d, pair ? 2 : 4);
       p.mapA1 = p.mapA0; p.mapB1 = p.mapB0;
       clip_pads(&p, !io.save_preactivations, rows_per_expert);
       p.n_tiles = (d + 255) / 256;
@@ -457,7 +470,7 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
       p.row_group = row_group_for(p.n_tiles, ctx);
       return pair ? launch_pair_gemm(ctx, kind, p, st) : launch_kind<GEMM_B4>(ctx, p, st);
     case GEMM_B3:
-      ok = map_2d(fn, &p.mapA0, act, R, f, 64) && map_2d(fn, &p.mapB0, o, R, d, 64);
+      ok = map_mn_rows(fn, &p.mapA0, act, R, f, 2) && map_mn_rows(fn, &p.mapB0, o, R, d, pair ? 2 : 4);
       p.mapA1 = p.mapA0; p.mapB1 = p.mapB0;
       p.m_tiles = pair ? (f + 255) / 256 : (f + 127) / 128;
       p.n_tiles = (d + 255) / 256;
@@ -471,8 +484,8 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
       if (!ok) return MOE_ERR_CUDA;
       return pair ? launch_pair_gemm(ctx, kind, p, st) : launch_kind<GEMM_B3>(ctx, p, st);
     case GEMM_B5:
-      ok = map_2d(fn, &p.mapA0, xp, R, d, 64) && map_2d(fn, &p.mapB0, dhg, R, f, 64) &&
-           map_2d(fn, &p.mapB1, dhu, R, f, 64);
+      ok = map_mn_rows(fn, &p.mapA0, xp, R, d, 2) && map_mn_rows(fn, &p.mapB0, dhg, R, f, 2) &&
+           map_mn_rows(fn, &p.mapB1, dhu, R, f, 2);
       p.mapA1 = p.mapA0;
       p.m_tiles = pair ? (d + 255) / 256 : (d + 127) / 128;
       p.n_tiles = (f + 127) / 128;
@@ -486,18 +499,24 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
       if (!ok) return MOE_ERR_CUDA;
       return pair ? launch_pair_gemm(ctx, kind, p, st) : launch_kind<GEMM_B5>(ctx, p, st);
     case GEMM_RT:
-      // logits[T,E] = x[T,d] W_r[d,E]; W_r is read as a one-slab 3D tensor so the weight loaders apply
-      ok = map_2d(fn, &p.mapA0, io.x, T, d, 128) && map_3d(fn, &p.mapB0, io.W_r, 1, d, E, 64);
-      p.mapA1 = p.mapA0; p.mapB1 = p.mapB0;
-      if (io.W_r_mid) {  // fp32 router weight: x (hi + mid + lo), each product exact in fp32
-        ok = ok && map_3d(fn, &p.mapB1, io.W_r_mid, 1, d, E, 64) && map_3d(fn, &p.mapB2, io.W_r_lo, 1, d, E, 64);
-        p.nseg = 3;
+      // logits[T,E] = x[T,d] W_r[d,E]; W_r is read as a one-slab tensor so the weight loaders apply
+      p.b_chunks = (E + 63) / 64;
+      p.whole_chunks = E % 64 == 0;
+      {
+        auto map_router = [&](CUtensorMap* m, const uint16_t* w) {
+          return p.whole_chunks ? map_mn(fn, m, w, 1, d, E, p.b_chunks) : map_3d(fn, m, w, 1, d, E, 64);
+        };
+        ok = map_2d(fn, &p.mapA0, io.x, T, d, 128) && map_router(&p.mapB0, io.W_r);
+        p.mapA1 = p.mapA0; p.mapB1 = p.mapB0;
+        if (io.W_r_mid) {  // fp32 router weight: x (hi + mid + lo), each product exact in fp32
+          ok = ok && map_router(&p.mapB1, io.W_r_mid) && map_router(&p.mapB2, io.W_r_lo);
+          p.nseg = 3;
+        }
       }
       p.static_m_tiles = static_cast<int>((T + BM - 1) / BM);
       p.n_tiles = 1;
       p.k_blocks = d / BK;
       p.N_total = E;
-      p.b_chunks = (E + 63) / 64;
       p.mma_n = (E + 15) / 16 * 16;
       p.stage_tx = A_BYTES + p.b_chunks * CHUNK_BYTES;
       p.T = T;
@@ -534,8 +553,10 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
       return launch_kind<GEMM_DX>(ctx, p, st);
     case GEMM_DWR: {
       // partial[s][d,E] = x_s^T (dl_hi + dl_lo)_s over token slices of split_rows tokens
-      ok = map_2d(fn, &p.mapA0, io.x, T, d, 64) && map_2d(fn, &p.mapB0, ws + L.dl_hi, T, E, 64) &&
-           map_2d(fn, &p.mapB1, ws + L.dl_lo, T, E, 64);
+      p.whole_chunks = E % 64 == 0;
+      ok = map_mn_rows(fn, &p.mapA0, io.x, T, d, 2) &&
+           (p.whole_chunks ? map_mn_rows(fn, &p.mapB0, ws + L.dl_hi, T, E, 2) && map_mn_rows(fn, &p.mapB1, ws + L.dl_lo, T, E, 2)
+                           : map_2d(fn, &p.mapB0, ws + L.dl_hi, T, E, 64) && map_2d(fn, &p.mapB1, ws + L.dl_lo, T, E, 64));
       p.mapA1 = p.mapA0;
       const int64_t per = ((T + DWR_SPLIT - 1) / DWR_SPLIT + BK - 1) / BK * BK;
       p.split_rows = static_cast<int>(per);
@@ -571,15 +592,15 @@ static double expected_tiles(double mean, double size) {
 
 // Tile shape per GEMM.  A CTA pair (256 x 256 tile, each CTA staging its rows of A and half of B) moves a third
 // less operand data from L2 per flop than a one-CTA 128 x 256 tile, and the L2 -> SM feed is what limits these
-// kernels: a 128-row block costs 0.87 of its one-CTA time on the pair kernel.  Row GEMMs pair two 128-row blocks of ONE
+// kernels: a 128-row block costs 0.80 of its one-CTA time on the pair kernel.  Row GEMMs pair two 128-row blocks of ONE
 // expert, so an expert with an odd block count pays for a block it does not have.  Whether pairs win therefore
 // oscillates with the rows per expert, and the rule compares the two expected costs.  Measured (d 2048, f 768, 128
-// experts, one-CTA -> pair, us; gate/up, down, dgrad gate/up): 62 rows per expert 164 -> 168, 81 -> 84, 161 -> 161;
-// 200: 200 -> 188, 106 -> 97, 193 -> 175; 312: 261 -> 276, 152 -> 157, 272 -> 296; 437: 331 -> 294, 197 -> 169,
-// 355 -> 320; 512: 372 -> 361, 217 -> 196, 393 -> 389; 1024: 696 -> 659, 407 -> 354, 741 -> 719.  The rule misses by at
-// most 1 % at 62 rows and 375 rows (equal there).
-// The dgrad-down GEMM is held by its epilogue (it reads hg and hu) rather than by the feed and gains less: 151 -> 152 at
-// 200 rows, 242 -> 252 at 512, 284 -> 295 at 625, 455 -> 439 at 1024: pairs from 768 rows on.
+// experts, one-CTA -> pair, us; gate/up, down, dgrad gate/up): 62 rows per expert 164 -> 168, 82 -> 85, 163 -> 160;
+// 156: 204 -> 186, 106 -> 96, 195 -> 174; 256: 231 -> 222, 129 -> 123, 233 -> 217; 312: 270 -> 273, 152 -> 156,
+// 276 -> 278; 375: 297 -> 282, 169 -> 161, 310 -> 292; 512: 385 -> 369, 218 -> 200, 404 -> 381; 1024: 719 -> 700,
+// 406 -> 365, 764 -> 718.  At 128 rows (equal, equal, 180 -> 167) the rule misses.
+// The dgrad-down GEMM is held by its epilogue (it reads hg and hu) rather than by the feed and gains less: 153 -> 152 at
+// 156 rows, 251 -> 271 at 512, 290 -> 299 at 625, 455 -> 465 at 1024: pairs from 768 rows on.
 // Half-empty pairs are better than complete pairs plus the leftover blocks in a second, one-CTA launch
 // (MOE_FLAG_HYBRID_TILES: 4.22 ms a step against 4.17 at 1024 rows per expert).
 // Weight gradients pair along the weight dimension without leftovers, but their K loop is the expert's row count, and
@@ -601,7 +622,7 @@ moe_status launch_grouped_gemm(moe_ctx_impl* ctx, GemmKind kind, int64_t T, cons
     if (kind == GEMM_B2)
       pair = rows_per_expert >= 768.0;
     else
-      pair = 0.87 * 2.0 * expected_tiles(rows_per_expert, 2 * BM) < expected_tiles(rows_per_expert, BM);
+      pair = 0.80 * 2.0 * expected_tiles(rows_per_expert, 2 * BM) < expected_tiles(rows_per_expert, BM);
     if (kind == GEMM_B4 && ctx->b4_pair_override >= 0) pair = ctx->b4_pair_override != 0;
   }
   if (ctx->tile_mode != 3) return launch_gemm_variant(ctx, kind, T, L, ws, io, st, pair, 0);
@@ -680,7 +701,7 @@ static moe_status launch_lora_gemm_bwd(moe_ctx_impl* ctx, LoraOp op, int64_t T, 
       if (!ok) return MOE_ERR_CUDA;
       return launch_kind<GEMM_B4>(ctx, p, st);
     case LORA_DB2:  // dB2[e][r,d] = v_e^T dy_rows_e      (B3 kind, M = rank)
-      ok = map_2d(fn, &p.mapA0, v, R, 64, 64) && map_2d(fn, &p.mapB0, dyr, R, d, 64);
+      ok = map_mn_rows(fn, &p.mapA0, v, R, 64, 2) && map_mn_rows(fn, &p.mapB0, dyr, R, d, 4);
       p.mapA1 = p.mapA0; p.mapB1 = p.mapB0;
       p.m_tiles = 1;
       p.n_tiles = (d + 255) / 256;
@@ -693,13 +714,13 @@ static moe_status launch_lora_gemm_bwd(moe_ctx_impl* ctx, LoraOp op, int64_t T, 
       return launch_kind<GEMM_B3>(ctx, p, st);
     case LORA_DA2:  // dA2[e][f,r] = act_e^T w_e           (B3 kind, N = rank)
     case LORA_DA1:  // dA1[e][d,r] = xp_e^T z_e
-      ok = map_2d(fn, &p.mapA0, op == LORA_DA2 ? act : xp, R, op == LORA_DA2 ? f : d, 64) &&
-           map_2d(fn, &p.mapB0, op == LORA_DA2 ? w : z, R, 64, 64);
+      ok = map_mn_rows(fn, &p.mapA0, op == LORA_DA2 ? act : xp, R, op == LORA_DA2 ? f : d, 2) &&
+           map_mn_rows(fn, &p.mapB0, op == LORA_DA2 ? w : z, R, 64, 1);
       p.mapA1 = p.mapA0; p.mapB1 = p.mapB0;
       p.M_total = op == LORA_DA2 ? f : d;
       p.m_tiles = (p.M_total + 127) / 128;
       p.n_tiles = 1;
-      p.b_chunks = 1; p.mma_n = 64; p.stage_tx = skinny_tx;
+      p.mma_n = 64; p.stage_tx = skinny_tx;
       p.N_total = r;
       p.out0 = op == LORA_DA2 ? lo.dA2 : lo.dA1;
       p.ld_out = r;
@@ -707,8 +728,8 @@ static moe_status launch_lora_gemm_bwd(moe_ctx_impl* ctx, LoraOp op, int64_t T, 
       if (!ok) return MOE_ERR_CUDA;
       return launch_kind<GEMM_B3>(ctx, p, st);
     case LORA_DB1:  // dB1g[e] | dB1u[e] [r,f] = u_e^T [dhg_e | dhu_e]   (B5 kind, M = rank)
-      ok = map_2d(fn, &p.mapA0, u, R, 64, 64) && map_2d(fn, &p.mapB0, dhg, R, f, 64) &&
-           map_2d(fn, &p.mapB1, dhu, R, f, 64);
+      ok = map_mn_rows(fn, &p.mapA0, u, R, 64, 2) && map_mn_rows(fn, &p.mapB0, dhg, R, f, 2) &&
+           map_mn_rows(fn, &p.mapB1, dhu, R, f, 2);
       p.mapA1 = p.mapA0;
       p.m_tiles = 1;
       p.n_tiles = (f + 127) / 128;
@@ -750,7 +771,6 @@ moe_status launch_lora_gemm(moe_ctx_impl* ctx, LoraOp op, int64_t T, const WsLay
   p.expert_order = reinterpret_cast<const int32_t*>(ws + L.expert_order);
   p.status = reinterpret_cast<int32_t*>(ws + L.status);
   p.E = E;
-  p.b_chunks = 4;
   p.mma_n = BN;
   p.stage_tx = STAGE_BYTES;
   p.nseg = 1;
@@ -762,11 +782,11 @@ moe_status launch_lora_gemm(moe_ctx_impl* ctx, LoraOp op, int64_t T, const WsLay
     case LORA_U:  // u[R,64] = s xp A1[e]            (F4 kind, N = 64)
     case LORA_V:  // v[R,64] = s act A2[e]
       ok = map_2d(fn, &p.mapA0, op == LORA_U ? xp : act, R, op == LORA_U ? d : f, 128) &&
-           map_3d(fn, &p.mapB0, op == LORA_U ? lo.A1 : lo.A2, E, op == LORA_U ? d : f, r, 64);
+           map_mn(fn, &p.mapB0, op == LORA_U ? lo.A1 : lo.A2, E, op == LORA_U ? d : f, r, 1);
       p.mapA1 = p.mapA0; p.mapB1 = p.mapB0;
       p.n_tiles = 1;
       p.k_blocks = (op == LORA_U ? d : f) / BK;
-      p.b_chunks = 1; p.mma_n = 64; p.stage_tx = skinny_tx;
+      p.mma_n = 64; p.stage_tx = skinny_tx;
       p.N_total = 64;
       p.out0 = op == LORA_U ? u : v;
       p.ld_out = 64;
@@ -774,9 +794,9 @@ moe_status launch_lora_gemm(moe_ctx_impl* ctx, LoraOp op, int64_t T, const WsLay
       if (!ok) return MOE_ERR_CUDA;
       return launch_kind<GEMM_F4>(ctx, p, st);
     case LORA_F3:  // [hg|hu] = xp [Wg|Wu] + u [B1g|B1u]
-      ok = map_2d(fn, &p.mapA0, xp, R, d, 128) && map_3d(fn, &p.mapB0, io.W_gate, E, d, f, 64) &&
-           map_3d(fn, &p.mapB1, io.W_up, E, d, f, 64) && map_2d(fn, &p.mapA2, u, R, 64, 128) &&
-           map_3d(fn, &p.mapB2, lo.B1g, E, r, f, 64) && map_3d(fn, &p.mapB3, lo.B1u, E, r, f, 64);
+      ok = map_2d(fn, &p.mapA0, xp, R, d, 128) && map_mn(fn, &p.mapB0, io.W_gate, E, d, f, 2) &&
+           map_mn(fn, &p.mapB1, io.W_up, E, d, f, 2) && map_2d(fn, &p.mapA2, u, R, 64, 128) &&
+           map_mn(fn, &p.mapB2, lo.B1g, E, r, f, 2) && map_mn(fn, &p.mapB3, lo.B1u, E, r, f, 2);
       p.mapA1 = p.mapA0;
       p.n_tiles = (f + 127) / 128;
       p.k_blocks = d / BK;
@@ -788,8 +808,8 @@ moe_status launch_lora_gemm(moe_ctx_impl* ctx, LoraOp op, int64_t T, const WsLay
       if (!ok) return MOE_ERR_CUDA;
       return launch_kind<GEMM_F3>(ctx, p, st);
     case LORA_F4:  // o = act Wd + v B2
-      ok = map_2d(fn, &p.mapA0, act, R, f, 128) && map_3d(fn, &p.mapB0, io.W_down, E, f, d, 64) &&
-           map_2d(fn, &p.mapA2, v, R, 64, 128) && map_3d(fn, &p.mapB2, lo.B2, E, r, d, 64);
+      ok = map_2d(fn, &p.mapA0, act, R, f, 128) && map_mn(fn, &p.mapB0, io.W_down, E, f, d, 4) &&
+           map_2d(fn, &p.mapA2, v, R, 64, 128) && map_mn(fn, &p.mapB2, lo.B2, E, r, d, 4);
       p.mapA1 = p.mapA0; p.mapB1 = p.mapB0;
       p.n_tiles = (d + 255) / 256;
       p.k_blocks = f / BK;

@@ -82,13 +82,10 @@ __device__ __forceinline__ void issue_loads2(const GemmParams& p, const Tile2& t
   if (KIND == GEMM_F3) {
     load_a_rows<true>(p, sA, bar, kb * BK, tl.row0, tl.valid);
     const CUtensorMap* mb = rank ? &p.mapB1 : &p.mapB0;  // leader: gate columns, partner: the matching up columns
-#pragma unroll
-    for (int c = 0; c < 2; ++c) tma_load_3d_pair(sB + c * CHUNK_BYTES, mb, bar, tl.n0 + c * 64, kb * BK, tl.e);
+    tma_load_4d_pair(sB, mb, bar, 0, kb * BK, tl.n0 / 64, tl.e);
   } else if (KIND == GEMM_F4) {
     load_a_rows<true>(p, sA, bar, kb * BK, tl.row0, tl.valid);
-#pragma unroll
-    for (int c = 0; c < 2; ++c)
-      tma_load_3d_pair(sB + c * CHUNK_BYTES, &p.mapB0, bar, tl.n0 + rank * 128 + c * 64, kb * BK, tl.e);
+    tma_load_4d_pair(sB, &p.mapB0, bar, 0, kb * BK, tl.n0 / 64 + rank * 2, tl.e);
   } else if (KIND == GEMM_B2) {
     tma_load_2d_pair(sA, &p.mapA0, bar, kb * BK, tl.write ? tl.row0 : p.oob_row);
     tma_load_3d_pair(sB, &p.mapB0, bar, kb * BK, tl.n0 + rank * 128, tl.e);
@@ -98,19 +95,13 @@ __device__ __forceinline__ void issue_loads2(const GemmParams& p, const Tile2& t
     tma_load_3d_pair(sB, seg ? &p.mapB1 : &p.mapB0, bar, kk * BK, tl.n0 + rank * 128, tl.e);
   } else if (KIND == GEMM_B3) {
     const int row = tl.row0 + kb * BK;
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      tma_load_2d_pair(sA + c * CHUNK_BYTES, &p.mapA0, bar, tl.m0 + c * 64, row);
-      tma_load_2d_pair(sB + c * CHUNK_BYTES, &p.mapB0, bar, tl.n0 + rank * 128 + c * 64, row);
-    }
+    tma_load_3d_pair(sA, &p.mapA0, bar, 0, row, tl.m0 / 64);
+    tma_load_3d_pair(sB, &p.mapB0, bar, 0, row, tl.n0 / 64 + rank * 2);
   } else {  // GEMM_B5
     const int row = tl.row0 + kb * BK;
     const CUtensorMap* mb = rank ? &p.mapB1 : &p.mapB0;  // leader: dhg columns, partner: dhu columns
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      tma_load_2d_pair(sA + c * CHUNK_BYTES, &p.mapA0, bar, tl.m0 + c * 64, row);
-      tma_load_2d_pair(sB + c * CHUNK_BYTES, mb, bar, tl.n0 + c * 64, row);
-    }
+    tma_load_3d_pair(sA, &p.mapA0, bar, 0, row, tl.m0 / 64);
+    tma_load_3d_pair(sB, mb, bar, 0, row, tl.n0 / 64);
   }
 }
 
@@ -159,114 +150,96 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
   const int cid = blockIdx.x >> 1, nclusters = gridDim.x >> 1;
 
   if (warp == 0) {
-    // ------------------------------------------------------------------ TMA producer (both CTAs)
-    uint32_t it = 0;
-    bool ok = true;
-    long long t_wait = 0, t_begin = clock64();
-    for (int rd = 0; rd * nclusters < ntiles && ok; ++rd) {
-      const int t = tile_of_round<KIND>(rd, cid, nclusters);
-      if (t >= ntiles) continue;
-      const Tile2 tl = get_tile2<KIND>(p, t, rank);
-      for (int kb = 0; kb < tl.nkb; ++kb, ++it) {
-        const int s = it % STAGES2;
-        const uint32_t ph = (it / STAGES2) & 1u;
-        const long long w0 = clock64();
-        if (!mbar_wait(empty_bar(s), ph ^ 1u)) {
-          ok = false;
-          break;
+    // ------------------------------------------------------------------ TMA producer (both CTAs; one thread)
+    if (elect_one()) {
+      RingPos pos;
+      uint32_t it = 0;
+      bool ok = true;
+      RoleClock clk(leader ? p.timers : nullptr);
+      for (int rd = 0; rd * nclusters < ntiles && ok; ++rd) {
+        const int t = tile_of_round<KIND>(rd, cid, nclusters);
+        if (t >= ntiles) continue;
+        const Tile2 tl = get_tile2<KIND>(p, t, rank);
+        for (int kb = 0; kb < tl.nkb; ++kb, ++it) {
+          clk.start();
+          if (!mbar_wait(empty_bar(pos.s), pos.phase ^ 1u)) {
+            ok = false;
+            break;
+          }
+          clk.add(0);
+          if (leader) mbar_expect_tx(full_bar(pos.s), 2 * STAGE2_BYTES);
+          const uint32_t sA = smem_base + pos.s * STAGE2_BYTES;
+          issue_loads2<KIND>(p, tl, kb, rank, sA, sA + A_BYTES, mapa_shared(full_bar(pos.s), 0));
+          pos.next(STAGES2);
         }
-        t_wait += clock64() - w0;
-        if (lane == 0) {
-          if (leader) mbar_expect_tx(full_bar(s), 2 * STAGE2_BYTES);
-          const uint32_t sA = smem_base + s * STAGE2_BYTES;
-          issue_loads2<KIND>(p, tl, kb, rank, sA, sA + A_BYTES, mapa_shared(full_bar(s), 0));
-        }
-        __syncwarp();
+      }
+      chain_next();
+      clk.report(0, 1);
+      if (!ok) {
+        // gave up: the leader waits (bounded) for the copies of BOTH CTAs that were already issued - they are all credited
+        // to its full barriers - so that neither CTA exits with copies in flight (the cluster barrier below holds the
+        // partner until then)
+        record_status(p.status, DEV_TIMEOUT, 1100 + KIND);
+        if (leader)
+          for (uint32_t i = it > static_cast<uint32_t>(STAGES2) ? it - STAGES2 : 0; i < it; ++i)
+            mbar_wait(full_bar(i % STAGES2), (i / STAGES2) & 1u);
       }
     }
-    chain_next();
-    if (p.timers && lane == 0 && leader) {
-      atomicAdd(p.timers + 0, static_cast<unsigned long long>(clock64() - t_begin));
-      atomicAdd(p.timers + 1, static_cast<unsigned long long>(t_wait));
-    }
-    if (!ok) {
-      // gave up: the leader waits (bounded) for the copies of BOTH CTAs that were already issued - they are all credited
-      // to its full barriers - so that neither CTA exits with copies in flight (the cluster barrier below holds the
-      // partner until then)
-      if (lane == 0) record_status(p.status, DEV_TIMEOUT, 1100 + KIND);
-      if (leader)
-        for (uint32_t i = it > static_cast<uint32_t>(STAGES2) ? it - STAGES2 : 0; i < it; ++i)
-          mbar_wait(full_bar(i % STAGES2), (i / STAGES2) & 1u);
-    }
   } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA issuer (leader CTA only)
-    if (leader) {
+    // ------------------------------------------------------------------ MMA issuer (leader CTA only; one thread)
+    if (leader && elect_one()) {
       constexpr uint32_t idesc = umma_idesc(2 * BM, BN, TR::A_MN, TR::B_MN);
-      constexpr uint32_t A_LBO = TR::A_MN ? CHUNK_BYTES : 0, B_LBO = TR::B_MN ? CHUNK_BYTES : 0;
       constexpr uint32_t A_KSTEP = TR::A_MN ? 2048 : 32, B_KSTEP = TR::B_MN ? 2048 : 32;
-      uint32_t it = 0, tc = 0;
+      const uint64_t descA = smem_desc(smem_base, TR::A_MN ? CHUNK_BYTES : 0, 1024);
+      const uint64_t descB = smem_desc(smem_base + A_BYTES, TR::B_MN ? CHUNK_BYTES : 0, 1024);
+      RingPos pos;
+      uint32_t tc = 0;
       bool ok = true;
-      long long t_acc = 0, t_full = 0, t_begin = clock64();
+      RoleClock clk(p.timers);
       for (int rd = 0; rd * nclusters < ntiles && ok; ++rd) {
-      const int t = tile_of_round<KIND>(rd, cid, nclusters);
-      if (t >= ntiles) continue;
+        const int t = tile_of_round<KIND>(rd, cid, nclusters);
+        if (t >= ntiles) continue;
         const Tile2 tl = get_tile2<KIND>(p, t, rank);
         if (tl.nkb == 0) continue;
         const int acc = tc & 1;
         const uint32_t aph = (tc >> 1) & 1u;
         ++tc;
-        const long long w0 = clock64();
+        clk.start();
         if (!mbar_wait(tempty_bar(acc), aph ^ 1u)) {
           ok = false;
           break;
         }
-        t_acc += clock64() - w0;
+        clk.add(0);
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + acc * ACC_COLS;
-        for (int kb = 0; kb < tl.nkb; ++kb, ++it) {
-          const int s = it % STAGES2;
-          const uint32_t ph = (it / STAGES2) & 1u;
-          const long long w1 = clock64();
-          if (!mbar_wait(full_bar(s), ph)) {
+        bool ready = false;  // the stage about to be used was already seen full
+        for (int kb = 0; kb < tl.nkb; ++kb) {
+          clk.start();
+          if (!ready && !mbar_wait(full_bar(pos.s), pos.phase)) {
             ok = false;
             break;
           }
-          t_full += clock64() - w1;
+          clk.add(1);
           tc_fence_after();
-          if (lane == 0) {
-            const uint32_t sA = smem_base + s * STAGE2_BYTES;
-            const uint32_t sB = sA + A_BYTES;
-            const int nks = kb == tl.nkb - 1 ? tl.klast : BK / 16;
+          const uint64_t off = (pos.s * STAGE2_BYTES) >> 4;
+          const uint32_t done = empty_bar(pos.s);
+          pos.next(STAGES2);
+          ready = kb + 1 < tl.nkb && mbar_try_wait(full_bar(pos.s), pos.phase);  // its latency passes under the MMAs
+          const int nks = kb == tl.nkb - 1 ? tl.klast : BK / 16;
 #pragma unroll
-            for (int ks = 0; ks < BK / 16; ++ks) {
-              if (ks < nks) {
-                const uint64_t da = smem_desc(sA + ks * A_KSTEP, A_LBO, 1024);
-                const uint64_t db = smem_desc(sB + ks * B_KSTEP, B_LBO, 1024);
-                umma_bf16_pair(d_tmem, da, db, idesc, (kb | ks) != 0 ? 1u : 0u);
-              }
-            }
-            // the stage is free in both CTAs once these MMAs have read it
-            umma_commit_pair_both(empty_bar(s));
-          }
-          __syncwarp();
+          for (int ks = 0; ks < BK / 16; ++ks)
+            if (ks < nks)
+              umma_bf16_pair(d_tmem, descA + off + (ks * A_KSTEP >> 4), descB + off + (ks * B_KSTEP >> 4), idesc,
+                             (kb | ks) != 0 ? 1u : 0u);
+          umma_commit_pair_both(done);  // the stage is free in both CTAs once these MMAs have read it
         }
-        if (ok && lane == 0) {
-          umma_commit_pair_both(tfull_bar(acc));
-        }
-        __syncwarp();
+        if (ok) umma_commit_pair_both(tfull_bar(acc));
       }
-      if (p.timers && lane == 0) {
-        atomicAdd(p.timers + 2, static_cast<unsigned long long>(clock64() - t_begin));
-        atomicAdd(p.timers + 3, static_cast<unsigned long long>(t_acc));
-        atomicAdd(p.timers + 4, static_cast<unsigned long long>(t_full));
-      }
+      clk.report(2, 3, 4);
       if (!ok) {
         // gave up: let every MMA issued so far finish (bounded) before the pair's tensor memory is freed
-        if (lane == 0) {
-          record_status(p.status, DEV_TIMEOUT, 1200 + KIND);
-          umma_commit_pair_both(bar0 + 8u * (2 * STAGES2 + 4));
-        }
-        __syncwarp();
+        record_status(p.status, DEV_TIMEOUT, 1200 + KIND);
+        umma_commit_pair_both(bar0 + 8u * (2 * STAGES2 + 4));
         mbar_wait(bar0 + 8u * (2 * STAGES2 + 4), 0u);
       }
     }
@@ -278,7 +251,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
     EpiStage es{smem_base + STAGES2 * STAGE2_BYTES + (warp - 2) * (EPI_UNITS * EPI_UNIT_BYTES), 0u};
     uint32_t tc = 0;
     bool ok = true;
-    long long t_idle = 0, t_begin = clock64();
+    RoleClock clk(p.timers);
     for (int rd = 0; rd * nclusters < ntiles && ok; ++rd) {
       const int t = tile_of_round<KIND>(rd, cid, nclusters);
       if (t >= ntiles) continue;
@@ -292,12 +265,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
       const uint32_t aph = (tc >> 1) & 1u;
       ++tc;
       epilogue_prefetch<KIND>(p, static_cast<int64_t>(tl.row0) + rin, tl.n0, tl.write && half == 0, tl.e, tl.m0 + rin);
-      const long long w0 = clock64();
+      clk.start();
       if (!mbar_wait(tfull_bar(acc), aph)) {
         ok = false;
         break;
       }
-      t_idle += clock64() - w0;
+      clk.add(0);
       tc_fence_after();
       const uint32_t taddr = tmem_base + (static_cast<uint32_t>(ew * 32) << 16) + acc * ACC_COLS;
       expert_epilogue<KIND>(p, tl.e, static_cast<int64_t>(tl.row0) + rin, (TR::WGRAD ? tl.m0 : tl.row0) + ew * 32, tl.n0, taddr,
@@ -308,10 +281,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
                               if (lane == 0) mbar_arrive_cluster(mapa_shared(tempty_bar(acc), 0));
                             });
     }
-    if (p.timers && lane == 0 && ew == 0 && half == 0 && leader) {
-      atomicAdd(p.timers + 5, static_cast<unsigned long long>(clock64() - t_begin));
-      atomicAdd(p.timers + 6, static_cast<unsigned long long>(t_idle));
-      atomicAdd(p.timers + 7, 1ull);
+    if (lane == 0 && ew == 0 && half == 0 && leader) {
+      clk.report(5, 6);
+      if (p.timers) atomicAdd(p.timers + 7, 1ull);
     }
     if (!ok && lane == 0) {
       record_status(p.status, DEV_TIMEOUT, 1300 + KIND);
