@@ -28,29 +28,36 @@
 namespace moe {
 
 template <int KIND>
-__global__ void __launch_bounds__(KIND == GEMM_RT ? 192 : GEMM_THREADS, 1)
+__global__ void __launch_bounds__(GEMM_THREADS, 1)
     grouped_gemm_kernel(const __grid_constant__ GemmParams p) {
   using TR = Traits<KIND>;
-  constexpr int EPI_WARPS = (KIND == GEMM_RT) ? 4 : 8;
-  constexpr int NST = STAGES;
+  constexpr int EPI_WARPS = 8;
   // The routing kind with E <= 128 stages only 32 KB per K block (16 KB of x, 16 KB of W_r): its stages are packed at
-  // that stride and the 96 KB this frees hold the scratch of its routing epilogue (80 KB) and the picks (16 KB).
+  // that stride and the 96 KB this frees hold the scratch of its routing epilogue (80 KB) and the picks (16 KB).  When no
+  // CTA has a second tile (up to 128 tokens per SM) the scratch lies over the stages, which are done with by then, and
+  // the ring has six of them: the main loop waits for memory (x and W_r come from HBM).
   constexpr uint32_t RT_STAGE_BYTES = A_BYTES + 2 * CHUNK_BYTES;
+  constexpr int MAX_STAGES = KIND == GEMM_RT ? 6 : STAGES;
+  const bool rt_packed = KIND == GEMM_RT && p.b_chunks <= 2;
+  const bool rt_overlay = rt_packed && p.static_m_tiles <= static_cast<int>(gridDim.x);
+  const int NST = rt_overlay ? 6 : STAGES;
+  static_assert(6 * RT_STAGE_BYTES <= STAGES * STAGE_BYTES + EPI_BYTES, "six packed stages do not fit");
   static_assert(STAGES * RT_STAGE_BYTES + ROUTE_SCRATCH_BYTES + 128 * ROUTE_SMEM_MAX_K * 8 <= STAGES * STAGE_BYTES + EPI_BYTES,
                 "routing scratch does not fit");
   extern __shared__ unsigned char gemm_smem_raw[];
-  __shared__ __align__(8) uint64_t bars[2 * STAGES + 5];  // full, empty, accumulator full / empty, drain (failure path)
+  __shared__ __align__(8) uint64_t bars[2 * MAX_STAGES + 5];  // full, empty, accumulator full / empty, drain (failure path)
   __shared__ uint32_t tmem_base_slot;
   __shared__ float s_bias[KIND == GEMM_RT ? MAX_E : 1];  // router bias (zero beyond E)
   __shared__ int s_hist[KIND == GEMM_RT ? 128 : 1];      // picks per expert of the tile (routing epilogue for E <= 128)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t smem_base = (smem_u32(gemm_smem_raw) + 1023u) & ~1023u;
-  const uint32_t stage_stride = (KIND == GEMM_RT && p.b_chunks <= 2) ? RT_STAGE_BYTES : STAGE_BYTES;
+  const uint32_t stage_stride = rt_packed ? RT_STAGE_BYTES : STAGE_BYTES;
+  const uint32_t rt_scratch = smem_base + (rt_overlay ? 0 : STAGES * RT_STAGE_BYTES);
   const uint32_t bar0 = smem_u32(bars);
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
-  auto empty_bar = [&](int s) { return bar0 + 8u * (STAGES + s); };
-  auto tfull_bar = [&](int a) { return bar0 + 8u * (2 * STAGES + a); };
-  auto tempty_bar = [&](int a) { return bar0 + 8u * (2 * STAGES + 2 + a); };
+  auto empty_bar = [&](int s) { return bar0 + 8u * (MAX_STAGES + s); };
+  auto tfull_bar = [&](int a) { return bar0 + 8u * (2 * MAX_STAGES + a); };
+  auto tempty_bar = [&](int a) { return bar0 + 8u * (2 * MAX_STAGES + 2 + a); };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < NST; ++s) {
@@ -61,7 +68,7 @@ __global__ void __launch_bounds__(KIND == GEMM_RT ? 192 : GEMM_THREADS, 1)
       mbar_init(tfull_bar(a), 1);
       mbar_init(tempty_bar(a), 32 * EPI_WARPS);
     }
-    mbar_init(bar0 + 8u * (2 * STAGES + 4), 1);
+    mbar_init(bar0 + 8u * (2 * MAX_STAGES + 4), 1);
     fence_mbar_init();
     tma_prefetch_desc(&p.mapA0);
     tma_prefetch_desc(&p.mapB0);
@@ -173,13 +180,13 @@ __global__ void __launch_bounds__(KIND == GEMM_RT ? 192 : GEMM_THREADS, 1)
       if (!ok) {
         // gave up: let every MMA issued so far finish (bounded) before the tensor memory is freed
         record_status(p.status, DEV_TIMEOUT, 200 + KIND);
-        umma_commit(bar0 + 8u * (2 * STAGES + 4));
-        mbar_wait(bar0 + 8u * (2 * STAGES + 4), 0u);
+        umma_commit(bar0 + 8u * (2 * MAX_STAGES + 4));
+        mbar_wait(bar0 + 8u * (2 * MAX_STAGES + 4), 0u);
       }
     }
   } else if (warp < 2 + EPI_WARPS) {
     // ------------------------------------------------------------------ epilogue (128 TMEM lanes; two warps per
-    // lane quadrant, each draining half of the tile's columns - the routing epilogue needs whole rows and uses one)
+    // lane quadrant, each draining half of the tile's columns; routing needs whole rows: one selects, one sums)
     const int ew = warp & 3;           // TMEM lane quadrant this warp may read
     const int half = (warp - 2) >> 2;  // which half of the columns
     EpiStage es{smem_base + STAGES * STAGE_BYTES + (warp - 2) * (EPI_UNITS * EPI_UNIT_BYTES), 0u};
@@ -223,12 +230,15 @@ __global__ void __launch_bounds__(KIND == GEMM_RT ? 192 : GEMM_THREADS, 1)
         mbar_arrive(tempty_bar(acc));
       };
       if (KIND == GEMM_RT) {
-        if (p.N_total <= 128 && p.top_k <= ROUTE_SMEM_MAX_K)
-          routing_epilogue_smem(p, s_bias, s_hist, smem_base + STAGES * RT_STAGE_BYTES,
-                                smem_base + STAGES * RT_STAGE_BYTES + ROUTE_SCRATCH_BYTES, row, tl.row0 / BM, ew, taddr,
-                                lane);
-        else
+        if (p.N_total <= 128 && p.top_k <= ROUTE_SMEM_MAX_K) {
+          if (half == 0)
+            routing_epilogue_smem(p, s_bias, s_hist, rt_scratch, rt_scratch + ROUTE_SCRATCH_BYTES, row, tl.row0 / BM,
+                                  ew, taddr, lane);
+          else
+            routing_softmax_sums(p, s_bias, row, tl.row0 / BM, ew, taddr, lane);
+        } else if (half == 0) {
           routing_epilogue_tmem(p, s_bias, row, tl.row0 / BM, ew, taddr, lane);
+        }
       } else if (KIND == GEMM_DWR) {
         // fp32 partial of dW_r for this token slice: hi and lo halves of dl share one accumulator pair
         const int m = tl.m0 + rin;
@@ -339,7 +349,7 @@ static moe_status launch_kind(moe_ctx_impl* ctx, const GemmParams& p, cudaStream
       return MOE_ERR_CUDA;
     ctx->attr_done[0][KIND] = 1;
   }
-  return launch_kernel(grouped_gemm_kernel<KIND>, ctx->sm_count, KIND == GEMM_RT ? 192 : GEMM_THREADS, GEMM_SMEM, st,
+  return launch_kernel(grouped_gemm_kernel<KIND>, ctx->sm_count, GEMM_THREADS, GEMM_SMEM, st,
                        p) == cudaSuccess
              ? MOE_OK
              : MOE_ERR_CUDA;
