@@ -234,28 +234,21 @@ __global__ void __launch_bounds__(TOK_TILE) hist_kernel(int64_t T, int E, int k,
   }
 }
 
-// One block: column scan of tile_counts (in place -> exclusive prefix along tiles), counts, canonical and
-// padded offsets, tile -> expert table, and the auxiliary loss from the router's partial column sums of p
-// (summed in a fixed order: reproducible).
 constexpr int SCAN_THREADS = 1024;
-__global__ void __launch_bounds__(SCAN_THREADS) scan_kernel(int64_t T, int E, int k, int tok_tiles, int psum_rows,
-                                                            int32_t* __restrict__ tile_counts, const TableOut tabs,
-                                                            const float* __restrict__ psum_part,
-                                                            float* __restrict__ psum, int32_t* __restrict__ counts_out,
-                                                            float* __restrict__ aux_out) {
-  chain_wait();
-  chain_next();
-  __shared__ int s_cnt[MAX_E];
-  __shared__ TableScratch s_tab;
-  __shared__ float s_term[MAX_E];
-  __shared__ float s_ps[SCAN_THREADS];
-  __shared__ int s_seg[SCAN_THREADS];
-  const int tid = threadIdx.x;
-  // column sums of p: G groups of threads stride over the partial rows
-  const int G = SCAN_THREADS / E;
+struct ScanScratch {
+  int cnt[MAX_E];
+  float term[MAX_E];
+  float ps[SCAN_THREADS];
+  int seg[SCAN_THREADS];
+  TableScratch tab;
+};
+
+// Partial column sums of p: G groups of threads stride over the router's partial rows; sixteen loads in flight per thread,
+// combined in a fixed order (reproducible).
+__device__ __forceinline__ void psum_columns(int E, int psum_rows, const float* __restrict__ psum_part, ScanScratch& sh) {
+  const int tid = threadIdx.x, G = SCAN_THREADS / E;
   if (tid < G * E) {
     const int g = tid / E, e = tid - g * E;
-    // sixteen loads in flight per thread; the partial sums are combined in a fixed order
     float acc[16];
 #pragma unroll
     for (int u = 0; u < 16; ++u) acc[u] = 0.f;
@@ -270,8 +263,50 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_kernel(int64_t T, int E, in
 #pragma unroll
       for (int u = 0; u < 8; ++u)
         if (u < st) acc[u] += acc[u + st];
-    s_ps[tid] = acc[0];
+    sh.ps[tid] = acc[0];
   }
+}
+
+// counts, column sums of p, auxiliary loss and the scheduling tables, from complete sh.cnt and sh.ps (block synchronised)
+__device__ __forceinline__ void finish_tables(int64_t T, int E, int k, ScanScratch& sh, const TableOut& tabs,
+                                              float* __restrict__ psum, int32_t* __restrict__ counts_out,
+                                              float* __restrict__ aux_out) {
+  const int tid = threadIdx.x, G = SCAN_THREADS / E;
+  for (int e = tid; e < E; e += SCAN_THREADS) {
+    const int run = sh.cnt[e];
+    counts_out[e] = run;
+    float ps = 0.f;
+    for (int g = 0; g < G; ++g) ps += sh.ps[g * E + e];
+    psum[e] = ps;
+    // aux term: (c_e / (T k)) * (Psum_e / T)
+    sh.term[e] = (T > 0) ? (static_cast<float>(run) / static_cast<float>(T * k)) * (ps / static_cast<float>(T)) : 0.f;
+  }
+  __syncthreads();
+  if (tid >= 32 && tid < 64) {  // the second warp sums the aux terms in a fixed order while the first one scans
+    const int lane = tid - 32;
+    float sterm = 0.f;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) sterm += (lane * 8 + u < E) ? sh.term[lane * 8 + u] : 0.f;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) sterm += __shfl_xor_sync(0xFFFFFFFFu, sterm, off);
+    if (lane == 0) aux_out[0] = sterm * static_cast<float>(E);
+  }
+  build_expert_tables(E, sh.cnt, sh.tab, tabs);
+}
+
+// One block: column scan of tile_counts (in place -> exclusive prefix along tiles), counts, canonical and
+// padded offsets, tile -> expert table, and the auxiliary loss from the router's partial column sums of p.
+__global__ void __launch_bounds__(SCAN_THREADS) scan_kernel(int64_t T, int E, int k, int tok_tiles, int psum_rows,
+                                                            int32_t* __restrict__ tile_counts, const TableOut tabs,
+                                                            const float* __restrict__ psum_part,
+                                                            float* __restrict__ psum, int32_t* __restrict__ counts_out,
+                                                            float* __restrict__ aux_out) {
+  chain_wait();
+  chain_next();
+  __shared__ ScanScratch sh;
+  const int tid = threadIdx.x;
+  const int G = SCAN_THREADS / E;
+  psum_columns(E, psum_rows, psum_part, sh);
   __syncthreads();
   // exclusive prefix of every expert's column of tile_counts along the tiles.  The G thread groups cut the tiles into G
   // consecutive segments; thread (g, e) sums its segment of column e (lanes of a warp touch consecutive experts, so the
@@ -292,12 +327,12 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_kernel(int64_t T, int E, in
 #pragma unroll
         for (int u = 0; u < 16; ++u) total += c[u];
       }
-      s_seg[tid] = total;
+      sh.seg[tid] = total;
     }
     __syncthreads();
     if (mine) {
       int run = 0;
-      for (int q = 0; q < g; ++q) run += s_seg[q * E + e];
+      for (int q = 0; q < g; ++q) run += sh.seg[q * E + e];
       for (int t0 = t_lo; t0 < t_hi; t0 += 16) {
         int c[16];
 #pragma unroll
@@ -308,30 +343,129 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_kernel(int64_t T, int E, in
           run += c[u];
         }
       }
-      if (g == G - 1) s_cnt[e] = run;  // the last segment ends with the column total (empty segments pass it on)
+      if (g == G - 1) sh.cnt[e] = run;  // the last segment ends with the column total (empty segments pass it on)
     }
   }
   __syncthreads();
-  for (int e = tid; e < E; e += SCAN_THREADS) {
-    const int run = s_cnt[e];
-    counts_out[e] = run;
-    float ps = 0.f;
-    for (int g = 0; g < G; ++g) ps += s_ps[g * E + e];
-    psum[e] = ps;
-    // aux term: (c_e / (T k)) * (Psum_e / T)
-    s_term[e] = (T > 0) ? (static_cast<float>(run) / static_cast<float>(T * k)) * (ps / static_cast<float>(T)) : 0.f;
+  finish_tables(T, E, k, sh, tabs, psum, counts_out, aux_out);
+}
+
+// The permutation in one kernel, while every block can afford to look at all tile histograms (PLACE_MAX_TILES): block 0
+// builds the counts, tables and the auxiliary loss; block b + 1 places the picks of token tile b.  Each block sums the
+// columns of tile_counts itself - over all tiles (expert totals, hence segment starts) and over the tiles before its own
+// (first rank) - so nothing waits for a scan by one block.  Bound by two rounds of L2 latency.  Measured against scan_kernel
+// followed by scatter_kernel: 241 tokens 13 -> 5 us, 16384 tokens 25 -> 14 us.  The histograms are read once per block, so the
+// traffic grows with the square of the token count: 0.13 GB from L2 at 512 tiles of 128 experts.
+constexpr int PLACE_MAX_TILES = 512;
+__global__ void __launch_bounds__(SCAN_THREADS) place_kernel(int64_t T, int E, int k, int tok_tiles, int psum_rows,
+                                                             const int32_t* __restrict__ tile_counts, const TableOut tabs,
+                                                             const float* __restrict__ psum_part,
+                                                             float* __restrict__ psum, int32_t* __restrict__ counts_out,
+                                                             float* __restrict__ aux_out, const int32_t* __restrict__ idx,
+                                                             const float* __restrict__ gates, int32_t* __restrict__ inv,
+                                                             float* __restrict__ row_gate, int32_t* __restrict__ perm_out,
+                                                             int32_t* dbg_status, int64_t rows_max) {
+  chain_wait();
+  chain_next();
+  __shared__ ScanScratch sh;
+  __shared__ int s_before[MAX_E], s_off[MAX_E], s_pad[MAX_E];
+  extern __shared__ uint32_t pl_masks[];  // [TOK_WARPS][E]
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int G = SCAN_THREADS / E;
+  const int my_tile = static_cast<int>(blockIdx.x) - 1;  // -1: tables
+  const int64_t i0 = static_cast<int64_t>(my_tile) * TOK_TILE * k;
+  const int64_t n_picks = my_tile < 0 ? 0 : min(static_cast<int64_t>(TOK_TILE) * k, T * k - i0);
+  if (my_tile >= 0)
+    for (int i = tid; i < TOK_WARPS * E; i += SCAN_THREADS) pl_masks[i] = 0u;
+  {
+    const int g = tid / E, e = tid - g * E;
+    if (tid < G * E) {
+      int total = 0, before = 0;
+      for (int b0 = g; b0 < tok_tiles; b0 += 16 * G) {
+        int c[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) c[u] = (b0 + u * G < tok_tiles) ? tile_counts[static_cast<int64_t>(b0 + u * G) * E + e] : 0;
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {
+          total += c[u];
+          before += (b0 + u * G < my_tile) ? c[u] : 0;
+        }
+      }
+      sh.seg[tid] = total;
+      if (my_tile >= 0) sh.ps[tid] = __int_as_float(before);  // (the column sums of p use this array in block 0 only)
+    }
   }
   __syncthreads();
-  if (tid >= 32 && tid < 64) {  // the second warp sums the aux terms in a fixed order while the first one scans
-    const int lane = tid - 32;
-    float sterm = 0.f;
-#pragma unroll
-    for (int u = 0; u < 8; ++u) sterm += (lane * 8 + u < E) ? s_term[lane * 8 + u] : 0.f;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) sterm += __shfl_xor_sync(0xFFFFFFFFu, sterm, off);
-    if (lane == 0) aux_out[0] = sterm * static_cast<float>(E);
+  for (int i = tid; i < n_picks; i += SCAN_THREADS) {
+    const int tok = i / k;
+    const int e = idx[i0 + i];
+    if (dbg_status && (e < 0 || e >= E)) continue;
+    atomicOr(&pl_masks[(tok >> 5) * E + e], 1u << (tok & 31));
   }
-  build_expert_tables(E, s_cnt, s_tab, tabs);
+  for (int e = tid; e < E; e += SCAN_THREADS) {
+    int total = 0, before = 0;
+    for (int g = 0; g < G; ++g) {
+      total += sh.seg[g * E + e];
+      if (my_tile >= 0) before += __float_as_int(sh.ps[g * E + e]);
+    }
+    sh.cnt[e] = total;
+    s_before[e] = before;
+  }
+  __syncthreads();
+  if (my_tile < 0) {
+    psum_columns(E, psum_rows, psum_part, sh);
+    __syncthreads();
+    finish_tables(T, E, k, sh, tabs, psum, counts_out, aux_out);
+    return;
+  }
+  if (tid < 32) {  // segment starts: lane L owns experts 8L .. 8L+7
+    int cn[8], pd[8], scn = 0, spd = 0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int e = lane * 8 + u, c = e < E ? sh.cnt[e] : 0;
+      cn[u] = scn;
+      pd[u] = spd;
+      scn += c;
+      spd += (c + ROW_PAD - 1) / ROW_PAD * ROW_PAD;
+    }
+    int icn = scn, ipd = spd;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int a = __shfl_up_sync(0xFFFFFFFFu, icn, off), b = __shfl_up_sync(0xFFFFFFFFu, ipd, off);
+      if (lane >= off) {
+        icn += a;
+        ipd += b;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int e = lane * 8 + u;
+      if (e < E) {
+        s_off[e] = icn - scn + cn[u];
+        s_pad[e] = ipd - spd + pd[u];
+      }
+    }
+  }
+  __syncthreads();
+  for (int i = tid; i < n_picks; i += SCAN_THREADS) {
+    const int tok = i / k;
+    const int e = idx[i0 + i];
+    if (dbg_status && (e < 0 || e >= E)) {  // debug checks: record and skip instead of touching memory out of range
+      record_status(dbg_status, DEV_BOUNDS, 501);
+      continue;
+    }
+    int rank = s_before[e];
+    for (int w = 0; w < (tok >> 5); ++w) rank += __popc(pl_masks[w * E + e]);
+    rank += __popc(pl_masks[(tok >> 5) * E + e] & ((1u << (tok & 31)) - 1u));
+    const int r = s_pad[e] + rank;
+    if (dbg_status && (r < 0 || r >= rows_max)) {
+      record_status(dbg_status, DEV_BOUNDS, 502);
+      continue;
+    }
+    inv[i0 + i] = r;
+    row_gate[r] = gates[i0 + i];
+    if (perm_out) perm_out[s_off[e] + rank] = static_cast<int32_t>(i0 + i);
+  }
 }
 
 __global__ void __launch_bounds__(TOK_TILE) scatter_kernel(int64_t T, int E, int k, const int32_t* __restrict__ idx,
@@ -484,6 +618,16 @@ void launch_permute(const Shape& s, int64_t T, const WsLayout& L, char* ws, cons
   const size_t msm = sizeof(uint32_t) * TOK_WARPS * s.E;
   if (tiles > 0 && !histogram_done) {
     launch_kernel(hist_kernel, tiles, TOK_TILE, msm, st, T, s.E, s.k, idx, tile_counts);
+  }
+  if (tiles > 0 && !tables_only && tiles <= PLACE_MAX_TILES) {
+    launch_kernel(place_kernel, tiles + 1, SCAN_THREADS, msm, st, T, s.E, s.k, tiles, psum_rows, tile_counts,
+                  table_pointers(L, ws), reinterpret_cast<const float*>(ws + L.psum_part),
+                  reinterpret_cast<float*>(ws + L.psum), counts_out, aux_out, idx,
+                  reinterpret_cast<const float*>(ws + L.gates), reinterpret_cast<int32_t*>(ws + L.inv),
+                  reinterpret_cast<float*>(ws + L.row_gate), perm_out,
+                  debug ? reinterpret_cast<int32_t*>(ws + L.status) : nullptr, L.rows_max);
+    launch_gather_rows(s, T, L, ws, x, reinterpret_cast<uint16_t*>(ws + L.xp), st, debug, clear_pads);
+    return;
   }
   launch_kernel(scan_kernel, 1, SCAN_THREADS, 0, st, T, s.E, s.k, tiles, psum_rows, tile_counts,
                 table_pointers(L, ws), reinterpret_cast<const float*>(ws + L.psum_part),
