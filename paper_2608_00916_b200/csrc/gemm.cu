@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
       const int acc = tc & 1;
       const uint32_t aph = (tc >> 1) & 1u;
       ++tc;
-      epilogue_prefetch<KIND>(p, static_cast<int64_t>(tl.row0) + rin, tl.n0, half == 0, tl.e, tl.m0 + rin);
+      epilogue_prefetch<KIND>(p, static_cast<int64_t>(tl.row0) + rin, tl.n0, half == 0);
       clk.start();
       if (!mbar_wait(tfull_bar(acc), aph)) {
         ok = false;
@@ -588,15 +588,12 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
 }
 
 // Expected number of `size`-row tiles of an expert when the loads scatter around `mean` like independent picks
-// (variance = mean): sum over j of P(load > j size).
+// (variance = mean): sum over j of P(load > j size); from eight tiles on the last one is half full on average.
 static double expected_tiles(double mean, double size) {
+  if (mean >= 8.0 * size) return mean / size + 0.5;
   const double sd = sqrt(mean > 1.0 ? mean : 1.0);
-  double n = 0.0;
-  for (int j = 0; j < 4096; ++j) {
-    const double above = 0.5 * erfc((j * size - mean) / (sd * 1.4142135623730951));
-    n += j == 0 ? 1.0 : above;
-    if (j > 0 && above < 1e-3) break;
-  }
+  double n = 1.0;
+  for (int j = 1; j < 16; ++j) n += 0.5 * erfc((j * size - mean) / (sd * 1.4142135623730951));
   return n;
 }
 

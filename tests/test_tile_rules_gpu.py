@@ -24,6 +24,14 @@ def test_tile_shape_boundaries(T, d, E, k, f, seed):
     check_all(Run(inp, k), ofw, obw, 0.05)
 
 
+@pytest.mark.parametrize("T", [65536 - 127, 65536, 65537])
+def test_permutation_on_both_sides_of_its_token_limit(T):
+    """512 tiles of 128 tokens are placed by one kernel, more by a scan and a scatter: same routing, same layer."""
+    inp = synth.make_inputs(synth.MoEShape(T, 64, 8, 2, 64), 77, x_std=1.0)
+    ofw, obw = oracle_run(inp, 2, 0.05)
+    check_all(Run(inp, 2), ofw, obw, 0.05)
+
+
 @pytest.mark.parametrize("T,d,E,k,f,seed,flags", [
     (5, 64, 16, 2, 64, 81, 0),       # experts with one row or none
     (150, 192, 16, 2, 320, 82, 0),   # about 19 rows: one group of 32 per tile
