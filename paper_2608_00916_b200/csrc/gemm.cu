@@ -614,6 +614,13 @@ static double expected_tiles(double mean, double size) {
 // with few K blocks the output leaves as fast as HBM takes it (a plain fill runs at 3.9 TB/s here) only from one-CTA
 // tiles, whose two CTAs do not have to meet: wgrad-down / wgrad-gate/up 162 -> 172 / 322 -> 330 at 312 rows, equal at
 // 375, 200 -> 187 / 399 -> 374 at 437, 222 -> 195 / 430 -> 392 at 512.
+static bool row_gemm_on_pairs(const moe_ctx_impl* ctx, GemmKind kind, double rows_per_expert) {
+  if (ctx->tile_mode != 0) return ctx->tile_mode == 1;
+  if (kind == GEMM_B4 && ctx->b4_pair_override >= 0) return ctx->b4_pair_override != 0;
+  if (kind == GEMM_B2) return rows_per_expert >= 768.0;
+  return 0.80 * 2.0 * expected_tiles(rows_per_expert, 2 * BM) < expected_tiles(rows_per_expert, BM);
+}
+
 moe_status launch_grouped_gemm(moe_ctx_impl* ctx, GemmKind kind, int64_t T, const WsLayout& L, char* ws,
                                const GemmIO& io, cudaStream_t st) {
   const bool row_kind = kind == GEMM_F3 || kind == GEMM_F4 || kind == GEMM_B2 || kind == GEMM_B4;
@@ -624,14 +631,7 @@ moe_status launch_grouped_gemm(moe_ctx_impl* ctx, GemmKind kind, int64_t T, cons
     return launch_gemm_variant(ctx, kind, T, L, ws, io, st, pair, 0);
   }
   if (!row_kind) return launch_gemm_variant(ctx, kind, T, L, ws, io, st, false, 0);
-  bool pair = ctx->tile_mode == 1;
-  if (ctx->tile_mode == 0) {
-    if (kind == GEMM_B2)
-      pair = rows_per_expert >= 768.0;
-    else
-      pair = 0.80 * 2.0 * expected_tiles(rows_per_expert, 2 * BM) < expected_tiles(rows_per_expert, BM);
-    if (kind == GEMM_B4 && ctx->b4_pair_override >= 0) pair = ctx->b4_pair_override != 0;
-  }
+  const bool pair = row_gemm_on_pairs(ctx, kind, rows_per_expert);
   if (ctx->tile_mode != 3) return launch_gemm_variant(ctx, kind, T, L, ws, io, st, pair, 0);
   const moe_status rc = launch_gemm_variant(ctx, kind, T, L, ws, io, st, true, 1);
   if (rc != MOE_OK) return rc;
@@ -641,7 +641,6 @@ moe_status launch_grouped_gemm(moe_ctx_impl* ctx, GemmKind kind, int64_t T, cons
 // Backward operations of the expert-LoRA variant (see launch_lora_gemm below, which prepares `p`).
 static moe_status launch_lora_gemm_bwd(moe_ctx_impl* ctx, LoraOp op, int64_t T, const WsLayout& L, char* ws,
                                        const GemmIO& io, const LoraArgs& lo, GemmParams p, cudaStream_t st) {
-  (void)T;
   const Shape& s = ctx->s;
   const int d = s.d, f = s.f, E = s.E, r = lo.rank;
   const int64_t R = L.rows_max;
@@ -651,6 +650,9 @@ static moe_status launch_lora_gemm_bwd(moe_ctx_impl* ctx, LoraOp op, int64_t T, 
            *dhu = B16(L.dhu), *dxp = B16(L.dxp), *u = B16(L.lora_u), *v = B16(L.lora_v), *w = B16(L.lora_w),
            *z = B16(L.lora_z);
   const uint32_t skinny_tx = A_BYTES + CHUNK_BYTES;
+  const bool pair = (op == LORA_B2 || op == LORA_B4) &&
+                    row_gemm_on_pairs(ctx, op == LORA_B2 ? GEMM_B2 : GEMM_B4, static_cast<double>(T) * s.k / E);
+  const int nb = pair ? 128 : 256;  // rows of a K-major B box
   bool ok = true;
   switch (op) {
     case LORA_W:  // w[R,64] = s dy_rows B2[e]^T      (B4 kind, one segment, K-major B of 64 rows)
@@ -680,8 +682,8 @@ static moe_status launch_lora_gemm_bwd(moe_ctx_impl* ctx, LoraOp op, int64_t T, 
       if (!ok) return MOE_ERR_CUDA;
       return launch_kind<GEMM_B4>(ctx, p, st);
     case LORA_B2:  // da = dy_rows Wd^T + w A2^T, SwiGLU-backward epilogue
-      ok = map_2d(fn, &p.mapA0, dyr, R, d, 128) && map_3d(fn, &p.mapB0, io.W_down, E, f, d, 256) &&
-           map_2d(fn, &p.mapA2, w, R, 64, 128) && map_3d(fn, &p.mapB2, lo.A2, E, f, r, 256);
+      ok = map_2d(fn, &p.mapA0, dyr, R, d, 128) && map_3d(fn, &p.mapB0, io.W_down, E, f, d, nb) &&
+           map_2d(fn, &p.mapA2, w, R, 64, 128) && map_3d(fn, &p.mapB2, lo.A2, E, f, r, nb);
       p.mapA1 = p.mapA0; p.mapB1 = p.mapB0;
       p.n_tiles = (f + 255) / 256;
       p.k_blocks = d / BK;
@@ -693,11 +695,11 @@ static moe_status launch_lora_gemm_bwd(moe_ctx_impl* ctx, LoraOp op, int64_t T, 
       p.outf = reinterpret_cast<float*>(ws + L.dg_part);
       p.rows_max = L.rows_max;
       if (!ok) return MOE_ERR_CUDA;
-      return launch_kind<GEMM_B2>(ctx, p, st);
+      return pair ? launch_pair_gemm(ctx, GEMM_B2, p, st) : launch_kind<GEMM_B2>(ctx, p, st);
     case LORA_B4:  // dxp = dhg Wg^T + dhu Wu^T + z A1^T
       ok = map_2d(fn, &p.mapA0, dhg, R, f, 128) && map_2d(fn, &p.mapA1, dhu, R, f, 128) &&
-           map_3d(fn, &p.mapB0, io.W_gate, E, d, f, 256) && map_3d(fn, &p.mapB1, io.W_up, E, d, f, 256) &&
-           map_2d(fn, &p.mapA2, z, R, 64, 128) && map_3d(fn, &p.mapB2, lo.A1, E, d, r, 256);
+           map_3d(fn, &p.mapB0, io.W_gate, E, d, f, nb) && map_3d(fn, &p.mapB1, io.W_up, E, d, f, nb) &&
+           map_2d(fn, &p.mapA2, z, R, 64, 128) && map_3d(fn, &p.mapB2, lo.A1, E, d, r, nb);
       p.n_tiles = (d + 255) / 256;
       p.k_blocks = f / BK;
       p.nseg = 2;
@@ -706,7 +708,7 @@ static moe_status launch_lora_gemm_bwd(moe_ctx_impl* ctx, LoraOp op, int64_t T, 
       p.out0 = dxp;
       p.ld_out = d;
       if (!ok) return MOE_ERR_CUDA;
-      return launch_kind<GEMM_B4>(ctx, p, st);
+      return pair ? launch_pair_gemm(ctx, GEMM_B4, p, st) : launch_kind<GEMM_B4>(ctx, p, st);
     case LORA_DB2:  // dB2[e][r,d] = v_e^T dy_rows_e      (B3 kind, M = rank)
       ok = map_mn_rows(fn, &p.mapA0, v, R, 64, 2) && map_mn_rows(fn, &p.mapB0, dyr, R, d, 4);
       p.mapA1 = p.mapA0; p.mapB1 = p.mapB0;
@@ -757,7 +759,8 @@ static moe_status launch_lora_gemm_bwd(moe_ctx_impl* ctx, LoraOp op, int64_t T, 
 // The adapted layer reuses the kernels above with different operands: the low-rank path enters each row GEMM as one
 // extra 64-deep K segment ([xp | u] [[W]; [B1]], ...), the four 64-wide row buffers u, v, w, z come from skinny
 // instances (N = 64) of the F4 / B4 kinds, and the adapter gradients from instances of the B3 / B5 kinds whose M or
-// N is the rank.  All on one-CTA tiles.
+// N is the rank.  The four large ones take the tile shape the plain layer would
+// (rank 16, 8192 tokens, 512 rows per expert: a step 2132 -> 2079 us), the others one-CTA tiles.
 moe_status launch_lora_gemm(moe_ctx_impl* ctx, LoraOp op, int64_t T, const WsLayout& L, char* ws, const GemmIO& io,
                             const LoraArgs& lo, cudaStream_t st) {
   const Shape& s = ctx->s;
@@ -775,6 +778,8 @@ moe_status launch_lora_gemm(moe_ctx_impl* ctx, LoraOp op, int64_t T, const WsLay
   p.pad_offsets = reinterpret_cast<const int32_t*>(ws + L.pad_offsets);
   p.counts = reinterpret_cast<const int32_t*>(ws + L.counts);
   p.pair_tab = reinterpret_cast<const int32_t*>(ws + L.pair_tab);
+  p.pair_count_slot = 2;
+  p.oob_row = static_cast<int>(R);
   p.expert_order = reinterpret_cast<const int32_t*>(ws + L.expert_order);
   p.status = reinterpret_cast<int32_t*>(ws + L.status);
   p.E = E;
@@ -784,6 +789,8 @@ moe_status launch_lora_gemm(moe_ctx_impl* ctx, LoraOp op, int64_t T, const WsLay
   p.out_scale = 1.f;
   p.row_gate = reinterpret_cast<const float*>(ws + L.row_gate);
   const uint32_t skinny_tx = A_BYTES + CHUNK_BYTES;  // a 128 x 64 A tile and one 64 x 64 B tile
+  const bool pair = (op == LORA_F3 || op == LORA_F4) &&
+                    row_gemm_on_pairs(ctx, op == LORA_F3 ? GEMM_F3 : GEMM_F4, static_cast<double>(T) * s.k / E);
   bool ok = true;
   switch (op) {
     case LORA_U:  // u[R,64] = s xp A1[e]            (F4 kind, N = 64)
@@ -813,10 +820,10 @@ moe_status launch_lora_gemm(moe_ctx_impl* ctx, LoraOp op, int64_t T, const WsLay
       p.ld_out = f;
       p.save_pre = 1;
       if (!ok) return MOE_ERR_CUDA;
-      return launch_kind<GEMM_F3>(ctx, p, st);
+      return pair ? launch_pair_gemm(ctx, GEMM_F3, p, st) : launch_kind<GEMM_F3>(ctx, p, st);
     case LORA_F4:  // o = act Wd + v B2
-      ok = map_2d(fn, &p.mapA0, act, R, f, 128) && map_mn(fn, &p.mapB0, io.W_down, E, f, d, 4) &&
-           map_2d(fn, &p.mapA2, v, R, 64, 128) && map_mn(fn, &p.mapB2, lo.B2, E, r, d, 4);
+      ok = map_2d(fn, &p.mapA0, act, R, f, 128) && map_mn(fn, &p.mapB0, io.W_down, E, f, d, pair ? 2 : 4) &&
+           map_2d(fn, &p.mapA2, v, R, 64, 128) && map_mn(fn, &p.mapB2, lo.B2, E, r, d, pair ? 2 : 4);
       p.mapA1 = p.mapA0; p.mapB1 = p.mapB0;
       p.n_tiles = (d + 255) / 256;
       p.k_blocks = f / BK;
@@ -825,7 +832,7 @@ moe_status launch_lora_gemm(moe_ctx_impl* ctx, LoraOp op, int64_t T, const WsLay
       p.out0 = o;
       p.ld_out = d;
       if (!ok) return MOE_ERR_CUDA;
-      return launch_kind<GEMM_F4>(ctx, p, st);
+      return pair ? launch_pair_gemm(ctx, GEMM_F4, p, st) : launch_kind<GEMM_F4>(ctx, p, st);
     default:
       break;
   }

@@ -70,7 +70,7 @@ __device__ __forceinline__ Tile2 get_tile2(const GemmParams& p, int t, int rank)
     tl.full = info.z == 2;
     tl.m0 = 0;
     tl.n0 = nt * Traits<KIND>::N_SPAN;
-    tl.nkb = p.k_blocks * p.nseg;
+    tl.nkb = p.k_blocks * p.nseg + p.k_blocks1;
   }
   return tl;
 }
@@ -79,6 +79,17 @@ __device__ __forceinline__ Tile2 get_tile2(const GemmParams& p, int t, int rank)
 template <int KIND>
 __device__ __forceinline__ void issue_loads2(const GemmParams& p, const Tile2& tl, int kb, int rank, uint32_t sA,
                                              uint32_t sB, uint32_t bar) {
+  if (!Traits<KIND>::WGRAD && kb >= p.k_blocks * p.nseg) {  // extra K segment of the low-rank adapter path
+    const int kk = kb - p.k_blocks * p.nseg;
+    tma_load_2d_pair(sA, &p.mapA2, bar, kk * BK, tl.write ? tl.row0 : p.oob_row);
+    if (KIND == GEMM_F3)
+      tma_load_4d_pair(sB, rank ? &p.mapB3 : &p.mapB2, bar, 0, kk * BK, tl.n0 / 64, tl.e);
+    else if (KIND == GEMM_F4)
+      tma_load_4d_pair(sB, &p.mapB2, bar, 0, kk * BK, tl.n0 / 64 + rank * 2, tl.e);
+    else
+      tma_load_3d_pair(sB, &p.mapB2, bar, kk * BK, tl.n0 + rank * 128, tl.e);
+    return;
+  }
   if (KIND == GEMM_F3) {
     load_a_rows<true>(p, sA, bar, kb * BK, tl.row0, tl.valid);
     const CUtensorMap* mb = rank ? &p.mapB1 : &p.mapB0;  // leader: gate columns, partner: the matching up columns

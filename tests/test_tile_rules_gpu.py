@@ -6,6 +6,7 @@ import torch
 from paper_2608_00916_b200 import synth
 from gpu_util import Run, oracle_run
 from test_gpu_parity import check_all
+from test_gpu_parity import test_expert_lora_against_the_oracle as lora_against_the_oracle
 
 pytestmark = pytest.mark.gpu
 
@@ -52,3 +53,12 @@ def test_scoring_never_uses_pad_rows(T, d, E, k, f, seed, flags):
     r.layer.poll()
     assert torch.equal(got["y"], train["y"])
     assert torch.isfinite(got["y"].float()).all()
+
+
+@pytest.mark.parametrize("T,d,E,k,f,rank,seed", [
+    (640, 192, 8, 2, 320, 16, 91),    # 160 rows per expert: gate/up, down and dgrad gate/up on pairs
+    (1024, 128, 8, 2, 192, 8, 92),    # 256: pairs whose second half is often empty
+    (3080, 192, 8, 2, 128, 64, 93),   # 770: dgrad-down on pairs as well, largest rank
+])
+def test_adapters_on_pairs(T, d, E, k, f, rank, seed):
+    lora_against_the_oracle(T, d, E, k, f, rank, seed)
