@@ -128,8 +128,9 @@ __global__ void __launch_bounds__(256) router_kernel(int64_t T, int d, int E, in
       int bi = 0x7FFFFFFF;
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
-        if (!((taken >> q) & 1u) && (bi == 0x7FFFFFFF || v[q] > bv)) {
-          bv = v[q];
+        const float sv = fmaxf(v[q], -INFINITY);  // NaN counts as -inf: all lanes agree on the order
+        if (!((taken >> q) & 1u) && (bi == 0x7FFFFFFF || sv > bv)) {
+          bv = sv;
           bi = lane + 32 * q;
         }
       }
@@ -205,6 +206,8 @@ void launch_router(const Shape& s, int64_t T, const uint16_t* x, const uint16_t*
 // the order inside an expert is the token order.  Each warp covers 32 consecutive tokens and records, per
 // expert, the 32-bit mask of its tokens that chose it (atomicOr: order-free, hence deterministic); ranks
 // are population counts of mask prefixes.  Tiles of TOK_TILE tokens are combined by a column scan.
+// The routers above and in gemm_common.cuh write k distinct experts in [0, E) for every token, NaN logits included.  The
+// kernels below index with them; a pick out of that range (an overwritten workspace) never leaves their tables.
 __device__ __forceinline__ void build_masks(uint32_t* masks /* [TOK_WARPS][E] */, const int32_t* __restrict__ idx, int64_t T,
                                             int E, int k, int64_t tile_t0) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -214,7 +217,7 @@ __device__ __forceinline__ void build_masks(uint32_t* masks /* [TOK_WARPS][E] */
   if (t < T) {
     for (int j = 0; j < k; ++j) {
       int e = idx[t * k + j];
-      atomicOr(&masks[warp * E + e], 1u << lane);
+      if (static_cast<unsigned>(e) < static_cast<unsigned>(E)) atomicOr(&masks[warp * E + e], 1u << lane);
     }
   }
   __syncthreads();
@@ -399,7 +402,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) place_kernel(int64_t T, int E, i
   for (int i = tid; i < n_picks; i += SCAN_THREADS) {
     const int tok = i / k;
     const int e = idx[i0 + i];
-    if (dbg_status && (e < 0 || e >= E)) continue;
+    if (static_cast<unsigned>(e) >= static_cast<unsigned>(E)) continue;
     atomicOr(&pl_masks[(tok >> 5) * E + e], 1u << (tok & 31));
   }
   for (int e = tid; e < E; e += SCAN_THREADS) {
@@ -450,8 +453,8 @@ __global__ void __launch_bounds__(SCAN_THREADS) place_kernel(int64_t T, int E, i
   for (int i = tid; i < n_picks; i += SCAN_THREADS) {
     const int tok = i / k;
     const int e = idx[i0 + i];
-    if (dbg_status && (e < 0 || e >= E)) {  // debug checks: record and skip instead of touching memory out of range
-      record_status(dbg_status, DEV_BOUNDS, 501);
+    if (static_cast<unsigned>(e) >= static_cast<unsigned>(E)) {
+      if (dbg_status) record_status(dbg_status, DEV_BOUNDS, 501);
       continue;
     }
     int rank = s_before[e];
@@ -487,8 +490,8 @@ __global__ void __launch_bounds__(TOK_TILE) scatter_kernel(int64_t T, int E, int
   if (t >= T) return;
   for (int j = 0; j < k; ++j) {
     const int e = idx[t * k + j];
-    if (dbg_status && (e < 0 || e >= E)) {  // debug checks: record and skip instead of touching memory out of range
-      record_status(dbg_status, DEV_BOUNDS, 501);
+    if (static_cast<unsigned>(e) >= static_cast<unsigned>(E)) {
+      if (dbg_status) record_status(dbg_status, DEV_BOUNDS, 501);
       continue;
     }
     int rank = tile_base[static_cast<int64_t>(blockIdx.x) * E + e];
