@@ -8,8 +8,8 @@ namespace moe {
 // y[t,:] = sum_{j<k} o[inv[t,j],:] where the rows of o already carry their gate (the gate-up epilogue folds it into
 // the activation); fp32 accumulation in slot order, one bf16 rounding.
 // One block per token; a thread owns 8 consecutive columns (16 bytes) and issues the k row loads back to back.
-__global__ void __launch_bounds__(256) combine_kernel(int d, int k, const uint16_t* __restrict__ o,
-                                                      const float* __restrict__ gates, const int32_t* __restrict__ inv,
+__global__ void __launch_bounds__(256) combine_kernel(int d, int k, const uint16_t* o,
+                                                      const float* gates, const int32_t* inv,
                                                       uint16_t* __restrict__ y, int32_t* dbg_status, int64_t rows_max) {
   chain_wait();
   chain_next();
@@ -31,7 +31,7 @@ __global__ void __launch_bounds__(256) combine_kernel(int d, int k, const uint16
     for (int i = 0; i < 8; ++i) acc[i] = 0.f;
 #pragma unroll 8
     for (int j = 0; j < k; ++j) {
-      const uint4 v = __ldg(reinterpret_cast<const uint4*>(o + static_cast<int64_t>(sr[j]) * d + c));
+      const uint4 v = *reinterpret_cast<const uint4*>(o + static_cast<int64_t>(sr[j]) * d + c);
       float a, b;
       unpack_bf16x2(v.x, a, b); acc[0] += a; acc[1] += b;
       unpack_bf16x2(v.y, a, b); acc[2] += a; acc[3] += b;
@@ -58,13 +58,13 @@ void launch_combine(const Shape& s, int64_t T, const uint16_t* o, const float* g
 // sums written by the dgrad-down epilogue (one slice per column tile) and is summed here in slice order.
 //   dl[t,e]  = p_e (dp_e - <p, dp>)                       auxiliary loss through P_e, dp_e = d_aux E c_e / (T k) / T
 //   dl[t,idx_j] += g_j (dg_j - sum_j' g_j' dg_j')         gates = softmax over the selected logits
-__global__ void __launch_bounds__(256) router_bwd_kernel(int64_t T, int E, int k, const float* __restrict__ logits,
-                                                         const int32_t* __restrict__ idx,
-                                                         const float* __restrict__ gates,
-                                                         const float* __restrict__ dg_part, int dg_tiles,
-                                                         int64_t rows_max, const int32_t* __restrict__ inv,
-                                                         float* __restrict__ dg,
-                                                         const int32_t* __restrict__ counts, float d_aux,
+__global__ void __launch_bounds__(256) router_bwd_kernel(int64_t T, int E, int k, const float* logits,
+                                                         const int32_t* idx,
+                                                         const float* gates,
+                                                         const float* dg_part, int dg_tiles,
+                                                         int64_t rows_max, const int32_t* inv,
+                                                         float* dg,
+                                                         const int32_t* counts, float d_aux,
                                                          float* __restrict__ dl, uint16_t* __restrict__ dl_hi,
                                                          uint16_t* __restrict__ dl_lo, int32_t* dbg_status) {
   chain_wait();
@@ -171,7 +171,7 @@ void launch_router_bwd(const Shape& s, int64_t T, const float* logits, const int
 constexpr int DW_BM = 64, DW_BK = 32;
 
 __global__ void __launch_bounds__(256) dwr_partial_kernel(int64_t T, int d, int E, const uint16_t* __restrict__ x,
-                                                          const float* __restrict__ dl, float* __restrict__ part) {
+                                                          const float* dl, float* __restrict__ part) {
   chain_wait();
   chain_next();
   // thread layout: 16 (row groups of 4) x 16 (column groups); columns handled: cg + 16*i for i < E/16 (<= 16)
@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(256) dwr_partial_kernel(int64_t T, int d, int 
     }
 }
 
-__global__ void dwr_reduce_kernel(int64_t n, const float* __restrict__ part, float* __restrict__ dW_r,
+__global__ void dwr_reduce_kernel(int64_t n, const float* part, float* __restrict__ dW_r,
                                   int accumulate) {
   chain_wait();
   chain_next();
@@ -243,7 +243,7 @@ __global__ void dwr_reduce_kernel(int64_t n, const float* __restrict__ part, flo
 }
 
 // db_r[e] = sum_t dl[t,e]: one block per 32 experts, 8 warps stride over the tokens, fixed-order final sum.
-__global__ void __launch_bounds__(256) dbr_kernel(int64_t T, int E, const float* __restrict__ dl,
+__global__ void __launch_bounds__(256) dbr_kernel(int64_t T, int E, const float* dl,
                                                   float* __restrict__ db_r, int accumulate) {
   chain_wait();
   chain_next();
@@ -283,9 +283,9 @@ void launch_dwr(const Shape& s, int64_t T, const uint16_t* x, const float* dl, f
 constexpr int UB_TOK = 8;
 
 __global__ void __launch_bounds__(256) unpermute_bwd_kernel(int64_t T, int d, int E, int k,
-                                                            const uint16_t* __restrict__ dxp,
-                                                            const int32_t* __restrict__ inv,
-                                                            const float* __restrict__ dl,
+                                                            const uint16_t* dxp,
+                                                            const int32_t* inv,
+                                                            const float* dl,
                                                             const uint16_t* __restrict__ W_r,
                                                             uint16_t* __restrict__ dx) {
   chain_wait();
@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(256) unpermute_bwd_kernel(int64_t T, int d, in
       const int64_t t = t0 + tk;
       if (t < T) {
         for (int j = 0; j < k; ++j) {
-          const uint4 v = __ldg(reinterpret_cast<const uint4*>(dxp + static_cast<int64_t>(s_inv[tk][j]) * d + c));
+          const uint4 v = *reinterpret_cast<const uint4*>(dxp + static_cast<int64_t>(s_inv[tk][j]) * d + c);
           float a, b;
           unpack_bf16x2(v.x, a, b); acc[tk][0] += a; acc[tk][1] += b;
           unpack_bf16x2(v.y, a, b); acc[tk][2] += a; acc[tk][3] += b;
@@ -372,9 +372,9 @@ __global__ void __launch_bounds__(256) unpermute_bwd_kernel(int64_t T, int d, in
 }
 
 // dx[t,:] = dxr[t,:] + sum_j dxp[inv[t,j],:]; one block per token, 16-byte accesses, all row loads in flight at once.
-__global__ void __launch_bounds__(256) unpermute_sum_kernel(int d, int k, const uint16_t* __restrict__ dxp,
-                                                            const int32_t* __restrict__ inv,
-                                                            const uint16_t* __restrict__ dxr,
+__global__ void __launch_bounds__(256) unpermute_sum_kernel(int d, int k, const uint16_t* dxp,
+                                                            const int32_t* inv,
+                                                            const uint16_t* dxr,
                                                             uint16_t* __restrict__ dx, int32_t* dbg_status,
                                                             int64_t rows_max) {
   chain_wait();
@@ -393,7 +393,7 @@ __global__ void __launch_bounds__(256) unpermute_sum_kernel(int d, int k, const 
   for (int c = threadIdx.x * 8; c < d; c += 256 * 8) {
     float acc[8];
     {
-      const uint4 v = __ldg(reinterpret_cast<const uint4*>(dxr + t * d + c));
+      const uint4 v = *reinterpret_cast<const uint4*>(dxr + t * d + c);
       unpack_bf16x2(v.x, acc[0], acc[1]);
       unpack_bf16x2(v.y, acc[2], acc[3]);
       unpack_bf16x2(v.z, acc[4], acc[5]);
@@ -401,7 +401,7 @@ __global__ void __launch_bounds__(256) unpermute_sum_kernel(int d, int k, const 
     }
 #pragma unroll 8
     for (int j = 0; j < k; ++j) {
-      const uint4 v = __ldg(reinterpret_cast<const uint4*>(dxp + static_cast<int64_t>(sr[j]) * d + c));
+      const uint4 v = *reinterpret_cast<const uint4*>(dxp + static_cast<int64_t>(sr[j]) * d + c);
       float a, b;
       unpack_bf16x2(v.x, a, b); acc[0] += a; acc[1] += b;
       unpack_bf16x2(v.y, a, b); acc[2] += a; acc[3] += b;

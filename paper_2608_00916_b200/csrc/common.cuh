@@ -313,7 +313,11 @@ inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, si
 }
 
 // ---- device helpers
-// Waits for the previous kernel of the chain (a no-op in a kernel launched plainly).
+// Waits for the previous kernel of the chain (a no-op in a kernel launched plainly).  A chained kernel is resident while
+// its predecessor still writes, so what an earlier kernel of the same call writes is not read-only for this one's
+// lifetime: pointers to such buffers carry no __restrict__ and are not read by __ldg, either of which would let the
+// compiler load through the non-coherent path or above this wait.  Both are for the call's inputs (x, dy, the weights)
+// and for what an earlier call left in the workspace.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Lets the next kernel of the chain be set up once every block of this one has got here or ended.
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -208,7 +208,7 @@ void launch_router(const Shape& s, int64_t T, const uint16_t* x, const uint16_t*
 // are population counts of mask prefixes.  Tiles of TOK_TILE tokens are combined by a column scan.
 // The routers above and in gemm_common.cuh write k distinct experts in [0, E) for every token, NaN logits included.  The
 // kernels below index with them; a pick out of that range (an overwritten workspace) never leaves their tables.
-__device__ __forceinline__ void build_masks(uint32_t* masks /* [TOK_WARPS][E] */, const int32_t* __restrict__ idx, int64_t T,
+__device__ __forceinline__ void build_masks(uint32_t* masks /* [TOK_WARPS][E] */, const int32_t* idx, int64_t T,
                                             int E, int k, int64_t tile_t0) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int i = tid; i < TOK_WARPS * E; i += TOK_TILE) masks[i] = 0u;
@@ -223,7 +223,7 @@ __device__ __forceinline__ void build_masks(uint32_t* masks /* [TOK_WARPS][E] */
   __syncthreads();
 }
 
-__global__ void __launch_bounds__(TOK_TILE) hist_kernel(int64_t T, int E, int k, const int32_t* __restrict__ idx,
+__global__ void __launch_bounds__(TOK_TILE) hist_kernel(int64_t T, int E, int k, const int32_t* idx,
                                                         int32_t* __restrict__ tile_counts) {
   chain_wait();
   chain_next();
@@ -248,7 +248,7 @@ struct ScanScratch {
 
 // Partial column sums of p: G groups of threads stride over the router's partial rows; sixteen loads in flight per thread,
 // combined in a fixed order (reproducible).
-__device__ __forceinline__ void psum_columns(int E, int psum_rows, const float* __restrict__ psum_part, ScanScratch& sh) {
+__device__ __forceinline__ void psum_columns(int E, int psum_rows, const float* psum_part, ScanScratch& sh) {
   const int tid = threadIdx.x, G = SCAN_THREADS / E;
   if (tid < G * E) {
     const int g = tid / E, e = tid - g * E;
@@ -300,8 +300,8 @@ __device__ __forceinline__ void finish_tables(int64_t T, int E, int k, ScanScrat
 // One block: column scan of tile_counts (in place -> exclusive prefix along tiles), counts, canonical and
 // padded offsets, tile -> expert table, and the auxiliary loss from the router's partial column sums of p.
 __global__ void __launch_bounds__(SCAN_THREADS) scan_kernel(int64_t T, int E, int k, int tok_tiles, int psum_rows,
-                                                            int32_t* __restrict__ tile_counts, const TableOut tabs,
-                                                            const float* __restrict__ psum_part,
+                                                            int32_t* tile_counts, const TableOut tabs,
+                                                            const float* psum_part,
                                                             float* __restrict__ psum, int32_t* __restrict__ counts_out,
                                                             float* __restrict__ aux_out) {
   chain_wait();
@@ -361,11 +361,11 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_kernel(int64_t T, int E, in
 // traffic grows with the square of the token count: 0.13 GB from L2 at 512 tiles of 128 experts.
 constexpr int PLACE_MAX_TILES = 512;
 __global__ void __launch_bounds__(SCAN_THREADS) place_kernel(int64_t T, int E, int k, int tok_tiles, int psum_rows,
-                                                             const int32_t* __restrict__ tile_counts, const TableOut tabs,
-                                                             const float* __restrict__ psum_part,
+                                                             const int32_t* tile_counts, const TableOut tabs,
+                                                             const float* psum_part,
                                                              float* __restrict__ psum, int32_t* __restrict__ counts_out,
-                                                             float* __restrict__ aux_out, const int32_t* __restrict__ idx,
-                                                             const float* __restrict__ gates, int32_t* __restrict__ inv,
+                                                             float* __restrict__ aux_out, const int32_t* idx,
+                                                             const float* gates, int32_t* __restrict__ inv,
                                                              float* __restrict__ row_gate, int32_t* __restrict__ perm_out,
                                                              int32_t* dbg_status, int64_t rows_max) {
   chain_wait();
@@ -471,11 +471,11 @@ __global__ void __launch_bounds__(SCAN_THREADS) place_kernel(int64_t T, int E, i
   }
 }
 
-__global__ void __launch_bounds__(TOK_TILE) scatter_kernel(int64_t T, int E, int k, const int32_t* __restrict__ idx,
-                                                           const int32_t* __restrict__ tile_base,
-                                                           const int32_t* __restrict__ offsets,
-                                                           const int32_t* __restrict__ pad_offsets,
-                                                           const float* __restrict__ gates,
+__global__ void __launch_bounds__(TOK_TILE) scatter_kernel(int64_t T, int E, int k, const int32_t* idx,
+                                                           const int32_t* tile_base,
+                                                           const int32_t* offsets,
+                                                           const int32_t* pad_offsets,
+                                                           const float* gates,
                                                            int32_t* __restrict__ inv,
                                                            float* __restrict__ row_gate,
                                                            int32_t* __restrict__ perm_out, int32_t* dbg_status,
@@ -515,9 +515,9 @@ __global__ void __launch_bounds__(TOK_TILE) scatter_kernel(int64_t T, int E, int
 // Blocks past the token range zero the pad rows, one expert per block.
 __global__ void __launch_bounds__(256) scatter_rows_kernel(int64_t T, int d, int k, int E, int tok_blocks,
                                                            const uint16_t* __restrict__ src,
-                                                           const int32_t* __restrict__ inv,
-                                                           const int32_t* __restrict__ counts,
-                                                           const int32_t* __restrict__ pad_offsets,
+                                                           const int32_t* inv,
+                                                           const int32_t* counts,
+                                                           const int32_t* pad_offsets,
                                                            uint16_t* __restrict__ rows, int32_t* dbg_status,
                                                            int64_t rows_max) {
   chain_wait();

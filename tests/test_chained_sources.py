@@ -1,0 +1,35 @@
+"""What the sources of chained kernels (launched while their predecessor still writes) have to keep to, read from the files."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2608_00916_b200", "csrc")
+FILES = ("route.cu", "combine.cu", "gemm.cu", "gemm2.cu", "gemm_common.cuh")
+# what the caller hands in, complete before the first kernel of the call: x / dy (src), the router's weight, bias and logits
+INPUTS = {"x", "src", "w", "W_r", "b_r", "logits_in"}
+
+
+def sources():
+    for name in FILES:
+        with open(os.path.join(CSRC, name)) as f:
+            yield name, f.read()
+
+
+def test_predecessor_outputs_are_not_declared_read_only():
+    kernels = 0
+    for name, text in sources():
+        for m in re.finditer(r"__global__ [^;{]*?(\w+)\(([^{;]*?)\) \{\s+chain_wait\(\);", text):
+            kernels += 1
+            for param in m.group(2).split(","):
+                if "const" in param and "__restrict__" in param:
+                    assert param.split()[-1] in INPUTS, f"{name}: {m.group(1)}: {param.strip()}"
+        for helper, what in (("build_masks", "idx"), ("psum_columns", "psum_part"), ("scan_kernel", "tile_counts")):
+            assert not re.search(helper + r"\([^{;]*__restrict__ " + what + r"\b", text), f"{name}: {helper}: {what}"
+    assert kernels >= 12
+
+
+def test_non_coherent_loads_are_of_inputs_only():
+    loads = [(name, arg) for name, text in sources() for arg in re.findall(r"__ldg\(([^;]*)\);", text)]
+    assert loads
+    for name, arg in loads:
+        # W_r, the rows of src (s4), and hg / hu (qh, qu), which the forward call has left in the workspace
+        assert re.search(r"\b(W_r|s4|qh|qu)\b", arg), f"{name}: __ldg({arg})"
