@@ -294,8 +294,14 @@ class Chain {
   static thread_local Chain* current_;
 };
 
-template <typename... P, typename... A>
-inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+// The arguments convert to the kernel's parameter types implicitly, as in <<<>>>, and not otherwise.
+template <typename T>
+struct Param {
+  using type = T;
+};
+template <typename... P>
+inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                 const typename Param<P>::type&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -306,7 +312,7 @@ inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, si
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = Chain::follows(st) ? 1 : 0;
-  const cudaError_t rc = cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+  const cudaError_t rc = cudaLaunchKernelEx(&cfg, kernel, args...);
   Chain::launched(st);
   note_launch();
   return rc;

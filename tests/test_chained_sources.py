@@ -1,6 +1,9 @@
 """What the sources of chained kernels (launched while their predecessor still writes) have to keep to, read from the files."""
 import os
 import re
+import subprocess
+
+from paper_2608_00916_b200 import build
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2608_00916_b200", "csrc")
 FILES = ("route.cu", "combine.cu", "gemm.cu", "gemm2.cu", "gemm_common.cuh")
@@ -33,3 +36,21 @@ def test_non_coherent_loads_are_of_inputs_only():
     for name, arg in loads:
         # W_r, the rows of src (s4), and hg / hu (qh, qu), which the forward call has left in the workspace
         assert re.search(r"\b(W_r|s4|qh|qu)\b", arg), f"{name}: __ldg({arg})"
+
+
+def compiles(tmp_path, argument):
+    src = tmp_path / "launch.cu"
+    src.write_text('#include "common.cuh"\n'
+                   "__global__ void kernel(const float* in, long n) {}\n"
+                   "void go(float* f, const unsigned short* u, cudaStream_t st) {\n"
+                   f"  moe::launch_kernel(kernel, 1, 32, 0, st, {argument}, 7);\n"
+                   "}\n")
+    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+    return subprocess.run([nvcc, *build.NVCC_FLAGS, "-I", CSRC, "-c", str(src), "-o", str(tmp_path / "launch.o")],
+                          stdout=subprocess.DEVNULL, stderr=subprocess.DEVNULL).returncode == 0
+
+
+def test_launch_arguments_convert_as_in_a_plain_launch(tmp_path):
+    assert compiles(tmp_path, "f") and compiles(tmp_path, "nullptr")
+    assert not compiles(tmp_path, "u")  # another pointer type
+    assert not compiles(tmp_path, "7")  # a number
