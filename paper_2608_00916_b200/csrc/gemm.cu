@@ -280,6 +280,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     }
   }
 
+  __syncwarp();  // the 31 lanes that passed by a one-thread role meet it here: what follows is executed by whole warps
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {

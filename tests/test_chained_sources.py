@@ -38,6 +38,15 @@ def test_non_coherent_loads_are_of_inputs_only():
         assert re.search(r"\b(W_r|s4|qh|qu)\b", arg), f"{name}: __ldg({arg})"
 
 
+def test_warps_reconverge_after_the_one_thread_roles():
+    """elect_one() sends one lane through a role's loop; the barriers and the tensor-memory instructions after it are for
+    whole warps."""
+    for name, text in sources():
+        if name in ("gemm.cu", "gemm2.cu"):
+            after = text[text.rindex("elect_one()"):]
+            assert re.search(r"\n  \}\n\n  __syncwarp\(\);[^\n]*\n  tc_fence_before\(\);\n  (__syncthreads|cluster_sync_all)", after), name
+
+
 def compiles(tmp_path, argument):
     src = tmp_path / "launch.cu"
     src.write_text('#include "common.cuh"\n'
