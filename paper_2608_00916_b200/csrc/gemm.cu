@@ -192,7 +192,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     EpiStage es{smem_base + STAGES * STAGE_BYTES + (warp - 2) * (EPI_UNITS * EPI_UNIT_BYTES), 0u};
     uint32_t tc = 0;
     bool ok = true;
-    RoleClock clk(p.timers);
+    auto clocked = [&]() { return p.timers && threadIdx.x == 64; };  // asked again each time: a flag would cost a register
+    if (clocked()) sum_cycles(p.timers + 5, false);  // total
     for (int rd = 0; rd * static_cast<int>(gridDim.x) < ntiles && ok; ++rd) {
       const int t = tile_of_round<KIND>(rd, blockIdx.x, gridDim.x);
       if (t >= ntiles) continue;
@@ -216,12 +217,12 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
       const uint32_t aph = (tc >> 1) & 1u;
       ++tc;
       epilogue_prefetch<KIND>(p, static_cast<int64_t>(tl.row0) + rin, tl.n0, half == 0);
-      clk.start();
+      if (clocked()) sum_cycles(p.timers + 6, false);  // waiting for a finished accumulator
       if (!mbar_wait(tfull_bar(acc), aph)) {
         ok = false;
         break;
       }
-      clk.add(0);
+      if (clocked()) sum_cycles(p.timers + 6, true);
       tc_fence_after();
       const uint32_t taddr = tmem_base + (static_cast<uint32_t>(ew * 32) << 16) + acc * ACC_COLS;
       const int64_t row = static_cast<int64_t>(tl.row0) + rin;
@@ -271,9 +272,9 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
       }
       if (KIND == GEMM_RT || KIND == GEMM_DWR) release();
     }
-    if (lane == 0 && ew == 0 && half == 0) {
-      clk.report(5, 6);  // total; waiting for a finished accumulator
-      if (p.timers) atomicAdd(p.timers + 7, 1ull);  // CTAs counted
+    if (clocked()) {
+      sum_cycles(p.timers + 5, true);
+      atomicAdd(p.timers + 7, 1ull);  // CTAs counted
     }
     if (!ok && lane == 0) {
       record_status(p.status, DEV_TIMEOUT, 300 + KIND);

@@ -262,7 +262,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
     EpiStage es{smem_base + STAGES2 * STAGE2_BYTES + (warp - 2) * (EPI_UNITS * EPI_UNIT_BYTES), 0u};
     uint32_t tc = 0;
     bool ok = true;
-    RoleClock clk(p.timers);
+    const bool clocked = p.timers && leader && threadIdx.x == 64;
+    if (clocked) sum_cycles(p.timers + 5, false);  // total
     for (int rd = 0; rd * nclusters < ntiles && ok; ++rd) {
       const int t = tile_of_round<KIND>(rd, cid, nclusters);
       if (t >= ntiles) continue;
@@ -276,12 +277,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
       const uint32_t aph = (tc >> 1) & 1u;
       ++tc;
       epilogue_prefetch<KIND>(p, static_cast<int64_t>(tl.row0) + rin, tl.n0, tl.write && half == 0);
-      clk.start();
+      if (clocked) sum_cycles(p.timers + 6, false);  // waiting for a finished accumulator
       if (!mbar_wait(tfull_bar(acc), aph)) {
         ok = false;
         break;
       }
-      clk.add(0);
+      if (clocked) sum_cycles(p.timers + 6, true);
       tc_fence_after();
       const uint32_t taddr = tmem_base + (static_cast<uint32_t>(ew * 32) << 16) + acc * ACC_COLS;
       expert_epilogue<KIND>(p, tl.e, static_cast<int64_t>(tl.row0) + rin, (TR::WGRAD ? tl.m0 : tl.row0) + ew * 32, tl.n0, taddr,
@@ -292,9 +293,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
                               if (lane == 0) mbar_arrive_cluster(mapa_shared(tempty_bar(acc), 0));
                             });
     }
-    if (lane == 0 && ew == 0 && half == 0 && leader) {
-      clk.report(5, 6);
-      if (p.timers) atomicAdd(p.timers + 7, 1ull);
+    if (clocked) {
+      sum_cycles(p.timers + 5, true);
+      atomicAdd(p.timers + 7, 1ull);  // CTAs counted
     }
     if (!ok && lane == 0) {
       record_status(p.status, DEV_TIMEOUT, 1300 + KIND);
