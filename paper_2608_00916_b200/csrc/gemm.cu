@@ -640,9 +640,20 @@ moe_status launch_grouped_gemm(moe_ctx_impl* ctx, GemmKind kind, int64_t T, cons
   return launch_gemm_variant(ctx, kind, T, L, ws, io, st, false, 2);
 }
 
+// The expert GEMM that an operation of the expert-LoRA variant is, with its low-rank segment (-1: a skinny one).
+static int lora_row_gemm(LoraOp op) {
+  switch (op) {
+    case LORA_F3: return GEMM_F3;
+    case LORA_F4: return GEMM_F4;
+    case LORA_B2: return GEMM_B2;
+    case LORA_B4: return GEMM_B4;
+    default: return -1;
+  }
+}
+
 // Backward operations of the expert-LoRA variant (see launch_lora_gemm below, which prepares `p`).
-static moe_status launch_lora_gemm_bwd(moe_ctx_impl* ctx, LoraOp op, int64_t T, const WsLayout& L, char* ws,
-                                       const GemmIO& io, const LoraArgs& lo, GemmParams p, cudaStream_t st) {
+static moe_status launch_lora_gemm_bwd(moe_ctx_impl* ctx, LoraOp op, const WsLayout& L, char* ws, const GemmIO& io,
+                                       const LoraArgs& lo, GemmParams p, bool pair, cudaStream_t st) {
   const Shape& s = ctx->s;
   const int d = s.d, f = s.f, E = s.E, r = lo.rank;
   const int64_t R = L.rows_max;
@@ -652,8 +663,6 @@ static moe_status launch_lora_gemm_bwd(moe_ctx_impl* ctx, LoraOp op, int64_t T, 
            *dhu = B16(L.dhu), *dxp = B16(L.dxp), *u = B16(L.lora_u), *v = B16(L.lora_v), *w = B16(L.lora_w),
            *z = B16(L.lora_z);
   const uint32_t skinny_tx = A_BYTES + CHUNK_BYTES;
-  const bool pair = (op == LORA_B2 || op == LORA_B4) &&
-                    row_gemm_on_pairs(ctx, op == LORA_B2 ? GEMM_B2 : GEMM_B4, static_cast<double>(T) * s.k / E);
   const int nb = pair ? 128 : 256;  // rows of a K-major B box
   bool ok = true;
   switch (op) {
@@ -791,8 +800,9 @@ moe_status launch_lora_gemm(moe_ctx_impl* ctx, LoraOp op, int64_t T, const WsLay
   p.out_scale = 1.f;
   p.row_gate = reinterpret_cast<const float*>(ws + L.row_gate);
   const uint32_t skinny_tx = A_BYTES + CHUNK_BYTES;  // a 128 x 64 A tile and one 64 x 64 B tile
-  const bool pair = (op == LORA_F3 || op == LORA_F4) &&
-                    row_gemm_on_pairs(ctx, op == LORA_F3 ? GEMM_F3 : GEMM_F4, static_cast<double>(T) * s.k / E);
+  const int kind = lora_row_gemm(op);
+  const bool pair = kind >= 0 && row_gemm_on_pairs(ctx, static_cast<GemmKind>(kind), static_cast<double>(T) * s.k / E);
+  if (kind >= 0 && ctx->gemm_timers) p.timers = reinterpret_cast<unsigned long long*>(ws + L.timers) + 8 * kind;
   bool ok = true;
   switch (op) {
     case LORA_U:  // u[R,64] = s xp A1[e]            (F4 kind, N = 64)
@@ -838,7 +848,7 @@ moe_status launch_lora_gemm(moe_ctx_impl* ctx, LoraOp op, int64_t T, const WsLay
     default:
       break;
   }
-  return launch_lora_gemm_bwd(ctx, op, T, L, ws, io, lo, p, st);
+  return launch_lora_gemm_bwd(ctx, op, L, ws, io, lo, p, pair, st);
 }
 
 }  // namespace moe

@@ -1,5 +1,5 @@
-"""Stage-by-stage parity at the sizes where the choice of tile shape changes and where a staging unit of the GEMM
-epilogues (32 rows x 64 columns) is only partly inside the output."""
+"""Stage-by-stage parity at the sizes where the choice of tile shape changes (and that it does change there), and where
+a staging unit of the GEMM epilogues (32 rows x 64 columns) is only partly inside the output."""
 import pytest
 import torch
 
@@ -11,12 +11,82 @@ from test_gpu_parity import test_expert_lora_against_the_oracle as lora_against_
 pytestmark = pytest.mark.gpu
 
 
+# The expert GEMMs in the order of their counters: with MOE_GEMM_TIMERS set a launch counts its CTAs (one of each pair).
+KINDS = ("F3", "F4", "B2", "B3", "B4", "B5")
+ROW = {"F3", "F4", "B4"}  # gate/up, down, dgrad gate/up; B2 is dgrad-down, B3 and B5 are the weight gradients
+
+
+@pytest.fixture
+def on_pairs(monkeypatch):
+    """GEMMs of the last step of a layer that ran on CTA pairs.  Call once with the layer and T before the step, to clear
+    the counters, and without T after it."""
+    monkeypatch.setenv("MOE_GEMM_TIMERS", "1")
+
+    def read(layer, T=None, lora=False):
+        if T is not None:
+            layer._ensure_ws(T)
+            if lora:
+                layer.ws = torch.empty(int(layer.lib.moe_lora_workspace_bytes(layer.h, T)), dtype=torch.uint8, device="cuda")
+            layer.ws.zero_()
+            return None
+        ctas = layer.buffer("timers", torch.int64).view(16, 8)[:6, 7].cpu().tolist()
+        sms = torch.cuda.get_device_properties(0).multi_processor_count
+        assert all(c in (0, sms // 2, sms) for c in ctas)
+        return {n for n, c in zip(KINDS, ctas) if c == sms // 2}
+
+    return read
+
+
+@pytest.mark.parametrize("T,pairs", [
+    (520, set()), (524, ROW),            # 130 and 131 rows per expert: the expected tiles of the two shapes cross,
+    (1048, ROW), (1052, set()),          # 262, 263: again,
+    (1468, set()), (1472, ROW),          # 367, 368: and again
+    (1532, ROW), (1536, ROW | {"B3", "B5"}),                          # 383, 384: weight gradients
+    (3068, ROW | {"B3", "B5"}), (3072, ROW | {"B2", "B3", "B5"}),     # 767, 768: dgrad-down
+])
+def test_tile_shape_of_each_gemm(T, pairs, on_pairs):
+    """The shape the rule selects on both sides of each of its lines, and the layer's parity there."""
+    inp = synth.make_inputs(synth.MoEShape(T, 128, 8, 2, 128), 70, x_std=1.0)
+    ofw, obw = oracle_run(inp, 2, 0.05)
+    r = Run(inp, 2)
+    on_pairs(r.layer, T)
+    check_all(r, ofw, obw, 0.05)
+    assert on_pairs(r.layer) == pairs
+
+
+@pytest.mark.parametrize("T,pairs", [(520, set()), (524, ROW), (1048, ROW), (1052, set()), (1468, set()), (1472, ROW),
+                                     (3072, ROW | {"B2"})])
+def test_tile_shape_of_the_adapted_gemms(T, pairs, on_pairs):
+    """The large GEMMs of an adapter step take the shapes of the plain layer; both shapes give the same bits."""
+    d, E, k, f = 128, 8, 2, 128
+    inp = synth.make_inputs(synth.MoEShape(T, d, E, k, f), 70, x_std=1.0)
+    lo = {n: torch.empty(*s, dtype=torch.bfloat16, device="cuda").normal_(0, 0.05) for n, s in (
+        ("A1", (E, d, 16)), ("B1_gate", (E, 16, f)), ("B1_up", (E, 16, f)), ("A2", (E, f, 16)), ("B2", (E, 16, d)))}
+
+    def step(flags):
+        r = Run(inp, k, flags=flags)
+        v = r.dev
+        on_pairs(r.layer, T, lora=True)
+        y = r.layer.lora_forward(v["x"], v["W_r"], v["W_gate"], v["W_up"], v["W_down"], lo, 2.0)["y"]
+        g = r.layer.lora_backward(v["dy"], 0.02)
+        r.layer.poll()
+        return on_pairs(r.layer), {"y": y, **g}
+
+    chosen, out = step(0)
+    assert chosen == pairs
+    for flags in (1, 2):  # forced: CTA pairs, one-CTA tiles
+        forced, other = step(flags)
+        assert forced == (ROW | {"B2"} if flags == 1 else set())
+        for n in out:
+            assert torch.equal(out[n], other[n]), n
+
+
 @pytest.mark.parametrize("T,d,E,k,f,seed", [
     (640, 192, 8, 2, 320, 71),    # 160 rows per expert: row GEMMs on pairs, weight gradients not
-    (1024, 128, 8, 2, 192, 72),   # 256: row GEMMs on one-CTA tiles
+    (1024, 128, 8, 2, 192, 72),   # 256: the same
     (1532, 192, 8, 2, 64, 73),    # 383: the last size with one-CTA weight gradients
     (1540, 320, 8, 2, 192, 74),   # 385: weight gradients on pairs, output rows and columns beyond the last full tile
-    (1750, 128, 8, 2, 320, 75),   # 437: row GEMMs on pairs again
+    (1750, 128, 8, 2, 320, 75),   # 437: the same
     (3080, 192, 8, 2, 128, 76),   # 770: dgrad-down on pairs as well
 ])
 def test_tile_shape_boundaries(T, d, E, k, f, seed):
