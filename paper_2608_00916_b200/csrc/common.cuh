@@ -101,8 +101,9 @@ struct moe_ctx_impl {
   int row_group_override;  // MOE_ROW_GROUP, if set (measurements of the tile order)
   int b4_pair_override;    // MOE_B4_PAIR = 0 / 1, if set (measurements: dgrad gate/up on one-CTA tiles / CTA pairs); else -1
   // cudaFuncSetAttribute (dynamic shared memory opt-in) is per device: remembered here, for the device the context is
-  // bound to, per kernel family (0: one-CTA kernels, 1: CTA-pair kernels) and GEMM kind
-  unsigned char attr_done[2][16];
+  // bound to, per kernel family (0: one-CTA kernels, 1: CTA-pair kernels, 2: one-CTA
+  // weight gradients that load and add) and GEMM kind
+  unsigned char attr_done[3][16];
   int profiling;
   cudaEvent_t ev[MOE_PROF_RING][MOE_NUM_STAGES][2];
   unsigned char ev_used[MOE_PROF_RING][MOE_NUM_STAGES];

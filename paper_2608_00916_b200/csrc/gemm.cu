@@ -27,7 +27,7 @@
 
 namespace moe {
 
-template <int KIND>
+template <int KIND, Accumulate ACC = Accumulate::NONE>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
     grouped_gemm_kernel(const __grid_constant__ GemmParams p) {
   using TR = Traits<KIND>;
@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
       const int acc = tc & 1;
       const uint32_t aph = (tc >> 1) & 1u;
       ++tc;
-      epilogue_prefetch<KIND>(p, static_cast<int64_t>(tl.row0) + rin, tl.n0, half == 0);
+      epilogue_prefetch<KIND, ACC>(p, static_cast<int64_t>(tl.row0) + rin, tl.n0, half == 0, tl.e, tl.m0 + rin);
       if (clocked()) sum_cycles(p.timers + 6, false);  // waiting for a finished accumulator
       if (!mbar_wait(tfull_bar(acc), aph)) {
         ok = false;
@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
           }
         }
       } else {
-        expert_epilogue<KIND>(p, tl.e, row, (TR::WGRAD ? tl.m0 : tl.row0) + ew * 32, tl.n0, taddr, true,
+        expert_epilogue<KIND, ACC>(p, tl.e, row, (TR::WGRAD ? tl.m0 : tl.row0) + ew * 32, tl.n0, taddr, true,
                               TR::WGRAD          ? p.M_total - (tl.m0 + ew * 32)
                               : KIND == GEMM_DX ? static_cast<int>(p.T - tl.row0 - ew * 32)
                               : p.clip_rows     ? tl.valid - ew * 32
@@ -343,18 +343,16 @@ static bool map_mn_rows(void* fn, CUtensorMap* m, const void* base, int64_t rows
   return map_chunks(fn, m, base, 1, rows, width, chunks, 3);
 }
 
-template <int KIND>
+template <int KIND, Accumulate ACC = Accumulate::NONE>
 static moe_status launch_kind(moe_ctx_impl* ctx, const GemmParams& p, cudaStream_t st) {
-  if (!ctx->attr_done[0][KIND]) {  // per device: the context is bound to one
-    if (cudaFuncSetAttribute(grouped_gemm_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(GEMM_SMEM)) != cudaSuccess)
+  auto* const kernel = grouped_gemm_kernel<KIND, ACC>;
+  unsigned char* const done = &ctx->attr_done[ACC == Accumulate::LOAD_ADD ? 2 : 0][KIND];
+  if (!*done) {  // per device: the context is bound to one
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(GEMM_SMEM)) != cudaSuccess)
       return MOE_ERR_CUDA;
-    ctx->attr_done[0][KIND] = 1;
+    *done = 1;
   }
-  return launch_kernel(grouped_gemm_kernel<KIND>, ctx->sm_count, GEMM_THREADS, GEMM_SMEM, st,
-                       p) == cudaSuccess
-             ? MOE_OK
-             : MOE_ERR_CUDA;
+  return launch_kernel(kernel, ctx->sm_count, GEMM_THREADS, GEMM_SMEM, st, p) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
 }
 
 // Row tiles (or pairs) walked together inside a column tile: 1 while the expert's weights are few column tiles wide (they
@@ -494,7 +492,9 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
       p.ld_out = d;
       p.expert_stride = static_cast<int64_t>(f) * d;
       if (!ok) return MOE_ERR_CUDA;
-      return pair ? launch_pair_gemm(ctx, kind, p, st) : launch_kind<GEMM_B3>(ctx, p, st);
+      return pair         ? launch_pair_gemm(ctx, kind, p, st)
+             : p.acc_fp32 ? launch_kind<GEMM_B3, Accumulate::LOAD_ADD>(ctx, p, st)
+                          : launch_kind<GEMM_B3>(ctx, p, st);
     case GEMM_B5:
       ok = map_mn_rows(fn, &p.mapA0, xp, R, d, 2) && map_mn_rows(fn, &p.mapB0, dhg, R, f, 2) &&
            map_mn_rows(fn, &p.mapB1, dhu, R, f, 2);
@@ -509,7 +509,9 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
       p.ld_out = f;
       p.expert_stride = static_cast<int64_t>(d) * f;
       if (!ok) return MOE_ERR_CUDA;
-      return pair ? launch_pair_gemm(ctx, kind, p, st) : launch_kind<GEMM_B5>(ctx, p, st);
+      return pair         ? launch_pair_gemm(ctx, kind, p, st)
+             : p.acc_fp32 ? launch_kind<GEMM_B5, Accumulate::LOAD_ADD>(ctx, p, st)
+                          : launch_kind<GEMM_B5>(ctx, p, st);
     case GEMM_RT:
       // logits[T,E] = x[T,d] W_r[d,E]; W_r is read as a one-slab tensor so the weight loaders apply
       p.b_chunks = (E + 63) / 64;
@@ -615,7 +617,8 @@ static double expected_tiles(double mean, double size) {
 // Weight gradients pair along the weight dimension without leftovers, but their K loop is the expert's row count, and
 // with few K blocks the output leaves as fast as HBM takes it (a plain fill runs at 3.9 TB/s here) only from one-CTA
 // tiles, whose two CTAs do not have to meet: wgrad-down / wgrad-gate/up 162 -> 172 / 322 -> 330 at 312 rows, equal at
-// 375, 200 -> 187 / 399 -> 374 at 437, 222 -> 195 / 430 -> 392 at 512.
+// 375, 200 -> 187 / 399 -> 374 at 437, 222 -> 195 / 430 -> 392 at 512.  When they accumulate in fp32 the line lies higher
+// (see Accumulate).
 static bool row_gemm_on_pairs(const moe_ctx_impl* ctx, GemmKind kind, double rows_per_expert) {
   if (ctx->tile_mode != 0) return ctx->tile_mode == 1;
   if (kind == GEMM_B4 && ctx->b4_pair_override >= 0) return ctx->b4_pair_override != 0;
@@ -629,7 +632,8 @@ moe_status launch_grouped_gemm(moe_ctx_impl* ctx, GemmKind kind, int64_t T, cons
   const bool wgrad_kind = kind == GEMM_B3 || kind == GEMM_B5;
   const double rows_per_expert = static_cast<double>(T) * ctx->s.k / ctx->s.E;
   if (wgrad_kind) {
-    const bool pair = ctx->tile_mode == 1 || ctx->tile_mode == 3 || (ctx->tile_mode == 0 && rows_per_expert >= 384.0);
+    const double line = io.dW_down_acc ? 704.0 : 384.0;
+    const bool pair = ctx->tile_mode == 1 || ctx->tile_mode == 3 || (ctx->tile_mode == 0 && rows_per_expert >= line);
     return launch_gemm_variant(ctx, kind, T, L, ws, io, st, pair, 0);
   }
   if (!row_kind) return launch_gemm_variant(ctx, kind, T, L, ws, io, st, false, 0);

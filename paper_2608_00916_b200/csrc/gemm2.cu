@@ -276,7 +276,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
       const int acc = tc & 1;
       const uint32_t aph = (tc >> 1) & 1u;
       ++tc;
-      epilogue_prefetch<KIND>(p, static_cast<int64_t>(tl.row0) + rin, tl.n0, tl.write && half == 0);
+      epilogue_prefetch<KIND, Accumulate::REDUCE>(p, static_cast<int64_t>(tl.row0) + rin, tl.n0, tl.write && half == 0);
       if (clocked) sum_cycles(p.timers + 6, false);  // waiting for a finished accumulator
       if (!mbar_wait(tfull_bar(acc), aph)) {
         ok = false;
@@ -285,7 +285,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
       if (clocked) sum_cycles(p.timers + 6, true);
       tc_fence_after();
       const uint32_t taddr = tmem_base + (static_cast<uint32_t>(ew * 32) << 16) + acc * ACC_COLS;
-      expert_epilogue<KIND>(p, tl.e, static_cast<int64_t>(tl.row0) + rin, (TR::WGRAD ? tl.m0 : tl.row0) + ew * 32, tl.n0, taddr,
+      expert_epilogue<KIND, Accumulate::REDUCE>(p, tl.e, static_cast<int64_t>(tl.row0) + rin, (TR::WGRAD ? tl.m0 : tl.row0) + ew * 32, tl.n0, taddr,
                             tl.write, TR::WGRAD ? p.M_total - (tl.m0 + ew * 32) : p.clip_rows ? tl.valid - ew * 32 : 32, es,
                             lane, half, [&]() {
                               tc_fence_before();

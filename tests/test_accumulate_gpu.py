@@ -8,9 +8,10 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("T,flags", [
-    (300, 1),   # CTA pairs
-    (300, 2),   # one-CTA tiles
-    (1700, 0),  # 425 rows per expert: pairs by the default rule
+    (300, 1),   # CTA pairs: reductions
+    (300, 2),   # one-CTA tiles: loads, additions, stores
+    (1700, 0),  # 425 rows per expert: one-CTA tiles by the default rule
+    (2900, 0),  # 725: pairs
 ])
 @pytest.mark.parametrize("exponent", [0, -85, -95, -103, -112])
 def test_accumulation_rounds_once_over_the_whole_range(T, flags, exponent):

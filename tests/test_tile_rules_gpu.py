@@ -4,8 +4,8 @@ import pytest
 import torch
 
 from paper_2608_00916_b200 import synth
-from gpu_util import Run, oracle_run
-from test_gpu_parity import check_all
+from gpu_util import Run, oracle_run, rel_fro
+from test_gpu_parity import TOL, check_all
 from test_gpu_parity import test_expert_lora_against_the_oracle as lora_against_the_oracle
 
 pytestmark = pytest.mark.gpu
@@ -52,6 +52,26 @@ def test_tile_shape_of_each_gemm(T, pairs, on_pairs):
     on_pairs(r.layer, T)
     check_all(r, ofw, obw, 0.05)
     assert on_pairs(r.layer) == pairs
+
+
+@pytest.mark.parametrize("T,pairs", [(1536, ROW), (2812, ROW), (2816, ROW | {"B3", "B5"})])
+def test_tile_shape_of_accumulating_gemms(T, pairs, on_pairs):
+    """384, 703 and 704 rows per expert: weight gradients that accumulate change shape later than those that do not; twice the
+    same micro-batch on buffers of zeros gives twice the oracle's gradient."""
+    d, E, k, f = 128, 8, 2, 192
+    inp = synth.make_inputs(synth.MoEShape(T, d, E, k, f), 70, x_std=1.0)
+    _, obw = oracle_run(inp, k, 0.05)
+    r = Run(inp, k)
+    acc = {"dW_r": torch.zeros(d, E, device="cuda"), "dW_gate": torch.zeros(E, d, f, device="cuda"),
+           "dW_up": torch.zeros(E, d, f, device="cuda"), "dW_down": torch.zeros(E, f, d, device="cuda")}
+    for _ in range(2):
+        on_pairs(r.layer, T)
+        r.forward()
+        r.layer.backward_accumulate(r.dev["dy"], 0.05, acc)
+        r.layer.poll()
+        assert on_pairs(r.layer) == pairs
+    for n in acc:
+        assert rel_fro(acc[n].cpu().numpy(), 2.0 * obw[n]) <= TOL, n
 
 
 @pytest.mark.parametrize("T,pairs", [(520, set()), (524, ROW), (1048, ROW), (1052, set()), (1468, set()), (1472, ROW),
