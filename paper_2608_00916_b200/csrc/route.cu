@@ -353,13 +353,18 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_kernel(int64_t T, int E, in
   finish_tables(T, E, k, sh, tabs, psum, counts_out, aux_out);
 }
 
-// The permutation in one kernel, while every block can afford to look at all tile histograms (PLACE_MAX_TILES): block 0
+// The permutation in one kernel, while every block can afford to look at all tile histograms (place_max_tiles): block 0
 // builds the counts, tables and the auxiliary loss; block b + 1 places the picks of token tile b.  Each block sums the
 // columns of tile_counts itself - over all tiles (expert totals, hence segment starts) and over the tiles before its own
-// (first rank) - so nothing waits for a scan by one block.  Bound by two rounds of L2 latency.  Measured against scan_kernel
-// followed by scatter_kernel: 241 tokens 13 -> 5 us, 16384 tokens 25 -> 14 us.  The histograms are read once per block, so the
-// traffic grows with the square of the token count: 0.13 GB from L2 at 512 tiles of 128 experts.
-constexpr int PLACE_MAX_TILES = 512;
+// (first rank) - so nothing waits for a scan by one block.  Bound by two rounds of L2 latency per wave of blocks.
+// Measured against scan_kernel followed by scatter_kernel at 128 experts: 241 tokens 13 -> 5 us, 16384 tokens 25 -> 14 us.
+//
+// The line.  The histograms are read once per block, so the traffic grows with the square of the token count, and with few
+// experts the 1024 / E partial sums per column, added up by one thread, weigh more than the tiles.  Permutation stage with rows
+// of 64 columns, scan and scatter -> place, us: 8 experts 26 -> 23 at 256 tiles, 34 -> 39 at 512; 16 experts 26 -> 23, 30 -> 31
+// at 384, 34 -> 37; 32 experts 36 -> 33 at 384, 42 -> 41 at 512, 56 -> 64 at 768; 64 experts 63 -> 58 at 512, 88 -> 91 at 768;
+// 128 experts 74 -> 67 at 512, 138 -> 154 at 1024; 256 experts 101 -> 91, 186 -> 227.
+static int place_max_tiles(int E) { return E < 32 ? 320 : 512; }
 __global__ void __launch_bounds__(SCAN_THREADS) place_kernel(int64_t T, int E, int k, int tok_tiles, int psum_rows,
                                                              const int32_t* tile_counts, const TableOut tabs,
                                                              const float* psum_part,
@@ -622,7 +627,7 @@ void launch_permute(const Shape& s, int64_t T, const WsLayout& L, char* ws, cons
   if (tiles > 0 && !histogram_done) {
     launch_kernel(hist_kernel, tiles, TOK_TILE, msm, st, T, s.E, s.k, idx, tile_counts);
   }
-  if (tiles > 0 && !tables_only && tiles <= PLACE_MAX_TILES) {
+  if (tiles > 0 && !tables_only && tiles <= place_max_tiles(s.E)) {
     launch_kernel(place_kernel, tiles + 1, SCAN_THREADS, msm, st, T, s.E, s.k, tiles, psum_rows, tile_counts,
                   table_pointers(L, ws), reinterpret_cast<const float*>(ws + L.psum_part),
                   reinterpret_cast<float*>(ws + L.psum), counts_out, aux_out, idx,

@@ -115,10 +115,11 @@ def test_tile_shape_boundaries(T, d, E, k, f, seed):
     check_all(Run(inp, k), ofw, obw, 0.05)
 
 
-@pytest.mark.parametrize("T", [65536 - 127, 65536, 65537])
-def test_permutation_on_both_sides_of_its_token_limit(T):
-    """512 tiles of 128 tokens are placed by one kernel, more by a scan and a scatter: same routing, same layer."""
-    inp = synth.make_inputs(synth.MoEShape(T, 64, 8, 2, 64), 77, x_std=1.0)
+@pytest.mark.parametrize("T,E", [(40960, 8), (40961, 8), (65536 - 127, 8), (65536, 8), (65537, 8), (65536, 32), (65537, 32)])
+def test_permutation_on_both_sides_of_its_token_limit(T, E):
+    """320 tiles of 128 tokens (512 from 32 experts on) are placed by one kernel, more by a scan and a scatter: same routing,
+    same layer."""
+    inp = synth.make_inputs(synth.MoEShape(T, 64, E, 2, 64), 77, x_std=1.0)
     ofw, obw = oracle_run(inp, 2, 0.05)
     check_all(Run(inp, 2), ofw, obw, 0.05)
 
