@@ -352,7 +352,8 @@ static moe_status launch_kind(moe_ctx_impl* ctx, const GemmParams& p, cudaStream
       return MOE_ERR_CUDA;
     *done = 1;
   }
-  return launch_kernel(kernel, ctx->sm_count, GEMM_THREADS, GEMM_SMEM, st, p) == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
+  launch_kernel(kernel, ctx->sm_count, GEMM_THREADS, GEMM_SMEM, st, p);
+  return cudaGetLastError() == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;  // reported here, and not by the next call once more
 }
 
 // Row tiles (or pairs) walked together inside a column tile: 1 while the expert's weights are few column tiles wide (they

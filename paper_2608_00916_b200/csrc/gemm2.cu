@@ -320,9 +320,8 @@ static moe_status launch_pair_kind(moe_ctx_impl* ctx, const GemmParams& p, cudaS
     ctx->attr_done[1][KIND] = 1;
   }
   const int grid = ctx->sm_count & ~1;  // whole pairs
-  return launch_kernel(grouped_gemm_pair_kernel<KIND>, grid, GEMM2_THREADS, GEMM2_SMEM, st, p) == cudaSuccess
-             ? MOE_OK
-             : MOE_ERR_CUDA;
+  launch_kernel(grouped_gemm_pair_kernel<KIND>, grid, GEMM2_THREADS, GEMM2_SMEM, st, p);
+  return cudaGetLastError() == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
 }
 
 moe_status launch_pair_gemm(moe_ctx_impl* ctx, GemmKind kind, const GemmParams& p, cudaStream_t st) {

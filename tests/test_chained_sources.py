@@ -47,6 +47,13 @@ def test_warps_reconverge_after_the_one_thread_roles():
             assert re.search(r"\n  \}\n\n  __syncwarp\(\);[^\n]*\n  tc_fence_before\(\);\n  (__syncthreads|cluster_sync_all)", after), name
 
 
+def test_a_failed_launch_of_a_gemm_is_reported_once():
+    """The runtime's last error is taken by the call that failed; left in place, the next call would return it again."""
+    for name, text in sources():
+        if name in ("gemm.cu", "gemm2.cu"):
+            assert re.search(r"  launch_kernel\([^;]*;\n  return cudaGetLastError\(\) == cudaSuccess \? MOE_OK : MOE_ERR_CUDA;", text), name
+
+
 def compiles(tmp_path, argument):
     src = tmp_path / "launch.cu"
     src.write_text('#include "common.cuh"\n'
