@@ -302,10 +302,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
     }
   }
 
-  __syncwarp();  // the 31 lanes that passed by a one-thread role meet it here: what follows is executed by whole warps
   tc_fence_before();
-  cluster_sync_all();  // the partner has stopped using this CTA's shared memory, barriers and tensor memory
+  cluster_sync_diverged();  // the partner has stopped using this CTA's shared memory, barriers and tensor memory
   if (warp == 1) {
+    __syncwarp();  // freeing tensor memory takes the whole warp
     tc_fence_after();
     tmem_dealloc_pair(tmem_base, TMEM_COLS);
   }
