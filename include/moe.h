@@ -56,10 +56,10 @@ typedef struct {
 
 /* Tile shape of the expert GEMMs.  By default the library chooses per GEMM between CTA pairs (256 x 256 tiles,
  * tcgen05 cta_group::2, each CTA staging half of B) and one-CTA 128 x 256 tiles: weight gradients run on pairs when
- * the experts average at least 384 rows, dgrad-down from 768, the other row GEMMs where the expected number of pairs
- * (an expert with an odd number of 128-row blocks gets a last pair whose second half is empty) costs less than the
- * expected number of one-CTA tiles.  The flags force
- * one shape everywhere (same results; for comparison measurements). */
+ * the experts average at least 384 rows (704 when they accumulate into fp32 buffers), dgrad-down from 768, the other row
+ * GEMMs where the expected number of pairs (an expert with an odd number of 128-row blocks gets a last pair whose second half
+ * is empty) costs less than the expected number of one-CTA tiles.  The flags force one shape everywhere (same results; for
+ * comparison measurements). */
 #define MOE_FLAG_CTA_PAIR_TILES 1
 #define MOE_FLAG_SINGLE_CTA_TILES 2
 /* Row GEMMs run every complete pair of 128-row blocks of an expert on a CTA pair and the leftover block of an odd
@@ -111,7 +111,7 @@ MOE_API size_t moe_workspace_bytes(const moe_ctx* ctx, int64_t T);
  * Names: "counts" "offsets" "pad_offsets" "logits" "idx" "gates" "inv" "row_gate" "xp" "hg" "hu" "act"
  * "o" "dhg" "dhu" "dxp" "dg" "dl".  Internal row buffers (xp, hg, hu, act, o, dhg, dhu, dxp) are laid out
  * expert-major with every expert's segment padded to a multiple of 128 rows ("pad_offsets"); pad rows
- * are zero.  "act" and "o" are stored already multiplied by the row's gate (so the combine is a plain sum); after
+ * are zero (after moe_forward_inference: unspecified).  "act" and "o" are stored already multiplied by the row's gate (so the combine is a plain sum); after
  * moe_backward "o" holds the gathered rows of dy.  Returns MOE_ERR_INVALID_ARG for an unknown name. */
 MOE_API moe_status moe_workspace_find(const moe_ctx* ctx, int64_t T, const char* name /* host */,
                               size_t* offset /* host */, size_t* bytes /* host */);
@@ -157,7 +157,8 @@ MOE_API moe_status moe_stage_times(moe_ctx* ctx, float* ms /* host */, int32_t* 
  *   W_gate,W_up [E,d,f] bf16        W_down [E,f,d] bf16
  * Outputs
  *   y          [T,d]   bf16
- *   topk_idx   [T,k]   int32, pick order (descending logit, ties ascending index)
+ *   topk_idx   [T,k]   int32, pick order (descending logit, ties ascending index); k distinct experts for every token: a
+ *                      NaN logit is ordered as -inf
  *   topk_w     [T,k]   fp32 gates, each row sums to 1
  *   expert_counts [E]  int32
  *   perm       [T*k]   int32 or NULL: perm[r] = t*k + j of the pair in row r of the expert-major order

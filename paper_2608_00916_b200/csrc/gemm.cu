@@ -18,8 +18,9 @@
 // row-major [K, cols] is an MN-major operand, and the UMMA instruction takes either.
 // Row buffers are expert-major with each expert's segment padded to 128 rows of zeros, so an M tile never
 // straddles two experts and the ragged K of the weight gradients needs no masking.
-// Warp roles: warp 0 TMA producer, warp 1 MMA issuer (owns the TMEM allocation), warps 2..9 epilogue (2..5 for the
-// routing kind).  The expert-LoRA variant runs on the same template (launch_lora_gemm at the end of this file).
+// Warp roles: warp 0 TMA producer, warp 1 MMA issuer (owns the TMEM allocation), warps 2..9 epilogue (of the two that
+// share a lane quadrant, the routing kind has one select experts and one sum the softmax).  The expert-LoRA variant runs
+// on the same template (launch_lora_gemm at the end of this file).
 // Every mbarrier wait is bounded; on a timeout the kernel records it in the status word and leaves.
 #include <math.h>
 
@@ -91,7 +92,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
 
   // The producer and the MMA issuer are one thread each.  What they do per K block (a wait, a few copies or four MMAs, a
   // commit) has to fit well inside the 512 cycles that the tensor core needs for it; run by a whole warp with one lane
-  // enabled, with a division for the stage index, it took 400 - 700 cycles and set the pace of every kernel here.
+  // enabled, with a division for the stage index, it took 400 - 700 cycles and set the pace of every kernel here.  With the
+  // issuer alone run by a whole warp gate/up at 1024 rows per expert takes 757 us instead of 688.
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     if (elect_one()) {
@@ -153,6 +155,9 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
         clk.add(0);
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + acc * ACC_COLS;
+        // Asking for the next stage before this one's MMAs are issued lets a copy that has landed be seen early; where none
+        // has, try_wait may hold the thread for a moment.  With it, without it and with test_wait in its place the row GEMMs at
+        // 62 to 1024 rows per expert take the same time, within 1 %.
         bool ready = false;  // the stage about to be used was already seen full
         for (int kb = 0; kb < tl.nkb; ++kb) {
           clk.start();
@@ -165,7 +170,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
           const uint64_t off = (pos.s * stage_stride) >> 4;
           const uint32_t done = empty_bar(pos.s);
           pos.next(NST);
-          ready = kb + 1 < tl.nkb && mbar_try_wait(full_bar(pos.s), pos.phase);  // its latency passes under the MMAs
+          ready = kb + 1 < tl.nkb && mbar_try_wait(full_bar(pos.s), pos.phase);
           const int nks = kb == tl.nkb - 1 ? tl.klast : BK / 16;
 #pragma unroll
           for (int ks = 0; ks < BK / 16; ++ks)
@@ -606,15 +611,21 @@ static double expected_tiles(double mean, double size) {
 
 // Tile shape per GEMM.  A CTA pair (256 x 256 tile, each CTA staging its rows of A and half of B) moves a third
 // less operand data from L2 per flop than a one-CTA 128 x 256 tile, and the L2 -> SM feed is what limits these
-// kernels: a 128-row block costs 0.80 of its one-CTA time on the pair kernel.  Row GEMMs pair two 128-row blocks of ONE
-// expert, so an expert with an odd block count pays for a block it does not have.  Whether pairs win therefore
-// oscillates with the rows per expert, and the rule compares the two expected costs.  Measured (d 2048, f 768, 128
-// experts, one-CTA -> pair, us; gate/up, down, dgrad gate/up): 62 rows per expert 164 -> 168, 82 -> 85, 163 -> 160;
-// 156: 204 -> 186, 106 -> 96, 195 -> 174; 256: 231 -> 222, 129 -> 123, 233 -> 217; 312: 270 -> 273, 152 -> 156,
-// 276 -> 278; 375: 297 -> 282, 169 -> 161, 310 -> 292; 512: 385 -> 369, 218 -> 200, 404 -> 381; 1024: 719 -> 700,
-// 406 -> 365, 764 -> 718.  At 128 rows (equal, equal, 180 -> 167) the rule misses.
-// The dgrad-down GEMM is held by its epilogue (it reads hg and hu) rather than by the feed and gains less: 153 -> 152 at
-// 156 rows, 251 -> 271 at 512, 290 -> 299 at 625, 455 -> 465 at 1024: pairs from 768 rows on.
+// kernels.  Row GEMMs pair two 128-row blocks of ONE expert, so an expert with an odd block count pays for a block it does not
+// have: a block on pairs costs less than a one-CTA block (0.76 - 0.81 at 256 and 300 rows, 0.85 - 0.87 from 512 on), but there
+// are more of them.  Whether pairs win therefore oscillates with the rows per expert, and the rule compares the expected
+// numbers of blocks, for experts loaded alike, under a threshold of 0.80 that is fitted to where the sign changes (it puts
+// the lines at 131, 263 and 368 rows).  Measured at
+// d 2048, f 768, 128 experts (one-CTA -> pair, us; gate/up, down, dgrad gate/up): 62 rows per expert 162 -> 167, 81 -> 84,
+// 156 -> 161; 128: 176 -> 177, 89 -> 91, 167 -> 168; 256: 230 -> 223, 131 -> 124, 232 -> 216; 300: 267 -> 274, 151 -> 156,
+// 265 -> 270; 512: 380 -> 358, 221 -> 208, 396 -> 375; 768: 535 -> 494, 310 -> 283, 559 -> 522; 1024: 689 -> 635, 400 -> 360,
+// 727 -> 670.  A few wide experts (d 4096, f 14336, 8 experts) leave a last round of pairs nearly empty at 512 and 768
+// rows, which the rule does not see: 865 -> 905, 432 -> 494, 891 -> 1070 at 512; 256: 522 -> 542, 308 -> 282, 643 -> 548;
+// 1024: 1524 -> 1494, 796 -> 754, 1698 -> 1611; 4096: 6604 -> 6187, 3138 -> 3065, 7312 -> 6943.
+// The dgrad-down GEMM is held by its epilogue (it reads hg and hu) rather than by the feed and gains less: 112 -> 125 at 62
+// rows, 127 -> 136 at 128, 166 -> 167 at 256, 181 -> 204 at 300, 248 -> 247 at 512, 333 -> 336 at 768, 418 -> 415 at 1024, 615 ->
+// 591 at 1536, 811 -> 788 at 2048; wide experts 301 -> 313 at 256, 510 -> 473 at 512, 702 -> 705 at 768, 881 -> 843 at 1024,
+// 3681 -> 3227 at 4096: pairs from 768 rows on, where the two are equal.
 // Half-empty pairs are better than complete pairs plus the leftover blocks in a second, one-CTA launch
 // (MOE_FLAG_HYBRID_TILES: 4.22 ms a step against 4.17 at 1024 rows per expert).
 // Weight gradients pair along the weight dimension without leftovers, but their K loop is the expert's row count, and
@@ -778,7 +789,8 @@ static moe_status launch_lora_gemm_bwd(moe_ctx_impl* ctx, LoraOp op, const WsLay
 // extra 64-deep K segment ([xp | u] [[W]; [B1]], ...), the four 64-wide row buffers u, v, w, z come from skinny
 // instances (N = 64) of the F4 / B4 kinds, and the adapter gradients from instances of the B3 / B5 kinds whose M or
 // N is the rank.  The four large ones take the tile shape the plain layer would
-// (rank 16, 8192 tokens, 512 rows per expert: a step 2132 -> 2079 us), the others one-CTA tiles.
+// (rank 16, 8192 tokens, 512 rows per expert: a step 2132 -> 2079 us), the others one-CTA tiles.  All walk the row tiles in
+// plain column order, also those of wide experts (row_group_for): adapters on such experts have not been timed.
 moe_status launch_lora_gemm(moe_ctx_impl* ctx, LoraOp op, int64_t T, const WsLayout& L, char* ws, const GemmIO& io,
                             const LoraArgs& lo, cudaStream_t st) {
   const Shape& s = ctx->s;

@@ -235,7 +235,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
           const uint64_t off = (pos.s * STAGE2_BYTES) >> 4;
           const uint32_t done = empty_bar(pos.s);
           pos.next(STAGES2);
-          ready = kb + 1 < tl.nkb && mbar_try_wait(full_bar(pos.s), pos.phase);  // its latency passes under the MMAs
+          ready = kb + 1 < tl.nkb && mbar_try_wait(full_bar(pos.s), pos.phase);
           const int nks = kb == tl.nkb - 1 ? tl.klast : BK / 16;
 #pragma unroll
           for (int ks = 0; ks < BK / 16; ++ks)

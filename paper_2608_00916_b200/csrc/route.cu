@@ -591,8 +591,6 @@ void launch_prepare(const WsLayout& L, char* ws, cudaStream_t st) {
                 reinterpret_cast<float*>(ws + L.row_gate), L.rows_alloc);
 }
 
-// tables_only: stop after the histogram and the scan (per-tile prefixes, counts, tables, aux loss); the expert-parallel
-// path places the rows itself
 // An fp32 value is the exact sum of three bf16 values (8 + 8 + 8 significand bits): the router contraction of an
 // fp32 weight runs as three bf16 tensor-core products, each exact in fp32.
 __global__ void __launch_bounds__(256) split_fp32_kernel(const float* __restrict__ w, uint16_t* __restrict__ hi,
@@ -617,6 +615,8 @@ void launch_split_fp32(const float* w, uint16_t* hi, uint16_t* mid, uint16_t* lo
   launch_kernel(split_fp32_kernel, static_cast<unsigned>((n + 255) / 256), 256, 0, st, w, hi, mid, lo, n);
 }
 
+// tables_only: stop after the histogram and the scan (per-tile prefixes, counts, tables, aux loss); the expert-parallel
+// path places the rows itself
 void launch_permute(const Shape& s, int64_t T, const WsLayout& L, char* ws, const uint16_t* x, int32_t* counts_out,
                     int32_t* perm_out, float* aux_out, int psum_rows, cudaStream_t st, bool tables_only,
                     bool histogram_done, bool debug, bool clear_pads) {
