@@ -43,8 +43,8 @@ WsLayout make_layout(const Shape& s, int64_t T, bool row_buffers) {
   L.fpair_tab = take(sizeof(int32_t) * 4 * L.max_m_tiles);
   L.single_tab = take(sizeof(int32_t) * s.E);
   L.tile_counts = take(sizeof(int32_t) * (L.tok_tiles + 1) * s.E);
-  // rows: one per SIMT router block, or four (one per epilogue warp) per 128-token tile of the tensor-core router
-  L.psum_part = take(sizeof(float) * (L.router_blocks + 4 * ((T + 127) / 128) + 1) * s.E);
+  // rows: one per SIMT router block; the tensor-core router writes at most as many
+  L.psum_part = take(sizeof(float) * (L.router_blocks + 1) * s.E);
   L.psum = take(sizeof(float) * s.E);
   L.logits = take(sizeof(float) * T * s.E);
   L.idx = take(sizeof(int32_t) * R);
@@ -382,7 +382,7 @@ static moe_status forward_impl(bool training, moe_ctx* ctx, int64_t T, const uin
   const bool tc_router = router_on_tensor_cores(s) && logits_in == nullptr;
   if (c->router_fp32 && (lora || !training)) return MOE_ERR_UNSUPPORTED;  // fp32 router weight: moe_forward / moe_backward
   Chain chain;
-  launch_prepare(L, ws, st);  // before any kernel that may record a status
+  if (T == 0 || !tc_router) launch_prepare(L, ws, st);  // before any kernel that may record a status
   if (c->router_fp32 && W_r) {
     // W_r points at fp32 values: split them into three exact bf16 terms, kept in the workspace for the backward pass
     const int64_t n = static_cast<int64_t>(s.d) * s.E, stride = n + 64;
@@ -395,7 +395,7 @@ static moe_status forward_impl(bool training, moe_ctx* ctx, int64_t T, const uin
   {
     StageTimer tm(c, st, 0);
     if (T > 0 && tc_router) {
-      rc = launch_grouped_gemm(c, GEMM_RT, T, L, ws, io, st);
+      rc = launch_router_tc(c, T, L, ws, io, st);
       if (rc != MOE_OK) return rc;
     } else {
       launch_router(s, T, x, W_r, b_r, logits_in, reinterpret_cast<float*>(ws + L.logits),
@@ -406,8 +406,8 @@ static moe_status forward_impl(bool training, moe_ctx* ctx, int64_t T, const uin
   {
     StageTimer tm(c, st, 1);
     launch_permute(s, T, L, ws, x, expert_counts, perm, aux_loss,
-                   static_cast<int>(router_psum_rows(s, T, logits_in != nullptr)), st, /*tables_only=*/false,
-                   /*histogram_done=*/tc_router && T > 0 && router_writes_histogram(s), c->debug_checks != 0,
+                   static_cast<int>(router_psum_rows(c, T, logits_in != nullptr)), st, /*tables_only=*/false,
+                   /*histogram_done=*/tc_router && T > 0, c->debug_checks != 0,
                    /*clear_pads=*/training);
   }
   if (T > 0) {

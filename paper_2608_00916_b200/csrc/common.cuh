@@ -104,6 +104,7 @@ struct moe_ctx_impl {
   // bound to, per kernel family (0: one-CTA kernels, 1: CTA-pair kernels, 2: one-CTA
   // weight gradients that load and add) and GEMM kind
   unsigned char attr_done[3][16];
+  unsigned router_attr;  // the same for the forms of the tensor-core router, one bit each
   int profiling;
   cudaEvent_t ev[MOE_PROF_RING][MOE_NUM_STAGES][2];
   unsigned char ev_used[MOE_PROF_RING][MOE_NUM_STAGES];
@@ -154,7 +155,7 @@ inline bool forward_matches(const moe_ctx_impl* c, const void* ws, int64_t T, in
 // binds the context to the current device on first use (api.cu)
 moe_status ensure_device(moe_ctx_impl* c);
 // ---- launchers (route.cu)
-// first kernel of a forward call: zero row gates, initialise the status block of a workspace seen for the first time
+// first kernel of a forward call whose router is not the tensor-core one: zero row gates, initialise the status block of a workspace seen for the first time
 void launch_prepare(const WsLayout& L, char* ws, cudaStream_t st);
 void launch_router(const Shape& s, int64_t T, const uint16_t* x, const uint16_t* W_r, const float* b_r,
                    const float* logits_in, float* logits, int32_t* idx, float* gates, int32_t* idx_out,
@@ -188,7 +189,7 @@ void launch_unpermute_bwd(const Shape& s, int64_t T, const uint16_t* dxp, const 
 void launch_unpermute_sum(const Shape& s, int64_t T, const uint16_t* dxp, const int32_t* inv, const uint16_t* dxr,
                           uint16_t* dx, cudaStream_t st, int32_t* dbg_status = nullptr, int64_t rows_max = 0);
 // ---- launchers (gemm.cu); each returns a CUDA / driver error as moe_status
-enum GemmKind { GEMM_F3 = 0, GEMM_F4, GEMM_B2, GEMM_B3, GEMM_B4, GEMM_B5, GEMM_RT, GEMM_DX, GEMM_DWR, GEMM_KINDS };
+enum GemmKind { GEMM_F3 = 0, GEMM_F4, GEMM_B2, GEMM_B3, GEMM_B4, GEMM_B5, GEMM_DX, GEMM_DWR, GEMM_KINDS };
 // Caller tensors a grouped-GEMM launch may need besides the workspace.
 struct GemmIO {
   bool save_preactivations = true;  // forward: also write hg, hu (needed by backward only)
@@ -243,11 +244,17 @@ moe_status launch_lora_gemm(moe_ctx_impl* ctx, LoraOp op, int64_t T, const WsLay
 
 // true when the tensor-core router / dW_r / dx kernels apply (their TMA maps need E % 8 == 0)
 inline bool router_on_tensor_cores(const Shape& s) { return s.E % 8 == 0; }
-// true when that router's epilogue also writes the per-tile histograms of the permutation (its shared-memory form)
-inline bool router_writes_histogram(const Shape& s) { return router_on_tensor_cores(s) && s.E <= 128 && s.k <= 16; }
-// psum_part rows written by the router: one per warp of a 128-token tile (tensor cores) or per ROUTER_TOK tokens (SIMT)
-inline int64_t router_psum_rows(const Shape& s, int64_t T, bool logits_given) {
-  return (router_on_tensor_cores(s) && !logits_given) ? 4 * ((T + 127) / 128) : (T + ROUTER_TOK - 1) / ROUTER_TOK;
+// ---- launchers (router.cu)
+// The tensor-core router: logits, picks, gates, column sums of p and the permutation's tile histograms.  Also what the first
+// kernel of a forward call does (launch_prepare): zero row gates, an initialised status block.
+moe_status launch_router_tc(moe_ctx_impl* ctx, int64_t T, const WsLayout& L, char* ws, const GemmIO& io, cudaStream_t st);
+// CTAs that share a 128-token tile in it
+int router_cluster(const Shape& s, int sm_count, int64_t T, bool fp32_weight);
+// psum_part rows written by the router: one per CTA with tokens (tensor cores) or per ROUTER_TOK tokens (SIMT)
+inline int64_t router_psum_rows(const moe_ctx_impl* c, int64_t T, bool logits_given) {
+  const int64_t tok = router_on_tensor_cores(c->s) && !logits_given
+                          ? TOK_TILE / router_cluster(c->s, c->sm_count, T, c->router_fp32 != 0) : ROUTER_TOK;
+  return (T + tok - 1) / tok;
 }
 
 // counts kernel launches of the library (process-wide; read through moe_kernel_launches)
@@ -328,6 +335,16 @@ inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, si
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Lets the next kernel of the chain be set up once every block of this one has got here or ended.
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Gives memory seen for the first time a clean status block.  One that already carries the cookie is left alone, so a failure
+// recorded by an earlier call stays visible until the host has reported it.
+__device__ __forceinline__ void init_status_block(int32_t* status, bool this_thread) {
+  if (this_thread && (status[2] != STATUS_COOKIE0 || status[3] != STATUS_COOKIE1)) {
+    status[0] = DEV_OK;
+    status[1] = 0;
+    status[2] = STATUS_COOKIE0;
+    status[3] = STATUS_COOKIE1;
+  }
+}
 // Records a device-side failure.  The first failure sticks: later ones do not overwrite it, and no kernel ever resets
 // the word (the host acknowledges it after reporting it, see moe_poll_status).
 __device__ __forceinline__ void record_status(int32_t* status, int code, int where) {

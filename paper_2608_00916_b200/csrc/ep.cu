@@ -327,16 +327,16 @@ moe_status moe_ep_route(moe_ctx* ctx, int64_t T, const uint16_t* x, const uint16
   if (rc != MOE_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   char* ws = static_cast<char*>(send_ws);
-  launch_prepare(L, ws, st);
+  if (T == 0) launch_prepare(L, ws, st);
   if (T > 0) {
     GemmIO io;
     io.x = x; io.W_r = W_r; io.b_r = b_r;
     io.idx_out = topk_idx; io.gates_out = topk_w;
-    rc = launch_grouped_gemm(c, GEMM_RT, T, L, ws, io, st);
+    rc = launch_router_tc(c, T, L, ws, io, st);
     if (rc != MOE_OK) return rc;
   }
-  launch_permute(s, T, L, ws, x, counts_local, nullptr, aux_loss, static_cast<int>(router_psum_rows(s, T, false)), st,
-                 /*tables_only=*/true, /*histogram_done=*/T > 0 && router_writes_histogram(s));
+  launch_permute(s, T, L, ws, x, counts_local, nullptr, aux_loss, static_cast<int>(router_psum_rows(c, T, false)), st,
+                 /*tables_only=*/true, /*histogram_done=*/T > 0);
   if (cudaGetLastError() != cudaSuccess) return MOE_ERR_CUDA;
   note_forward(c, send_ws, T, FWD_EP);  // the later phases on this sender workspace must name the same T
   return MOE_OK;

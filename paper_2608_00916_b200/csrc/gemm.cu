@@ -7,9 +7,8 @@
 //   B4  dxp     = dhg W_gate[e]^T + dhu W_up[e]^T   (one accumulator, two K segments)
 //   B3  dW_down[e]          = act_e^T dy_rows_e     (K = rows of expert e, one CTA owns a whole output tile)
 //   B5  dW_gate[e]|dW_up[e] = xp_e^T [dhg_e|dhu_e]
-// and the three contractions of the router, whose operands are bf16 (or fp32 split exactly into two bf16 terms),
-// so that a bf16 MMA with fp32 accumulation is an fp32 contraction up to summation order:
-//   RT  logits = x W_r (+ b_r)                      + routing epilogue (top-k, gates, softmax column sums)
+// and the two contractions of the router's backward pass, whose operands are bf16 (or fp32 split exactly into two bf16
+// terms), so that a bf16 MMA with fp32 accumulation is an fp32 contraction up to summation order:
 //   DX  dxr    = dl_hi W_r^T + dl_lo W_r^T          (router term of dx; the unpermute kernel adds the dxp rows)
 //   DWR dW_r partial[s] = x_s^T (dl_hi + dl_lo)_s   (token slices s; partials are summed by a small kernel)
 // Tiles are 128 x 256 with K steps of 64; operands arrive by TMA into 128-byte-swizzled shared memory (4 stages),
@@ -18,13 +17,13 @@
 // row-major [K, cols] is an MN-major operand, and the UMMA instruction takes either.
 // Row buffers are expert-major with each expert's segment padded to 128 rows of zeros, so an M tile never
 // straddles two experts and the ragged K of the weight gradients needs no masking.
-// Warp roles: warp 0 TMA producer, warp 1 MMA issuer (owns the TMEM allocation), warps 2..9 epilogue (of the two that
-// share a lane quadrant, the routing kind has one select experts and one sum the softmax).  The expert-LoRA variant runs
-// on the same template (launch_lora_gemm at the end of this file).
+// Warp roles: warp 0 TMA producer, warp 1 MMA issuer (owns the TMEM allocation), warps 2..9 epilogue.  The expert-LoRA
+// variant runs on the same template (launch_lora_gemm at the end of this file); the router's forward pass is in router.cu.
 // Every mbarrier wait is bounded; on a timeout the kernel records it in the status word and leaves.
 #include <math.h>
 
 #include "gemm_common.cuh"
+#include "tensor_maps.cuh"
 
 namespace moe {
 
@@ -33,35 +32,19 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     grouped_gemm_kernel(const __grid_constant__ GemmParams p) {
   using TR = Traits<KIND>;
   constexpr int EPI_WARPS = 8;
-  // The routing kind with E <= 128 stages only 32 KB per K block (16 KB of x, 16 KB of W_r): its stages are packed at
-  // that stride and the 96 KB this frees hold the scratch of its routing epilogue (80 KB) and the picks (16 KB).  When no
-  // CTA has a second tile (up to 128 tokens per SM) the scratch lies over the stages, which are done with by then, and
-  // the ring has six of them: the main loop waits for memory (x and W_r come from HBM).
-  constexpr uint32_t RT_STAGE_BYTES = A_BYTES + 2 * CHUNK_BYTES;
-  constexpr int MAX_STAGES = KIND == GEMM_RT ? 6 : STAGES;
-  const bool rt_packed = KIND == GEMM_RT && p.b_chunks <= 2;
-  const bool rt_overlay = rt_packed && p.static_m_tiles <= static_cast<int>(gridDim.x);
-  const int NST = rt_overlay ? 6 : STAGES;
-  static_assert(6 * RT_STAGE_BYTES <= STAGES * STAGE_BYTES + EPI_BYTES, "six packed stages do not fit");
-  static_assert(STAGES * RT_STAGE_BYTES + ROUTE_SCRATCH_BYTES + 128 * ROUTE_SMEM_MAX_K * 8 <= STAGES * STAGE_BYTES + EPI_BYTES,
-                "routing scratch does not fit");
   extern __shared__ unsigned char gemm_smem_raw[];
-  __shared__ __align__(8) uint64_t bars[2 * MAX_STAGES + 5];  // full, empty, accumulator full / empty, drain (failure path)
+  __shared__ __align__(8) uint64_t bars[2 * STAGES + 5];  // full, empty, accumulator full / empty, drain (failure path)
   __shared__ uint32_t tmem_base_slot;
-  __shared__ float s_bias[KIND == GEMM_RT ? MAX_E : 1];  // router bias (zero beyond E)
-  __shared__ int s_hist[KIND == GEMM_RT ? 128 : 1];      // picks per expert of the tile (routing epilogue for E <= 128)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t smem_base = (smem_u32(gemm_smem_raw) + 1023u) & ~1023u;
-  const uint32_t stage_stride = rt_packed ? RT_STAGE_BYTES : STAGE_BYTES;
-  const uint32_t rt_scratch = smem_base + (rt_overlay ? 0 : STAGES * RT_STAGE_BYTES);
   const uint32_t bar0 = smem_u32(bars);
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
-  auto empty_bar = [&](int s) { return bar0 + 8u * (MAX_STAGES + s); };
-  auto tfull_bar = [&](int a) { return bar0 + 8u * (2 * MAX_STAGES + a); };
-  auto tempty_bar = [&](int a) { return bar0 + 8u * (2 * MAX_STAGES + 2 + a); };
+  auto empty_bar = [&](int s) { return bar0 + 8u * (STAGES + s); };
+  auto tfull_bar = [&](int a) { return bar0 + 8u * (2 * STAGES + a); };
+  auto tempty_bar = [&](int a) { return bar0 + 8u * (2 * STAGES + 2 + a); };
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < NST; ++s) {
+    for (int s = 0; s < STAGES; ++s) {
       mbar_init(full_bar(s), 1);
       mbar_init(empty_bar(s), 1);
     }
@@ -69,7 +52,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
       mbar_init(tfull_bar(a), 1);
       mbar_init(tempty_bar(a), 32 * EPI_WARPS);
     }
-    mbar_init(bar0 + 8u * (2 * MAX_STAGES + 4), 1);
+    mbar_init(bar0 + 8u * (2 * STAGES + 4), 1);
     fence_mbar_init();
     tma_prefetch_desc(&p.mapA0);
     tma_prefetch_desc(&p.mapB0);
@@ -79,11 +62,6 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     tmem_relinquish();
   }
   chain_wait();  // everything above touches only this CTA's own state
-  if (KIND == GEMM_RT)
-    for (int i = threadIdx.x; i < MAX_E; i += blockDim.x) {
-      s_bias[i] = (p.bias && i < p.N_total) ? p.bias[i] : 0.f;
-      if (i < 128) s_hist[i] = 0;
-    }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -112,10 +90,10 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
             break;
           }
           clk.add(0);
-          const uint32_t sA = smem_base + pos.s * stage_stride;
+          const uint32_t sA = smem_base + pos.s * STAGE_BYTES;
           mbar_expect_tx(full_bar(pos.s), p.stage_tx);
           issue_loads<KIND>(p, tl, kb, sA, sA + A_BYTES, full_bar(pos.s));
-          pos.next(NST);
+          pos.next(STAGES);
         }
       }
       chain_next();  // not earlier: blocks of the next kernel that only wait would sit beside the main loop
@@ -124,8 +102,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
         // gave up: the copies already issued still land in this CTA's shared memory - wait for them (bounded again)
         // before the CTA may exit
         record_status(p.status, DEV_TIMEOUT, 100 + KIND);
-        for (uint32_t i = it > static_cast<uint32_t>(NST) ? it - NST : 0; i < it; ++i)
-          mbar_wait(full_bar(i % NST), (i / NST) & 1u);
+        for (uint32_t i = it > static_cast<uint32_t>(STAGES) ? it - STAGES : 0; i < it; ++i)
+          mbar_wait(full_bar(i % STAGES), (i / STAGES) & 1u);
       }
     }
   } else if (warp == 1) {
@@ -167,9 +145,9 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
           }
           clk.add(1);
           tc_fence_after();
-          const uint64_t off = (pos.s * stage_stride) >> 4;
+          const uint64_t off = (pos.s * STAGE_BYTES) >> 4;
           const uint32_t done = empty_bar(pos.s);
-          pos.next(NST);
+          pos.next(STAGES);
           ready = kb + 1 < tl.nkb && mbar_try_wait(full_bar(pos.s), pos.phase);
           const int nks = kb == tl.nkb - 1 ? tl.klast : BK / 16;
 #pragma unroll
@@ -185,13 +163,13 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
       if (!ok) {
         // gave up: let every MMA issued so far finish (bounded) before the tensor memory is freed
         record_status(p.status, DEV_TIMEOUT, 200 + KIND);
-        umma_commit(bar0 + 8u * (2 * MAX_STAGES + 4));
-        mbar_wait(bar0 + 8u * (2 * MAX_STAGES + 4), 0u);
+        umma_commit(bar0 + 8u * (2 * STAGES + 4));
+        mbar_wait(bar0 + 8u * (2 * STAGES + 4), 0u);
       }
     }
   } else if (warp < 2 + EPI_WARPS) {
     // ------------------------------------------------------------------ epilogue (128 TMEM lanes; two warps per
-    // lane quadrant, each draining half of the tile's columns; routing needs whole rows: one selects, one sums)
+    // lane quadrant, each draining half of the tile's columns)
     const int ew = warp & 3;           // TMEM lane quadrant this warp may read
     const int half = (warp - 2) >> 2;  // which half of the columns
     EpiStage es{smem_base + STAGES * STAGE_BYTES + (warp - 2) * (EPI_UNITS * EPI_UNIT_BYTES), 0u};
@@ -235,17 +213,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
         tc_fence_before();
         mbar_arrive(tempty_bar(acc));
       };
-      if (KIND == GEMM_RT) {
-        if (p.N_total <= 128 && p.top_k <= ROUTE_SMEM_MAX_K) {
-          if (half == 0)
-            routing_epilogue_smem(p, s_bias, s_hist, rt_scratch, rt_scratch + ROUTE_SCRATCH_BYTES, row, tl.row0 / BM,
-                                  ew, taddr, lane);
-          else
-            routing_softmax_sums(p, s_bias, row, tl.row0 / BM, ew, taddr, lane);
-        } else if (half == 0) {
-          routing_epilogue_tmem(p, s_bias, row, tl.row0 / BM, ew, taddr, lane);
-        }
-      } else if (KIND == GEMM_DWR) {
+      if (KIND == GEMM_DWR) {
         // fp32 partial of dW_r for this token slice: hi and lo halves of dl share one accumulator pair
         const int m = tl.m0 + rin;
 #pragma unroll 1
@@ -275,7 +243,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                                                 : 32,
                               es, lane, half, release);
       }
-      if (KIND == GEMM_RT || KIND == GEMM_DWR) release();
+      if (KIND == GEMM_DWR) release();
     }
     if (clocked()) {
       sum_cycles(p.timers + 5, true);
@@ -298,58 +266,6 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
 }
 
 // ------------------------------------------------------------------------------------------ host side
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-// bf16 row-major [rows, width] -> 2D map with box {64, box_rows}
-static bool map_2d(void* fn, CUtensorMap* m, const void* base, int64_t rows, int64_t width, int box_rows) {
-  cuuint64_t dims[2] = {static_cast<cuuint64_t>(width), static_cast<cuuint64_t>(rows)};
-  cuuint64_t strides[1] = {static_cast<cuuint64_t>(width) * 2};
-  cuuint32_t box[2] = {64, static_cast<cuuint32_t>(box_rows)};
-  cuuint32_t es[2] = {1, 1};
-  return reinterpret_cast<EncodeTiledFn>(fn)(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims,
-                                             strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                                             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                                             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-// bf16 [E, rows, width] -> 3D map with box {64, box_rows, 1}
-static bool map_3d(void* fn, CUtensorMap* m, const void* base, int64_t E, int64_t rows, int64_t width,
-                   int box_rows) {
-  cuuint64_t dims[3] = {static_cast<cuuint64_t>(width), static_cast<cuuint64_t>(rows), static_cast<cuuint64_t>(E)};
-  cuuint64_t strides[2] = {static_cast<cuuint64_t>(width) * 2, static_cast<cuuint64_t>(width) * rows * 2};
-  cuuint32_t box[3] = {64, static_cast<cuuint32_t>(box_rows), 1};
-  cuuint32_t es[3] = {1, 1, 1};
-  return reinterpret_cast<EncodeTiledFn>(fn)(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims,
-                                             strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                                             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                                             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// MN-major operands, `chunks` 64-column chunks of 64 K rows in one box that lands in shared memory chunk by chunk.  The
-// chunk is a dimension of the map (64 columns apart), so the width has to be a multiple of 64, or at most 64 with one
-// chunk in use (columns beyond the width read as zeros).
-static bool map_chunks(void* fn, CUtensorMap* m, const void* base, int64_t E, int64_t rows, int64_t width, int chunks,
-                       int rank) {
-  cuuint64_t dims[4] = {static_cast<cuuint64_t>(width < 64 ? width : 64), static_cast<cuuint64_t>(rows),
-                        static_cast<cuuint64_t>((width + 63) / 64), static_cast<cuuint64_t>(E)};
-  cuuint64_t strides[3] = {static_cast<cuuint64_t>(width) * 2, 128, static_cast<cuuint64_t>(width) * rows * 2};
-  cuuint32_t box[4] = {64, 64, static_cast<cuuint32_t>(chunks), 1};
-  cuuint32_t es[4] = {1, 1, 1, 1};
-  return reinterpret_cast<EncodeTiledFn>(fn)(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void*>(base), dims,
-                                             strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                                             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                                             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-// bf16 weights [E, rows, width]: coordinates (0, row, chunk, expert)
-static bool map_mn(void* fn, CUtensorMap* m, const void* base, int64_t E, int64_t rows, int64_t width, int chunks) {
-  return map_chunks(fn, m, base, E, rows, width, chunks, 4);
-}
-// bf16 rows [rows, width]: coordinates (0, row, chunk)
-static bool map_mn_rows(void* fn, CUtensorMap* m, const void* base, int64_t rows, int64_t width, int chunks) {
-  return map_chunks(fn, m, base, 1, rows, width, chunks, 3);
-}
-
 template <int KIND, Accumulate ACC = Accumulate::NONE>
 static moe_status launch_kind(moe_ctx_impl* ctx, const GemmParams& p, cudaStream_t st) {
   auto* const kernel = grouped_gemm_kernel<KIND, ACC>;
@@ -520,40 +436,6 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
       return pair         ? launch_pair_gemm(ctx, kind, p, st)
              : p.acc_fp32 ? launch_kind<GEMM_B5, Accumulate::LOAD_ADD>(ctx, p, st)
                           : launch_kind<GEMM_B5>(ctx, p, st);
-    case GEMM_RT:
-      // logits[T,E] = x[T,d] W_r[d,E]; W_r is read as a one-slab tensor so the weight loaders apply
-      p.b_chunks = (E + 63) / 64;
-      p.whole_chunks = E % 64 == 0;
-      {
-        auto map_router = [&](CUtensorMap* m, const uint16_t* w) {
-          return p.whole_chunks ? map_mn(fn, m, w, 1, d, E, p.b_chunks) : map_3d(fn, m, w, 1, d, E, 64);
-        };
-        ok = map_2d(fn, &p.mapA0, io.x, T, d, 128) && map_router(&p.mapB0, io.W_r);
-        p.mapA1 = p.mapA0; p.mapB1 = p.mapB0;
-        if (io.W_r_mid) {  // fp32 router weight: x (hi + mid + lo), each product exact in fp32
-          ok = ok && map_router(&p.mapB1, io.W_r_mid) && map_router(&p.mapB2, io.W_r_lo);
-          p.nseg = 3;
-        }
-      }
-      p.static_m_tiles = static_cast<int>((T + BM - 1) / BM);
-      p.n_tiles = 1;
-      p.k_blocks = d / BK;
-      p.N_total = E;
-      p.mma_n = (E + 15) / 16 * 16;
-      p.stage_tx = A_BYTES + p.b_chunks * CHUNK_BYTES;
-      p.T = T;
-      p.top_k = s.k;
-      p.bias = io.b_r;
-      p.logits = reinterpret_cast<float*>(ws + L.logits);
-      p.logits_out = io.logits_out;
-      p.idx = reinterpret_cast<int32_t*>(ws + L.idx);
-      p.gates = reinterpret_cast<float*>(ws + L.gates);
-      p.idx_out = io.idx_out;
-      p.gates_out = io.gates_out;
-      p.psum_part = reinterpret_cast<float*>(ws + L.psum_part);
-      p.tile_counts = reinterpret_cast<int32_t*>(ws + L.tile_counts);  // written by the shared-memory routing epilogue
-      if (!ok) return MOE_ERR_CUDA;
-      return launch_kind<GEMM_RT>(ctx, p, st);
     case GEMM_DX:
       // dxr[T,d] = dl_hi W_r^T + dl_lo W_r^T
       ok = map_2d(fn, &p.mapA0, ws + L.dl_hi, T, E, 128) && map_2d(fn, &p.mapA1, ws + L.dl_lo, T, E, 128) &&
@@ -568,7 +450,6 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
       p.k_blocks = (E + BK - 1) / BK;
       p.N_total = d;
       p.T = T;
-      p.top_k = s.k;
       p.out0 = reinterpret_cast<uint16_t*>(ws + L.dxr);
       p.ld_out = d;
       if (!ok) return MOE_ERR_CUDA;

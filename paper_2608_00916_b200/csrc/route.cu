@@ -1,7 +1,7 @@
 // Router (fp32 logits, softmax, top-k with lowest-index tie-break, renormalised gates) and the
 // deterministic token permutation (per-tile histogram, prefix scan, stable scatter, row copy).  The router kernel here
 // is the SIMT path (expert counts that are not a multiple of 8, or caller-supplied logits); otherwise the logits are
-// contracted on the tensor cores (gemm.cu, kind RT).
+// contracted on the tensor cores (router.cu).
 #include <algorithm>
 
 #include "common.cuh"
@@ -206,7 +206,7 @@ void launch_router(const Shape& s, int64_t T, const uint16_t* x, const uint16_t*
 // the order inside an expert is the token order.  Each warp covers 32 consecutive tokens and records, per
 // expert, the 32-bit mask of its tokens that chose it (atomicOr: order-free, hence deterministic); ranks
 // are population counts of mask prefixes.  Tiles of TOK_TILE tokens are combined by a column scan.
-// The routers above and in gemm_common.cuh write k distinct experts in [0, E) for every token, NaN logits included.  The
+// The routers above and in router.cu write k distinct experts in [0, E) for every token, NaN logits included.  The
 // kernels below index with them; a pick out of that range (an overwritten workspace) never leaves their tables.
 __device__ __forceinline__ void build_masks(uint32_t* masks /* [TOK_WARPS][E] */, const int32_t* idx, int64_t T,
                                             int E, int k, int64_t tile_t0) {
@@ -568,19 +568,13 @@ void launch_gather_rows(const Shape& s, int64_t T, const WsLayout& L, const char
       debug ? reinterpret_cast<int32_t*>(const_cast<char*>(ws) + L.status) : nullptr, L.rows_max);
 }
 
-// First kernel of every forward call: clears the row gates (pad rows must read 0) and makes sure the workspace's status
-// block is initialised.  A status block that already carries the cookie is left alone, so a failure recorded by an
-// earlier call stays visible until the host has reported it; memory seen for the first time gets a clean block.
+// First kernel of a forward call without the tensor-core router, which does the same: clears the row gates (pad rows must
+// read 0) and makes sure the workspace's status block is initialised.
 __global__ void __launch_bounds__(256) prepare_kernel(int32_t* __restrict__ status, float* __restrict__ row_gate,
                                                       int64_t rows) {
   chain_wait();
   chain_next();
-  if (blockIdx.x == 0 && threadIdx.x == 0 && (status[2] != STATUS_COOKIE0 || status[3] != STATUS_COOKIE1)) {
-    status[0] = DEV_OK;
-    status[1] = 0;
-    status[2] = STATUS_COOKIE0;
-    status[3] = STATUS_COOKIE1;
-  }
+  init_status_block(status, blockIdx.x == 0 && threadIdx.x == 0);
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x; i < rows; i += static_cast<int64_t>(gridDim.x) * 256)
     row_gate[i] = 0.f;
 }

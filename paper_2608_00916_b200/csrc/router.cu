@@ -1,0 +1,491 @@
+// Router on the tensor cores: logits = x W_r (+ b_r), softmax statistics, top-k, gates, and the permutation's per-tile
+// histogram, in one kernel.  x and W_r are bf16 (an fp32 W_r comes as three exact bf16 terms), so that a bf16 MMA with fp32
+// accumulation is an fp32 contraction up to summation order.
+//
+// A cluster of CL CTAs takes one tile of 128 tokens and splits the K blocks; every CTA contracts its share into tensor
+// memory (128 tokens x E), copies it to shared memory, and then routes 128 / CL of the tokens, adding up the CL partial
+// sums of their logits through distributed shared memory in rank order.  What bounds it: up to a few thousand tokens the
+// latency of fetching x and W_r through few SMs (one CTA per tile fetches d * (256 + 2 E) bytes: 1 MB at d 2048, E 128) and of
+// routing the tokens, hence the split; from there on the stream of x from HBM, two CTAs to an SM.
+//
+// Three steps between barriers.  (1) A warp per token: the sum of the partial logits, which replaces the row in this CTA's
+// shared memory, the softmax and its column sums; a lane holds NV / 4 groups of four columns.  (2) A thread per token: top-k
+// as a three-level tournament, groups of four columns, supers of four groups, the maxima of the supers in registers; a round
+// takes the largest super (lowest among equals), the group and the column in it, removes the column and repairs the maxima
+// above it, which is the rule "largest, lowest index among equals" because the levels partition the columns in order.
+// (3) The picks and gates leave as whole lines.
+//
+// A CTA routes a handful of tokens and every instruction of that arrives cold, about 450 cycles for each eight of them.  So
+// while the operands are on their way the waiting warps run the steps once on whatever shared memory holds, each warp one
+// step, so that the code is fetched side by side; what this first pass stores is overwritten by the same threads.
+#include <string.h>
+
+#include "common.cuh"
+#include "ptx.cuh"
+#include "tensor_maps.cuh"
+
+namespace moe {
+
+constexpr int RO_TOK = 128;                    // tokens of a tile (the permutation's token tile as well)
+constexpr int RO_WARPS = 12;                   // routing warps
+constexpr int RO_THREADS = 64 + 32 * RO_WARPS;  // warps: 0 TMA producer, 1 MMA issuer, 2.. routing
+constexpr int RO_BK = 64;
+constexpr int RO_A_BYTES = RO_TOK * RO_BK * 2;   // 16 KB of x per K block
+constexpr int RO_CHUNK_BYTES = 64 * RO_BK * 2;   // 8 KB per 64 columns of W_r
+constexpr int RO_MAX_STAGES = 4;
+static_assert(RO_TOK == TOK_TILE, "the histogram written here is the permutation's");
+
+struct RouterParams {
+  CUtensorMap map_x, map_w0, map_w1, map_w2;
+  int32_t* status;
+  float* row_gate;       // cleared here: pad rows must read 0
+  int64_t rows;
+  const float* bias;     // [E] or null
+  float* logits;         // [T, E] saved logits
+  float* logits_out;     // optional copy for the caller
+  int32_t *idx, *idx_out;
+  float *gates, *gates_out;
+  float* psum_part;      // [CTAs with tokens, E] column sums of p
+  int32_t* tile_counts;  // [tiles, E] picks of every 128-token tile
+  int64_t T;
+  int E, k;
+  int k_blocks, k_total;  // K blocks of one bf16 term of W_r, and of all terms
+  int b_chunks, whole_chunks;
+  int mma_n, stages;
+  uint32_t stage_bytes, tmem_cols;
+};
+
+__device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void red_cluster_add(uint32_t addr, int v) {
+  asm volatile("red.relaxed.cluster.shared::cluster.add.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
+__device__ __forceinline__ float4 lds_f4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
+  return v;
+}
+__device__ __forceinline__ void sts_f4(uint32_t addr, float4 v) {
+  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+__device__ __forceinline__ float max4(float4 v) { return fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)); }
+// index (0..3) of the first component equal to m
+__device__ __forceinline__ int first_eq4(float4 v, float m) { return v.x == m ? 0 : (v.y == m ? 1 : (v.z == m ? 2 : 3)); }
+__device__ __forceinline__ float4 without(float4 v, int i, float by) {
+  return make_float4(i == 0 ? by : v.x, i == 1 ? by : v.y, i == 2 ? by : v.z, i == 3 ? by : v.w);
+}
+__device__ __forceinline__ int lds_int(uint32_t addr) {
+  int v;
+  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ float warp_max(float v) {  // NaN is dropped
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v = fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, off));
+  return v;
+}
+__device__ __forceinline__ float warp_sum(float v) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
+  return v;
+}
+
+// A NaN logit counts as -inf in the selection, and every token gets k distinct experts whatever its logits are (the
+// permutation indexes its tables with the picks): once nothing larger than -inf is left, the lowest index that is not among
+// the j picks so far is taken.  picks: the token's picks {exponential, column}, `pitch` bytes apart.
+__device__ __forceinline__ int lowest_untaken(int j, uint32_t picks, uint32_t pitch) {
+  int e = 0;
+#pragma unroll 1
+  for (int q = 0; q < j;) {
+    if (lds_int(picks + q * pitch + 4) == e) {
+      ++e;
+      q = 0;
+    } else {
+      ++q;
+    }
+  }
+  return e;
+}
+
+// Top-k of one token: `row` its logits (missing columns are -inf), `maxima` the maxima of its groups, both in shared memory and
+// used up.  Leaves the picks and returns 1 / sum of their exponentials.
+template <int SUPERS>
+__device__ __forceinline__ float select_topk(int k, uint32_t row, uint32_t maxima, uint32_t picks, uint32_t pick_pitch, int* s_hist,
+                                             int count) {
+  float sm[SUPERS];
+#pragma unroll
+  for (int q = 0; q < SUPERS; ++q) sm[q] = max4(lds_f4(maxima + q * 16));
+  float vmax = 0.f, zs = 0.f;
+#pragma unroll 1
+  for (int j = 0; j < k; ++j) {
+    float best = sm[0];
+#pragma unroll
+    for (int q = 1; q < SUPERS; ++q) best = fmaxf(best, sm[q]);
+    int s = SUPERS - 1;
+#pragma unroll
+    for (int q = SUPERS - 2; q >= 0; --q) s = (sm[q] == best) ? q : s;
+    const float4 g4 = lds_f4(maxima + s * 16);
+    const int gi = first_eq4(g4, best), g = s * 4 + gi;
+    const float4 v4 = lds_f4(row + g * 16);
+    const int ci = first_eq4(v4, best);
+    int col = g * 4 + ci;
+    if (!(best > -INFINITY)) col = lowest_untaken(j, picks, pick_pitch);
+    if (j == 0) vmax = best;
+    const float ex = expf(best - vmax);
+    zs += ex;
+    asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(picks + j * pick_pitch), "r"(__float_as_uint(ex)), "r"(col) : "memory");
+    atomicAdd(&s_hist[col], count);  // the tile's histogram (integer adds: order-free)
+    const float4 nv = without(v4, ci, -INFINITY);
+    sts_f4(row + g * 16, nv);
+    const float4 ng = without(g4, gi, max4(nv));
+    sts_f4(maxima + s * 16, ng);
+    const float ns = max4(ng);
+#pragma unroll
+    for (int q = 0; q < SUPERS; ++q) sm[q] = (q == s) ? ns : sm[q];
+  }
+  return 1.f / zs;
+}
+
+__device__ __forceinline__ void routing_sync() { asm volatile("bar.sync 1, %0;" ::"n"(32 * RO_WARPS) : "memory"); }
+
+template <int CL>
+__device__ __forceinline__ void cluster_or_block_sync() {
+  if (CL > 1)
+    cluster_sync_diverged();
+  else
+    block_sync_diverged();
+}
+
+template <int CL, int NV>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, NV == 4 ? 2 : 1)
+    router_cluster_kernel(const __grid_constant__ RouterParams p) {
+  extern __shared__ unsigned char ro_smem_raw[];
+  __shared__ __align__(8) uint64_t bars[2 * RO_MAX_STAGES + 1];  // full, empty, accumulator complete
+  __shared__ uint32_t tmem_base_slot;
+  __shared__ int s_hist[32 * NV];
+  __shared__ __align__(16) float s_psum[RO_WARPS][32 * NV];
+  __shared__ __align__(16) float s_first[40 * NV + 4];  // a row, its maxima and a pick for the first pass of the selection
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int rank = CL > 1 ? static_cast<int>(cluster_ctarank()) : 0;
+  const int tile = blockIdx.x / CL;
+  const int64_t t0 = static_cast<int64_t>(tile) * RO_TOK;
+  const uint32_t smem_base = (smem_u32(ro_smem_raw) + 1023u) & ~1023u;
+  const uint32_t bar0 = smem_u32(bars);
+  const uint32_t acc_bar = bar0 + 8u * (2 * RO_MAX_STAGES);
+  auto full_bar = [&](int s) { return bar0 + 8u * s; };
+  auto empty_bar = [&](int s) { return bar0 + 8u * (RO_MAX_STAGES + s); };
+  const int kb0 = p.k_total * rank / CL, kb1 = p.k_total * (rank + 1) / CL;  // this CTA's K blocks
+
+  if (tid == 0) {
+    for (int s = 0; s < p.stages; ++s) {
+      mbar_init(full_bar(s), 1);
+      mbar_init(empty_bar(s), 1);
+    }
+    mbar_init(acc_bar, 1);
+    fence_mbar_init();
+    tma_prefetch_desc(&p.map_x);
+    tma_prefetch_desc(&p.map_w0);
+  }
+  if (warp == 1) {
+    tmem_alloc(smem_u32(&tmem_base_slot), p.tmem_cols);
+    tmem_relinquish();
+  }
+  for (int i = tid; i < 32 * NV; i += RO_THREADS) s_hist[i] = 0;
+  chain_wait();  // everything above touches only this CTA's own state
+  init_status_block(p.status, blockIdx.x == 0 && tid == 0);  // long before a wait of this kernel can run out
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = tmem_base_slot;
+
+  if (warp == 0) {
+    if (elect_one()) {  // TMA producer
+      int s = 0;
+      uint32_t phase = 0, it = 0;
+      bool ok = true;
+      for (int kb = kb0; kb < kb1; ++kb, ++it) {
+        if (!mbar_wait(empty_bar(s), phase ^ 1u)) {
+          ok = false;
+          break;
+        }
+        const uint32_t sA = smem_base + s * p.stage_bytes, sB = sA + RO_A_BYTES, bar = full_bar(s);
+        const int seg = kb / p.k_blocks, kk = (kb - seg * p.k_blocks) * RO_BK;
+        const CUtensorMap* mw = seg == 0 ? &p.map_w0 : (seg == 1 ? &p.map_w1 : &p.map_w2);
+        mbar_expect_tx(bar, p.stage_bytes);
+        tma_load_2d(sA, &p.map_x, bar, kk, static_cast<int>(t0));
+        if (p.whole_chunks) {
+          tma_load_4d(sB, mw, bar, 0, kk, 0, 0);
+        } else {  // E is not a multiple of 64: a box per chunk, the last one clipped
+          for (int c = 0; c < p.b_chunks; ++c) tma_load_3d(sB + c * RO_CHUNK_BYTES, mw, bar, c * 64, kk, 0);
+        }
+        if (++s == p.stages) {
+          s = 0;
+          phase ^= 1u;
+        }
+      }
+      chain_next();
+      if (!ok) {  // gave up: the copies in flight land in this CTA's shared memory before it leaves (bounded again)
+        record_status(p.status, DEV_TIMEOUT, 106);
+        const uint32_t n = static_cast<uint32_t>(p.stages);
+        for (uint32_t i = it > n ? it - n : 0; i < it; ++i) mbar_wait(full_bar(i % n), (i / n) & 1u);
+      }
+    }
+  } else if (warp == 1) {
+    if (elect_one()) {  // MMA issuer
+      const uint32_t idesc = umma_idesc(RO_TOK, p.mma_n, 0, 1);
+      const uint64_t descA = smem_desc(smem_base, 0, 1024);
+      const uint64_t descB = smem_desc(smem_base + RO_A_BYTES, RO_CHUNK_BYTES, 1024);
+      int s = 0;
+      uint32_t phase = 0;
+      bool ok = true;
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (!mbar_wait(full_bar(s), phase)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint64_t off = (static_cast<uint64_t>(s) * p.stage_bytes) >> 4;
+#pragma unroll
+        for (int ks = 0; ks < RO_BK / 16; ++ks)
+          umma_bf16(tmem_base, descA + off + (ks * 32 >> 4), descB + off + (ks * 2048 >> 4), idesc, (kb != kb0 || ks != 0) ? 1u : 0u);
+        umma_commit(empty_bar(s));
+        if (++s == p.stages) {
+          s = 0;
+          phase ^= 1u;
+        }
+      }
+      if (!ok) record_status(p.status, DEV_TIMEOUT, 206);
+      // also after giving up: the MMAs issued so far finish before the waiting warps go on and the tensor memory is freed
+      umma_commit(acc_bar);
+      if (!ok) mbar_wait(acc_bar, 0u);
+    }
+  } else {
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * (RO_WARPS * 32) + (tid - 64); i < p.rows;
+         i += static_cast<int64_t>(gridDim.x) * (RO_WARPS * 32))
+      p.row_gate[i] = 0.f;
+  }
+
+  const uint32_t part = smem_base;  // partial logits of the tile, over the operand stages
+  constexpr uint32_t PITCH = 32 * NV * 4 + 16;  // rows 16 bytes apart in the banks
+  if (warp < 2) cluster_or_block_sync<CL>();
+  if (warp >= 2) {
+    constexpr int MINE = RO_TOK / CL;  // this CTA's tokens of the tile
+    constexpr uint32_t MAX_PITCH = 32 * (NV / 4) * 4 + 16;
+    const uint32_t maxima = part + RO_TOK * PITCH;              // of the groups of four columns: MINE rows
+    const uint32_t picks = maxima + MINE * MAX_PITCH;           // {exponential, column}: k rows of MINE (and one, in other banks)
+    const uint32_t pick_pitch = MINE * 8 + 8, recip = picks + p.k * pick_pitch;  // 1 / sum of the exponentials
+    const int w = warp - 2, E = p.E, k = p.k;
+    const int64_t first = t0 + rank * MINE, left = p.T - first;
+    const int tokens = left < MINE ? static_cast<int>(left) : MINE;  // of which are there (may be negative)
+    float acc[NV];
+#pragma unroll
+    for (int q = 0; q < NV; ++q) acc[q] = 0.f;
+#pragma unroll 1
+    for (int pass = w % 3;; pass = 3) {  // 0, 1, 2: that step only, before there is anything to route; 3: all of them
+      const bool all = pass == 3;
+      if (all || pass == 0) {
+#pragma unroll 1
+        for (int i = w; i < (all ? tokens : w + 1); i += RO_WARPS) {
+          const uint32_t mrow = maxima + (i < MINE ? i : 0) * MAX_PITCH;
+          float v[NV];
+          float vmax = -INFINITY;
+#pragma unroll
+          for (int q = 0; q < NV / 4; ++q) {
+            const int col = 4 * (lane + 32 * q);
+            const uint32_t a = part + (rank * MINE + (i < MINE ? i : 0)) * PITCH + col * 4;
+            float4 x[CL];
+#pragma unroll
+            for (int r = 0; r < CL; ++r) x[r] = ld_cluster_f4(CL > 1 ? mapa_shared(a, all ? r : rank) : a);
+            float4 sum = x[0];
+#pragma unroll
+            for (int r = 1; r < CL; ++r) sum = make_float4(sum.x + x[r].x, sum.y + x[r].y, sum.z + x[r].z, sum.w + x[r].w);
+            if (col < E) {  // E is a multiple of 8: the four columns exist or do not
+              if (p.bias) {
+                const float4 b = *reinterpret_cast<const float4*>(p.bias + col);
+                sum = make_float4(sum.x + b.x, sum.y + b.y, sum.z + b.z, sum.w + b.w);
+              }
+              if (i < tokens) {
+                const int64_t at = (first + i) * E + col;
+                *reinterpret_cast<float4*>(p.logits + at) = sum;
+                if (p.logits_out) *reinterpret_cast<float4*>(p.logits_out + at) = sum;
+              }
+            } else {
+              sum = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+            }
+            if (all) sts_f4(a, sum);
+            v[4 * q] = sum.x;
+            v[4 * q + 1] = sum.y;
+            v[4 * q + 2] = sum.z;
+            v[4 * q + 3] = sum.w;
+            const float m = max4(sum);
+            if (all) asm volatile("st.shared.f32 [%0], %1;" ::"r"(mrow + (lane + 32 * q) * 4), "f"(m) : "memory");
+            vmax = fmaxf(vmax, m);
+          }
+          vmax = warp_max(vmax);
+          float z = 0.f;
+#pragma unroll
+          for (int q = 0; q < NV; ++q) {
+            v[q] = expf(v[q] - vmax);
+            z += v[q];
+          }
+          const float rz = 1.f / warp_sum(z);
+#pragma unroll
+          for (int q = 0; q < NV; ++q) acc[q] = fmaf(v[q], rz, acc[q]);
+        }
+      }
+      if (all) routing_sync();
+      const int t = tid - 64;
+      if (all ? t < tokens : pass == 1) {
+        const uint32_t scratch = smem_u32(s_first);
+        const float rz = select_topk<2 * NV>(all ? k : 1, all ? part + (rank * MINE + t) * PITCH : scratch,
+                                             all ? maxima + t * MAX_PITCH : scratch + 32 * NV * 4,
+                                             all ? picks + t * 8 : scratch + 40 * NV * 4, pick_pitch, s_hist, all ? 1 : 0);
+        asm volatile("st.shared.f32 [%0], %1;" ::"r"(all ? recip + t * 4 : scratch + 40 * NV * 4 + 8), "f"(rz) : "memory");
+      }
+      if (all) routing_sync();
+      if (all || pass == 2) {
+#pragma unroll 1
+        for (int i = t; i < tokens * k; i += 32 * RO_WARPS) {
+          const int tok = i / k, j = i - tok * k;
+          uint32_t exb, col;
+          asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(exb), "=r"(col) : "r"(picks + j * pick_pitch + tok * 8) : "memory");
+          const float g = __uint_as_float(exb) * __int_as_float(lds_int(recip + tok * 4));
+          const int64_t at = first * k + i;
+          p.idx[at] = static_cast<int32_t>(col);
+          p.gates[at] = g;
+          p.idx_out[at] = static_cast<int32_t>(col);
+          p.gates_out[at] = g;
+          if (!all) break;
+        }
+      }
+      if (all) break;
+      // partial logits: tensor memory -> shared memory (the operand stages have all been consumed)
+      const bool ok = mbar_wait(acc_bar, 0u);
+      if (!ok && lane == 0) record_status(p.status, DEV_TIMEOUT, 306);
+      tc_fence_after();
+      const int ew = warp & 3, row = ew * 32 + lane;
+      if (ok)
+        for (int c = w >> 2; c * 16 < E; c += RO_WARPS / 4) {
+          uint32_t r[16];
+          tmem_ld16(tmem_base + (static_cast<uint32_t>(ew * 32) << 16) + c * 16, r);
+          tmem_ld_wait();
+#pragma unroll
+          for (int b = 0; b < 4; ++b)
+            st_shared_v4(part + row * PITCH + c * 64 + b * 16, r[4 * b], r[4 * b + 1], r[4 * b + 2], r[4 * b + 3]);
+        }
+      tc_fence_before();
+      cluster_or_block_sync<CL>();
+#pragma unroll
+      for (int q = 0; q < NV; ++q) acc[q] = 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < NV; ++q) s_psum[w][4 * (lane + 32 * (q / 4)) + q % 4] = acc[q];
+    routing_sync();
+    const int e = tid - 64;
+    if (e < E) {
+      float s = 0.f;
+#pragma unroll 4
+      for (int u = 0; u < RO_WARPS; ++u) s += s_psum[u][e];
+      if (tokens > 0) p.psum_part[static_cast<int64_t>(blockIdx.x) * E + e] = s;
+      if (CL > 1 && rank != 0) red_cluster_add(mapa_shared(smem_u32(&s_hist[e]), 0), s_hist[e]);
+      if (CL == 1) p.tile_counts[static_cast<int64_t>(tile) * E + e] = s_hist[e];
+    }
+  }
+  if (CL > 1) {
+    cluster_sync_diverged();  // nobody reads this CTA's shared memory any more; the counts of the tile are complete
+    if (rank == 0 && tid >= 64 && tid - 64 < p.E) p.tile_counts[static_cast<int64_t>(tile) * p.E + tid - 64] = s_hist[tid - 64];
+  }
+  if (warp == 1) {
+    __syncwarp();  // freeing tensor memory takes the whole warp
+    tc_fence_after();
+    tmem_dealloc(tmem_base, p.tmem_cols);
+  }
+}
+
+// CTAs per token tile: four while each has an SM to itself, two while two share one (E <= 128), never more than there are K
+// blocks.  Router stage at d 2048, 128 experts, us, with one / two / four / eight: 128 tokens 30 / 23 / 18 / 18, 2048 30 / 23 /
+// 19 / 22, 4736 (148 CTAs of four) 30 / 24 / 23 / 34, 8192 32 / 25 / 25 / 40, 9472 32 / 27 / 36 / 51, 16384 35 / 32 / 42, 18944
+// (296 CTAs of two) 36 / 35 / 53, 24576 40 / 49 / 57.  One CTA per tile in the persistent GEMM template, its 128 tokens routed by
+// four warps: 28 at 128 to 4096 tokens, 31 at 8192, 33 at 16384, 48 at 32768, where this kernel takes 18 to 24, 25, 32 and 44.
+int router_cluster(const Shape& s, int sm_count, int64_t T, bool fp32_weight) {
+  const int64_t tiles = (T + RO_TOK - 1) / RO_TOK;
+  const int k_total = s.d / RO_BK * (fp32_weight ? 3 : 1);
+  const int cl = tiles * 4 <= sm_count ? 4 : tiles * 2 <= sm_count * (s.E <= 128 ? 2 : 1) ? 2 : 1;
+  return cl <= k_total ? cl : k_total < 2 ? 1 : 2;
+}
+
+template <int CL, int NV>
+static moe_status launch_one(moe_ctx_impl* ctx, const RouterParams& p, int tiles, size_t smem, cudaStream_t st) {
+  auto* const kernel = router_cluster_kernel<CL, NV>;
+  constexpr int slot = (CL == 1 ? 0 : CL == 2 ? 1 : 2) + (NV == 4 ? 0 : 4);
+  if (!(ctx->router_attr & (1u << slot))) {  // per device: the context is bound to one (and to one top-k)
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+      return MOE_ERR_CUDA;
+    ctx->router_attr |= 1u << slot;
+  }
+  launch_kernel(kernel, tiles * CL, RO_THREADS, smem, st, p);
+  return cudaGetLastError() == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
+}
+
+moe_status launch_router_tc(moe_ctx_impl* ctx, int64_t T, const WsLayout& L, char* ws, const GemmIO& io, cudaStream_t st) {
+  const Shape& s = ctx->s;
+  void* fn = ctx->encode_fn;
+  RouterParams p;
+  memset(&p, 0, sizeof(p));
+  p.E = s.E;
+  p.k = s.k;
+  p.T = T;
+  p.b_chunks = (s.E + 63) / 64;
+  p.whole_chunks = s.E % 64 == 0;
+  auto map_w = [&](CUtensorMap* m, const uint16_t* w) {  // W_r as a one-slab tensor of weights
+    return p.whole_chunks ? map_mn(fn, m, w, 1, s.d, s.E, p.b_chunks) : map_3d(fn, m, w, 1, s.d, s.E, 64);
+  };
+  bool ok = map_2d(fn, &p.map_x, io.x, T, s.d, RO_TOK) && map_w(&p.map_w0, io.W_r);
+  if (io.W_r_mid) ok = ok && map_w(&p.map_w1, io.W_r_mid) && map_w(&p.map_w2, io.W_r_lo);
+  if (!ok) return MOE_ERR_CUDA;
+  p.k_blocks = s.d / RO_BK;
+  p.k_total = p.k_blocks * (io.W_r_mid ? 3 : 1);
+  p.mma_n = (s.E + 15) / 16 * 16;
+  p.stage_bytes = RO_A_BYTES + p.b_chunks * RO_CHUNK_BYTES;
+  const bool narrow = s.E <= 128;
+  p.stages = narrow ? 3 : RO_MAX_STAGES;
+  p.tmem_cols = s.E <= 32 ? 32 : s.E <= 64 ? 64 : s.E <= 128 ? 128 : 256;
+  p.status = reinterpret_cast<int32_t*>(ws + L.status);
+  p.row_gate = reinterpret_cast<float*>(ws + L.row_gate);
+  p.rows = L.rows_alloc;
+  p.bias = io.b_r;
+  p.logits = reinterpret_cast<float*>(ws + L.logits);
+  p.logits_out = io.logits_out;
+  p.idx = reinterpret_cast<int32_t*>(ws + L.idx);
+  p.gates = reinterpret_cast<float*>(ws + L.gates);
+  p.idx_out = io.idx_out;
+  p.gates_out = io.gates_out;
+  p.psum_part = reinterpret_cast<float*>(ws + L.psum_part);
+  p.tile_counts = reinterpret_cast<int32_t*>(ws + L.tile_counts);
+  const int tiles = static_cast<int>((T + RO_TOK - 1) / RO_TOK);
+  const int cl = router_cluster(s, ctx->sm_count, T, io.W_r_mid != nullptr);
+  // three stages of 32 KB (E <= 128) or four of up to 48 KB, and over them what the routing needs: 128 rows of partial logits,
+  // for the CTA's tokens the maxima of their groups, and {pick, column} and 1 / sum for k picks
+  const size_t nv = narrow ? 4 : 8, mine = RO_TOK / cl;
+  const size_t ring = narrow ? 3 * (RO_A_BYTES + 2 * RO_CHUNK_BYTES) : RO_MAX_STAGES * (RO_A_BYTES + 4 * RO_CHUNK_BYTES);
+  const size_t routing = RO_TOK * (128 * nv + 16) + mine * (32 * nv + 16) + s.k * (mine * 8 + 8) + mine * 4;
+  const size_t smem = (ring > routing ? ring : routing) + 1024;
+  if (narrow) {
+    switch (cl) {
+      case 4: return launch_one<4, 4>(ctx, p, tiles, smem, st);
+      case 2: return launch_one<2, 4>(ctx, p, tiles, smem, st);
+      default: return launch_one<1, 4>(ctx, p, tiles, smem, st);
+    }
+  }
+  switch (cl) {
+    case 4: return launch_one<4, 8>(ctx, p, tiles, smem, st);
+    case 2: return launch_one<2, 8>(ctx, p, tiles, smem, st);
+    default: return launch_one<1, 8>(ctx, p, tiles, smem, st);
+  }
+}
+
+}  // namespace moe

@@ -1,0 +1,30 @@
+"""The properties of test_chained_sources.py, read from the kernels in files of their own."""
+import pytest
+
+import test_chained_sources as rules
+
+
+@pytest.fixture(autouse=True)
+def files(monkeypatch):
+    monkeypatch.setattr(rules, "FILES", ("router.cu",))
+
+
+def test_predecessor_outputs_are_read_by_ordinary_loads():
+    for name, text in rules.sources():
+        assert "__restrict__" not in text, name
+        assert "chain_wait();" in text and "chain_next();" in text, name
+        assert "__ldg" not in text, name
+
+
+def test_barriers_after_the_one_thread_roles_do_not_need_whole_warps():
+    """One lane of a warp is in its role's loop while the others wait: the barriers of whole blocks and clusters that follow take
+    threads one by one, and the warp that frees tensor memory comes together first."""
+    for name, text in rules.sources():
+        after = text[text.index("elect_one()"):]
+        assert "__syncthreads()" not in after and "cluster_sync_all()" not in after, name
+        assert "if (warp == 1) {\n    __syncwarp();" in after, name
+
+
+def test_a_failed_launch_is_reported_once():
+    for name, text in rules.sources():
+        assert text.count("launch_kernel(") == text.count("return cudaGetLastError() == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;"), name

@@ -1,0 +1,59 @@
+"""The tensor-core router at the sizes where it changes form: the number of CTAs that share a token tile, the columns a lane
+holds, and token counts around the tokens of a CTA and of a tile."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2608_00916_b200 import synth
+from gpu_util import Run, oracle_run
+from test_gpu_parity import check_all, check_routing
+from test_routing_nonfinite import check_picks
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("T,d,E,k", [
+    (1, 512, 128, 8), (31, 512, 128, 8), (33, 512, 128, 8),        # four CTAs to a tile, 32 tokens each, most of them idle
+    (129, 512, 64, 6), (2047, 512, 128, 16),
+    (200, 64, 16, 2), (200, 128, 16, 2), (200, 192, 24, 4),        # no more CTAs than K blocks
+    (33, 512, 256, 32), (300, 512, 136, 8),                        # two groups of four columns to a lane
+    (4736, 512, 40, 3), (4737, 512, 40, 3),                        # 148 SMs: four CTAs to a tile, two
+    (18944, 128, 16, 2), (18945, 128, 16, 2),                      # two, one
+    (4737, 256, 200, 4), (9473, 256, 136, 2),                      # one CTA per SM: two, one
+])
+def test_routing_in_every_form(T, d, E, k):
+    inp = synth.make_inputs(synth.MoEShape(T, d, E, k, 64), 300 + T % 97, x_std=1.0)
+    ofw, obw = oracle_run(inp, k, 0.05)
+    check_all(Run(inp, k), ofw, obw, 0.05, stages=T < 3000)
+
+
+@pytest.mark.parametrize("T,d", [(40, 64), (40, 192), (700, 512), (5000, 128)])
+def test_fp32_router_weight_splits_over_its_terms(T, d):
+    """The K blocks of an fp32 weight's three terms are shared out like those of one."""
+    from paper_2608_00916_b200.binding import FLAG_ROUTER_FP32, MoELayer
+    E, k, f = 32, 4, 64
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d)
+    n = lambda *s: torch.empty(*s, device="cuda").normal_(generator=g)
+    x, W_r = n(T, d).bfloat16(), n(d, E) / d**0.5
+    Wg, Wu, Wd = ((0.1 * n(E, *s)).bfloat16() for s in ((d, f), (d, f), (f, d)))
+    layer = MoELayer(d, E, f, k, FLAG_ROUTER_FP32)
+    out = layer.forward(x, W_r, Wg, Wu, Wd, want_logits=True)
+    layer.poll()
+    ref = x.double() @ W_r.double()
+    # fp32 sums of 3 d exact products of a unit-variance row: 3 d ulps of the partial sums would be the worst case
+    assert (out["logits"].double() - ref).abs().max().item() <= 3 * d * 2.0**-24 * 8
+    check_picks(out, k, E)
+
+
+def test_small_and_large_clusters_agree_on_ties():
+    """Tokens with exactly equal logits (two equal columns of W_r, repeated) take the lowest index in every form."""
+    d, E, k = 512, 128, 8
+    for T in (16, 5000, 20000):
+        inp = synth.make_inputs(synth.MoEShape(T, d, E, k, 64), 5, x_std=1.0, guard=False)
+        inp["W_r"][:, 64:] = inp["W_r"][:, :64]
+        r = Run(inp, k)
+        fw = r.forward()
+        logits, idx = fw["logits"].cpu().numpy(), fw["idx"].cpu().numpy()
+        assert np.array_equal(logits[:, :64], logits[:, 64:])
+        assert np.array_equal(idx, np.argsort(-logits, axis=1, kind="stable")[:, :k])
