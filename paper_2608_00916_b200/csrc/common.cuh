@@ -102,8 +102,8 @@ struct moe_ctx_impl {
   int b4_pair_override;    // MOE_B4_PAIR = 0 / 1, if set (measurements: dgrad gate/up on one-CTA tiles / CTA pairs); else -1
   // cudaFuncSetAttribute (dynamic shared memory opt-in) is per device: remembered here, for the device the context is
   // bound to, per kernel family (0: one-CTA kernels, 1: CTA-pair kernels, 2: one-CTA
-  // weight gradients that load and add) and GEMM kind
-  unsigned char attr_done[3][16];
+  // weight gradients that load and add, 3: row GEMMs with the tokens as N) and GEMM kind
+  unsigned char attr_done[4][16];
   unsigned router_attr;  // the same for the forms of the tensor-core router, one bit each
   int profiling;
   cudaEvent_t ev[MOE_PROF_RING][MOE_NUM_STAGES][2];
@@ -225,6 +225,9 @@ struct LoraArgs {
   const uint16_t *A1 = nullptr, *B1g = nullptr, *B1u = nullptr, *A2 = nullptr, *B2 = nullptr;
   uint16_t *dA1 = nullptr, *dB1g = nullptr, *dB1u = nullptr, *dA2 = nullptr, *dB2 = nullptr;
 };
+// row GEMMs with the tokens as the N operand; lo: with the extra K segment of the adapters (gemm_tokens.cu)
+moe_status launch_token_gemm(moe_ctx_impl* ctx, GemmKind kind, const WsLayout& L, char* ws, const GemmIO& io, const LoraArgs* lo,
+                             cudaStream_t st);
 enum LoraOp {
   LORA_U = 0,  // u = s xp A1
   LORA_F3,     // [hg|hu] = xp [Wg|Wu] + u [B1g|B1u], SwiGLU epilogue

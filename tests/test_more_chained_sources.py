@@ -6,14 +6,14 @@ import test_chained_sources as rules
 
 @pytest.fixture(autouse=True)
 def files(monkeypatch):
-    monkeypatch.setattr(rules, "FILES", ("router.cu",))
+    monkeypatch.setattr(rules, "FILES", ("router.cu", "gemm_tokens.cu"))
 
 
 def test_predecessor_outputs_are_read_by_ordinary_loads():
     for name, text in rules.sources():
         assert "__restrict__" not in text, name
         assert "chain_wait();" in text and "chain_next();" in text, name
-        assert "__ldg" not in text, name
+    rules.test_non_coherent_loads_are_of_inputs_only()  # hg and hu, which the forward call has left
 
 
 def test_barriers_after_the_one_thread_roles_do_not_need_whole_warps():
