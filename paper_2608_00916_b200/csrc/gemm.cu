@@ -43,6 +43,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
   auto tfull_bar = [&](int a) { return bar0 + 8u * (2 * STAGES + a); };
   auto tempty_bar = [&](int a) { return bar0 + 8u * (2 * STAGES + 2 + a); };
 
+  constexpr bool teams = EpilogueTeams<KIND, ACC>::value;
+
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(full_bar(s), 1);
@@ -50,7 +52,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(tfull_bar(a), 1);
-      mbar_init(tempty_bar(a), 32 * EPI_WARPS);
+      mbar_init(tempty_bar(a), (teams ? 16 : 32) * EPI_WARPS);
     }
     mbar_init(bar0 + 8u * (2 * STAGES + 4), 1);
     fence_mbar_init();
@@ -169,7 +171,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     }
   } else if (warp < 2 + EPI_WARPS) {
     // ------------------------------------------------------------------ epilogue (128 TMEM lanes; two warps per
-    // lane quadrant, each draining half of the tile's columns)
+    // lane quadrant, each draining half of the tile's columns, or every other tile: EpilogueTeams)
     const int ew = warp & 3;           // TMEM lane quadrant this warp may read
     const int half = (warp - 2) >> 2;  // which half of the columns
     EpiStage es{smem_base + STAGES * STAGE_BYTES + (warp - 2) * (EPI_UNITS * EPI_UNIT_BYTES), 0u};
@@ -199,7 +201,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
       const int acc = tc & 1;
       const uint32_t aph = (tc >> 1) & 1u;
       ++tc;
-      epilogue_prefetch<KIND, ACC>(p, static_cast<int64_t>(tl.row0) + rin, tl.n0, half == 0, tl.e, tl.m0 + rin);
+      if (teams && acc != half) continue;  // the other team's tile
+      epilogue_prefetch<KIND, ACC>(p, static_cast<int64_t>(tl.row0) + rin, tl.n0, teams || half == 0, tl.e, tl.m0 + rin);
       if (clocked()) sum_cycles(p.timers + 6, false);  // waiting for a finished accumulator
       if (!mbar_wait(tfull_bar(acc), aph)) {
         ok = false;
@@ -209,7 +212,10 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
       tc_fence_after();
       const uint32_t taddr = tmem_base + (static_cast<uint32_t>(ew * 32) << 16) + acc * ACC_COLS;
       const int64_t row = static_cast<int64_t>(tl.row0) + rin;
+      int part = teams ? 0 : half;  // which half of the columns
+      const int last = teams ? 1 : half;
       auto release = [&]() {
+        if (part != last) return;
         tc_fence_before();
         mbar_arrive(tempty_bar(acc));
       };
@@ -236,12 +242,14 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
           }
         }
       } else {
-        expert_epilogue<KIND, ACC>(p, tl.e, row, (TR::WGRAD ? tl.m0 : tl.row0) + ew * 32, tl.n0, taddr, true,
-                              TR::WGRAD          ? p.M_total - (tl.m0 + ew * 32)
-                              : KIND == GEMM_DX ? static_cast<int>(p.T - tl.row0 - ew * 32)
-                              : p.clip_rows     ? tl.valid - ew * 32
-                                                : 32,
-                              es, lane, half, release);
+#pragma unroll 1
+        for (; part <= last; ++part)
+          expert_epilogue<KIND, ACC>(p, tl.e, row, (TR::WGRAD ? tl.m0 : tl.row0) + ew * 32, tl.n0, taddr, true,
+                                     TR::WGRAD          ? p.M_total - (tl.m0 + ew * 32)
+                                     : KIND == GEMM_DX ? static_cast<int>(p.T - tl.row0 - ew * 32)
+                                     : p.clip_rows     ? tl.valid - ew * 32
+                                                       : 32,
+                                     es, lane, part, release);
       }
       if (KIND == GEMM_DWR) release();
     }

@@ -116,8 +116,10 @@ __device__ __forceinline__ void issue_loads2(const GemmParams& p, const Tile2& t
   }
 }
 
+// The bound of 512 threads keeps the weight gradients at 128 registers: blocks of the bandwidth-bound kernels on the second
+// stream have to fit beside them.
 template <int KIND>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Traits<KIND>::WGRAD ? 512 : GEMM2_THREADS, 1)
     grouped_gemm_pair_kernel(const __grid_constant__ GemmParams p) {
   using TR = Traits<KIND>;
   extern __shared__ unsigned char gemm2_smem_raw[];
@@ -134,6 +136,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
   auto tfull_bar = [&](int a) { return bar0 + 8u * (2 * STAGES2 + a); };
   auto tempty_bar = [&](int a) { return bar0 + 8u * (2 * STAGES2 + 2 + a); };
 
+  constexpr bool teams = EpilogueTeams<KIND, Accumulate::REDUCE>::value;
+
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES2; ++s) {
       mbar_init(full_bar(s), 1);   // used in the leader only: its producer's arrive + the bytes of both CTAs
@@ -141,7 +145,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(tfull_bar(a), 1);   // one commit from the leader's MMA thread
-      mbar_init(tempty_bar(a), 16);  // used in the leader only: 8 epilogue warps of each CTA
+      mbar_init(tempty_bar(a), teams ? 8 : 16);  // used in the leader only: 8 epilogue warps of each CTA, or 4
     }
     mbar_init(bar0 + 8u * (2 * STAGES2 + 4), 1);
     fence_mbar_init();
@@ -256,7 +260,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
     }
   } else {
     // ------------------------------------------------------------------ epilogue (8 warps per CTA, own 128 rows:
-    // two warps per TMEM lane quadrant, each draining half of the tile's columns)
+    // two warps per TMEM lane quadrant, each draining half of the tile's columns, or every other tile: EpilogueTeams)
     const int ew = warp & 3;
     const int half = (warp - 2) >> 2;
     EpiStage es{smem_base + STAGES2 * STAGE2_BYTES + (warp - 2) * (EPI_UNITS * EPI_UNIT_BYTES), 0u};
@@ -276,6 +280,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
       const int acc = tc & 1;
       const uint32_t aph = (tc >> 1) & 1u;
       ++tc;
+      if (teams && acc != half) continue;  // the other team's tile
       epilogue_prefetch<KIND, Accumulate::REDUCE>(p, static_cast<int64_t>(tl.row0) + rin, tl.n0, tl.write && half == 0);
       if (clocked) sum_cycles(p.timers + 6, false);  // waiting for a finished accumulator
       if (!mbar_wait(tfull_bar(acc), aph)) {
@@ -285,13 +290,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM2_THREADS, 1)
       if (clocked) sum_cycles(p.timers + 6, true);
       tc_fence_after();
       const uint32_t taddr = tmem_base + (static_cast<uint32_t>(ew * 32) << 16) + acc * ACC_COLS;
-      expert_epilogue<KIND, Accumulate::REDUCE>(p, tl.e, static_cast<int64_t>(tl.row0) + rin, (TR::WGRAD ? tl.m0 : tl.row0) + ew * 32, tl.n0, taddr,
-                            tl.write, TR::WGRAD ? p.M_total - (tl.m0 + ew * 32) : p.clip_rows ? tl.valid - ew * 32 : 32, es,
-                            lane, half, [&]() {
-                              tc_fence_before();
-                              __syncwarp();
-                              if (lane == 0) mbar_arrive_cluster(mapa_shared(tempty_bar(acc), 0));
-                            });
+      const int last = teams ? 1 : half;
+#pragma unroll 1
+      for (int part = teams ? 0 : half; part <= last; ++part)
+        expert_epilogue<KIND, Accumulate::REDUCE>(
+            p, tl.e, static_cast<int64_t>(tl.row0) + rin, (TR::WGRAD ? tl.m0 : tl.row0) + ew * 32, tl.n0, taddr, tl.write,
+            TR::WGRAD ? p.M_total - (tl.m0 + ew * 32) : p.clip_rows ? tl.valid - ew * 32 : 32, es, lane, part, [&]() {
+              if (part != last) return;
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive_cluster(mapa_shared(tempty_bar(acc), 0));
+            });
     }
     if (clocked) {
       sum_cycles(p.timers + 5, true);
