@@ -145,7 +145,7 @@ def kernel_launches() -> int:
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()  # an int becomes a pointer in the call, by the argument types of load_library
 
 
 def listwise_loss(scores, teacher=None, s_temp: float = 1.0, t_temp: float = 1.0, want_grad: bool = True):
@@ -204,6 +204,7 @@ class MoELayer:
         self.ws = None
         self.T = None
         self._saved = None
+        self._ws_need = {}  # (T, inference) -> bytes: a function of the shape
 
     def __del__(self):
         try:
@@ -233,14 +234,18 @@ class MoELayer:
 
     def _ensure_ws(self, T: int, inference: bool = False):
         import torch
-        need = self.inference_workspace_bytes(T) if inference else self.workspace_bytes(T)
+        need = self._ws_need.get((T, inference))
+        if need is None:
+            if len(self._ws_need) >= 64:
+                self._ws_need.clear()
+            need = self._ws_need[(T, inference)] = self.inference_workspace_bytes(T) if inference else self.workspace_bytes(T)
         if self.ws is None or self.ws.numel() < need:
             self.ws = torch.empty(max(need, 256), dtype=torch.uint8, device="cuda")
         self.T = T
 
     def _stream(self):
         import torch
-        return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
     # ---- calls
     def forward(self, x, W_r, W_gate, W_up, W_down, b_r=None, logits_in=None, want_logits=False, want_perm=True,
@@ -249,21 +254,22 @@ class MoELayer:
         import torch
         T = x.shape[0]
         d, E, f, k = self.d, self.E, self.f, self.k
-        assert x.dtype == torch.bfloat16 and tuple(x.shape) == (T, d) and x.is_contiguous()
-        wr_dtype = torch.float32 if (self.flags & FLAG_ROUTER_FP32) else torch.bfloat16
-        assert tuple(W_r.shape) == (d, E) and W_r.dtype == wr_dtype and W_r.is_contiguous()
+        bf16, f32, i32, empty = torch.bfloat16, torch.float32, torch.int32, torch.empty
+        assert x.dtype == bf16 and x.shape == (T, d) and x.is_contiguous()
+        wr_dtype = f32 if (self.flags & FLAG_ROUTER_FP32) else bf16
+        assert W_r.shape == (d, E) and W_r.dtype == wr_dtype and W_r.is_contiguous()
         for w, shp in ((W_gate, (E, d, f)), (W_up, (E, d, f)), (W_down, (E, f, d))):
-            assert tuple(w.shape) == shp and w.dtype == torch.bfloat16 and w.is_contiguous()
+            assert w.shape == shp and w.dtype == bf16 and w.is_contiguous()
         self._ensure_ws(T, inference)
         dev = x.device
         out = {
-            "y": torch.empty(T, d, dtype=torch.bfloat16, device=dev),
-            "idx": torch.empty(T, k, dtype=torch.int32, device=dev),
-            "gates": torch.empty(T, k, dtype=torch.float32, device=dev),
-            "counts": torch.empty(E, dtype=torch.int32, device=dev),
-            "perm": torch.empty(T * k, dtype=torch.int32, device=dev) if want_perm else None,
-            "aux": torch.empty(1, dtype=torch.float32, device=dev),
-            "logits": torch.empty(T, E, dtype=torch.float32, device=dev) if want_logits else None,
+            "y": torch.empty_like(x),
+            "idx": empty(T, k, dtype=i32, device=dev),
+            "gates": empty(T, k, dtype=f32, device=dev),
+            "counts": empty(E, dtype=i32, device=dev),
+            "perm": empty(T * k, dtype=i32, device=dev) if want_perm else None,
+            "aux": empty(1, dtype=f32, device=dev),
+            "logits": empty(T, E, dtype=f32, device=dev) if want_logits else None,
         }
         if b_r is not None:
             assert b_r.dtype == torch.float32 and b_r.numel() == E
