@@ -227,7 +227,7 @@ struct LoraArgs {
 };
 // row GEMMs with the tokens as the N operand; lo: with the extra K segment of the adapters (gemm_tokens.cu)
 moe_status launch_token_gemm(moe_ctx_impl* ctx, GemmKind kind, const WsLayout& L, char* ws, const GemmIO& io, const LoraArgs* lo,
-                             cudaStream_t st);
+                             bool small, cudaStream_t st);
 enum LoraOp {
   LORA_U = 0,  // u = s xp A1
   LORA_F3,     // [hg|hu] = xp [Wg|Wu] + u [B1g|B1u], SwiGLU epilogue

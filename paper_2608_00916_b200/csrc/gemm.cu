@@ -531,29 +531,32 @@ static bool row_gemm_on_pairs(const moe_ctx_impl* ctx, GemmKind kind, double row
 
 // Row GEMMs with the tokens as the N operand (gemm_tokens.cu): no padding rows in the MMAs, but longer epilogues (the results
 // have to be transposed), so the K loop must be long, and where an expert's rows fill the other tiles anyway there is nothing
-// to gain.  Pairs or one-CTA tiles, whichever is better -> tokens, us, at d 2048, f 768, 128 experts:
-//   rows        15          62          128         256         512         768         1024        2048          4096
-//   gate/up     164 -> 156  164 -> 159  172 -> 170  209 -> 207  342 -> 339  480 -> 477  632 -> 630  1211 -> 1230  2377 -> 2439
-//   down        81 -> 81    81 -> 83    92 -> 90    119 -> 118  198 -> 198  273 -> 284  360 -> 372  658 -> 695    1225 -> 1359
-//   dgrad-down  109 -> 95   109 -> 102  125 -> 119  165 -> 146  247 -> 229  328 -> 304  419 -> 386  784 -> 756    1559 -> 1531
-//   dgrad-g/u   155 -> 151  154 -> 152  171 -> 161  206 -> 196  350 -> 333  506 -> 490  677 -> 660  1255 -> 1246  2348 -> 2405
+// to gain.  Pairs or one-CTA tiles, whichever the rule above takes -> tokens, us, at d 2048, f 768, 128 experts:
+//   rows        15          62          256         512         768         1024        2048          4096
+//   gate/up     165 -> 154  165 -> 158  221 -> 208  350 -> 319  487 -> 453  629 -> 592  1198 -> 1157  2399 -> 2385
+//   down        80 -> 81    81 -> 84    122 -> 121  198 -> 198  275 -> 282  352 -> 362  647 -> 670    1218 -> 1315
+//   dgrad-down  114 -> 92   113 -> 101  168 -> 146  252 -> 219  337 -> 299  414 -> 371  775 -> 735    1554 -> 1551
+//   dgrad-g/u   156 -> 152  156 -> 154  215 -> 198  360 -> 322  518 -> 474  670 -> 624  1228 -> 1174  2362 -> 2370
 // and at d 4096, f 14336, 8 experts, whose row tiles are walked in groups:
 //   rows        64          128         256         512         768           1024          4096
-//   gate/up     340 -> 345  379 -> 363  500 -> 466  783 -> 755  1122 -> 1102  1418 -> 1392  6186 -> 6354
-//   down        147 -> 158  218 -> 166  271 -> 245  476 -> 458  582 -> 582    755 -> 756    3047 -> 3189
-//   dgrad-down  210 -> 194  226 -> 213  304 -> 279  484 -> 422  635 -> 621    795 -> 789    3167 -> 3538
-//   dgrad-g/u   314 -> 329  449 -> 341  531 -> 492  924 -> 928  1181 -> 1263  1502 -> 1597  6156 -> 6345
-// In forward-only calls, which skip the pad rows, they gain more: scoring 241 tokens 238 -> 232 us, 2048 tokens 335 -> 316.
-// Smaller widths: at d 1024, f 1536, 32 experts dgrad-down 43 -> 31, 45 -> 43, 93 -> 85 at 32, 128 and 512 rows, but gate/up (16 K
-// blocks, three outputs) 52 -> 57, 57 -> 60, 101 -> 105; at d 512 the two forms take the same time.
+//   gate/up     341 -> 331  379 -> 358  508 -> 454  847 -> 756  1172 -> 1098  1501 -> 1401  6189 -> 6391
+//   down        148 -> 154  217 -> 164  279 -> 253  469 -> 440  655 -> 659    754 -> 778    3082 -> 3290
+//   dgrad-down  209 -> 184  226 -> 210  320 -> 281  496 -> 428  639 -> 588    845 -> 780    3218 -> 3420
+//   dgrad-g/u   314 -> 313  449 -> 336  539 -> 496  933 -> 876  1316 -> 1408  1526 -> 1721  6231 -> 6520
+// Smaller widths: at d 1024, f 1536, 32 experts dgrad-down 43 -> 31, 45 -> 43, 93 -> 85, 172 -> 146 at 32, 128, 512, 1024 rows, but
+// gate/up (16 K blocks, three outputs) 53 -> 56, 57 -> 61, 101 -> 107, 166 -> 184.  At d 256 to 768 only dgrad-down gains, whose
+// other form is slow to start, and that only with few rows: d 256, f 512, 8 experts 19 -> 13 at 16 rows, 19 -> 15 at 64, 19 -> 19 at
+// 256; d 512, f 768 21 -> 15 at 64, 21 -> 21 at 256; d 768, f 512, 64 experts 25 -> 21 at 16 rows.
 static bool row_gemm_by_tokens(const moe_ctx_impl* ctx, GemmKind kind, double rows_per_expert) {
   const int d = ctx->s.d, f = ctx->s.f;
-  if (ctx->tile_mode != 0 || d < 1024 || f < 512) return false;
+  if (ctx->tile_mode != 0) return false;
+  if (kind == GEMM_B2 && rows_per_expert < 128.0) return true;
+  if (d < 1024 || f < 512) return false;
   switch (kind) {
-    case GEMM_F3: return d >= 2048 && rows_per_expert < 1100.0;
-    case GEMM_F4: return (d <= 3072 || rows_per_expert >= 96.0) && rows_per_expert < 640.0;
-    case GEMM_B2: return f <= 3072 || rows_per_expert < 1100.0;
-    case GEMM_B4: return d <= 3072 ? rows_per_expert < 3072.0 : rows_per_expert >= 96.0 && rows_per_expert < 512.0;
+    case GEMM_F3: return d >= 2048 && rows_per_expert < (f <= 1536 ? 3072.0 : 1536.0);
+    case GEMM_F4: return rows_per_expert >= 96.0 && rows_per_expert < 640.0;
+    case GEMM_B2: return f <= 3072 || rows_per_expert < 1536.0;
+    case GEMM_B4: return rows_per_expert < (d <= 3072 ? 3072.0 : 640.0);
     default: return false;
   }
 }
@@ -569,7 +572,7 @@ moe_status launch_grouped_gemm(moe_ctx_impl* ctx, GemmKind kind, int64_t T, cons
     return launch_gemm_variant(ctx, kind, T, L, ws, io, st, pair, 0);
   }
   if (!row_kind) return launch_gemm_variant(ctx, kind, T, L, ws, io, st, false, 0);
-  if (row_gemm_by_tokens(ctx, kind, rows_per_expert)) return launch_token_gemm(ctx, kind, L, ws, io, nullptr, st);
+  if (row_gemm_by_tokens(ctx, kind, rows_per_expert)) return launch_token_gemm(ctx, kind, L, ws, io, nullptr, rows_per_expert < 80.0, st);
   const bool pair = row_gemm_on_pairs(ctx, kind, rows_per_expert);
   if (ctx->tile_mode != 3) return launch_gemm_variant(ctx, kind, T, L, ws, io, st, pair, 0);
   const moe_status rc = launch_gemm_variant(ctx, kind, T, L, ws, io, st, true, 1);
@@ -739,9 +742,10 @@ moe_status launch_lora_gemm(moe_ctx_impl* ctx, LoraOp op, int64_t T, const WsLay
   p.row_gate = reinterpret_cast<const float*>(ws + L.row_gate);
   const uint32_t skinny_tx = A_BYTES + CHUNK_BYTES;  // a 128 x 64 A tile and one 64 x 64 B tile
   const int kind = lora_row_gemm(op);
-  if (kind >= 0 && row_gemm_by_tokens(ctx, static_cast<GemmKind>(kind), static_cast<double>(T) * s.k / E))
-    return launch_token_gemm(ctx, static_cast<GemmKind>(kind), L, ws, io, &lo, st);
-  const bool pair = kind >= 0 && row_gemm_on_pairs(ctx, static_cast<GemmKind>(kind), static_cast<double>(T) * s.k / E);
+  const double rows_per_expert = static_cast<double>(T) * s.k / E;
+  if (kind >= 0 && row_gemm_by_tokens(ctx, static_cast<GemmKind>(kind), rows_per_expert))
+    return launch_token_gemm(ctx, static_cast<GemmKind>(kind), L, ws, io, &lo, rows_per_expert < 80.0, st);
+  const bool pair = kind >= 0 && row_gemm_on_pairs(ctx, static_cast<GemmKind>(kind), rows_per_expert);
   if (kind >= 0 && ctx->gemm_timers) p.timers = reinterpret_cast<unsigned long long*>(ws + L.timers) + 8 * kind;
   bool ok = true;
   switch (op) {

@@ -29,25 +29,28 @@
 
 namespace moe {
 
-constexpr int TK_STAGES = 6;
+constexpr int TK_MAX_STAGES = 8;
 // Epilogue groups of four warps, a lane quadrant each.  With two, and the gates of a unit fetched in that unit, dgrad-down was
 // held by its epilogue (3300 cycles a unit): 154 / 249 / 318 / 414 us at 256 / 512 / 768 / 1024 rows per expert against 146 / 229 /
 // 302 / 375.
 constexpr int TK_GROUPS = 3;
 constexpr int TK_THREADS = 64 + 128 * TK_GROUPS;  // warps: 0 TMA producer, 1 MMA issuer, 2.. epilogue
-constexpr int TK_MAX_N = 256;    // tokens of a tile
-constexpr int TK_STAGE_BYTES = A_BYTES + (TK_MAX_N / 2) * BK * 2;  // 16 KB of weights, up to 16 KB of tokens
+// Tiles hold up to 256 tokens, a stage 16 KB of weights and up to 16 KB of tokens, and the ring six of them; with few rows per
+// expert (p.small) up to 128 tokens, so that eight stages fit (and the host has half as many maps to encode, 0.65 us each).
+// Gate/up and dgrad-down, us, six stages -> eight: 154 / 93 -> 153 / 91 at 4 rows per expert, 158 / 101 -> 159 / 101 at 62, 160 / 106 ->
+// 166 / 107 at 94 (a second tile per expert), at d 4096, f 14336 340 / 190 -> 331 / 184 at 64, 357 / 211 -> 368 / 215 at 128: below 80.
+constexpr int TK_RING_BYTES = 6 * 32768;
 // Staging of an epilogue group, 16 tokens: hg, hu and act at 2 KB and 4 KB of values on their way between the gate and the up
 // warps (F3), hg and hu at 4 KB and 256 bytes of dg partials (B2), two buffers of 4 KB (F4, B4).
 constexpr int TK_SWAP = 6144, TK_DG = 8192, TK_EPI_BYTES = 10240;
-constexpr size_t TK_SMEM = static_cast<size_t>(TK_STAGES) * TK_STAGE_BYTES + TK_GROUPS * TK_EPI_BYTES + 1024;
+constexpr size_t TK_SMEM = static_cast<size_t>(TK_RING_BYTES) + TK_GROUPS * TK_EPI_BYTES + 1024;
 
 struct TokenGemmParams {
   CUtensorMap a0, a1;      // weights: F3 gate and up, B4 gate and up (its two K segments), F4 and B2 down
   CUtensorMap ax0, ax1;    // the same for the extra K segment of the low-rank adapters
-  CUtensorMap b[2][8];     // rows of segment 0, of segment 1 (B4); boxes of 16, 32, .. 128 rows
-  CUtensorMap bx;          // rows of the extra segment; 128 rows
-  const int32_t *sched, *pair_tab, *pad_offsets, *counts;
+  CUtensorMap b[2][8];     // rows of segment 0, of segment 1 (B4); boxes of 16, 32, .. 128 rows (small: .. 64)
+  CUtensorMap bx;          // rows of the extra segment; 128 rows (small: 64)
+  const int32_t *sched, *pair_tab, *tile_expert, *pad_offsets, *counts;
   int32_t* status;
   unsigned long long* timers;
   int n_tiles;             // weight tiles
@@ -62,6 +65,7 @@ struct TokenGemmParams {
   int64_t rows_max;
   int save_pre;            // F3: also store hg, hu
   int clip_rows;           // pad rows are not stored
+  int small;               // few rows per expert
 };
 
 template <int KIND>
@@ -78,41 +82,30 @@ struct TokenTile {
   int nt;       // weight tile
 };
 
-// An expert's rows are cut into as many tiles as it has pairs of 128-row blocks, all of one size but for the last.
+__device__ __forceinline__ int token_tiles(const TokenGemmParams& p) { return p.sched[p.small ? 0 : 2] * p.n_tiles; }
+
+// An expert's rows are cut into as many tiles as it has pairs of 128-row blocks (small: blocks), all of one size but for the last.
 __device__ __forceinline__ TokenTile get_token_tile(const TokenGemmParams& p, int t) {
   TokenTile tl;
-  int pr;
-  row_tile_order(t, p.n_tiles, p.row_group, p.sched[2], pr, tl.nt);
-  const int4 info = *reinterpret_cast<const int4*>(p.pair_tab + 4 * pr);  // expert, first row of the pair
-  tl.e = info.x;
-  const int first = p.pad_offsets[tl.e], count = p.counts[tl.e];
-  const int b = (info.y - first) / TK_MAX_N, tiles = (count + TK_MAX_N - 1) / TK_MAX_N;
+  int ri, b, first;
+  row_tile_order(t, p.n_tiles, p.row_group, p.sched[p.small ? 0 : 2], ri, tl.nt);
+  if (p.small) {
+    tl.e = p.tile_expert[ri];
+    first = p.pad_offsets[tl.e];
+    b = ri - first / BM;
+  } else {
+    const int4 info = *reinterpret_cast<const int4*>(p.pair_tab + 4 * ri);  // expert, first row of the pair
+    tl.e = info.x;
+    first = p.pad_offsets[tl.e];
+    b = (info.y - first) / (2 * BM);
+  }
+  const int count = p.counts[tl.e], most = p.small ? BM : 2 * BM, tiles = (count + most - 1) / most;
   const int size = ((count + tiles - 1) / tiles + 15) & ~15, left = count - b * size;
   tl.n = min(size, (left + 15) & ~15);
   tl.row0 = first + b * size;
   tl.stored = p.clip_rows ? min(tl.n, left) : tl.n;
   tl.zeros = !p.clip_rows && b == tiles - 1 ? (count + ROW_PAD - 1) / ROW_PAD * ROW_PAD - (b * size + tl.n) : 0;
   return tl;
-}
-
-template <int KIND>
-__device__ __forceinline__ void issue_token_loads(const TokenGemmParams& p, const TokenTile& tl, int kb, int rank, uint32_t sA,
-                                                  uint32_t sB, uint32_t bar) {
-  const int seg = kb / p.k_blocks;
-  const bool extra = seg >= p.nseg;
-  const int kk = (kb - (extra ? p.nseg : seg) * p.k_blocks) * BK;
-  const CUtensorMap *a0 = extra ? &p.ax0 : &p.a0, *a1 = extra ? &p.ax1 : &p.a1;
-  if (KIND == GEMM_F3) {
-    const int chunk = tl.nt * 2 + rank;
-    tma_load_4d_pair(sA, a0, bar, 0, kk, chunk, tl.e);
-    tma_load_4d_pair(sA + CHUNK_BYTES, a1, bar, 0, kk, chunk, tl.e);
-  } else if (KIND == GEMM_F4) {
-    tma_load_4d_pair(sA, a0, bar, 0, kk, tl.nt * 4 + rank * 2, tl.e);
-  } else {  // B2, B4: K-major weights
-    tma_load_3d_pair(sA, KIND == GEMM_B4 && seg == 1 && !extra ? a1 : a0, bar, kk, tl.nt * 256 + rank * 128, tl.e);
-  }
-  tma_load_2d_pair(sB, extra ? &p.bx : &p.b[KIND == GEMM_B4 ? seg : 0][((tl.n >> 1) + 15) / 16 - 1], bar, kk,
-                   tl.row0 + rank * (tl.n >> 1));
 }
 
 // 16 TMEM lanes x 16 columns: register 4 j + 2 i + b of a thread is lane 8 i + thread / 4, column 8 j + 2 (thread % 4) + b.
@@ -392,7 +385,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TK_THREADS, 1)
     token_gemm_kernel(const __grid_constant__ TokenGemmParams p) {
   constexpr int A_MN = TokenTraits<KIND>::A_MN;
   extern __shared__ unsigned char tk_smem_raw[];
-  __shared__ __align__(8) uint64_t bars[2 * TK_STAGES + 5];  // full, empty, accumulator full / empty, drain (failure path)
+  __shared__ __align__(8) uint64_t bars[2 * TK_MAX_STAGES + 5];  // full, empty, accumulator full / empty, drain (failure path)
   __shared__ uint32_t tmem_base_slot;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -401,12 +394,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TK_THREADS, 1)
   const uint32_t smem_base = (smem_u32(tk_smem_raw) + 1023u) & ~1023u;
   const uint32_t bar0 = smem_u32(bars);
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
-  auto empty_bar = [&](int s) { return bar0 + 8u * (TK_STAGES + s); };
-  auto tfull_bar = [&](int a) { return bar0 + 8u * (2 * TK_STAGES + a); };
-  auto tempty_bar = [&](int a) { return bar0 + 8u * (2 * TK_STAGES + 2 + a); };
+  auto empty_bar = [&](int s) { return bar0 + 8u * (TK_MAX_STAGES + s); };
+  auto tfull_bar = [&](int a) { return bar0 + 8u * (2 * TK_MAX_STAGES + a); };
+  auto tempty_bar = [&](int a) { return bar0 + 8u * (2 * TK_MAX_STAGES + 2 + a); };
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < TK_STAGES; ++s) {
+    for (int s = 0; s < TK_MAX_STAGES; ++s) {
       mbar_init(full_bar(s), 1);   // used in the leader only: its producer's arrive + the bytes of both CTAs
       mbar_init(empty_bar(s), 1);  // one commit from the leader's MMA thread
     }
@@ -414,7 +407,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TK_THREADS, 1)
       mbar_init(tfull_bar(a), 1);    // one commit from the leader's MMA thread
       mbar_init(tempty_bar(a), 8 * TK_GROUPS);  // used in the leader only: the epilogue warps of both CTAs
     }
-    mbar_init(bar0 + 8u * (2 * TK_STAGES + 4), 1);
+    mbar_init(bar0 + 8u * (2 * TK_MAX_STAGES + 4), 1);
     fence_mbar_init();
     tma_prefetch_desc(&p.a0);
     tma_prefetch_desc(&p.a1);
@@ -428,8 +421,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TK_THREADS, 1)
   cluster_sync_all();  // barriers of both CTAs are initialised before anyone signals across the pair
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_slot;
-  const int ntiles = p.sched[2] * p.n_tiles;
+  const int ntiles = token_tiles(p);
   const int cid = blockIdx.x >> 1, nclusters = gridDim.x >> 1;
+  const uint32_t stages = p.small ? 8 : 6, stage_bytes = TK_RING_BYTES / stages;
   const int nkb = p.k_blocks * p.nseg + p.k_blocks1;
 
   if (warp == 0) {
@@ -439,21 +433,46 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TK_THREADS, 1)
       uint32_t it = 0;
       bool ok = true;
       RoleClock clk(leader ? p.timers : nullptr);
+      // The loop over the K blocks is kept short: what this thread takes to issue the copies of a stage that has become free
+      // counts like latency.  With a division for the segment, the choice of the maps and the address of the barrier in it gate/up
+      // took 343 us at 512 rows per expert (326 now) and 632 at 1024 (600), dgrad gate/up 664 at 1024 (638), scoring 241 tokens 230
+      // (225).
+      const uint32_t full0 = mapa_shared(full_bar(0), 0);
       for (int t = cid; t < ntiles && ok; t += nclusters) {
         const TokenTile tl = get_token_tile(p, t);
-        // bytes of a K block of both CTAs: the copy of a CTA's tokens is rounded up to 16 rows (extra segment: 128)
-        const uint32_t tx = 2 * (A_BYTES + ((tl.n >> 1) + 15) / 16 * 16 * BK * 2);
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
-          clk.start();
-          if (!mbar_wait(empty_bar(pos.s), pos.phase ^ 1u)) {
-            ok = false;
-            break;
+        const int box = ((tl.n >> 1) + 15) / 16 - 1;  // the copy of this CTA's tokens: 16 (box + 1) rows, of the extra segment all
+        const int y = tl.row0 + rank * (tl.n >> 1);
+        const int wx = KIND == GEMM_F3 ? tl.nt * 2 + rank : KIND == GEMM_F4 ? tl.nt * 4 + rank * 2 : tl.nt * 256 + rank * 128;
+        const int segs = p.nseg + (p.k_blocks1 ? 1 : 0);
+#pragma unroll 1
+        for (int seg = 0; seg < segs && ok; ++seg) {
+          const bool extra = seg == p.nseg;
+          const CUtensorMap* const a0 = extra ? &p.ax0 : KIND == GEMM_B4 && seg == 1 ? &p.a1 : &p.a0;
+          const CUtensorMap* const a1 = extra ? &p.ax1 : &p.a1;  // F3: the up columns
+          const CUtensorMap* const b = extra ? &p.bx : &p.b[KIND == GEMM_B4 ? seg : 0][box];
+          const uint32_t tx = 2 * (extra ? stage_bytes : A_BYTES + (box + 1) * 16 * BK * 2);  // of both CTAs
+          const int k_end = (extra ? p.k_blocks1 : p.k_blocks) * BK;
+#pragma unroll 1
+          for (int kk = 0; kk < k_end; kk += BK, ++it) {
+            clk.start();
+            if (!mbar_wait(empty_bar(pos.s), pos.phase ^ 1u)) {
+              ok = false;
+              break;
+            }
+            clk.add(0);
+            if (leader) mbar_expect_tx(full_bar(pos.s), tx);
+            const uint32_t sA = smem_base + pos.s * stage_bytes, bar = full0 + 8u * pos.s;
+            if (KIND == GEMM_F3) {
+              tma_load_4d_pair(sA, a0, bar, 0, kk, wx, tl.e);
+              tma_load_4d_pair(sA + CHUNK_BYTES, a1, bar, 0, kk, wx, tl.e);
+            } else if (KIND == GEMM_F4) {
+              tma_load_4d_pair(sA, a0, bar, 0, kk, wx, tl.e);
+            } else {  // B2, B4: K-major weights
+              tma_load_3d_pair(sA, a0, bar, kk, wx, tl.e);
+            }
+            tma_load_2d_pair(sA + A_BYTES, b, bar, kk, y);
+            pos.next(stages);
           }
-          clk.add(0);
-          if (leader) mbar_expect_tx(full_bar(pos.s), kb < p.k_blocks * p.nseg ? tx : 2 * TK_STAGE_BYTES);
-          const uint32_t sA = smem_base + pos.s * TK_STAGE_BYTES;
-          issue_token_loads<KIND>(p, tl, kb, rank, sA, sA + A_BYTES, mapa_shared(full_bar(pos.s), 0));
-          pos.next(TK_STAGES);
         }
       }
       chain_next();
@@ -463,8 +482,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TK_THREADS, 1)
         // barriers, so that neither CTA exits with copies in flight (the cluster barrier below holds the partner until then)
         record_status(p.status, DEV_TIMEOUT, 2100 + KIND);
         if (leader)
-          for (uint32_t i = it > static_cast<uint32_t>(TK_STAGES) ? it - TK_STAGES : 0; i < it; ++i)
-            mbar_wait(full_bar(i % TK_STAGES), (i / TK_STAGES) & 1u);
+          for (uint32_t i = it > stages ? it - stages : 0; i < it; ++i) mbar_wait(full_bar(i % stages), (i / stages) & 1u);
       }
     }
   } else if (warp == 1) {
@@ -499,9 +517,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TK_THREADS, 1)
           }
           clk.add(1);
           tc_fence_after();
-          const uint64_t off = (pos.s * TK_STAGE_BYTES) >> 4;
+          const uint64_t off = (pos.s * stage_bytes) >> 4;
           const uint32_t done = empty_bar(pos.s);
-          pos.next(TK_STAGES);
+          pos.next(stages);
           ready = kb + 1 < nkb && mbar_try_wait(full_bar(pos.s), pos.phase);
 #pragma unroll
           for (int ks = 0; ks < BK / 16; ++ks)
@@ -514,15 +532,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TK_THREADS, 1)
       if (!ok) {
         // gave up: let every MMA issued so far finish (bounded) before the pair's tensor memory is freed
         record_status(p.status, DEV_TIMEOUT, 2200 + KIND);
-        umma_commit_pair_both(bar0 + 8u * (2 * TK_STAGES + 4));
-        mbar_wait(bar0 + 8u * (2 * TK_STAGES + 4), 0u);
+        umma_commit_pair_both(bar0 + 8u * (2 * TK_MAX_STAGES + 4));
+        mbar_wait(bar0 + 8u * (2 * TK_MAX_STAGES + 4), 0u);
       }
     }
   } else {
     // ------------------------------------------------------------------ epilogue
     const int q = warp & 3;
     const int group = (warp - 2) >> 2;
-    const uint32_t staging = smem_base + TK_STAGES * TK_STAGE_BYTES + group * TK_EPI_BYTES;
+    const uint32_t staging = smem_base + TK_RING_BYTES + group * TK_EPI_BYTES;
     uint32_t tc = 0;
     bool ok = true;
     const bool clocked = p.timers && leader && threadIdx.x == 64;
@@ -589,14 +607,14 @@ static moe_status launch_token_kind(moe_ctx_impl* ctx, const TokenGemmParams& p,
 }
 
 moe_status launch_token_gemm(moe_ctx_impl* ctx, GemmKind kind, const WsLayout& L, char* ws, const GemmIO& io, const LoraArgs* lo,
-                             cudaStream_t st) {
+                             bool small, cudaStream_t st) {
   const Shape& s = ctx->s;
   const int d = s.d, f = s.f, E = s.E, r = lo ? lo->rank : 0;
   const int64_t R = L.rows_max;
   void* fn = ctx->encode_fn;
   auto B16 = [&](size_t off) { return reinterpret_cast<uint16_t*>(ws + off); };
   auto rows = [&](CUtensorMap (&m)[8], const uint16_t* base, int64_t width) {
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < (small ? 4 : 8); ++i)
       if (!map_2d(fn, &m[i], base, R, width, 16 * (i + 1))) return false;
     return true;
   };
@@ -604,6 +622,8 @@ moe_status launch_token_gemm(moe_ctx_impl* ctx, GemmKind kind, const WsLayout& L
   memset(&p, 0, sizeof(p));
   p.sched = reinterpret_cast<const int32_t*>(ws + L.sched);
   p.pair_tab = reinterpret_cast<const int32_t*>(ws + L.pair_tab);
+  p.tile_expert = reinterpret_cast<const int32_t*>(ws + L.tile_expert);
+  p.small = small ? 1 : 0;
   p.pad_offsets = reinterpret_cast<const int32_t*>(ws + L.pad_offsets);
   p.counts = reinterpret_cast<const int32_t*>(ws + L.counts);
   p.status = reinterpret_cast<int32_t*>(ws + L.status);
@@ -615,7 +635,7 @@ moe_status launch_token_gemm(moe_ctx_impl* ctx, GemmKind kind, const WsLayout& L
     case GEMM_F3:
       ok = map_mn(fn, &p.a0, io.W_gate, E, d, f, 1) && map_mn(fn, &p.a1, io.W_up, E, d, f, 1) && rows(p.b[0], B16(L.xp), d) &&
            (!lo || (map_mn(fn, &p.ax0, lo->B1g, E, r, f, 1) && map_mn(fn, &p.ax1, lo->B1u, E, r, f, 1) &&
-                    map_2d(fn, &p.bx, B16(L.lora_u), R, 64, 128)));
+                    map_2d(fn, &p.bx, B16(L.lora_u), R, 64, small ? 64 : 128)));
       p.n_tiles = (f + 127) / 128;
       p.k_blocks = d / BK;
       p.N_total = f;
@@ -626,7 +646,7 @@ moe_status launch_token_gemm(moe_ctx_impl* ctx, GemmKind kind, const WsLayout& L
       break;
     case GEMM_F4:
       ok = map_mn(fn, &p.a0, io.W_down, E, f, d, 2) && rows(p.b[0], B16(L.act), f) &&
-           (!lo || (map_mn(fn, &p.ax0, lo->B2, E, r, d, 2) && map_2d(fn, &p.bx, B16(L.lora_v), R, 64, 128)));
+           (!lo || (map_mn(fn, &p.ax0, lo->B2, E, r, d, 2) && map_2d(fn, &p.bx, B16(L.lora_v), R, 64, small ? 64 : 128)));
       p.n_tiles = (d + 255) / 256;
       p.k_blocks = f / BK;
       p.N_total = d;
@@ -635,7 +655,7 @@ moe_status launch_token_gemm(moe_ctx_impl* ctx, GemmKind kind, const WsLayout& L
       break;
     case GEMM_B2:
       ok = map_3d(fn, &p.a0, io.W_down, E, f, d, 128) && rows(p.b[0], B16(L.o), d) &&
-           (!lo || (map_3d(fn, &p.ax0, lo->A2, E, f, r, 128) && map_2d(fn, &p.bx, B16(L.lora_w), R, 64, 128)));
+           (!lo || (map_3d(fn, &p.ax0, lo->A2, E, f, r, 128) && map_2d(fn, &p.bx, B16(L.lora_w), R, 64, small ? 64 : 128)));
       p.n_tiles = (f + 255) / 256;
       p.k_blocks = d / BK;
       p.N_total = f;
@@ -648,7 +668,7 @@ moe_status launch_token_gemm(moe_ctx_impl* ctx, GemmKind kind, const WsLayout& L
     case GEMM_B4:
       ok = map_3d(fn, &p.a0, io.W_gate, E, d, f, 128) && map_3d(fn, &p.a1, io.W_up, E, d, f, 128) && rows(p.b[0], B16(L.dhg), f) &&
            rows(p.b[1], B16(L.dhu), f) &&
-           (!lo || (map_3d(fn, &p.ax0, lo->A1, E, d, r, 128) && map_2d(fn, &p.bx, B16(L.lora_z), R, 64, 128)));
+           (!lo || (map_3d(fn, &p.ax0, lo->A1, E, d, r, 128) && map_2d(fn, &p.bx, B16(L.lora_z), R, 64, small ? 64 : 128)));
       p.n_tiles = (d + 255) / 256;
       p.nseg = 2;
       p.k_blocks = f / BK;
