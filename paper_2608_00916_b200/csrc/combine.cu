@@ -264,14 +264,15 @@ __global__ void __launch_bounds__(256) dbr_kernel(int64_t T, int E, const float*
 }
 
 void launch_dwr(const Shape& s, int64_t T, const uint16_t* x, const float* dl, float* part, float* dW_r,
-                float* db_r, bool partials_ready, cudaStream_t st, bool accumulate) {
+                float* db_r, bool partials_ready, cudaStream_t st, bool accumulate, bool complete) {
   const int64_t n = static_cast<int64_t>(s.d) * s.E;
-  if (!partials_ready) {
+  if (!partials_ready && !complete) {
     dim3 grid(s.d / DW_BM, DWR_SPLIT);
     launch_kernel(dwr_partial_kernel, grid, 256, sizeof(float) * DW_BK * s.E, st, T, s.d, s.E, x, dl, part);
   }
-  launch_kernel(dwr_reduce_kernel, static_cast<unsigned>((n + 255) / 256), 256, 0, st, n, part, dW_r,
-                accumulate ? 1 : 0);
+  if (!complete)
+    launch_kernel(dwr_reduce_kernel, static_cast<unsigned>((n + 255) / 256), 256, 0, st, n, part, dW_r,
+                  accumulate ? 1 : 0);
   if (db_r) {
     launch_kernel(dbr_kernel, (s.E + 31) / 32, 256, 0, st, T, s.E, dl, db_r, accumulate ? 1 : 0);
   }

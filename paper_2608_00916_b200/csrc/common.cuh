@@ -180,9 +180,9 @@ void launch_router_bwd(const Shape& s, int64_t T, const float* logits, const int
                        const int32_t* counts, float d_aux, float* dl, uint16_t* dl_hi, uint16_t* dl_lo,
                        cudaStream_t st, int32_t* dbg_status = nullptr);
 // dg_tiles == 0: dg[t,j] has been filled by the caller (expert-parallel path) and is read instead of the partials
-// SIMT dW_r (any E) and the shared partial reduction / db_r
+// SIMT dW_r (any E) and the shared partial reduction / db_r; complete: dW_r needs neither
 void launch_dwr(const Shape& s, int64_t T, const uint16_t* x, const float* dl, float* part, float* dW_r,
-                float* db_r, bool partials_ready, cudaStream_t st, bool accumulate = false);
+                float* db_r, bool partials_ready, cudaStream_t st, bool accumulate = false, bool complete = false);
 void launch_unpermute_bwd(const Shape& s, int64_t T, const uint16_t* dxp, const int32_t* inv, const float* dl,
                           const uint16_t* W_r, uint16_t* dx, cudaStream_t st);
 // dx[t,:] = dxr[t,:] + sum_j dxp[inv[t,j],:]  (router term already contracted on the tensor cores)
@@ -206,6 +206,8 @@ struct GemmIO {
   uint16_t* dW_down = nullptr;
   uint16_t* dx = nullptr;
   int e_first = 0, e_count = 0;  // weight gradients: e_count > 0 restricts the launch to experts [e_first, e_first + e_count)
+  float* dW_r = nullptr;         // not null: the router weight gradient is written, or added, here and not as partials
+  bool dW_r_accumulate = false;
   float* dW_gate_acc = nullptr;  // accumulate mode: fp32 buffers the weight gradients are added to
   float* dW_up_acc = nullptr;
   float* dW_down_acc = nullptr;

@@ -233,11 +233,15 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
             float* dst = p.outf + (static_cast<int64_t>(tl.e) * p.M_total + m) * p.N_total + col;
 #pragma unroll
             for (int i = 0; i < 32; i += 4) {
-              if (col + i < p.N_total)
-                *reinterpret_cast<float4*>(dst + i) = make_float4(
-                    __uint_as_float(rh[i]) + __uint_as_float(rl[i]), __uint_as_float(rh[i + 1]) + __uint_as_float(rl[i + 1]),
-                    __uint_as_float(rh[i + 2]) + __uint_as_float(rl[i + 2]),
-                    __uint_as_float(rh[i + 3]) + __uint_as_float(rl[i + 3]));
+              if (col + i >= p.N_total) continue;
+              float4 v = make_float4(
+                  __uint_as_float(rh[i]) + __uint_as_float(rl[i]), __uint_as_float(rh[i + 1]) + __uint_as_float(rl[i + 1]),
+                  __uint_as_float(rh[i + 2]) + __uint_as_float(rl[i + 2]), __uint_as_float(rh[i + 3]) + __uint_as_float(rl[i + 3]));
+              if (p.acc_fp32) {
+                const float4 old = *reinterpret_cast<const float4*>(dst + i);
+                v = make_float4(old.x + v.x, old.y + v.y, old.z + v.z, old.w + v.w);
+              }
+              *reinterpret_cast<float4*>(dst + i) = v;
             }
           }
         }
@@ -469,15 +473,18 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
            (p.whole_chunks ? map_mn_rows(fn, &p.mapB0, ws + L.dl_hi, T, E, 2) && map_mn_rows(fn, &p.mapB1, ws + L.dl_lo, T, E, 2)
                            : map_2d(fn, &p.mapB0, ws + L.dl_hi, T, E, 64) && map_2d(fn, &p.mapB1, ws + L.dl_lo, T, E, 64));
       p.mapA1 = p.mapA0;
-      const int64_t per = ((T + DWR_SPLIT - 1) / DWR_SPLIT + BK - 1) / BK * BK;
+      // (few tokens, io.dW_r: one slice, straight into dW_r)
+      const int slices = io.dW_r ? 1 : DWR_SPLIT;
+      const int64_t per = ((T + slices - 1) / slices + BK - 1) / BK * BK;
       p.split_rows = static_cast<int>(per);
       p.rows_total = static_cast<int>((T + BK - 1) / BK * BK);
-      p.E = DWR_SPLIT;  // slices play the role of experts in the tile list
+      p.E = slices;  // slices play the role of experts in the tile list
       p.m_tiles = (d + 127) / 128;
       p.n_tiles = (E + 127) / 128;
       p.M_total = d;
       p.N_total = E;
-      p.outf = reinterpret_cast<float*>(ws + L.dwr_part);
+      p.outf = io.dW_r ? io.dW_r : reinterpret_cast<float*>(ws + L.dwr_part);
+      p.acc_fp32 = io.dW_r && io.dW_r_accumulate;
       if (!ok) return MOE_ERR_CUDA;
       return launch_kind<GEMM_DWR>(ctx, p, st);
     }
