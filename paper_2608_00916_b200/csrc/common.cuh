@@ -12,7 +12,7 @@ namespace moe {
 
 constexpr int ROW_PAD = 128;     // every expert's row segment starts and ends on a multiple of this
 constexpr int TOK_TILE = 128;    // tokens per tile of the permutation (histogram / scatter blocks: 4 warps x 32); equal to
-                                 // the token tile of the tensor-core router, whose epilogue writes the tile histograms
+                                 // the token tile of the tensor-core router, which writes the tile histograms
 constexpr int TOK_WARPS = TOK_TILE / 32;
 constexpr int ROUTER_TOK = 16;   // tokens per block in the router kernel
 constexpr int MAX_E = 256;
