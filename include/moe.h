@@ -58,7 +58,8 @@ typedef struct {
  * tcgen05 cta_group::2, each CTA staging half of B) and one-CTA 128 x 256 tiles: weight gradients run on pairs when
  * the experts average at least 384 rows (704 when they accumulate into fp32 buffers), dgrad-down from 768, the other row
  * GEMMs where the expected number of pairs (an expert with an odd number of 128-row blocks gets a last pair whose second half
- * is empty) costs less than the expected number of one-CTA tiles.  The flags force one shape everywhere (same results; for
+ * is empty) costs less than the expected number of one-CTA tiles; for the widths and rows per expert where that is faster the
+ * row GEMMs take the tokens as the N operand instead.  The flags force one row-tile shape everywhere (same results; for
  * comparison measurements). */
 #define MOE_FLAG_CTA_PAIR_TILES 1
 #define MOE_FLAG_SINGLE_CTA_TILES 2
