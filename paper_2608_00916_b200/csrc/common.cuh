@@ -254,11 +254,11 @@ inline bool router_on_tensor_cores(const Shape& s) { return s.E % 8 == 0; }
 // kernel of a forward call does (launch_prepare): zero row gates, an initialised status block.
 moe_status launch_router_tc(moe_ctx_impl* ctx, int64_t T, const WsLayout& L, char* ws, const GemmIO& io, cudaStream_t st);
 // CTAs that share a 128-token tile in it
-int router_cluster(const Shape& s, int sm_count, int64_t T, bool fp32_weight);
+int router_cluster(const Shape& s, int sm_count, int64_t T);
 // psum_part rows written by the router: one per CTA with tokens (tensor cores) or per ROUTER_TOK tokens (SIMT)
 inline int64_t router_psum_rows(const moe_ctx_impl* c, int64_t T, bool logits_given) {
   const int64_t tok = router_on_tensor_cores(c->s) && !logits_given
-                          ? TOK_TILE / router_cluster(c->s, c->sm_count, T, c->router_fp32 != 0) : ROUTER_TOK;
+                          ? TOK_TILE / router_cluster(c->s, c->sm_count, T) : ROUTER_TOK;
   return (T + tok - 1) / tok;
 }
 

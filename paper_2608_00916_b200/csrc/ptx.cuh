@@ -185,9 +185,11 @@ __device__ __forceinline__ void cluster_sync_all() {
 }
 // The barriers of a block and of a cluster for warps whose lanes may not be together (after a one-thread role).
 __device__ __forceinline__ void block_sync_diverged() { asm volatile("barrier.sync 0;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_diverged() {
-  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  cluster_arrive();
+  cluster_wait();
 }
 // arrive on an mbarrier that may live in the peer CTA (shared::cluster address)
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {

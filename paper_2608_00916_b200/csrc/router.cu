@@ -2,23 +2,26 @@
 // histogram, in one kernel.  x and W_r are bf16 (an fp32 W_r comes as three exact bf16 terms), so that a bf16 MMA with fp32
 // accumulation is an fp32 contraction up to summation order.
 //
-// A cluster of CL CTAs takes one tile of 128 tokens and splits the K blocks; every CTA contracts its share into tensor
-// memory (128 tokens x E), copies it to shared memory, and then routes 128 / CL of the tokens, adding up the CL partial
-// sums of their logits through distributed shared memory in rank order.  What bounds it: up to a few thousand tokens the
-// latency of fetching x and W_r through few SMs (one CTA per tile fetches d * (256 + 2 E) bytes: 1 MB at d 2048, E 128) and of
-// routing the tokens, hence the split; from there on the stream of x from HBM, two CTAs to an SM.
+// CL CTAs share the 128 tokens of a tile, each contracts and routes 128 / CL of them: W_r^T is the M operand (128 experts, twice
+// above 128 of them), the CTA's tokens are N.  Every logit is one sum over all K blocks in their order, so that a token's logits,
+// and with them its experts, are the same bits whatever the number of tokens of the call selects.  (Splitting the K blocks over
+// the CTAs instead fetches a part of W_r per CTA, not all of it, and took 17 us where this takes 19 up to 1000 tokens; but its sums
+// change with the split, and a token near a tie got other experts in another batch.)  The CTAs of a tile are a cluster only
+// to add up the tile's histogram.  What bounds it: up to some ten thousand tokens the latency of fetching W_r and the tokens
+// through one SM each and of routing, hence the split; from there on the stream of x from HBM, two CTAs to an SM.
 //
-// Three steps between barriers.  (1) A warp per token: the sum of the partial logits, which replaces the row in this CTA's
-// shared memory, the softmax and its column sums; a lane holds NV / 4 groups of four columns.  (2) A thread per token: top-k
-// as a three-level tournament, groups of four columns, supers of four groups, the maxima of the supers in registers; a round
-// takes the largest super (lowest among equals), the group and the column in it, removes the column and repairs the maxima
-// above it, which is the rule "largest, lowest index among equals" because the levels partition the columns in order.
-// (3) The picks and gates leave as whole lines.
+// Three steps between barriers.  (1) A warp per token: bias, softmax and its column sums; a lane holds NV / 4 groups of four
+// columns.  (2) A thread per token: top-k as a three-level tournament, groups of four columns, supers of four groups, the maxima
+// of the supers in registers; a round takes the largest super (lowest among equals), the group and the column in it, removes the
+// column and repairs the maxima above it, which is the rule "largest, lowest index among equals" because the levels partition the
+// columns in order.  (3) The picks and gates leave as whole lines.
 //
 // A CTA routes a handful of tokens and every instruction of that arrives cold, about 450 cycles for each eight of them.  So
 // while the operands are on their way the waiting warps run the steps once on whatever shared memory holds, each warp one
 // step, so that the code is fetched side by side; what this first pass stores is overwritten by the same threads.
 #include <string.h>
+
+#include <algorithm>
 
 #include "common.cuh"
 #include "ptx.cuh"
@@ -30,9 +33,13 @@ constexpr int RO_TOK = 128;                    // tokens of a tile (the permutat
 constexpr int RO_WARPS = 12;                   // routing warps
 constexpr int RO_THREADS = 64 + 32 * RO_WARPS;  // warps: 0 TMA producer, 1 MMA issuer, 2.. routing
 constexpr int RO_BK = 64;
-constexpr int RO_A_BYTES = RO_TOK * RO_BK * 2;   // 16 KB of x per K block
-constexpr int RO_CHUNK_BYTES = 64 * RO_BK * 2;   // 8 KB per 64 columns of W_r
-constexpr int RO_MAX_STAGES = 4;
+constexpr int RO_CHUNK_BYTES = 64 * RO_BK * 2;   // 8 KB per 64 columns of W_r and K block
+constexpr int RO_MAX_STAGES = 16;
+// Bytes of the operand stages.  Every CTA fetches all of W_r, and waits for latency more than for bandwidth, so the copies in
+// flight count: 100 -> 200 KB at d 2048 and 128 experts 20 -> 19 us at 128 tokens, 26 -> 23 at 8192, 35 -> 31 at 16384.  But 200 KB
+// take an SM, so they are for launches whose CTAs have one each; more of them share one (49 us at 20000 tokens with 200 KB, 41 at
+// 24576 with 100).  Above 128 experts an SM holds one CTA anyway.
+constexpr int RO_RING = 100 * 1024, RO_DEEP_RING = 200 * 1024;
 static_assert(RO_TOK == TOK_TILE, "the histogram written here is the permutation's");
 
 struct RouterParams {
@@ -50,16 +57,11 @@ struct RouterParams {
   int64_t T;
   int E, k;
   int k_blocks, k_total;  // K blocks of one bf16 term of W_r, and of all terms
-  int b_chunks, whole_chunks;
-  int mma_n, stages;
-  uint32_t stage_bytes, tmem_cols;
+  int w_chunks, whole_chunks;  // 64-column chunks of W_r; E is a multiple of 64, so they are one copy
+  int stages;
+  uint32_t w_bytes, stage_bytes;  // of a stage: W_r, and with the tokens
 };
 
-__device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
-  float4 v;
-  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
-  return v;
-}
 __device__ __forceinline__ void red_cluster_add(uint32_t addr, int v) {
   asm volatile("red.relaxed.cluster.shared::cluster.add.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
@@ -152,17 +154,11 @@ __device__ __forceinline__ float select_topk(int k, uint32_t row, uint32_t maxim
 
 __device__ __forceinline__ void routing_sync() { asm volatile("bar.sync 1, %0;" ::"n"(32 * RO_WARPS) : "memory"); }
 
-template <int CL>
-__device__ __forceinline__ void cluster_or_block_sync() {
-  if (CL > 1)
-    cluster_sync_diverged();
-  else
-    block_sync_diverged();
-}
-
 template <int CL, int NV>
 __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, NV == 4 ? 2 : 1)
     router_cluster_kernel(const __grid_constant__ RouterParams p) {
+  constexpr int MINE = RO_TOK / CL;             // this CTA's tokens of the tile
+  constexpr uint32_t ACCS = NV / 4, TMEM_COLS = ACCS * MINE;  // an accumulator for each 128 experts, a column per token
   extern __shared__ unsigned char ro_smem_raw[];
   __shared__ __align__(8) uint64_t bars[2 * RO_MAX_STAGES + 1];  // full, empty, accumulator complete
   __shared__ uint32_t tmem_base_slot;
@@ -172,13 +168,14 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, NV == 4
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int rank = CL > 1 ? static_cast<int>(cluster_ctarank()) : 0;
   const int tile = blockIdx.x / CL;
-  const int64_t t0 = static_cast<int64_t>(tile) * RO_TOK;
+  const int64_t first = static_cast<int64_t>(tile) * RO_TOK + rank * MINE, left = p.T - first;
+  const int tokens = left < MINE ? static_cast<int>(left) : MINE;  // of which are there (may be negative)
+  const int k_blocks = tokens > 0 ? p.k_total : 0;
   const uint32_t smem_base = (smem_u32(ro_smem_raw) + 1023u) & ~1023u;
   const uint32_t bar0 = smem_u32(bars);
   const uint32_t acc_bar = bar0 + 8u * (2 * RO_MAX_STAGES);
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
   auto empty_bar = [&](int s) { return bar0 + 8u * (RO_MAX_STAGES + s); };
-  const int kb0 = p.k_total * rank / CL, kb1 = p.k_total * (rank + 1) / CL;  // this CTA's K blocks
 
   if (tid == 0) {
     for (int s = 0; s < p.stages; ++s) {
@@ -191,7 +188,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, NV == 4
     tma_prefetch_desc(&p.map_w0);
   }
   if (warp == 1) {
-    tmem_alloc(smem_u32(&tmem_base_slot), p.tmem_cols);
+    tmem_alloc(smem_u32(&tmem_base_slot), TMEM_COLS);
     tmem_relinquish();
   }
   for (int i = tid; i < 32 * NV; i += RO_THREADS) s_hist[i] = 0;
@@ -200,6 +197,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, NV == 4
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (CL > 1) cluster_arrive();  // the counts are cleared: waited for where they are added to
   const uint32_t tmem_base = tmem_base_slot;
 
   if (warp == 0) {
@@ -207,24 +205,29 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, NV == 4
       int s = 0;
       uint32_t phase = 0, it = 0;
       bool ok = true;
-      for (int kb = kb0; kb < kb1; ++kb, ++it) {
-        if (!mbar_wait(empty_bar(s), phase ^ 1u)) {
-          ok = false;
-          break;
-        }
-        const uint32_t sA = smem_base + s * p.stage_bytes, sB = sA + RO_A_BYTES, bar = full_bar(s);
-        const int seg = kb / p.k_blocks, kk = (kb - seg * p.k_blocks) * RO_BK;
-        const CUtensorMap* mw = seg == 0 ? &p.map_w0 : (seg == 1 ? &p.map_w1 : &p.map_w2);
-        mbar_expect_tx(bar, p.stage_bytes);
-        tma_load_2d(sA, &p.map_x, bar, kk, static_cast<int>(t0));
-        if (p.whole_chunks) {
-          tma_load_4d(sB, mw, bar, 0, kk, 0, 0);
-        } else {  // E is not a multiple of 64: a box per chunk, the last one clipped
-          for (int c = 0; c < p.b_chunks; ++c) tma_load_3d(sB + c * RO_CHUNK_BYTES, mw, bar, c * 64, kk, 0);
-        }
-        if (++s == p.stages) {
-          s = 0;
-          phase ^= 1u;
+      // (what this thread takes to refill a stage counts like latency: no divisions and no choice of maps in the loop)
+      const int k_end = tokens > 0 ? p.k_blocks * RO_BK : 0, segs = p.k_total / p.k_blocks;
+      for (int seg = 0; seg < segs && ok; ++seg) {
+        const CUtensorMap* const mw = seg == 0 ? &p.map_w0 : (seg == 1 ? &p.map_w1 : &p.map_w2);
+#pragma unroll 1
+        for (int kk = 0; kk < k_end; kk += RO_BK, ++it) {
+          const uint32_t sW = smem_base + s * p.stage_bytes, bar = full_bar(s);
+          if (!mbar_wait(empty_bar(s), phase ^ 1u)) {
+            ok = false;
+            break;
+          }
+          mbar_expect_tx(bar, p.stage_bytes);
+          if (p.whole_chunks) {
+            tma_load_4d(sW, mw, bar, 0, kk, 0, 0);
+          } else {  // E is not a multiple of 64: a box per chunk, the last one clipped
+#pragma unroll 1
+            for (int c = 0; c < p.w_chunks; ++c) tma_load_3d(sW + c * RO_CHUNK_BYTES, mw, bar, c * 64, kk, 0);
+          }
+          tma_load_2d(sW + p.w_bytes, &p.map_x, bar, kk, static_cast<int>(first));
+          if (++s == p.stages) {
+            s = 0;
+            phase ^= 1u;
+          }
         }
       }
       chain_next();
@@ -236,13 +239,14 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, NV == 4
     }
   } else if (warp == 1) {
     if (elect_one()) {  // MMA issuer
-      const uint32_t idesc = umma_idesc(RO_TOK, p.mma_n, 0, 1);
-      const uint64_t descA = smem_desc(smem_base, 0, 1024);
-      const uint64_t descB = smem_desc(smem_base + RO_A_BYTES, RO_CHUNK_BYTES, 1024);
+      // (experts beyond the chunks of W_r are whatever lies behind them; their accumulator lanes are not read)
+      constexpr uint32_t idesc = umma_idesc(128, MINE, 1, 0);
+      const uint64_t descW = smem_desc(smem_base, RO_CHUNK_BYTES, 1024);
+      const uint64_t descX = smem_desc(smem_base + p.w_bytes, 0, 1024);
       int s = 0;
       uint32_t phase = 0;
       bool ok = true;
-      for (int kb = kb0; kb < kb1; ++kb) {
+      for (int kb = 0; kb < k_blocks; ++kb) {
         if (!mbar_wait(full_bar(s), phase)) {
           ok = false;
           break;
@@ -251,7 +255,10 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, NV == 4
         const uint64_t off = (static_cast<uint64_t>(s) * p.stage_bytes) >> 4;
 #pragma unroll
         for (int ks = 0; ks < RO_BK / 16; ++ks)
-          umma_bf16(tmem_base, descA + off + (ks * 32 >> 4), descB + off + (ks * 2048 >> 4), idesc, (kb != kb0 || ks != 0) ? 1u : 0u);
+#pragma unroll
+          for (uint32_t h = 0; h < ACCS; ++h)
+            umma_bf16(tmem_base + h * MINE, descW + off + ((h * 2 * RO_CHUNK_BYTES + ks * 2048) >> 4), descX + off + (ks * 32 >> 4), idesc,
+                      (kb | ks) != 0 ? 1u : 0u);
         umma_commit(empty_bar(s));
         if (++s == p.stages) {
           s = 0;
@@ -260,7 +267,10 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, NV == 4
       }
       if (!ok) record_status(p.status, DEV_TIMEOUT, 206);
       // also after giving up: the MMAs issued so far finish before the waiting warps go on and the tensor memory is freed
-      umma_commit(acc_bar);
+      if (k_blocks > 0)
+        umma_commit(acc_bar);
+      else
+        mbar_arrive(acc_bar);
       if (!ok) mbar_wait(acc_bar, 0u);
     }
   } else {
@@ -269,18 +279,14 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, NV == 4
       p.row_gate[i] = 0.f;
   }
 
-  const uint32_t part = smem_base;  // partial logits of the tile, over the operand stages
+  const uint32_t part = smem_base;  // the logits of this CTA's tokens, over the operand stages
   constexpr uint32_t PITCH = 32 * NV * 4 + 16;  // rows 16 bytes apart in the banks
-  if (warp < 2) cluster_or_block_sync<CL>();
   if (warp >= 2) {
-    constexpr int MINE = RO_TOK / CL;  // this CTA's tokens of the tile
     constexpr uint32_t MAX_PITCH = 32 * (NV / 4) * 4 + 16;
-    const uint32_t maxima = part + RO_TOK * PITCH;              // of the groups of four columns: MINE rows
+    const uint32_t maxima = part + MINE * PITCH;                // of the groups of four columns
     const uint32_t picks = maxima + MINE * MAX_PITCH;           // {exponential, column}: k rows of MINE (and one, in other banks)
     const uint32_t pick_pitch = MINE * 8 + 8, recip = picks + p.k * pick_pitch;  // 1 / sum of the exponentials
     const int w = warp - 2, E = p.E, k = p.k;
-    const int64_t first = t0 + rank * MINE, left = p.T - first;
-    const int tokens = left < MINE ? static_cast<int>(left) : MINE;  // of which are there (may be negative)
     float acc[NV];
 #pragma unroll
     for (int q = 0; q < NV; ++q) acc[q] = 0.f;
@@ -290,19 +296,14 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, NV == 4
       if (all || pass == 0) {
 #pragma unroll 1
         for (int i = w; i < (all ? tokens : w + 1); i += RO_WARPS) {
-          const uint32_t mrow = maxima + (i < MINE ? i : 0) * MAX_PITCH;
+          const uint32_t mrow = maxima + i * MAX_PITCH;
           float v[NV];
           float vmax = -INFINITY;
 #pragma unroll
           for (int q = 0; q < NV / 4; ++q) {
             const int col = 4 * (lane + 32 * q);
-            const uint32_t a = part + (rank * MINE + (i < MINE ? i : 0)) * PITCH + col * 4;
-            float4 x[CL];
-#pragma unroll
-            for (int r = 0; r < CL; ++r) x[r] = ld_cluster_f4(CL > 1 ? mapa_shared(a, all ? r : rank) : a);
-            float4 sum = x[0];
-#pragma unroll
-            for (int r = 1; r < CL; ++r) sum = make_float4(sum.x + x[r].x, sum.y + x[r].y, sum.z + x[r].z, sum.w + x[r].w);
+            const uint32_t a = part + i * PITCH + col * 4;
+            float4 sum = lds_f4(a);
             if (col < E) {  // E is a multiple of 8: the four columns exist or do not
               if (p.bias) {
                 const float4 b = *reinterpret_cast<const float4*>(p.bias + col);
@@ -341,7 +342,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, NV == 4
       const int t = tid - 64;
       if (all ? t < tokens : pass == 1) {
         const uint32_t scratch = smem_u32(s_first);
-        const float rz = select_topk<2 * NV>(all ? k : 1, all ? part + (rank * MINE + t) * PITCH : scratch,
+        const float rz = select_topk<2 * NV>(all ? k : 1, all ? part + t * PITCH : scratch,
                                              all ? maxima + t * MAX_PITCH : scratch + 32 * NV * 4,
                                              all ? picks + t * 8 : scratch + 40 * NV * 4, pick_pitch, s_hist, all ? 1 : 0);
         asm volatile("st.shared.f32 [%0], %1;" ::"r"(all ? recip + t * 4 : scratch + 40 * NV * 4 + 8), "f"(rz) : "memory");
@@ -363,67 +364,88 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, NV == 4
         }
       }
       if (all) break;
-      // partial logits: tensor memory -> shared memory (the operand stages have all been consumed)
+      // logits: tensor memory (lane = expert, column = token) -> shared memory (the operand stages have all been consumed)
       const bool ok = mbar_wait(acc_bar, 0u);
       if (!ok && lane == 0) record_status(p.status, DEV_TIMEOUT, 306);
       tc_fence_after();
-      const int ew = warp & 3, row = ew * 32 + lane;
-      if (ok)
-        for (int c = w >> 2; c * 16 < E; c += RO_WARPS / 4) {
+      const int ew = warp & 3;
+      if (ok && tokens > 0)
+#pragma unroll 1
+        for (int c = w >> 2; c < static_cast<int>(ACCS) * (MINE / 16); c += RO_WARPS / 4) {
+          const int e = c / (MINE / 16) * 128 + ew * 32 + lane, tok0 = c % (MINE / 16) * 16;
           uint32_t r[16];
           tmem_ld16(tmem_base + (static_cast<uint32_t>(ew * 32) << 16) + c * 16, r);
           tmem_ld_wait();
+          if (e < E)
 #pragma unroll
-          for (int b = 0; b < 4; ++b)
-            st_shared_v4(part + row * PITCH + c * 64 + b * 16, r[4 * b], r[4 * b + 1], r[4 * b + 2], r[4 * b + 3]);
+            for (int i = 0; i < 16; ++i) asm volatile("st.shared.b32 [%0], %1;" ::"r"(part + (tok0 + i) * PITCH + e * 4), "r"(r[i]) : "memory");
         }
       tc_fence_before();
-      cluster_or_block_sync<CL>();
+      routing_sync();
 #pragma unroll
       for (int q = 0; q < NV; ++q) acc[q] = 0.f;
     }
 #pragma unroll
     for (int q = 0; q < NV; ++q) s_psum[w][4 * (lane + 32 * (q / 4)) + q % 4] = acc[q];
     routing_sync();
+    if (CL > 1) cluster_wait();  // the tile's first CTA has cleared its counts
     const int e = tid - 64;
     if (e < E) {
       float s = 0.f;
 #pragma unroll 4
       for (int u = 0; u < RO_WARPS; ++u) s += s_psum[u][e];
       if (tokens > 0) p.psum_part[static_cast<int64_t>(blockIdx.x) * E + e] = s;
-      if (CL > 1 && rank != 0) red_cluster_add(mapa_shared(smem_u32(&s_hist[e]), 0), s_hist[e]);
+      if (CL > 1 && rank != 0 && tokens > 0) red_cluster_add(mapa_shared(smem_u32(&s_hist[e]), 0), s_hist[e]);
       if (CL == 1) p.tile_counts[static_cast<int64_t>(tile) * E + e] = s_hist[e];
     }
+  } else if (CL > 1) {
+    cluster_wait();
   }
-  if (CL > 1) {
-    cluster_sync_diverged();  // nobody reads this CTA's shared memory any more; the counts of the tile are complete
-    if (rank == 0 && tid >= 64 && tid - 64 < p.E) p.tile_counts[static_cast<int64_t>(tile) * p.E + tid - 64] = s_hist[tid - 64];
-  }
+  if (CL > 1)
+    cluster_sync_diverged();  // the counts of the tile are complete
+  else
+    block_sync_diverged();  // tensor memory has been read
+  if (CL > 1 && rank == 0 && tid >= 64 && tid - 64 < p.E) p.tile_counts[static_cast<int64_t>(tile) * p.E + tid - 64] = s_hist[tid - 64];
   if (warp == 1) {
     __syncwarp();  // freeing tensor memory takes the whole warp
     tc_fence_after();
-    tmem_dealloc(tmem_base, p.tmem_cols);
+    tmem_dealloc(tmem_base, TMEM_COLS);
   }
 }
 
-// CTAs per token tile: four while each has an SM to itself, two while two share one (E <= 128), never more than there are K
-// blocks.  Router stage at d 2048, 128 experts, us, with one / two / four / eight: 128 tokens 30 / 23 / 18 / 18, 2048 30 / 23 /
-// 19 / 22, 4736 (148 CTAs of four) 30 / 24 / 23 / 34, 8192 32 / 25 / 25 / 40, 9472 32 / 27 / 36 / 51, 16384 35 / 32 / 42, 18944
-// (296 CTAs of two) 36 / 35 / 53, 24576 40 / 49 / 57.  One CTA per tile in the persistent GEMM template, its 128 tokens routed by
-// four warps: 28 at 128 to 4096 tokens, 31 at 8192, 33 at 16384, 48 at 32768, where this kernel takes 18 to 24, 25, 32 and 44.
-int router_cluster(const Shape& s, int sm_count, int64_t T, bool fp32_weight) {
+// CTAs per token tile: as many as have an SM each.  Clusters of four do not fill the chip (they lie within a part of it), so
+// they go up to eight ninths of the SMs.  Router stage, us, with one / two / four at d 2048 and 128 experts: 128 tokens 25 / 21 / 19,
+// 4096 (128 CTAs of four) 25 / 21 / 20, 4736 (148) 25 / 22 / 24 or more, 8192 26 / 23 / 25, 9472 (148 CTAs of two) 27 / 24 / 37, 12000
+// 29 / 31 / 39, 16384 31 / 34 / 45, 18944 33 / 35 / 55, 32768 47 / 58 / 80; with 256 experts 33 / 27 / 23 at 128, 31 / 27 / 24 at 4096, 34 /
+// 29 / 58 at 9472, 35 / 49 / 60 at 12000.  Rows of W_r of less than 64 bytes come slowly however few they are, and all CTAs ask for the
+// same lines, so that with few experts fewer CTAs are better sooner: d 4096 and 8 experts 29 / 27 / 25 at 128 tokens, 29 / 27 / 27 at
+// 2048, 30 / 31 / 37 at 4096, 37 / 39 / 57 at 8192; d 256 and 8 experts 16 / 14 / 14 at 2048, 17 / 16 / 17 at 4096.
+// One CTA per tile in the persistent GEMM template, four warps routing: 27 at 128 to 4096 tokens, 28 at 8192, 32 at 16384, 54 at 32768.
+int router_cluster(const Shape& s, int sm_count, int64_t T) {
   const int64_t tiles = (T + RO_TOK - 1) / RO_TOK;
-  const int k_total = s.d / RO_BK * (fp32_weight ? 3 : 1);
-  const int cl = tiles * 4 <= sm_count ? 4 : tiles * 2 <= sm_count * (s.E <= 128 ? 2 : 1) ? 2 : 1;
-  return cl <= k_total ? cl : k_total < 2 ? 1 : 2;
+  if (s.E < 32 && tiles > 16) return 1;
+  return tiles * 4 * 9 <= sm_count * 8 ? 4 : tiles * 2 <= sm_count ? 2 : 1;
 }
 
 template <int CL, int NV>
-static moe_status launch_one(moe_ctx_impl* ctx, const RouterParams& p, int tiles, size_t smem, cudaStream_t st) {
+static moe_status launch_one(moe_ctx_impl* ctx, RouterParams& p, int tiles, cudaStream_t st) {
   auto* const kernel = router_cluster_kernel<CL, NV>;
+  // the stages (and what an MMA reads behind an odd number of chunks), and over them what the routing needs: the logits of the
+  // CTA's tokens, the maxima of their groups, and {pick, column} and 1 / sum for k picks
+  constexpr size_t mine = RO_TOK / CL;
+  const size_t routing = mine * (128 * NV + 16) + mine * (32 * NV + 16) + p.k * (mine * 8 + 8) + mine * 4;
+  auto smem_of = [&](int stages) {
+    const size_t ring = stages * p.stage_bytes + (p.w_chunks & 1) * RO_CHUNK_BYTES;
+    return (ring > routing ? ring : routing) + 1024;
+  };
+  auto stages_in = [&](int ring) { return std::min(ring / static_cast<int>(p.stage_bytes), RO_MAX_STAGES); };
+  p.w_bytes = p.w_chunks * RO_CHUNK_BYTES;
+  p.stage_bytes = p.w_bytes + mine * RO_BK * 2;
+  p.stages = stages_in(NV > 4 || tiles * CL <= ctx->sm_count ? RO_DEEP_RING : RO_RING);
+  const size_t smem = smem_of(p.stages), smem_most = smem_of(stages_in(RO_DEEP_RING));
   constexpr int slot = (CL == 1 ? 0 : CL == 2 ? 1 : 2) + (NV == 4 ? 0 : 4);
   if (!(ctx->router_attr & (1u << slot))) {  // per device: the context is bound to one (and to one top-k)
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess)
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_most)) != cudaSuccess)
       return MOE_ERR_CUDA;
     ctx->router_attr |= 1u << slot;
   }
@@ -439,21 +461,17 @@ moe_status launch_router_tc(moe_ctx_impl* ctx, int64_t T, const WsLayout& L, cha
   p.E = s.E;
   p.k = s.k;
   p.T = T;
-  p.b_chunks = (s.E + 63) / 64;
+  p.w_chunks = (s.E + 63) / 64;
   p.whole_chunks = s.E % 64 == 0;
   auto map_w = [&](CUtensorMap* m, const uint16_t* w) {  // W_r as a one-slab tensor of weights
-    return p.whole_chunks ? map_mn(fn, m, w, 1, s.d, s.E, p.b_chunks) : map_3d(fn, m, w, 1, s.d, s.E, 64);
+    return p.whole_chunks ? map_mn(fn, m, w, 1, s.d, s.E, p.w_chunks) : map_3d(fn, m, w, 1, s.d, s.E, 64);
   };
-  bool ok = map_2d(fn, &p.map_x, io.x, T, s.d, RO_TOK) && map_w(&p.map_w0, io.W_r);
+  const int cl = router_cluster(s, ctx->sm_count, T);
+  bool ok = map_2d(fn, &p.map_x, io.x, T, s.d, RO_TOK / cl) && map_w(&p.map_w0, io.W_r);
   if (io.W_r_mid) ok = ok && map_w(&p.map_w1, io.W_r_mid) && map_w(&p.map_w2, io.W_r_lo);
   if (!ok) return MOE_ERR_CUDA;
   p.k_blocks = s.d / RO_BK;
   p.k_total = p.k_blocks * (io.W_r_mid ? 3 : 1);
-  p.mma_n = (s.E + 15) / 16 * 16;
-  p.stage_bytes = RO_A_BYTES + p.b_chunks * RO_CHUNK_BYTES;
-  const bool narrow = s.E <= 128;
-  p.stages = narrow ? 3 : RO_MAX_STAGES;
-  p.tmem_cols = s.E <= 32 ? 32 : s.E <= 64 ? 64 : s.E <= 128 ? 128 : 256;
   p.status = reinterpret_cast<int32_t*>(ws + L.status);
   p.row_gate = reinterpret_cast<float*>(ws + L.row_gate);
   p.rows = L.rows_alloc;
@@ -467,24 +485,17 @@ moe_status launch_router_tc(moe_ctx_impl* ctx, int64_t T, const WsLayout& L, cha
   p.psum_part = reinterpret_cast<float*>(ws + L.psum_part);
   p.tile_counts = reinterpret_cast<int32_t*>(ws + L.tile_counts);
   const int tiles = static_cast<int>((T + RO_TOK - 1) / RO_TOK);
-  const int cl = router_cluster(s, ctx->sm_count, T, io.W_r_mid != nullptr);
-  // three stages of 32 KB (E <= 128) or four of up to 48 KB, and over them what the routing needs: 128 rows of partial logits,
-  // for the CTA's tokens the maxima of their groups, and {pick, column} and 1 / sum for k picks
-  const size_t nv = narrow ? 4 : 8, mine = RO_TOK / cl;
-  const size_t ring = narrow ? 3 * (RO_A_BYTES + 2 * RO_CHUNK_BYTES) : RO_MAX_STAGES * (RO_A_BYTES + 4 * RO_CHUNK_BYTES);
-  const size_t routing = RO_TOK * (128 * nv + 16) + mine * (32 * nv + 16) + s.k * (mine * 8 + 8) + mine * 4;
-  const size_t smem = (ring > routing ? ring : routing) + 1024;
-  if (narrow) {
+  if (s.E <= 128) {
     switch (cl) {
-      case 4: return launch_one<4, 4>(ctx, p, tiles, smem, st);
-      case 2: return launch_one<2, 4>(ctx, p, tiles, smem, st);
-      default: return launch_one<1, 4>(ctx, p, tiles, smem, st);
+      case 4: return launch_one<4, 4>(ctx, p, tiles, st);
+      case 2: return launch_one<2, 4>(ctx, p, tiles, st);
+      default: return launch_one<1, 4>(ctx, p, tiles, st);
     }
   }
   switch (cl) {
-    case 4: return launch_one<4, 8>(ctx, p, tiles, smem, st);
-    case 2: return launch_one<2, 8>(ctx, p, tiles, smem, st);
-    default: return launch_one<1, 8>(ctx, p, tiles, smem, st);
+    case 4: return launch_one<4, 8>(ctx, p, tiles, st);
+    case 2: return launch_one<2, 8>(ctx, p, tiles, st);
+    default: return launch_one<1, 8>(ctx, p, tiles, st);
   }
 }
 

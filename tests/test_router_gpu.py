@@ -15,11 +15,14 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("T,d,E,k", [
     (1, 512, 128, 8), (31, 512, 128, 8), (33, 512, 128, 8),        # four CTAs to a tile, 32 tokens each, most of them idle
     (129, 512, 64, 6), (2047, 512, 128, 16),
-    (200, 64, 16, 2), (200, 128, 16, 2), (200, 192, 24, 4),        # no more CTAs than K blocks
+    (200, 64, 16, 2), (200, 128, 16, 2), (200, 192, 24, 4),        # one to three K blocks
     (33, 512, 256, 32), (300, 512, 136, 8),                        # two groups of four columns to a lane
-    (4736, 512, 40, 3), (4737, 512, 40, 3),                        # 148 SMs: four CTAs to a tile, two
-    (18944, 128, 16, 2), (18945, 128, 16, 2),                      # two, one
-    (4737, 256, 200, 4), (9473, 256, 136, 2),                      # one CTA per SM: two, one
+    (4736, 512, 40, 3), (4737, 512, 40, 3),                        # 148 SMs: two CTAs to a tile
+    (18944, 128, 16, 2), (18945, 128, 16, 2),                      # one: on an SM of its own, or two to an SM
+    (4737, 256, 200, 4), (9473, 256, 136, 2),                      # more than 128 experts: two CTAs to a tile, one
+    (4096, 256, 40, 3), (4097, 256, 40, 3),                        # four CTAs to a tile, two
+    (9472, 128, 40, 3), (9473, 128, 40, 3),                        # two, one
+    (2048, 128, 16, 2), (2049, 128, 16, 2),                        # fewer than 32 experts: four, one
 ])
 def test_routing_in_every_form(T, d, E, k):
     inp = synth.make_inputs(synth.MoEShape(T, d, E, k, 64), 300 + T % 97, x_std=1.0)
