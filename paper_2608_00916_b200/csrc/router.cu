@@ -305,9 +305,9 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, NV == 4
             const uint32_t a = part + i * PITCH + col * 4;
             float4 sum = lds_f4(a);
             if (col < E) {  // E is a multiple of 8: the four columns exist or do not
-              if (p.bias) {
-                const float4 b = *reinterpret_cast<const float4*>(p.bias + col);
-                sum = make_float4(sum.x + b.x, sum.y + b.y, sum.z + b.z, sum.w + b.w);
+              if (p.bias) {  // by words: it may lie anywhere in a buffer of parameters
+                const float* const b = p.bias + col;
+                sum = make_float4(sum.x + b[0], sum.y + b[1], sum.z + b[2], sum.w + b[3]);
               }
               if (i < tokens) {
                 const int64_t at = (first + i) * E + col;

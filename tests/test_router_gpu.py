@@ -60,3 +60,37 @@ def test_small_and_large_clusters_agree_on_ties():
         logits, idx = fw["logits"].cpu().numpy(), fw["idx"].cpu().numpy()
         assert np.array_equal(logits[:, :64], logits[:, 64:])
         assert np.array_equal(idx, np.argsort(-logits, axis=1, kind="stable")[:, :k])
+
+
+@pytest.mark.parametrize("E,k", [(16, 2), (136, 4)])
+@pytest.mark.parametrize("offset", [1, 2, 3])
+def test_a_bias_anywhere_in_a_parameter_buffer(E, k, offset):
+    """A view into a flat buffer of fp32 parameters is aligned to 4 bytes only: same results as from an aligned bias, through the
+    plain, forward-only, adapter and expert-parallel calls."""
+    from paper_2608_00916_b200 import ep
+    T, d, f, r = 300, 128, 64, 8
+    g = torch.Generator(device="cuda")
+    g.manual_seed(E)
+    n = lambda *s: torch.empty(*s, device="cuda").normal_(generator=g)
+    x, W_r = n(T, d).bfloat16(), (n(d, E) / d**0.5).bfloat16()
+    W = [(0.1 * n(E, *s)).bfloat16() for s in ((d, f), (d, f), (f, d))]
+    lora = {m: (0.1 * n(E, *s)).bfloat16() for m, s in
+            (("A1", (d, r)), ("B1_gate", (r, f)), ("B1_up", (r, f)), ("A2", (f, r)), ("B2", (r, d)))}
+    aligned = n(E)
+    flat = torch.zeros(E + 4, device="cuda")
+    view = flat[offset:offset + E]
+    view.copy_(aligned)
+    from paper_2608_00916_b200.binding import MoELayer
+
+    def calls(b_r):
+        layer = MoELayer(d, E, f, k)
+        outs = [layer.forward(x, W_r, *W, b_r=b_r, want_logits=True), layer.forward(x, W_r, *W, b_r=b_r, inference=True),
+                layer.lora_forward(x, W_r, *W, lora, 2.0, b_r=b_r)]
+        layer.poll()
+        rank = ep.EPRank(d, E, f, k, 1, 0, T * k)
+        rank.set_peers([rank.own_ws.data_ptr()])
+        return outs + [rank.route(x, W_r, b_r)]
+
+    for want, got in zip(calls(aligned), calls(view)):
+        for name in want:
+            assert want[name] is None or torch.equal(want[name], got[name]), name
