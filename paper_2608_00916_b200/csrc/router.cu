@@ -431,21 +431,20 @@ template <int CL, int NV>
 static moe_status launch_one(moe_ctx_impl* ctx, RouterParams& p, int tiles, cudaStream_t st) {
   auto* const kernel = router_cluster_kernel<CL, NV>;
   // the stages (and what an MMA reads behind an odd number of chunks), and over them what the routing needs: the logits of the
-  // CTA's tokens, the maxima of their groups, and {pick, column} and 1 / sum for k picks
+  // CTA's tokens, the maxima of their groups, and {pick, column} and 1 / sum for k picks (with one CTA per tile and more than 20
+  // picks that leaves no room for two CTAs on an SM)
   constexpr size_t mine = RO_TOK / CL;
-  const size_t routing = mine * (128 * NV + 16) + mine * (32 * NV + 16) + p.k * (mine * 8 + 8) + mine * 4;
-  auto smem_of = [&](int stages) {
-    const size_t ring = stages * p.stage_bytes + (p.w_chunks & 1) * RO_CHUNK_BYTES;
-    return (ring > routing ? ring : routing) + 1024;
-  };
-  auto stages_in = [&](int ring) { return std::min(ring / static_cast<int>(p.stage_bytes), RO_MAX_STAGES); };
+  auto routing = [](int k) { return mine * (128 * NV + 16) + mine * (32 * NV + 16) + k * (mine * 8 + 8) + mine * 4; };
+  auto smem_of = [](size_t ring, size_t over) { return (ring > over ? ring : over) + 1024; };
   p.w_bytes = p.w_chunks * RO_CHUNK_BYTES;
   p.stage_bytes = p.w_bytes + mine * RO_BK * 2;
-  p.stages = stages_in(NV > 4 || tiles * CL <= ctx->sm_count ? RO_DEEP_RING : RO_RING);
-  const size_t smem = smem_of(p.stages), smem_most = smem_of(stages_in(RO_DEEP_RING));
+  const uint32_t room = NV > 4 || tiles * CL <= ctx->sm_count ? RO_DEEP_RING : RO_RING;
+  p.stages = std::min<int>(room / p.stage_bytes, RO_MAX_STAGES);
+  const size_t smem = smem_of(p.stages * p.stage_bytes + (p.w_chunks & 1) * RO_CHUNK_BYTES, routing(p.k));
   constexpr int slot = (CL == 1 ? 0 : CL == 2 ? 1 : 2) + (NV == 4 ? 0 : 4);
-  if (!(ctx->router_attr & (1u << slot))) {  // per device: the context is bound to one (and to one top-k)
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_most)) != cudaSuccess)
+  if (!(ctx->router_attr & (1u << slot))) {  // per device (the context is bound to one), and for every context on it: the most of all
+    const size_t most = smem_of(RO_DEEP_RING + RO_CHUNK_BYTES, routing(MAX_K));
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most)) != cudaSuccess)
       return MOE_ERR_CUDA;
     ctx->router_attr |= 1u << slot;
   }

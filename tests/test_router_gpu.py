@@ -94,3 +94,15 @@ def test_a_bias_anywhere_in_a_parameter_buffer(E, k, offset):
     for want, got in zip(calls(aligned), calls(view)):
         for name in want:
             assert want[name] is None or torch.equal(want[name], got[name]), name
+
+
+@pytest.mark.parametrize("d,E,k,other", [(64, 16, 16, 2), (64, 256, 32, 4)])
+def test_layers_that_share_a_form_of_the_router(d, E, k, other):
+    """The shared-memory limit of a kernel belongs to the device, not to a layer: one that needs less leaves room for the other."""
+    T, f = 20000, 64
+    inp = synth.make_inputs(synth.MoEShape(T, d, E, k, f), 9, x_std=1.0, guard=False)
+    large, small = Run(inp, k), Run(inp, other)
+    first = {n: t.clone() for n, t in large.forward().items() if t is not None}
+    small.forward()
+    again = large.forward()
+    assert all(torch.equal(first[n], again[n]) for n in first)
