@@ -121,7 +121,6 @@ static moe_status status_to_code(int v) {
   return v == DEV_OK ? MOE_OK : (v == DEV_BOUNDS ? MOE_ERR_DEVICE_BOUNDS : MOE_ERR_DEVICE_TIMEOUT);
 }
 
-static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 struct StageTimer {
   moe_ctx_impl* c;
@@ -523,11 +522,7 @@ static moe_status backward_impl(moe_ctx* ctx, int64_t T, const uint16_t* dy, flo
   // after that GEMM and joined before the final unpermute, where it fills the tails of the three big GEMMs instead of
   // standing in line behind them.  Without tokens, or with MOE_FLAG_NO_SIDE_STREAM, it runs in line.
   bool forked = false;
-  // Few tokens: dW_r from one slice of them, without partials and the kernel that adds them up.  us, partials and sum -> one
-  // slice, at d 2048 and 128 experts: 15 -> 13 at 128 and 256 tokens, 15 -> 15 at 512, 15 -> 17 at 1000; at d 256 and 8 experts
-  // 10 -> 9 at 64, 10 -> 10 at 256, 11 -> 11 at 512, 11 -> 15 at 1024, and one launch less for the host.
-  constexpr int64_t ONE_SLICE_TOKENS = 512;
-  const bool one_slice = T > 0 && T <= ONE_SLICE_TOKENS && aligned16(dW_r);
+  const bool one_slice = dwr_in_one_slice(T, dW_r);
   auto router_chain = [&]() -> moe_status {
     cudaStream_t rs = st;
     if (T > 0 && c->use_side_stream) {

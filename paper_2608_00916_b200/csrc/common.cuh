@@ -247,6 +247,12 @@ enum LoraOp {
 moe_status launch_lora_gemm(moe_ctx_impl* ctx, LoraOp op, int64_t T, const WsLayout& L, char* ws, const GemmIO& io,
                             const LoraArgs& lo, cudaStream_t st);
 
+inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+// Few tokens: dW_r from one slice of them, without partials and the kernel that adds them up (the plain and the expert-parallel
+// backward pass alike).  us, partials and sum -> one slice, at d 2048 and 128 experts: 15 -> 13 at 128 and 256 tokens, 15 -> 15 at
+// 512, 15 -> 17 at 1000; at d 256 and 8 experts 10 -> 9 at 64, 10 -> 10 at 256, 11 -> 11 at 512, 11 -> 15 at 1024, and one launch
+// less for the host.
+inline bool dwr_in_one_slice(int64_t T, const void* dW_r) { return T > 0 && T <= 512 && aligned16(dW_r); }
 // true when the tensor-core router / dW_r / dx kernels apply (their TMA maps need E % 8 == 0)
 inline bool router_on_tensor_cores(const Shape& s) { return s.E % 8 == 0; }
 // ---- launchers (router.cu)

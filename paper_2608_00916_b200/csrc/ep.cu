@@ -214,8 +214,6 @@ __global__ void __launch_bounds__(256) ep_gather_dg_kernel(int64_t n, int E_loc,
   dg[i] = s;
 }
 
-static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
-
 struct EpLayouts {
   WsLayout send, own;
   int64_t T_equiv;
@@ -515,11 +513,13 @@ moe_status moe_ep_router_backward(moe_ctx* ctx, int64_t T, float d_aux, const ui
                     reinterpret_cast<uint16_t*>(ws + L.dl_lo), st);
   GemmIO io;
   io.x = x; io.W_r = W_r;
+  const bool one_slice = dwr_in_one_slice(T, dW_r);
   if (T > 0) {
+    if (one_slice) io.dW_r = dW_r;
     rc = launch_grouped_gemm(c, GEMM_DWR, T, L, ws, io, st);
     if (rc != MOE_OK) return rc;
   }
-  launch_dwr(s, T, x, dl, reinterpret_cast<float*>(ws + L.dwr_part), dW_r, db_r, T > 0, st, false);
+  launch_dwr(s, T, x, dl, reinterpret_cast<float*>(ws + L.dwr_part), dW_r, db_r, T > 0, st, false, one_slice);
   if (T > 0) {
     rc = launch_grouped_gemm(c, GEMM_DX, T, L, ws, io, st);
     if (rc != MOE_OK) return rc;

@@ -111,6 +111,26 @@ def test_ep_with_one_rank_equals_the_plain_layer():
         assert torch.equal(owner[0][n], bw[n]), n
 
 
+@pytest.mark.parametrize("T", [1, 64, 512, 513])
+def test_ep_with_one_rank_equals_the_plain_layer_at_few_tokens(T):
+    """Also where the plain layer takes the router weight gradient from one slice of the tokens."""
+    from gpu_util import Run
+    shape = synth.MoEShape(T, 256, 16, 4, 128)
+    r = Run(synth.make_inputs(shape, 36), shape.k)
+    fw, bw = r.forward(), r.backward(0.03)
+    grp = ep.LocalGroup(shape.d, shape.E, shape.f, shape.k, 1, shape.T * shape.k)
+    v = r.dev
+    efw, _ = grp.forward([v["x"]], v["W_r"], v["W_gate"], v["W_up"], v["W_down"])
+    sender, owner = grp.backward([v["dy"]], 0.03, want_db=True)
+    grp.poll()
+    for n in ("idx", "gates", "y", "aux"):
+        assert torch.equal(efw[0][n], fw[n]), n
+    for n in ("dx", "dW_r", "db_r"):
+        assert torch.equal(sender[0][n], bw[n]), n
+    for n in ("dW_gate", "dW_up", "dW_down"):
+        assert torch.equal(owner[0][n], bw[n]), n
+
+
 def test_dist_group_with_one_rank():
     """ep.DistGroup - the multi-process form (NCCL all_gather of the counts, owner workspace in symmetric memory and
     mapped through its rendezvous, group barriers between phases) - on a one-rank group in a child process: bitwise the
