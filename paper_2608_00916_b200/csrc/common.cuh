@@ -357,7 +357,9 @@ __device__ __forceinline__ void init_status_block(int32_t* status, bool this_thr
   }
 }
 // Records a device-side failure.  The first failure sticks: later ones do not overwrite it, and no kernel ever resets
-// the word (the host acknowledges it after reporting it, see moe_poll_status).
+// the word (the host acknowledges it after reporting it, see moe_poll_status).  `where` of a timeout: 100 producer, 200 MMA
+// issuer, 300 epilogue of the one-CTA GEMMs, each plus the GEMM's kind; the same plus 1000 on CTA pairs, plus 2000 with the tokens
+// as N; 3100, 3200, 3300 the router; 9000 the self-test.
 __device__ __forceinline__ void record_status(int32_t* status, int code, int where) {
   if (atomicCAS(status, DEV_OK, code) == DEV_OK) status[1] = where;
 }

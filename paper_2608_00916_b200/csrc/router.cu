@@ -232,7 +232,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, NV == 4
       }
       chain_next();
       if (!ok) {  // gave up: the copies in flight land in this CTA's shared memory before it leaves (bounded again)
-        record_status(p.status, DEV_TIMEOUT, 106);
+        record_status(p.status, DEV_TIMEOUT, 3100);
         const uint32_t n = static_cast<uint32_t>(p.stages);
         for (uint32_t i = it > n ? it - n : 0; i < it; ++i) mbar_wait(full_bar(i % n), (i / n) & 1u);
       }
@@ -265,7 +265,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, NV == 4
           phase ^= 1u;
         }
       }
-      if (!ok) record_status(p.status, DEV_TIMEOUT, 206);
+      if (!ok) record_status(p.status, DEV_TIMEOUT, 3200);
       // also after giving up: the MMAs issued so far finish before the waiting warps go on and the tensor memory is freed
       if (k_blocks > 0)
         umma_commit(acc_bar);
@@ -366,7 +366,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, NV == 4
       if (all) break;
       // logits: tensor memory (lane = expert, column = token) -> shared memory (the operand stages have all been consumed)
       const bool ok = mbar_wait(acc_bar, 0u);
-      if (!ok && lane == 0) record_status(p.status, DEV_TIMEOUT, 306);
+      if (!ok && lane == 0) record_status(p.status, DEV_TIMEOUT, 3300);
       tc_fence_after();
       const int ew = warp & 3;
       if (ok && tokens > 0)
