@@ -19,7 +19,9 @@
  *
  * Conventions
  *   - Every pointer is a DEVICE pointer unless its comment says "host".  Tensors are dense row-major.
- *   - bf16 tensors are passed as uint16_t bit patterns.  Pointers must be 16-byte aligned.
+ *   - bf16 tensors are passed as uint16_t bit patterns.  They, an fp32 router weight, the fp32 buffers that dW_gate, dW_up and
+ *     dW_down accumulate into and the workspaces must be 16-byte aligned (MOE_ERR_INVALID_ARG otherwise); the other fp32 and int32
+ *     arrays (b_r, logits, dW_r, indices, counts and so on) may lie anywhere in a larger buffer.
  *   - The caller owns every buffer, the workspace included.  No entry point allocates or frees device
  *     memory.
  *   - All work is enqueued on the caller's CUDA stream (passed as void* = cudaStream_t).  Neither

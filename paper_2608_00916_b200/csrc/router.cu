@@ -80,6 +80,17 @@ __device__ __forceinline__ int first_eq4(float4 v, float m) { return v.x == m ? 
 __device__ __forceinline__ float4 without(float4 v, int i, float by) {
   return make_float4(i == 0 ? by : v.x, i == 1 ? by : v.y, i == 2 ? by : v.z, i == 3 ? by : v.w);
 }
+// The caller's copy of the logits, whose alignment nothing checks
+__device__ __forceinline__ void store_caller(float* out, float4 v) {
+  if ((reinterpret_cast<uintptr_t>(out) & 15u) == 0) {
+    *reinterpret_cast<float4*>(out) = v;
+  } else {
+    out[0] = v.x;
+    out[1] = v.y;
+    out[2] = v.z;
+    out[3] = v.w;
+  }
+}
 __device__ __forceinline__ int lds_int(uint32_t addr) {
   int v;
   asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
@@ -312,7 +323,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, NV == 4
               if (i < tokens) {
                 const int64_t at = (first + i) * E + col;
                 *reinterpret_cast<float4*>(p.logits + at) = sum;
-                if (p.logits_out) *reinterpret_cast<float4*>(p.logits_out + at) = sum;
+                if (p.logits_out) store_caller(p.logits_out + at, sum);
               }
             } else {
               sum = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);

@@ -106,3 +106,36 @@ def test_layers_that_share_a_form_of_the_router(d, E, k, other):
     small.forward()
     again = large.forward()
     assert all(torch.equal(first[n], again[n]) for n in first)
+
+
+@pytest.mark.parametrize("E,k", [(16, 2), (136, 4), (12, 2)])
+@pytest.mark.parametrize("offset", [1, 2, 3])
+def test_fp32_and_int32_outputs_anywhere_in_a_buffer(E, k, offset):
+    """C entry points: logits, gates, indices, counts, order, aux loss and dW_r that are aligned to 4 bytes only."""
+    import ctypes as C
+    T, d, f = 300, 128, 64
+    inp = synth.make_inputs(synth.MoEShape(T, d, E, k, f), 11, x_std=1.0, guard=False)
+    r = Run(inp, k)
+    fw = r.forward()
+    bw = r.backward(0.05)
+    shapes = {"idx": (T, k), "gates": (T, k), "counts": (E,), "perm": (T * k,), "aux": (1,), "logits": (T, E), "dW_r": (d, E)}
+    flat, out = {}, {}
+    for n, s in shapes.items():
+        want = fw[n] if n in fw else bw[n]
+        flat[n] = torch.full((want.numel() + 8,), 7, dtype=want.dtype, device="cuda")
+        out[n] = flat[n][offset:offset + want.numel()].view(s)
+    y, layer, v = torch.empty_like(fw["y"]), r.layer, r.dev
+    p = lambda t: C.c_void_p(t.data_ptr())
+    stream = C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    assert layer.lib.moe_forward(layer.h, T, p(v["x"]), p(v["W_r"]), None, None, p(v["W_gate"]), p(v["W_up"]), p(v["W_down"]), p(y),
+                                 p(out["idx"]), p(out["gates"]), p(out["counts"]), p(out["perm"]), p(out["aux"]), p(out["logits"]),
+                                 p(layer.ws), layer.ws.numel(), stream) == 0
+    layer.backward(v["dy"], 0.05, grads={"dW_r": out["dW_r"]})
+    layer.poll()
+    for n in shapes:
+        want = fw[n] if n in fw else bw[n]
+        if n == "dW_r":  # partial sums instead of one slice of the tokens
+            assert (out[n] - want).norm().item() <= 1e-5 * want.norm().item()
+        else:
+            assert torch.equal(out[n].reshape(want.shape), want), n
+        assert (flat[n][:offset] == 7).all() and (flat[n][offset + want.numel():] == 7).all(), n
