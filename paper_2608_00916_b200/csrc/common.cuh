@@ -35,7 +35,8 @@ struct Shape {
 // Byte offsets of every internal buffer inside the caller's workspace (all 256-byte aligned).
 struct WsLayout {
   size_t status;       // int32[16]   [0] device status (first failure sticks), [1] where it happened, [2..3] cookie
-  size_t timers;       // int64[GEMM_KINDS][8] cycle counters of the GEMM roles (filled only when MOE_GEMM_TIMERS is set)
+  size_t timers;       // int64[2 GEMM_KINDS][8] cycle counters of the GEMM roles (filled only when MOE_GEMM_TIMERS is set);
+                       // second half: row GEMMs with the tokens as N
   size_t counts;       // int32[E]    rows per expert
   size_t offsets;      // int32[E+1]  exclusive scan of counts (canonical, unpadded)
   size_t pad_offsets;  // int32[E+1]  exclusive scan of counts rounded up to ROW_PAD
@@ -227,6 +228,8 @@ struct LoraArgs {
   const uint16_t *A1 = nullptr, *B1g = nullptr, *B1u = nullptr, *A2 = nullptr, *B2 = nullptr;
   uint16_t *dA1 = nullptr, *dB1g = nullptr, *dB1u = nullptr, *dA2 = nullptr, *dB2 = nullptr;
 };
+// consecutive row tiles that a row GEMM walks inside one column tile
+int row_group_for(int n_tiles, const moe_ctx_impl* ctx);
 // row GEMMs with the tokens as the N operand; lo: with the extra K segment of the adapters (gemm_tokens.cu)
 moe_status launch_token_gemm(moe_ctx_impl* ctx, GemmKind kind, const WsLayout& L, char* ws, const GemmIO& io, const LoraArgs* lo,
                              bool small, cudaStream_t st);

@@ -294,7 +294,7 @@ static moe_status launch_kind(moe_ctx_impl* ctx, const GemmParams& p, cudaStream
 // Row tiles (or pairs) walked together inside a column tile: 1 while the expert's weights are few column tiles wide (they
 // stay in L2 between row tiles: Qwen3-30B-A3B shape), 16 for wide experts (coarse shape: at 112 column tiles an expert's
 // gate and up slabs are 235 MB and were read from DRAM once per row pair).  MOE_ROW_GROUP overrides (measurements).
-static int row_group_for(int n_tiles, const moe_ctx_impl* ctx) {
+int row_group_for(int n_tiles, const moe_ctx_impl* ctx) {
   if (ctx->row_group_override > 0) return ctx->row_group_override;
   return n_tiles > 12 ? 16 : 1;
 }
@@ -556,7 +556,7 @@ static bool row_gemm_on_pairs(const moe_ctx_impl* ctx, GemmKind kind, double row
 // 256; d 512, f 768 21 -> 15 at 64, 21 -> 21 at 256; d 768, f 512, 64 experts 25 -> 21 at 16 rows.
 static bool row_gemm_by_tokens(const moe_ctx_impl* ctx, GemmKind kind, double rows_per_expert) {
   const int d = ctx->s.d, f = ctx->s.f;
-  if (ctx->tile_mode != 0) return false;
+  if (ctx->tile_mode != 0 || (kind == GEMM_B4 && ctx->b4_pair_override >= 0)) return false;
   if (kind == GEMM_B2 && rows_per_expert < 128.0) return true;
   if (d < 1024 || f < 512) return false;
   switch (kind) {
@@ -718,8 +718,9 @@ static moe_status launch_lora_gemm_bwd(moe_ctx_impl* ctx, LoraOp op, const WsLay
 // extra 64-deep K segment ([xp | u] [[W]; [B1]], ...), the four 64-wide row buffers u, v, w, z come from skinny
 // instances (N = 64) of the F4 / B4 kinds, and the adapter gradients from instances of the B3 / B5 kinds whose M or
 // N is the rank.  The four large ones take the tile shape the plain layer would
-// (rank 16, 8192 tokens, 512 rows per expert: a step 2132 -> 2079 us), the others one-CTA tiles.  All walk the row tiles in
-// plain column order, also those of wide experts (row_group_for): adapters on such experts have not been timed.
+// (rank 16, 8192 tokens, 512 rows per expert: a step 2132 -> 2079 us), the others one-CTA tiles.  On row tiles they
+// walk in plain column order, also those of wide experts, with the tokens as N as the plain layer does (row_group_for): adapters
+// on such experts have not been timed.
 moe_status launch_lora_gemm(moe_ctx_impl* ctx, LoraOp op, int64_t T, const WsLayout& L, char* ws, const GemmIO& io,
                             const LoraArgs& lo, cudaStream_t st) {
   const Shape& s = ctx->s;

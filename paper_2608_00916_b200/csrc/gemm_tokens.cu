@@ -627,7 +627,7 @@ moe_status launch_token_gemm(moe_ctx_impl* ctx, GemmKind kind, const WsLayout& L
   p.pad_offsets = reinterpret_cast<const int32_t*>(ws + L.pad_offsets);
   p.counts = reinterpret_cast<const int32_t*>(ws + L.counts);
   p.status = reinterpret_cast<int32_t*>(ws + L.status);
-  p.timers = ctx->gemm_timers ? reinterpret_cast<unsigned long long*>(ws + L.timers) + 8 * kind : nullptr;
+  p.timers = ctx->gemm_timers ? reinterpret_cast<unsigned long long*>(ws + L.timers) + 8 * (GEMM_KINDS + kind) : nullptr;
   p.nseg = 1;
   p.k_blocks1 = lo ? 1 : 0;
   bool ok = true;
@@ -680,7 +680,7 @@ moe_status launch_token_gemm(moe_ctx_impl* ctx, GemmKind kind, const WsLayout& L
   }
   if (!ok) return MOE_ERR_CUDA;
   p.ld_out = p.N_total;
-  p.row_group = p.n_tiles > 12 ? 16 : 1;
+  p.row_group = row_group_for(p.n_tiles, ctx);
   switch (kind) {
     case GEMM_F3: return launch_token_kind<GEMM_F3>(ctx, p, st);
     case GEMM_F4: return launch_token_kind<GEMM_F4>(ctx, p, st);

@@ -28,3 +28,8 @@ def test_barriers_after_the_one_thread_roles_do_not_need_whole_warps():
 def test_a_failed_launch_is_reported_once():
     for name, text in rules.sources():
         assert text.count("launch_kernel(") == text.count("return cudaGetLastError() == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;"), name
+
+
+def test_every_row_gemm_walks_its_tiles_in_groups_by_one_rule():
+    text = dict(rules.sources())["gemm_tokens.cu"]
+    assert "p.row_group = row_group_for(" in text

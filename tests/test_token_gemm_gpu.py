@@ -50,3 +50,51 @@ def test_one_expert_takes_every_token():
     inp = synth.make_inputs(synth.MoEShape(700, 2048, 16, 2, 512), 7, x_std=1.0, skew=True)
     ofw, obw = oracle_run(inp, 2, 0.1)
     check_all(Run(inp, 2), ofw, obw, 0.1)
+
+
+def forms(layer, T=None, inference=False):
+    """Which form each row GEMM of a layer's last step took: "one" CTA tiles, CTA "pairs" or "tokens" as N (from the CTAs that
+    MOE_GEMM_TIMERS counts, one of each pair, apart for the two kinds of operands).  With T, before the step: clears the counters."""
+    if T is not None:
+        layer._ensure_ws(T, inference)
+        layer.ws.zero_()
+        return None
+    ctas = layer.buffer("timers", torch.int64).view(2, 8, 8)[:, :, 7].cpu().tolist()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    out = {}
+    for i, name in ((0, "F3"), (1, "F4"), (2, "B2"), (4, "B4")):
+        rows, tokens = ctas[0][i], ctas[1][i]
+        assert (rows, tokens) in ((sms, 0), (sms // 2, 0), (0, sms // 2)), (name, rows, tokens)
+        out[name] = "tokens" if tokens else "pairs" if rows == sms // 2 else "one"
+    return out
+
+
+def step_forms(T, d, E, k, f):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(T)
+    n = lambda *s: torch.empty(*s, device="cuda").normal_(0, 0.05, generator=g).bfloat16()
+    from paper_2608_00916_b200.binding import MoELayer
+    layer = MoELayer(d, E, f, k)
+    forms(layer, T)
+    layer.forward(n(T, d), n(d, E), n(E, d, f), n(E, d, f), n(E, f, d))
+    grads = layer.backward(n(T, d), 0.01)
+    layer.poll()
+    return forms(layer), grads["dx"]
+
+
+def test_measurement_switches_act_on_every_form(monkeypatch):
+    """MOE_B4_PAIR puts dgrad gate/up on one-CTA tiles or pairs where the rule would take the tokens as N; the order in which
+    MOE_ROW_GROUP walks the tiles changes no bit."""
+    monkeypatch.setenv("MOE_GEMM_TIMERS", "1")
+    chosen, dx = step_forms(1000, 2048, 8, 2, 512)  # 250 rows per expert
+    assert set(chosen.values()) == {"tokens"}
+    for value, form in (("0", "one"), ("1", "pairs")):
+        monkeypatch.setenv("MOE_B4_PAIR", value)
+        forced, other = step_forms(1000, 2048, 8, 2, 512)
+        assert forced == {**chosen, "B4": form}
+        assert torch.equal(other, dx)
+    monkeypatch.delenv("MOE_B4_PAIR")
+    for value in ("2", "5"):
+        monkeypatch.setenv("MOE_ROW_GROUP", value)
+        grouped, other = step_forms(1000, 2048, 8, 2, 512)
+        assert grouped == chosen and torch.equal(other, dx)
