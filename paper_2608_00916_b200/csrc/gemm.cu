@@ -538,32 +538,45 @@ static bool row_gemm_on_pairs(const moe_ctx_impl* ctx, GemmKind kind, double row
 
 // Row GEMMs with the tokens as the N operand (gemm_tokens.cu): no padding rows in the MMAs, but longer epilogues (the results
 // have to be transposed), so the K loop must be long, and where an expert's rows fill the other tiles anyway there is nothing
-// to gain.  Pairs or one-CTA tiles, whichever the rule above takes -> tokens, us, at d 2048, f 768, 128 experts:
-//   rows        15          62          256         512         768         1024        2048          4096
-//   gate/up     165 -> 154  165 -> 158  221 -> 208  350 -> 319  487 -> 453  629 -> 592  1198 -> 1157  2399 -> 2385
-//   down        80 -> 81    81 -> 84    122 -> 121  198 -> 198  275 -> 282  352 -> 362  647 -> 670    1218 -> 1315
-//   dgrad-down  114 -> 92   113 -> 101  168 -> 146  252 -> 219  337 -> 299  414 -> 371  775 -> 735    1554 -> 1551
-//   dgrad-g/u   156 -> 152  156 -> 154  215 -> 198  360 -> 322  518 -> 474  670 -> 624  1228 -> 1174  2362 -> 2370
-// and at d 4096, f 14336, 8 experts, whose row tiles are walked in groups:
-//   rows        64          128         256         512         768           1024          4096
-//   gate/up     341 -> 331  379 -> 358  508 -> 454  847 -> 756  1172 -> 1098  1501 -> 1401  6189 -> 6391
-//   down        148 -> 154  217 -> 164  279 -> 253  469 -> 440  655 -> 659    754 -> 778    3082 -> 3290
-//   dgrad-down  209 -> 184  226 -> 210  320 -> 281  496 -> 428  639 -> 588    845 -> 780    3218 -> 3420
-//   dgrad-g/u   314 -> 313  449 -> 336  539 -> 496  933 -> 876  1316 -> 1408  1526 -> 1721  6231 -> 6520
-// Smaller widths: at d 1024, f 1536, 32 experts dgrad-down 43 -> 31, 45 -> 43, 93 -> 85, 172 -> 146 at 32, 128, 512, 1024 rows, but
-// gate/up (16 K blocks, three outputs) 53 -> 56, 57 -> 61, 101 -> 107, 166 -> 184.  At d 256 to 768 only dgrad-down gains, whose
-// other form is slow to start, and that only with few rows: d 256, f 512, 8 experts 19 -> 13 at 16 rows, 19 -> 15 at 64, 19 -> 19 at
-// 256; d 512, f 768 21 -> 15 at 64, 21 -> 21 at 256; d 768, f 512, 64 experts 25 -> 21 at 16 rows.
-static bool row_gemm_by_tokens(const moe_ctx_impl* ctx, GemmKind kind, double rows_per_expert) {
+// to gain.  The other tiles begin to need a second block of 128 rows where the experts average 120, and that is the main line.
+// Pairs or one-CTA tiles, whichever the rule above takes -> tokens, us, at d 2048, f 768, 128 experts:
+//   rows        8           32          64          96          120         128         256         512         640
+//   gate/up     165 -> 154  165 -> 158  165 -> 162  163 -> 160  167 -> 164  174 -> 169  220 -> 207  348 -> 316  418 -> 386
+//   down        81 -> 80    81 -> 82    81 -> 84    81 -> 82    85 -> 88    91 -> 91    121 -> 120  198 -> 200  235 -> 239
+//   dgrad-down  111 -> 91   111 -> 96   111 -> 102  112 -> 106  124 -> 115  127 -> 118  168 -> 147  251 -> 221  301 -> 258
+//   dgrad-g/u   156 -> 150  156 -> 152  156 -> 156  155 -> 155  164 -> 158  171 -> 161  215 -> 196  360 -> 323  437 -> 396
+// (the down GEMM ties by stage, but whole calls gain by it at 128 and 256 rows: scoring 2048 tokens 311, 312 -> 306, 307, a training
+// step of 4096 1426, 1434 -> 1399, 1431; 1024, 2048, 4096 rows: gate/up 629 -> 592, 1198 -> 1157, 2399 -> 2385, dgrad-g/u 670 -> 624, 1228 -> 1174, 2362 -> 2370) and at
+// d 4096, f 14336, 8 experts, whose row tiles are walked in groups:
+//   rows        8           64          96          128         256         512         640           768           1536
+//   gate/up     341 -> 327  342 -> 330  342 -> 345  362 -> 356  507 -> 457  795 -> 766  999 -> 917    1161 -> 1077  2092 -> 2137
+//   down        147 -> 150  148 -> 153  147 -> 158  222 -> 163  280 -> 260  485 -> 475  556 -> 532    642 -> 679    1097 -> 1170
+//   dgrad-down  213 -> 176  214 -> 186  214 -> 199  233 -> 211  321 -> 282  492 -> 417  545 -> 508    643 -> 588    1166 -> 1164
+//   dgrad-g/u   313 -> 306  314 -> 312  314 -> 328  462 -> 333  541 -> 502  936 -> 942  1115 -> 1151  1295 -> 1428  2224 -> 2438
+// Between, at 64 / 96 / 128 / 256 / 640 / 2048 rows:
+//   gate/up     d 3072, f 1536: 121 -> 124, 121 -> 126, 146 -> 130, 162 -> 151, 306 -> 276, 862 -> 831; d 4096, f 3072: 156 -> 161, 156 ->
+//               167, 167 -> 175, 239 -> 218, 426 -> 393, 1203 -> 1166; d 2048, f 512: 65 -> 68, 66 -> 69, 72 -> 72, 92 -> 90, 146 -> 139;
+//               d 1024, f 512: 40 -> 44, 39 -> 44, 44 -> 48, 56 -> 57, 88 -> 94, 211 -> 240; f 1536: 53 -> 57, 54 -> 58, 57 -> 62, 70 -> 75
+//   down        d 2048, f 512: 35 -> 41, 35 -> 40, 40 -> 43, 56 -> 58, 94 -> 103; d 1024, f 768: 31 -> 34, 30 -> 33, 33 -> 35, 42 -> 44, 66 -> 67;
+//               f 1536: 30 -> 32, 30 -> 32, 37 -> 33, 41 -> 41, 65 -> 62, 159 -> 154; d 2048, f 1536: 79 -> 78, 78 -> 78, 90 -> 83, 110 -> 103, 222
+//               -> 213, 592 -> 595; d 3072, f 1536: 60 -> 63, 60 -> 64, 74 -> 66, 87 -> 81, 167 -> 155, 441 -> 435
+//   dgrad-down  faster from d 1024, f 512 on (72 -> 74 there at 512, f 4096 412 -> 378 at 2048); at narrower widths a gain where its other form is slow
+//               to start: d 128, f 512 19 -> 13, 19 -> 14, 19 -> 17 at 16, 64, 120; d 768, f 768 23 -> 19, 23 -> 21, 25 -> 26; d 256, f 1024 33 ->
+//               25, 33 -> 30, 44 -> 39 (33 -> 35 at 96); d 64, f 64 13 -> 11, 13 -> 13, 13 -> 15: up to 96 rows
+//   dgrad-g/u   d 1024, f 512: 41 -> 42, 40 -> 44, 46 -> 45, 54 -> 52, 81 -> 77, 210 -> 204; f 768: 55 -> 56, 55 -> 58, 60 -> 58, 72 -> 68; f 1536: 56
+//               -> 54, 56 -> 57, 68 -> 59, 72 -> 70; d 1536, f 1024: 60 -> 55, 60 -> 56, 59 -> 58; d 3072, f 1536: 123 -> 122, 123 -> 126, 150 ->
+//               130, 163 -> 150, 316 -> 285, 882 -> 857; d 4096, f 3072: 156 -> 157, 155 -> 164, 177 -> 170, 235 -> 216, 452 -> 417, 1229 -> 1220
+static bool row_gemm_by_tokens(const moe_ctx_impl* ctx, GemmKind kind, double rows) {
   const int d = ctx->s.d, f = ctx->s.f;
   if (ctx->tile_mode != 0 || (kind == GEMM_B4 && ctx->b4_pair_override >= 0)) return false;
-  if (kind == GEMM_B2 && rows_per_expert < 128.0) return true;
-  if (d < 1024 || f < 512) return false;
+  if (d < 1024 || f < 512) return kind == GEMM_B2 && rows < 96.0;
   switch (kind) {
-    case GEMM_F3: return d >= 2048 && rows_per_expert < (f <= 1536 ? 3072.0 : 1536.0);
-    case GEMM_F4: return rows_per_expert >= 96.0 && rows_per_expert < 640.0;
-    case GEMM_B2: return f <= 3072 || rows_per_expert < 1536.0;
-    case GEMM_B4: return rows_per_expert < (d <= 3072 ? 3072.0 : 640.0);
+    case GEMM_F3:
+      return d >= 2048 && (rows < 48.0 || rows >= 120.0 || (d < 3072 && f >= 768)) && rows < (f <= 1536 ? 3072.0 : 1536.0);
+    case GEMM_F4: return (f >= 1536 || (d >= 2048 && f >= 768)) && rows >= 120.0 && rows < 640.0;
+    case GEMM_B2: return f <= 3072 || rows < 1536.0;
+    case GEMM_B4:
+      return (rows >= 120.0 || (static_cast<int64_t>(d) * f >= 1 << 20 && (rows < 80.0 || d < 3072))) && rows < (d <= 3072 ? 3072.0 : 640.0);
     default: return false;
   }
 }
