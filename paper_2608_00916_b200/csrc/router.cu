@@ -3,12 +3,17 @@
 // accumulation is an fp32 contraction up to summation order.
 //
 // CL CTAs share the 128 tokens of a tile, each contracts and routes 128 / CL of them: W_r^T is the M operand (128 experts, twice
-// above 128 of them), the CTA's tokens are N.  Every logit is one sum over all K blocks in their order, so that a token's logits,
-// and with them its experts, are the same bits whatever the number of tokens of the call selects.  (Splitting the K blocks over
-// the CTAs instead fetches a part of W_r per CTA, not all of it, and took 17 us where this takes 19 up to 1000 tokens; but its sums
-// change with the split, and a token near a tie got other experts in another batch.)  The CTAs of a tile are a cluster only
-// to add up the tile's histogram.  What bounds it: up to some ten thousand tokens the latency of fetching W_r and the tokens
-// through one SM each and of routing, hence the split; from there on the stream of x from HBM, two CTAs to an SM.
+// above 128 of them), the CTA's tokens are N.  The K blocks are summed in four chains (fewer below four K blocks), each in an
+// accumulator of its own, and the chains in their order: the tensor core drops what lies below the last place of an accumulator,
+// so that the error grows with the length of a chain (rms 2.1e-6 with one chain, 0.5e-6 with four at d 2048 and unit-variance
+// logits).
+// The order of the sums depends on d alone, so that a token's logits, and with them its experts, are the same bits whatever the
+// number of tokens of the call selects.  (Splitting the K blocks over the CTAs instead fetches a part of W_r per CTA, not all of
+// it, and took 17 us where this takes 19 up to 1000 tokens; but its sums change with the split, and a token near a tie got other
+// experts in another batch.)  The CTAs of a tile are a cluster only to add up the tile's histogram.  What bounds it: up to some ten
+// thousand tokens the latency of fetching W_r and the tokens through one SM each and of routing, hence the split; from there on the
+// stream of x from HBM.  With one CTA per tile the accumulators fill tensor memory, so that an SM holds one CTA: 42 -> 56 us at
+// 24576 tokens, 49 -> 60 at 32768 against one chain and two CTAs.
 //
 // Three steps between barriers.  (1) A warp per token: bias, softmax and its column sums; a lane holds NV / 4 groups of four
 // columns.  (2) A thread per token: top-k as a three-level tournament, groups of four columns, supers of four groups, the maxima
@@ -35,11 +40,10 @@ constexpr int RO_THREADS = 64 + 32 * RO_WARPS;  // warps: 0 TMA producer, 1 MMA 
 constexpr int RO_BK = 64;
 constexpr int RO_CHUNK_BYTES = 64 * RO_BK * 2;   // 8 KB per 64 columns of W_r and K block
 constexpr int RO_MAX_STAGES = 16;
+constexpr int RO_CHAINS = 4;  // partial sums of a logit
 // Bytes of the operand stages.  Every CTA fetches all of W_r, and waits for latency more than for bandwidth, so the copies in
-// flight count: 100 -> 200 KB at d 2048 and 128 experts 20 -> 19 us at 128 tokens, 26 -> 23 at 8192, 35 -> 31 at 16384.  But 200 KB
-// take an SM, so they are for launches whose CTAs have one each; more of them share one (49 us at 20000 tokens with 200 KB, 41 at
-// 24576 with 100).  Above 128 experts an SM holds one CTA anyway.
-constexpr int RO_RING = 100 * 1024, RO_DEEP_RING = 200 * 1024;
+// flight count: 100 -> 200 KB at d 2048 and 128 experts 20 -> 19 us at 128 tokens, 26 -> 23 at 8192, 35 -> 31 at 16384 (one chain).
+constexpr int RO_RING = 200 * 1024;
 static_assert(RO_TOK == TOK_TILE, "the histogram written here is the permutation's");
 
 struct RouterParams {
@@ -56,7 +60,7 @@ struct RouterParams {
   int32_t* tile_counts;  // [tiles, E] picks of every 128-token tile
   int64_t T;
   int E, k;
-  int k_blocks, k_total;  // K blocks of one bf16 term of W_r, and of all terms
+  int k_blocks, k_total, chains;  // K blocks of one bf16 term of W_r, and of all terms; chains they are summed in
   int w_chunks, whole_chunks;  // 64-column chunks of W_r; E is a multiple of 64, so they are one copy
   int stages;
   uint32_t w_bytes, stage_bytes;  // of a stage: W_r, and with the tokens
@@ -166,10 +170,10 @@ __device__ __forceinline__ float select_topk(int k, uint32_t row, uint32_t maxim
 __device__ __forceinline__ void routing_sync() { asm volatile("bar.sync 1, %0;" ::"n"(32 * RO_WARPS) : "memory"); }
 
 template <int CL, int NV>
-__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, NV == 4 ? 2 : 1)
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, 1)
     router_cluster_kernel(const __grid_constant__ RouterParams p) {
   constexpr int MINE = RO_TOK / CL;             // this CTA's tokens of the tile
-  constexpr uint32_t ACCS = NV / 4, TMEM_COLS = ACCS * MINE;  // an accumulator for each 128 experts, a column per token
+  constexpr uint32_t ACCS = NV / 4, TMEM_COLS = RO_CHAINS * ACCS * MINE;  // per chain an accumulator for each 128 experts, a column per token
   extern __shared__ unsigned char ro_smem_raw[];
   __shared__ __align__(8) uint64_t bars[2 * RO_MAX_STAGES + 1];  // full, empty, accumulator complete
   __shared__ uint32_t tmem_base_slot;
@@ -257,7 +261,13 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, NV == 4
       int s = 0;
       uint32_t phase = 0;
       bool ok = true;
+      int chain = 0, first_kb = 0, next_kb = p.k_total / p.chains;  // chain c: K blocks c k_total / chains and on
       for (int kb = 0; kb < k_blocks; ++kb) {
+        if (kb == next_kb) {
+          ++chain;
+          first_kb = kb;
+          next_kb = p.k_total * (chain + 1) / p.chains;
+        }
         if (!mbar_wait(full_bar(s), phase)) {
           ok = false;
           break;
@@ -268,8 +278,8 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, NV == 4
         for (int ks = 0; ks < RO_BK / 16; ++ks)
 #pragma unroll
           for (uint32_t h = 0; h < ACCS; ++h)
-            umma_bf16(tmem_base + h * MINE, descW + off + ((h * 2 * RO_CHUNK_BYTES + ks * 2048) >> 4), descX + off + (ks * 32 >> 4), idesc,
-                      (kb | ks) != 0 ? 1u : 0u);
+            umma_bf16(tmem_base + (chain * ACCS + h) * MINE, descW + off + ((h * 2 * RO_CHUNK_BYTES + ks * 2048) >> 4), descX + off + (ks * 32 >> 4), idesc,
+                      kb != first_kb || ks != 0 ? 1u : 0u);
         umma_commit(empty_bar(s));
         if (++s == p.stages) {
           s = 0;
@@ -384,12 +394,22 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, NV == 4
 #pragma unroll 1
         for (int c = w >> 2; c < static_cast<int>(ACCS) * (MINE / 16); c += RO_WARPS / 4) {
           const int e = c / (MINE / 16) * 128 + ew * 32 + lane, tok0 = c % (MINE / 16) * 16;
-          uint32_t r[16];
-          tmem_ld16(tmem_base + (static_cast<uint32_t>(ew * 32) << 16) + c * 16, r);
+          uint32_t r[RO_CHAINS][16];
+#pragma unroll
+          for (int q = 0; q < RO_CHAINS; ++q)
+            if (q < p.chains) tmem_ld16(tmem_base + (static_cast<uint32_t>(ew * 32) << 16) + q * (ACCS * MINE) + c * 16, r[q]);
           tmem_ld_wait();
+          float sum[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) sum[i] = __uint_as_float(r[0][i]);
+#pragma unroll
+          for (int q = 1; q < RO_CHAINS; ++q)
+            if (q < p.chains)
+#pragma unroll
+              for (int i = 0; i < 16; ++i) sum[i] += __uint_as_float(r[q][i]);
           if (e < E)
 #pragma unroll
-            for (int i = 0; i < 16; ++i) asm volatile("st.shared.b32 [%0], %1;" ::"r"(part + (tok0 + i) * PITCH + e * 4), "r"(r[i]) : "memory");
+            for (int i = 0; i < 16; ++i) asm volatile("st.shared.f32 [%0], %1;" ::"r"(part + (tok0 + i) * PITCH + e * 4), "f"(sum[i]) : "memory");
         }
       tc_fence_before();
       routing_sync();
@@ -424,37 +444,35 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, NV == 4
   }
 }
 
-// CTAs per token tile: as many as have an SM each.  Clusters of four do not fill the chip (they lie within a part of it), so
-// they go up to eight ninths of the SMs.  Router stage, us, with one / two / four at d 2048 and 128 experts: 128 tokens 25 / 21 / 19,
-// 4096 (128 CTAs of four) 25 / 21 / 20, 4736 (148) 25 / 22 / 24 or more, 8192 26 / 23 / 25, 9472 (148 CTAs of two) 27 / 24 / 37, 12000
-// 29 / 31 / 39, 16384 31 / 34 / 45, 18944 33 / 35 / 55, 32768 47 / 58 / 80; with 256 experts 33 / 27 / 23 at 128, 31 / 27 / 24 at 4096, 34 /
-// 29 / 58 at 9472, 35 / 49 / 60 at 12000.  Rows of W_r of less than 64 bytes come slowly however few they are, and all CTAs ask for the
-// same lines, so that with few experts fewer CTAs are better sooner: d 4096 and 8 experts 29 / 27 / 25 at 128 tokens, 29 / 27 / 27 at
-// 2048, 30 / 31 / 37 at 4096, 37 / 39 / 57 at 8192; d 256 and 8 experts 16 / 14 / 14 at 2048, 17 / 16 / 17 at 4096.
+// CTAs per token tile: as many as have an SM each, and more than one wave of them only where there is no choice.  Clusters of four
+// do not fill the chip (they lie within a part of it), so they go up to eight ninths of the SMs.  Router stage, us, with one / two /
+// four at d 2048 and 128 experts: 128 tokens 25 / 23 / 20, 4096 (128 CTAs of four) 26 / 24 / 21, 4737 (152) 26 / 24 / 35, 8192 27 / 25 / 35,
+// 9472 (148 CTAs of two) 29 / 26 / 49, 9473 29 / 39 / 49, 16384 33 / 45 / 65, 32768 59 / 85 / 129.  Above 128 experts one CTA's accumulators
+// do not fit: 256 experts, two / four: 28 / 25 at 128 tokens, 29 / 25 at 4096, 29 / 43 at 4737, 54 / 82 at 16384.  With few experts the rows
+// of W_r are short and come slowly however few they are, and all CTAs ask for the same lines, so that two are worse than one: d 4096
+// and 8 experts 32 / 33 at 4737, 37 / 43 at 8192, 39 / 46 at 9472; d 256 and 8 experts 19 / 18 at 4737, 20 / 20 at 8192.
 // One CTA per tile in the persistent GEMM template, four warps routing: 27 at 128 to 4096 tokens, 28 at 8192, 32 at 16384, 54 at 32768.
 int router_cluster(const Shape& s, int sm_count, int64_t T) {
   const int64_t tiles = (T + RO_TOK - 1) / RO_TOK;
-  if (s.E < 32 && tiles > 16) return 1;
-  return tiles * 4 * 9 <= sm_count * 8 ? 4 : tiles * 2 <= sm_count ? 2 : 1;
+  if (tiles * 4 * 9 <= sm_count * 8) return 4;
+  return s.E <= 128 && (s.E < 32 || tiles * 2 > sm_count) ? 1 : 2;
 }
 
 template <int CL, int NV>
 static moe_status launch_one(moe_ctx_impl* ctx, RouterParams& p, int tiles, cudaStream_t st) {
   auto* const kernel = router_cluster_kernel<CL, NV>;
   // the stages (and what an MMA reads behind an odd number of chunks), and over them what the routing needs: the logits of the
-  // CTA's tokens, the maxima of their groups, and {pick, column} and 1 / sum for k picks (with one CTA per tile and more than 20
-  // picks that leaves no room for two CTAs on an SM)
+  // CTA's tokens, the maxima of their groups, and {pick, column} and 1 / sum for k picks
   constexpr size_t mine = RO_TOK / CL;
   auto routing = [](int k) { return mine * (128 * NV + 16) + mine * (32 * NV + 16) + k * (mine * 8 + 8) + mine * 4; };
   auto smem_of = [](size_t ring, size_t over) { return (ring > over ? ring : over) + 1024; };
   p.w_bytes = p.w_chunks * RO_CHUNK_BYTES;
   p.stage_bytes = p.w_bytes + mine * RO_BK * 2;
-  const uint32_t room = NV > 4 || tiles * CL <= ctx->sm_count ? RO_DEEP_RING : RO_RING;
-  p.stages = std::min<int>(room / p.stage_bytes, RO_MAX_STAGES);
+  p.stages = std::min<int>(RO_RING / p.stage_bytes, RO_MAX_STAGES);
   const size_t smem = smem_of(p.stages * p.stage_bytes + (p.w_chunks & 1) * RO_CHUNK_BYTES, routing(p.k));
   constexpr int slot = (CL == 1 ? 0 : CL == 2 ? 1 : 2) + (NV == 4 ? 0 : 4);
   if (!(ctx->router_attr & (1u << slot))) {  // per device (the context is bound to one), and for every context on it: the most of all
-    const size_t most = smem_of(RO_DEEP_RING + RO_CHUNK_BYTES, routing(MAX_K));
+    const size_t most = smem_of(RO_RING + RO_CHUNK_BYTES, routing(MAX_K));
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most)) != cudaSuccess)
       return MOE_ERR_CUDA;
     ctx->router_attr |= 1u << slot;
@@ -482,6 +500,7 @@ moe_status launch_router_tc(moe_ctx_impl* ctx, int64_t T, const WsLayout& L, cha
   if (!ok) return MOE_ERR_CUDA;
   p.k_blocks = s.d / RO_BK;
   p.k_total = p.k_blocks * (io.W_r_mid ? 3 : 1);
+  p.chains = p.k_total >= RO_CHAINS ? RO_CHAINS : p.k_total >= 2 ? 2 : 1;
   p.status = reinterpret_cast<int32_t*>(ws + L.status);
   p.row_gate = reinterpret_cast<float*>(ws + L.row_gate);
   p.rows = L.rows_alloc;
@@ -502,11 +521,7 @@ moe_status launch_router_tc(moe_ctx_impl* ctx, int64_t T, const WsLayout& L, cha
       default: return launch_one<1, 4>(ctx, p, tiles, st);
     }
   }
-  switch (cl) {
-    case 4: return launch_one<4, 8>(ctx, p, tiles, st);
-    case 2: return launch_one<2, 8>(ctx, p, tiles, st);
-    default: return launch_one<1, 8>(ctx, p, tiles, st);
-  }
+  return cl == 4 ? launch_one<4, 8>(ctx, p, tiles, st) : launch_one<2, 8>(ctx, p, tiles, st);
 }
 
 }  // namespace moe
