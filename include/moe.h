@@ -30,6 +30,8 @@
  *   - Errors are return codes.  Argument errors are found before anything is launched.  A device-side
  *     problem (a bounded wait that ran out) sets a status word inside the workspace; the kernels leave
  *     cleanly and moe_poll_status reports it.
+ *   - A token's logits, topk_idx, topk_w and y do not depend on the other tokens of the call or on their number: they are the
+ *     same bits alone and in any batch.
  *   - Inputs must be finite.  One moe_ctx serves one stream at a time.
  */
 #ifndef MOE_B200_H

@@ -12,7 +12,9 @@ pytestmark = pytest.mark.gpu
     (512, 128, 8, 64, 20000, 0),                # 32, 64 and 128 tokens of a tile to a CTA of the router
     (320, 136, 4, 64, 20000, 0),                # two lanes' columns: an accumulator for each 128 experts
     (128, 24, 2, 64, 20000, FLAG_ROUTER_FP32),  # the three terms of an fp32 router weight
+    (192, 12, 3, 64, 9000, 0),                  # the router for expert counts that are not a multiple of 8
     (2048, 128, 8, 512, 9000, 0),               # row GEMMs on tokens, on pairs and on one-CTA tiles
+    (1024, 32, 4, 1536, 9000, 0),               # the down GEMM as well
 ])
 def test_a_token_alone_and_in_a_batch(d, E, k, f, T, flags):
     g = torch.Generator(device="cuda")
