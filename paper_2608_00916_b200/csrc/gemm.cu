@@ -521,14 +521,17 @@ static double expected_tiles(double mean, double size) {
 // The dgrad-down GEMM is held by its epilogue (it reads hg and hu) rather than by the feed and gains less: 112 -> 125 at 62
 // rows, 127 -> 136 at 128, 166 -> 167 at 256, 181 -> 204 at 300, 248 -> 247 at 512, 333 -> 336 at 768, 418 -> 415 at 1024, 615 ->
 // 591 at 1536, 811 -> 788 at 2048; wide experts 301 -> 313 at 256, 510 -> 473 at 512, 702 -> 705 at 768, 881 -> 843 at 1024,
-// 3681 -> 3227 at 4096: pairs from 768 rows on, where the two are equal.
+// 3681 -> 3227 at 4096: pairs from 768 rows on, where the two are equal (reached by widths below d 1024 or f 512 and by wide experts
+// only: the rest take the tokens as N, see below).
 // Half-empty pairs are better than complete pairs plus the leftover blocks in a second, one-CTA launch
 // (MOE_FLAG_HYBRID_TILES: 4.22 ms a step against 4.17 at 1024 rows per expert).
 // Weight gradients pair along the weight dimension without leftovers, but their K loop is the expert's row count, and
 // with few K blocks the output leaves as fast as HBM takes it (tile-shaped stores reach 6 TB/s here) only from one-CTA
-// tiles, whose two CTAs do not have to meet: wgrad-down / wgrad-gate/up 162 -> 172 / 322 -> 330 at 312 rows, equal at
-// 375, 200 -> 187 / 399 -> 374 at 437, 222 -> 195 / 430 -> 392 at 512.  When they accumulate in fp32 the line lies higher
-// (see Accumulate).
+// tiles, whose two CTAs do not have to meet.  One-CTA -> pairs, us, wgrad-down / gate/up at d 2048, f 768, 128 experts: 89 / 167 ->
+// 104 / 196 at 62 rows, 132 / 257 -> 139 / 272 at 256, 146 / 293 -> 147 / 302 at 312, 163 / 332 -> 158 / 323 at 375, 181 / 377 -> 171 /
+// 352 at 437, 202 / 419 -> 186 / 384 at 512, 342 / 691 -> 289 / 621 at 1024; d 1024, f 768, 64 experts 47 / 76 -> 47 / 78 at 312, 51 / 85 ->
+// 51 / 82 at 375; d 4096, f 14336, 8 experts 265 / 569 -> 273 / 604 at 256, 294 / 661 -> 296 / 644 at 312, 339 / 780 -> 327 / 715 at 375.
+// The line stands at 384.  When they accumulate in fp32 it lies higher (see Accumulate).
 static bool row_gemm_on_pairs(const moe_ctx_impl* ctx, GemmKind kind, double rows_per_expert) {
   if (ctx->tile_mode != 0) return ctx->tile_mode == 1;
   if (kind == GEMM_B4 && ctx->b4_pair_override >= 0) return ctx->b4_pair_override != 0;
