@@ -293,10 +293,25 @@ static moe_status launch_kind(moe_ctx_impl* ctx, const GemmParams& p, cudaStream
 
 // Row tiles (or pairs) walked together inside a column tile: 1 while the expert's weights are few column tiles wide (they
 // stay in L2 between row tiles: Qwen3-30B-A3B shape), 16 for wide experts (coarse shape: at 112 column tiles an expert's
-// gate and up slabs are 235 MB and were read from DRAM once per row pair).  MOE_ROW_GROUP overrides (measurements).
+// gate and up slabs are 235 MB and were read from DRAM once per row pair).  A group ends with its expert (expert_tile_order): a
+// step at that shape then reads 1.9 GB less for gate/up, 4 GB less for dgrad gate/up and takes, with 512 / 1024 / 4096 rows per
+// expert and the weight gradients in groups as well, 4640 -> 4275, 8130 -> 7590 and 31200 -> 28600 us (at the power cap, where a
+// byte from DRAM costs what 110 flops do).  MOE_ROW_GROUP overrides (measurements).
 int row_group_for(int n_tiles, const moe_ctx_impl* ctx) {
   if (ctx->row_group_override > 0) return ctx->row_group_override;
   return n_tiles > 12 ? 16 : 1;
+}
+
+// The same for a weight gradient on CTA pairs: 256-row tiles of the output walked together inside a column tile.  With column
+// tiles fastest every row tile reads the operand of the columns (`columns` wide, the expert's rows long) from DRAM again once
+// that operand has outgrown L2; walked in groups, row and column operands are shared by the pairs that run at the same time.
+// wgrad gate/up at d 4096, f 14336, 4096 rows per expert: 25.9 -> 6.6 GB read, 6013 -> 5110 us; at 1024 rows (59 MB) 2.34 -> 0.56 GB,
+// 1426 -> 1285 us, a step 6414 -> 6275 at 768 rows, 4616 -> 4547 at 512 (29 MB).  With 15 MB (256 rows, one-CTA tiles) nothing is read
+// twice either way and rows of adjacent columns leave together: 662 -> 704 us in groups.  Hence above 24 MB, and where there are more
+// column tiles than a group has rows.
+static int wgrad_group_for(int n_tiles, double rows_per_expert, int64_t columns, const moe_ctx_impl* ctx) {
+  if (ctx->row_group_override > 0) return ctx->row_group_override;
+  return n_tiles > 16 && rows_per_expert * static_cast<double>(columns) * 2.0 >= 24e6 ? 16 : 1;
 }
 
 // Forward-only calls leave pad rows alone (nothing reads them afterwards), which at few rows per expert is most of what
@@ -425,6 +440,7 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
       p.out0 = dW_down;
       p.accf0 = io.dW_down_acc;
       p.acc_fp32 = io.dW_down_acc != nullptr;
+      p.row_group = wgrad_group_for(p.n_tiles, rows_per_expert, d, ctx);
       p.ld_out = d;
       p.expert_stride = static_cast<int64_t>(f) * d;
       if (!ok) return MOE_ERR_CUDA;
@@ -442,6 +458,7 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
       p.out0 = dW_gate; p.out1 = dW_up;
       p.accf0 = io.dW_gate_acc; p.accf1 = io.dW_up_acc;
       p.acc_fp32 = io.dW_gate_acc != nullptr;
+      p.row_group = wgrad_group_for(p.n_tiles, rows_per_expert, 2 * f, ctx);
       p.ld_out = f;
       p.expert_stride = static_cast<int64_t>(d) * f;
       if (!ok) return MOE_ERR_CUDA;

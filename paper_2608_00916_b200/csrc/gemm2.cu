@@ -51,8 +51,10 @@ __device__ __forceinline__ Tile2 get_tile2(const GemmParams& p, int t, int rank)
     const int slot = t / per;
     tl.e = p.expert_grouped ? p.e_first + slot : p.expert_order[slot];  // else: longest K loops first
     const int rem = t - slot * per;
-    tl.m0 = (rem / p.n_tiles) * 2 * BM + rank * BM;
-    tl.n0 = (rem % p.n_tiles) * Traits<KIND>::N_SPAN;
+    int mt, nt;
+    row_tile_order(rem, p.n_tiles, p.row_group, p.m_tiles, mt, nt);
+    tl.m0 = mt * 2 * BM + rank * BM;
+    tl.n0 = nt * Traits<KIND>::N_SPAN;
     tl.row0 = p.pad_offsets[tl.e];
     tl.nkb = (p.counts[tl.e] + BK - 1) / BK;  // the rest of the 128-row padding is zeros
     tl.klast = last_k_steps(p.counts[tl.e]);
@@ -61,7 +63,14 @@ __device__ __forceinline__ Tile2 get_tile2(const GemmParams& p, int t, int rank)
     tl.full = true;
   } else {
     int pr, nt;
-    row_tile_order(t, p.n_tiles, p.row_group, p.sched[p.pair_count_slot], pr, nt);
+    if (p.row_group > 1 && p.pair_count_slot == 2) {
+      const int q = t / p.n_tiles;
+      const int4 at = *reinterpret_cast<const int4*>(p.pair_tab + 4 * q);
+      const int row0 = p.pad_offsets[at.x], rows = p.pad_offsets[at.x + 1] - row0;
+      expert_tile_order(t, p.n_tiles, p.row_group, q - (at.y - row0) / (2 * BM), (rows + 2 * BM - 1) / (2 * BM), pr, nt);
+    } else {
+      row_tile_order(t, p.n_tiles, p.row_group, p.sched[p.pair_count_slot], pr, nt);
+    }
     const int4 info = *reinterpret_cast<const int4*>(p.pair_tab + 4 * pr);  // expert, first row, blocks (1 or 2)
     tl.e = info.x;
     tl.row0 = info.y + rank * BM;

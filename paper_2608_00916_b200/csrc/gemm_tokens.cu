@@ -88,7 +88,14 @@ __device__ __forceinline__ int token_tiles(const TokenGemmParams& p) { return p.
 __device__ __forceinline__ TokenTile get_token_tile(const TokenGemmParams& p, int t) {
   TokenTile tl;
   int ri, b, first;
-  row_tile_order(t, p.n_tiles, p.row_group, p.sched[p.small ? 0 : 2], ri, tl.nt);
+  if (p.row_group > 1) {
+    const int q = t / p.n_tiles, e = p.small ? p.tile_expert[q] : p.pair_tab[4 * q], most = p.small ? BM : 2 * BM;
+    first = p.pad_offsets[e];
+    b = p.small ? q - first / BM : (p.pair_tab[4 * q + 1] - first) / most;
+    expert_tile_order(t, p.n_tiles, p.row_group, q - b, (p.pad_offsets[e + 1] - first + most - 1) / most, ri, tl.nt);
+  } else {
+    row_tile_order(t, p.n_tiles, p.row_group, p.sched[p.small ? 0 : 2], ri, tl.nt);
+  }
   if (p.small) {
     tl.e = p.tile_expert[ri];
     first = p.pad_offsets[tl.e];

@@ -1,0 +1,41 @@
+"""The order in which the tiles of the expert GEMMs are walked: every tile once, whatever the loads and the group size."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2608_00916_b200 import synth
+from paper_2608_00916_b200.binding import MoELayer
+from gpu_util import Run, oracle_run
+from test_gpu_parity import check_all
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("flags", [0, 1, 2])  # the default rule, CTA pairs, one-CTA tiles
+@pytest.mark.parametrize("T,d,E,k,f", [(900, 1088, 8, 2, 640), (1500, 320, 5, 2, 704), (2600, 576, 2, 1, 320)])
+def test_group_size_changes_no_bit(T, d, E, k, f, flags, monkeypatch):
+    """Experts with no rows, a few and up to 21 row tiles; groups that do not divide them, ragged last tiles in both directions."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(T)
+    n = lambda *s: torch.empty(*s, device="cuda").normal_(0, 0.05, generator=g).bfloat16()
+    x, W, dy = n(T, d), (n(d, E), n(E, d, f), n(E, d, f), n(E, f, d)), n(T, d)
+    b_r = torch.linspace(-2.0, 2.0, E, device="cuda")
+
+    def step():
+        layer = MoELayer(d, E, f, k, flags)
+        out = layer.forward(x, *W, b_r=b_r)
+        grads = layer.backward(dy, 0.01)
+        layer.poll()
+        return [out["y"]] + [grads[m] for m in ("dx", "dW_gate", "dW_up", "dW_down")]
+
+    plain = step()
+    for group in ("2", "3", "7", "40"):
+        monkeypatch.setenv("MOE_ROW_GROUP", group)
+        assert all(torch.equal(a, b) for a, b in zip(step(), plain)), group
+
+
+def test_weight_gradient_of_a_wide_expert():
+    """2800 rows, 17 column tiles: by its own rule gate/up walks the three row tiles (the last one short) inside a column tile."""
+    inp = synth.make_inputs(synth.MoEShape(22400, 576, 8, 1, 2176), 31, x_std=1.0)
+    ofw, obw = oracle_run(inp, 1, 0.05, dtype=np.float32)
+    check_all(Run(inp, 1), ofw, obw, 0.05, stages=False)
