@@ -70,9 +70,7 @@ typedef struct {
 /* Row GEMMs run every complete pair of 128-row blocks of an expert on a CTA pair and the leftover block of an odd
  * count on a one-CTA tile (two launches, no half-empty pairs); weight gradients run on pairs. */
 #define MOE_FLAG_HYBRID_TILES 16
-/* moe_backward normally runs the router's gradient chain (dl, dW_r, db_r, the router term of dx) on a second stream of
- * the context, forked and joined inside the call (the caller's stream sees one ordered call; the pattern is legal
- * inside a stream capture).  This flag keeps everything on the caller's stream. */
+/* Accepted and without effect: every call uses the caller's stream only. */
 #define MOE_FLAG_NO_SIDE_STREAM 8
 /* The router weight W_r is passed as fp32 [d,E] instead of bf16 (moe_forward / moe_backward only; E must be a multiple
  * of 8).  Every fp32 value is the exact sum of three bf16 values, so the logits are still an fp32 contraction of exact
@@ -147,8 +145,8 @@ MOE_API moe_status moe_selftest_timeout(moe_ctx* ctx, void* workspace, void* cud
  * Stage order: 0 router, 1 permute (histogram, scan, scatter, gather), 2 gate/up GEMM + SwiGLU,
  * 3 down GEMM, 4 combine, 5 combine-bwd (gather of dy rows), 6 dgrad-down + SwiGLU-bwd (+ dg), 7 wgrad-down, 8 dgrad gate/up,
  * 9 wgrad gate/up, 10 router-bwd (dl), 11 dW_r, 12 unpermute-bwd (dx), 13 router term of dx, 14..15 unused.
- * Stages 10, 11 and 13 run on the context's second stream beside stages 7..9 (unless MOE_FLAG_NO_SIDE_STREAM), so the
- * stage times then add up to more than the step. */
+ * The events keep the kernels of a call apart; without them stages 10 and 12 run beside stages 7 and 9 and each GEMM begins
+ * while the one before it drains, so the stage times add up to more than the step. */
 #define MOE_PROF_RING 64
 MOE_API moe_status moe_set_profiling(moe_ctx* ctx, int enable);
 MOE_API moe_status moe_stage_times(moe_ctx* ctx, float* ms /* host */, int32_t* steps /* host */);

@@ -100,14 +100,6 @@ moe_status ensure_device(moe_ctx_impl* c) {
   c->gemm_timers = getenv("MOE_GEMM_TIMERS") != nullptr;
   c->row_group_override = getenv("MOE_ROW_GROUP") ? atoi(getenv("MOE_ROW_GROUP")) : 0;
   c->b4_pair_override = getenv("MOE_B4_PAIR") ? atoi(getenv("MOE_B4_PAIR")) : -1;
-  if (c->use_side_stream) {
-    if (cudaStreamCreateWithFlags(&c->s_side, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&c->ev_b4, cudaEventDisableTiming) != cudaSuccess)
-      return MOE_ERR_CUDA;
-    c->side_created = 1;
-  }
   memset(c->attr_done, 0, sizeof(c->attr_done));
   return MOE_OK;
 }
@@ -155,7 +147,6 @@ moe_status moe_create(const moe_config* cfg, moe_ctx** out) {
   memset(c, 0, sizeof(*c));
   c->s = Shape{cfg->d, cfg->E, cfg->f, cfg->top_k};
   c->device = -1;  // bound by the first call that launches work
-  c->use_side_stream = (cfg->flags & MOE_FLAG_NO_SIDE_STREAM) ? 0 : 1;
   c->router_fp32 = (cfg->flags & MOE_FLAG_ROUTER_FP32) ? 1 : 0;
   c->debug_checks = (cfg->flags & MOE_FLAG_DEBUG_CHECKS) ? 1 : 0;
   c->tile_mode = (cfg->flags & MOE_FLAG_CTA_PAIR_TILES) ? 1
@@ -175,12 +166,6 @@ void moe_destroy(moe_ctx* ctx) {
         cudaEventDestroy(c->ev[r][i][1]);
       }
   if (c->own) moe_destroy(reinterpret_cast<moe_ctx*>(c->own));
-  if (c->side_created) {
-    cudaStreamDestroy(c->s_side);
-    cudaEventDestroy(c->ev_fork);
-    cudaEventDestroy(c->ev_join);
-    cudaEventDestroy(c->ev_b4);
-  }
   if (c->e2e_created) {
     cudaStreamDestroy(c->s_in);
     cudaStreamDestroy(c->s_out);
@@ -412,6 +397,7 @@ static moe_status forward_impl(bool training, moe_ctx* ctx, int64_t T, const uin
   if (T > 0) {
     {
       StageTimer tm(c, st, 2);
+      io.next_early = true;
       if (lora) {
         rc = launch_lora_gemm(c, LORA_U, T, L, ws, io, *lora, st);
         if (rc == MOE_OK) rc = launch_lora_gemm(c, LORA_F3, T, L, ws, io, *lora, st);
@@ -424,8 +410,10 @@ static moe_status forward_impl(bool training, moe_ctx* ctx, int64_t T, const uin
       StageTimer tm(c, st, 3);
       if (lora) {
         rc = launch_lora_gemm(c, LORA_V, T, L, ws, io, *lora, st);
+        io.next_early = false;
         if (rc == MOE_OK) rc = launch_lora_gemm(c, LORA_F4, T, L, ws, io, *lora, st);
       } else {
+        io.next_early = false;  // the combine only waits
         rc = launch_grouped_gemm(c, GEMM_F4, T, L, ws, io, st);
       }
     }
@@ -517,86 +505,73 @@ static moe_status backward_impl(moe_ctx* ctx, int64_t T, const uint16_t* dy, flo
     StageTimer tm(c, st, 5);
     launch_gather_rows(s, T, L, ws, dy, reinterpret_cast<uint16_t*>(ws + L.o), st, c->debug_checks != 0);
   }
-  // The router's gradient chain (dl, dW_r, db_r and the router term of dx) needs only the dg partials that the
-  // dgrad-down GEMM leaves behind.  It is small and latency-bound, so it runs on a second stream of the context, forked
-  // after that GEMM and joined before the final unpermute, where it fills the tails of the three big GEMMs instead of
-  // standing in line behind them.  Without tokens, or with MOE_FLAG_NO_SIDE_STREAM, it runs in line.
-  bool forked = false;
+  // One chain of kernels.  The small ones run beside the GEMM in front of them, whose blocks leave them registers enough: dl
+  // (which needs the dgrad-down GEMM) beside the weight gradient of down, dx (dgrad gate/up and dl) beside that of gate and up.
+  // The two GEMMs over dl come in as the blocks of dgrad gate/up leave.
+  int32_t* const dbg = c->debug_checks ? reinterpret_cast<int32_t*>(ws + L.status) : nullptr;
+  const uint16_t* const dxp = reinterpret_cast<const uint16_t*>(ws + L.dxp);
   const bool one_slice = dwr_in_one_slice(T, dW_r);
-  auto router_chain = [&]() -> moe_status {
-    cudaStream_t rs = st;
-    if (T > 0 && c->use_side_stream) {
-      if (cudaEventRecord(c->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(c->s_side, c->ev_fork, 0) != cudaSuccess)
-        return MOE_ERR_CUDA;
-      rs = c->s_side;
-      chain.waits(rs);
-      forked = true;
-    }
+  auto router_gradient = [&]() {
+    StageTimer tm(c, st, 10);
+    launch_router_bwd(s, T, reinterpret_cast<const float*>(ws + L.logits), reinterpret_cast<const int32_t*>(ws + L.idx),
+                      gates, reinterpret_cast<const float*>(ws + L.dg_part), 2 * ((s.f + 255) / 256), L.rows_max, inv,
+                      reinterpret_cast<float*>(ws + L.dg), reinterpret_cast<const int32_t*>(ws + L.counts), d_aux, dl,
+                      reinterpret_cast<uint16_t*>(ws + L.dl_hi), reinterpret_cast<uint16_t*>(ws + L.dl_lo), st, dbg, /*ready=*/true);
+  };
+  // the router term of dx, and dW_r in slices of the tokens
+  auto router_gemms = [&]() -> moe_status {
+    if (!tc_router || T == 0) return MOE_OK;
+    GemmIO rio = io;
+    rio.ready = true;
     {
-      StageTimer tm(c, rs, 10);
-      launch_router_bwd(s, T, reinterpret_cast<const float*>(ws + L.logits), reinterpret_cast<const int32_t*>(ws + L.idx),
-                        gates, reinterpret_cast<const float*>(ws + L.dg_part), 2 * ((s.f + 255) / 256), L.rows_max, inv,
-                        reinterpret_cast<float*>(ws + L.dg), reinterpret_cast<const int32_t*>(ws + L.counts), d_aux, dl,
-                        reinterpret_cast<uint16_t*>(ws + L.dl_hi), reinterpret_cast<uint16_t*>(ws + L.dl_lo), rs,
-                        c->debug_checks ? reinterpret_cast<int32_t*>(ws + L.status) : nullptr);
-    }
-    {
-      StageTimer tm(c, rs, 11);
-      if (tc_router && T > 0) {
-        if (one_slice) {
-          io.dW_r = dW_r;
-          io.dW_r_accumulate = accumulate;
-        }
-        const moe_status r2 = launch_grouped_gemm(c, GEMM_DWR, T, L, ws, io, rs);
-        if (r2 != MOE_OK) return r2;
-      }
-      launch_dwr(s, T, x, dl, reinterpret_cast<float*>(ws + L.dwr_part), dW_r, db_r, tc_router && T > 0, rs, accumulate,
-                 tc_router && one_slice);
-    }
-    if (tc_router && T > 0) {
-      StageTimer tm(c, rs, 13);
-      const moe_status r2 = launch_grouped_gemm(c, GEMM_DX, T, L, ws, io, rs);
+      StageTimer tm(c, st, 13);
+      const moe_status r2 = launch_grouped_gemm(c, GEMM_DX, T, L, ws, rio, st);
       if (r2 != MOE_OK) return r2;
     }
-    return MOE_OK;
-  };
-  // dx = router term + sum of the dxp rows needs the dgrad gate/up GEMM (dxp) and the router chain (dxr), but not the
-  // last weight-gradient GEMM: with the second stream it runs beside that GEMM (it is bandwidth-bound, fits on the SMs
-  // next to the GEMM's CTAs and uses the DRAM bandwidth the GEMM leaves idle); the call joins the two streams at its end.
-  auto finish_dx = [&](bool after_last_gemm) -> moe_status {
-    if (forked == after_last_gemm) return MOE_OK;  // forked: right after the dgrad GEMM; in line: at the very end
-    cudaStream_t xs = st;
-    if (forked) {
-      if (cudaEventRecord(c->ev_b4, st) != cudaSuccess || cudaStreamWaitEvent(c->s_side, c->ev_b4, 0) != cudaSuccess)
-        return MOE_ERR_CUDA;
-      xs = c->s_side;
-      chain.waits(xs);
+    StageTimer tm(c, st, 11);
+    if (one_slice) {
+      rio.dW_r = dW_r;
+      rio.dW_r_accumulate = accumulate;
     }
-    {
-      StageTimer tm(c, xs, 12);
-      if (tc_router && T > 0) {
-        launch_unpermute_sum(s, T, reinterpret_cast<const uint16_t*>(ws + L.dxp), inv,
-                             reinterpret_cast<const uint16_t*>(ws + L.dxr), dx, xs,
-                             c->debug_checks ? reinterpret_cast<int32_t*>(ws + L.status) : nullptr, L.rows_max);
-      } else {
-        launch_unpermute_bwd(s, T, reinterpret_cast<const uint16_t*>(ws + L.dxp), inv, dl, W_r, dx, xs);
-      }
-    }
-    if (forked && cudaEventRecord(c->ev_join, c->s_side) != cudaSuccess) return MOE_ERR_CUDA;
-    return MOE_OK;
+    return launch_grouped_gemm(c, GEMM_DWR, T, L, ws, rio, st);
   };
+  auto finish_dx = [&]() {
+    StageTimer tm(c, st, 12);
+    if (tc_router && T > 0) {
+      launch_unpermute_sum(s, T, dxp, inv, reinterpret_cast<const uint16_t*>(ws + L.dxr), dx, st, dbg, L.rows_max, /*ready=*/true);
+    } else {
+      launch_unpermute_bwd(s, T, dxp, inv, dl, W_r, dx, st);
+    }
+  };
+  io.next_early = true;
   if (lora) {
     // base weights frozen: no dW_gate / dW_up / dW_down; the adapter gradients come from skinny GEMMs
-    const LoraOp seq[4][2] = {{LORA_W, LORA_B2}, {LORA_DB2, LORA_DA2}, {LORA_Z, LORA_B4}, {LORA_DB1, LORA_DA1}};
-    for (int g = 0; g < 4 && rc == MOE_OK; ++g) {
-      const bool row_ops = (g == 0 || g == 2);  // row GEMMs have no tiles without tokens; weight gradients zero-fill
-      if (!(row_ops && T == 0)) {
-        StageTimer tm(c, st, 6 + g);
-        rc = launch_lora_gemm(c, seq[g][0], T, L, ws, io, *lora, st);
-        if (rc == MOE_OK) rc = launch_lora_gemm(c, seq[g][1], T, L, ws, io, *lora, st);
-      }
-      if (g == 0 && rc == MOE_OK) rc = router_chain();
-      if (g == 2 && rc == MOE_OK) rc = finish_dx(false);
+    auto run = [&](LoraOp op, bool ready) {
+      io.ready = ready;
+      if (rc == MOE_OK) rc = launch_lora_gemm(c, op, T, L, ws, io, *lora, st);
+    };
+    if (T > 0) {  // row GEMMs have no tiles without tokens; weight gradients zero-fill
+      StageTimer tm(c, st, 6);
+      run(LORA_W, false);
+      run(LORA_B2, false);
+    }
+    {
+      StageTimer tm(c, st, 7);
+      run(LORA_DB2, true);
+      run(LORA_DA2, true);
+    }
+    if (rc == MOE_OK) router_gradient();
+    if (T > 0) {
+      StageTimer tm(c, st, 8);
+      run(LORA_Z, true);
+      run(LORA_B4, false);
+    }
+    if (rc == MOE_OK) rc = router_gemms();
+    {
+      StageTimer tm(c, st, 9);  // dx included, which runs beside both
+      run(LORA_DB1, true);
+      if (rc == MOE_OK) finish_dx();
+      run(LORA_DA1, true);
     }
     if (rc != MOE_OK) return rc;
   } else {
@@ -604,8 +579,6 @@ static moe_status backward_impl(moe_ctx* ctx, int64_t T, const uint16_t* dy, flo
       StageTimer tm(c, st, 6);
       rc = launch_grouped_gemm(c, GEMM_B2, T, L, ws, io, st);
     }
-    if (rc != MOE_OK) return rc;
-    rc = router_chain();
     if (rc != MOE_OK) return rc;
     // weight gradients: one launch, or one per range of experts with an event after each
     auto wgrad = [&](GemmKind kind, int ev_base) -> moe_status {
@@ -623,17 +596,18 @@ static moe_status backward_impl(moe_ctx* ctx, int64_t T, const uint16_t* dy, flo
       }
       return MOE_OK;
     };
+    io.ready = true;  // from here on: only the dgrad-down GEMM's results are read, and the dy rows
     {
       StageTimer tm(c, st, 7);
       rc = wgrad(GEMM_B3, 0);
     }
     if (rc != MOE_OK) return rc;
+    router_gradient();
     if (T > 0) {
       StageTimer tm(c, st, 8);
       rc = launch_grouped_gemm(c, GEMM_B4, T, L, ws, io, st);
     }
-    if (rc != MOE_OK) return rc;
-    rc = finish_dx(false);
+    if (rc == MOE_OK) rc = router_gemms();
     if (rc != MOE_OK) return rc;
     {
       StageTimer tm(c, st, 9);
@@ -641,9 +615,8 @@ static moe_status backward_impl(moe_ctx* ctx, int64_t T, const uint16_t* dy, flo
     }
     if (rc != MOE_OK) return rc;
   }
-  rc = finish_dx(true);
-  if (rc != MOE_OK) return rc;
-  if (forked && cudaStreamWaitEvent(st, c->ev_join, 0) != cudaSuccess) return MOE_ERR_CUDA;
+  if (!lora) finish_dx();
+  launch_dwr(s, T, x, dl, reinterpret_cast<float*>(ws + L.dwr_part), dW_r, db_r, tc_router && T > 0, st, accumulate, tc_router && one_slice);
   if (c->profiling) c->prof_step++;
   return cudaGetLastError() == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
 }

@@ -66,9 +66,8 @@ __global__ void __launch_bounds__(256) router_bwd_kernel(int64_t T, int E, int k
                                                          float* dg,
                                                          const int32_t* counts, float d_aux,
                                                          float* __restrict__ dl, uint16_t* __restrict__ dl_hi,
-                                                         uint16_t* __restrict__ dl_lo, int32_t* dbg_status) {
-  chain_wait();
-  chain_next();
+                                                         uint16_t* __restrict__ dl_lo, int32_t* dbg_status, int ready) {
+  chain_enter(ready);
   const int lane = threadIdx.x & 31;
   const int64_t t = static_cast<int64_t>(blockIdx.x) * 8 + (threadIdx.x >> 5);
   if (t >= T) return;
@@ -153,15 +152,16 @@ __global__ void __launch_bounds__(256) router_bwd_kernel(int64_t T, int E, int k
       dl_lo[t * E + e] = *reinterpret_cast<const uint16_t*>(&l);
     }
   }
+  chain_leave(ready);
 }
 
 void launch_router_bwd(const Shape& s, int64_t T, const float* logits, const int32_t* idx, const float* gates,
                        const float* dg_part, int dg_tiles, int64_t rows_max, const int32_t* inv, float* dg,
                        const int32_t* counts, float d_aux, float* dl, uint16_t* dl_hi, uint16_t* dl_lo,
-                       cudaStream_t st, int32_t* dbg_status) {
+                       cudaStream_t st, int32_t* dbg_status, bool ready) {
   if (T == 0) return;
   launch_kernel(router_bwd_kernel, static_cast<unsigned>((T + 7) / 8), 256, 0, st, T, s.E, s.k, logits, idx, gates,
-                dg_part, dg_tiles, rows_max, inv, dg, counts, d_aux, dl, dl_hi, dl_lo, dbg_status);
+                dg_part, dg_tiles, rows_max, inv, dg, counts, d_aux, dl, dl_hi, dl_lo, dbg_status, ready ? 1 : 0);
 }
 
 // ------------------------------------------------------------------------------------------ dW_r, db_r
@@ -377,9 +377,8 @@ __global__ void __launch_bounds__(256) unpermute_sum_kernel(int d, int k, const 
                                                             const int32_t* inv,
                                                             const uint16_t* dxr,
                                                             uint16_t* __restrict__ dx, int32_t* dbg_status,
-                                                            int64_t rows_max) {
-  chain_wait();
-  chain_next();
+                                                            int64_t rows_max, int ready) {
+  chain_enter(ready);
   const int64_t t = blockIdx.x;
   __shared__ int sr[MAX_K];
   if (threadIdx.x < k) {
@@ -416,13 +415,14 @@ __global__ void __launch_bounds__(256) unpermute_sum_kernel(int d, int k, const 
     w.w = pack_bf16x2(acc[6], acc[7]);
     *reinterpret_cast<uint4*>(dx + t * d + c) = w;
   }
+  chain_leave(ready);
 }
 
 void launch_unpermute_sum(const Shape& s, int64_t T, const uint16_t* dxp, const int32_t* inv, const uint16_t* dxr,
-                          uint16_t* dx, cudaStream_t st, int32_t* dbg_status, int64_t rows_max) {
+                          uint16_t* dx, cudaStream_t st, int32_t* dbg_status, int64_t rows_max, bool ready) {
   if (T == 0) return;
   launch_kernel(unpermute_sum_kernel, static_cast<unsigned>(T), 256, 0, st, s.d, s.k, dxp, inv, dxr, dx, dbg_status,
-                rows_max);
+                rows_max, ready ? 1 : 0);
 }
 
 void launch_unpermute_bwd(const Shape& s, int64_t T, const uint16_t* dxp, const int32_t* inv, const float* dl,

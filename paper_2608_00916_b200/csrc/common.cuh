@@ -92,10 +92,6 @@ struct moe_ctx_impl {
   void* encode_fn;  // cuTensorMapEncodeTiled, fetched through the runtime
   int router_fp32;      // W_r is passed as fp32 (MOE_FLAG_ROUTER_FP32)
   int debug_checks;     // MOE_FLAG_DEBUG_CHECKS: index checks in the permutation / combine / router-gradient kernels
-  int use_side_stream;  // backward runs the router's gradient chain on s_side, beside the big GEMMs
-  int side_created;
-  cudaStream_t s_side;
-  cudaEvent_t ev_fork, ev_join, ev_b4;
   int tile_mode;    // 0: choose per GEMM, 1: always CTA pairs (odd blocks as half-empty pairs), 2: always one-CTA tiles,
                     // 3: row GEMMs as full pairs + one-CTA tiles for the leftover blocks, weight gradients on pairs
   int gemm_timers;  // MOE_GEMM_TIMERS was set when the context first touched its device
@@ -179,7 +175,7 @@ void launch_gather_rows(const Shape& s, int64_t T, const WsLayout& L, const char
 void launch_router_bwd(const Shape& s, int64_t T, const float* logits, const int32_t* idx, const float* gates,
                        const float* dg_part, int dg_tiles, int64_t rows_max, const int32_t* inv, float* dg,
                        const int32_t* counts, float d_aux, float* dl, uint16_t* dl_hi, uint16_t* dl_lo,
-                       cudaStream_t st, int32_t* dbg_status = nullptr);
+                       cudaStream_t st, int32_t* dbg_status = nullptr, bool ready = false);
 // dg_tiles == 0: dg[t,j] has been filled by the caller (expert-parallel path) and is read instead of the partials
 // SIMT dW_r (any E) and the shared partial reduction / db_r; complete: dW_r needs neither
 void launch_dwr(const Shape& s, int64_t T, const uint16_t* x, const float* dl, float* part, float* dW_r,
@@ -188,11 +184,13 @@ void launch_unpermute_bwd(const Shape& s, int64_t T, const uint16_t* dxp, const 
                           const uint16_t* W_r, uint16_t* dx, cudaStream_t st);
 // dx[t,:] = dxr[t,:] + sum_j dxp[inv[t,j],:]  (router term already contracted on the tensor cores)
 void launch_unpermute_sum(const Shape& s, int64_t T, const uint16_t* dxp, const int32_t* inv, const uint16_t* dxr,
-                          uint16_t* dx, cudaStream_t st, int32_t* dbg_status = nullptr, int64_t rows_max = 0);
+                          uint16_t* dx, cudaStream_t st, int32_t* dbg_status = nullptr, int64_t rows_max = 0, bool ready = false);
 // ---- launchers (gemm.cu); each returns a CUDA / driver error as moe_status
 enum GemmKind { GEMM_F3 = 0, GEMM_F4, GEMM_B2, GEMM_B3, GEMM_B4, GEMM_B5, GEMM_DX, GEMM_DWR, GEMM_KINDS };
 // Caller tensors a grouped-GEMM launch may need besides the workspace.
 struct GemmIO {
+  bool ready = false;       // the kernel on the stream before the GEMM writes nothing that it reads
+  bool next_early = false;  // the one after it is another GEMM, or one that needs nothing of it
   bool save_preactivations = true;  // forward: also write hg, hu (needed by backward only)
   const uint16_t* x = nullptr;
   const uint16_t* W_r = nullptr;      // bf16 router weight, or the leading bf16 term of an fp32 one
@@ -274,12 +272,11 @@ inline int64_t router_psum_rows(const moe_ctx_impl* c, int64_t T, bool logits_gi
 // counts kernel launches of the library (process-wide; read through moe_kernel_launches)
 void note_launch(int n = 1);
 
-// The kernels of one call, in order, on the caller's stream and on the context's second one.  A kernel that directly
-// follows another one of the same call on its stream is launched chained (programmatic stream serialization): it is set
-// up while its predecessor drains, and chain_wait(), called by every such kernel before its first access to global
-// memory, returns when the predecessor has completed and its writes are visible.  The first kernel of a call, and the
-// first one on a stream after that stream was told to wait for an event, depend on more than the kernel before them and
-// are launched plainly.  The object lives on the stack of the call and is seen by the launches of its own thread only;
+// The kernels of one call, in order, on the caller's stream.  A kernel that directly follows another one of the same call is
+// launched chained (programmatic stream serialization): it is set up while its predecessor drains, and chain_wait() returns when
+// the predecessor has completed and its writes are visible.  Small kernels call it before their first access to global memory;
+// GEMMs and the kernels that run beside them in front of what the predecessor has written (chain_warp in gemm_common.cuh,
+// chain_enter).  The first kernel of a call depends on more than the kernel before it and is launched plainly.  The object lives on the stack of the call and is seen by the launches of its own thread only;
 // without one every launch is plain.  Measured: the gap between two kernels falls from 1.5 - 2.5 us to below 1 us.
 class Chain {
  public:
@@ -287,11 +284,6 @@ class Chain {
   ~Chain() { current_ = outer_; }
   Chain(const Chain&) = delete;
   void operator=(const Chain&) = delete;
-  // the stream now also waits for an event
-  void waits(cudaStream_t st) {
-    for (Entry& e : e_)
-      if (e.used && e.st == st) e.used = false;
-  }
   static bool follows(cudaStream_t st) {
     if (current_)
       for (const Entry& e : current_->e_)
@@ -349,6 +341,15 @@ inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, si
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Lets the next kernel of the chain be set up once every block of this one has got here or ended.
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// A small kernel whose inputs were complete before its predecessor in the chain began (ready) runs beside that one: chain_enter()
+// first, chain_leave() last, where one block waits for the predecessor, so that this kernel's end still stands for that one's.
+__device__ __forceinline__ void chain_enter(int ready) {
+  if (!ready) chain_wait();
+  chain_next();
+}
+__device__ __forceinline__ void chain_leave(int ready) {
+  if (ready && blockIdx.x == 0 && blockIdx.y == 0) chain_wait();
+}
 // Gives memory seen for the first time a clean status block.  One that already carries the cookie is left alone, so a failure
 // recorded by an earlier call stays visible until the host has reported it.
 __device__ __forceinline__ void init_status_block(int32_t* status, bool this_thread) {

@@ -63,7 +63,9 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     tmem_alloc(smem_u32(&tmem_base_slot), TMEM_COLS);
     tmem_relinquish();
   }
-  chain_wait();  // everything above touches only this CTA's own state
+  // Row GEMMs of the experts wait for the kernel before them in front of their rows (chain_warp).
+  constexpr bool PRELOAD = !TR::WGRAD && !TR::STATIC_M;
+  if (!PRELOAD && !p.ready) chain_wait();  // everything above touches only this CTA's own state
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -81,11 +83,27 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
       uint32_t it = 0;
       bool ok = true;
       RoleClock clk(p.timers);
-      for (int rd = 0; rd * static_cast<int>(gridDim.x) < ntiles && ok; ++rd) {
+      int kb = 0;  // the first K block of the first tile that is not on its way yet
+      Tile tl = {};
+      if (PRELOAD) {
+        const bool any = static_cast<int>(blockIdx.x) < ntiles;
+        if (any) tl = get_tile<KIND>(p, blockIdx.x);
+        const int pre = any ? min(STAGES, p.k_blocks) : 0;
+        for (int i = 0; i < pre; ++i) {
+          mbar_expect_tx(full_bar(i), p.stage_tx);
+          issue_loads<KIND, 2>(p, tl, i, 0, smem_base + i * STAGE_BYTES + A_BYTES, full_bar(i));
+        }
+        if (!p.ready) chain_wait();
+        for (; kb < pre; ++kb, ++it) {
+          issue_loads<KIND, 1>(p, tl, kb, smem_base + kb * STAGE_BYTES, 0, full_bar(kb));
+          pos.next(STAGES);
+        }
+      }
+      for (int rd = 0; rd * static_cast<int>(gridDim.x) < ntiles && ok; ++rd, kb = 0) {
         const int t = tile_of_round<KIND>(rd, blockIdx.x, gridDim.x);
         if (t >= ntiles) continue;
-        const Tile tl = get_tile<KIND>(p, t);
-        for (int kb = 0; kb < tl.nkb; ++kb, ++it) {
+        if (!PRELOAD || rd) tl = get_tile<KIND>(p, t);
+        for (; kb < tl.nkb; ++kb, ++it) {
           clk.start();
           if (!mbar_wait(empty_bar(pos.s), pos.phase ^ 1u)) {
             ok = false;
@@ -98,7 +116,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
           pos.next(STAGES);
         }
       }
-      chain_next();  // not earlier: blocks of the next kernel that only wait would sit beside the main loop
+      chain_next();  // not earlier without next_early: blocks of the next kernel that only wait would sit beside the main loop
       clk.report(0, 1);  // total; waiting for a free stage
       if (!ok) {
         // gave up: the copies already issued still land in this CTA's shared memory - wait for them (bounded again)
@@ -177,6 +195,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     EpiStage es{smem_base + STAGES * STAGE_BYTES + (warp - 2) * (EPI_UNITS * EPI_UNIT_BYTES), 0u};
     uint32_t tc = 0;
     bool ok = true;
+    if (PRELOAD && !p.ready) chain_wait();  // for what it reads itself
     auto clocked = [&]() { return p.timers && threadIdx.x == 64; };  // asked again each time: a flag would cost a register
     if (clocked()) sum_cycles(p.timers + 5, false);  // total
     for (int rd = 0; rd * static_cast<int>(gridDim.x) < ntiles && ok; ++rd) {
@@ -264,6 +283,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     if (!ok && lane == 0) {
       record_status(p.status, DEV_TIMEOUT, 300 + KIND);
     }
+  } else {
+    chain_warp(p.next_early);
   }
 
   // 31 lanes of the producer's and the issuer's warps have passed by their roles: the barrier takes threads one by one.  (A
@@ -368,6 +389,8 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
     p.e_first = io.e_first;
     p.expert_grouped = 1;
   }
+  p.ready = io.ready ? 1 : 0;
+  p.next_early = io.next_early ? 1 : 0;
   p.mma_n = BN;
   p.stage_tx = STAGE_BYTES;
   p.nseg = (kind == GEMM_B4 || kind == GEMM_DX) ? 2 : 1;
@@ -776,6 +799,8 @@ moe_status launch_lora_gemm(moe_ctx_impl* ctx, LoraOp op, int64_t T, const WsLay
   p.expert_order = reinterpret_cast<const int32_t*>(ws + L.expert_order);
   p.status = reinterpret_cast<int32_t*>(ws + L.status);
   p.E = E;
+  p.ready = io.ready ? 1 : 0;
+  p.next_early = io.next_early ? 1 : 0;
   p.mma_n = BN;
   p.stage_tx = STAGE_BYTES;
   p.nseg = 1;

@@ -23,7 +23,7 @@
 namespace moe {
 
 constexpr int STAGES2 = 6;
-constexpr int GEMM2_THREADS = 320;  // warps: 0 TMA producer, 1 MMA issuer, 2..9 epilogue (two per TMEM lane quadrant)
+constexpr int GEMM2_THREADS = 352;  // warps: 0 TMA producer, 1 MMA issuer, 2..9 epilogue (two per TMEM lane quadrant), 10 chain
 constexpr int BH_BYTES = 128 * BK * 2;              // this CTA's half of B: 16 KB
 constexpr int STAGE2_BYTES = A_BYTES + BH_BYTES;    // 32 KB
 constexpr size_t GEMM2_SMEM = static_cast<size_t>(STAGES2) * STAGE2_BYTES + EPI_BYTES + 1024;
@@ -39,7 +39,7 @@ struct Tile2 {
 template <int KIND>
 __device__ __forceinline__ int total_tiles2(const GemmParams& p) {
   if (Traits<KIND>::WGRAD) return p.E * p.m_tiles * p.n_tiles;  // m_tiles = 256-row pairs of the output
-  return p.sched[p.pair_count_slot] * p.n_tiles;                // number of row-block pairs in the table in use
+  return __ldcg(p.sched + p.pair_count_slot) * p.n_tiles;       // number of row-block pairs in the table in use
 }
 
 template <int KIND>
@@ -65,13 +65,13 @@ __device__ __forceinline__ Tile2 get_tile2(const GemmParams& p, int t, int rank)
     int pr, nt;
     if (p.row_group > 1 && p.pair_count_slot == 2) {
       const int q = t / p.n_tiles;
-      const int4 at = *reinterpret_cast<const int4*>(p.pair_tab + 4 * q);
-      const int row0 = p.pad_offsets[at.x], rows = p.pad_offsets[at.x + 1] - row0;
+      const int4 at = __ldcg(reinterpret_cast<const int4*>(p.pair_tab + 4 * q));
+      const int row0 = __ldcg(p.pad_offsets + at.x), rows = __ldcg(p.pad_offsets + at.x + 1) - row0;
       expert_tile_order(t, p.n_tiles, p.row_group, q - (at.y - row0) / (2 * BM), (rows + 2 * BM - 1) / (2 * BM), pr, nt);
     } else {
-      row_tile_order(t, p.n_tiles, p.row_group, p.sched[p.pair_count_slot], pr, nt);
+      row_tile_order(t, p.n_tiles, p.row_group, __ldcg(p.sched + p.pair_count_slot), pr, nt);
     }
-    const int4 info = *reinterpret_cast<const int4*>(p.pair_tab + 4 * pr);  // expert, first row, blocks (1 or 2)
+    const int4 info = __ldcg(reinterpret_cast<const int4*>(p.pair_tab + 4 * pr));  // expert, first row, blocks (1 or 2)
     tl.e = info.x;
     tl.row0 = info.y + rank * BM;
     tl.write = rank < info.z;
@@ -84,11 +84,12 @@ __device__ __forceinline__ Tile2 get_tile2(const GemmParams& p, int t, int rank)
   return tl;
 }
 
-// Loads of one K block for the CTA of rank `rank`: its rows of A and its 128-column half of B.
-template <int KIND>
+// Loads of one K block for the CTA of rank `rank`: its rows of A and its 128-column half of B (PART as in issue_loads).
+template <int KIND, int PART = 3>
 __device__ __forceinline__ void issue_loads2(const GemmParams& p, const Tile2& tl, int kb, int rank, uint32_t sA,
                                              uint32_t sB, uint32_t bar) {
-  if (!Traits<KIND>::WGRAD && kb >= p.k_blocks * p.nseg) {  // extra K segment of the low-rank adapter path
+  constexpr bool A = (PART & 1) != 0, B = (PART & 2) != 0;
+  if (!Traits<KIND>::WGRAD && PART == 3 && kb >= p.k_blocks * p.nseg) {  // extra K segment of the low-rank adapter path
     const int kk = kb - p.k_blocks * p.nseg;
     tma_load_2d_pair(sA, &p.mapA2, bar, kk * BK, tl.write ? tl.row0 : p.oob_row);
     if (KIND == GEMM_F3)
@@ -100,19 +101,19 @@ __device__ __forceinline__ void issue_loads2(const GemmParams& p, const Tile2& t
     return;
   }
   if (KIND == GEMM_F3) {
-    load_a_rows<true>(p, sA, bar, kb * BK, tl.row0, tl.valid);
+    if (A) load_a_rows<true>(p, sA, bar, kb * BK, tl.row0, tl.valid);
     const CUtensorMap* mb = rank ? &p.mapB1 : &p.mapB0;  // leader: gate columns, partner: the matching up columns
-    tma_load_4d_pair(sB, mb, bar, 0, kb * BK, tl.n0 / 64, tl.e);
+    if (B) tma_load_4d_pair(sB, mb, bar, 0, kb * BK, tl.n0 / 64, tl.e);
   } else if (KIND == GEMM_F4) {
-    load_a_rows<true>(p, sA, bar, kb * BK, tl.row0, tl.valid);
-    tma_load_4d_pair(sB, &p.mapB0, bar, 0, kb * BK, tl.n0 / 64 + rank * 2, tl.e);
+    if (A) load_a_rows<true>(p, sA, bar, kb * BK, tl.row0, tl.valid);
+    if (B) tma_load_4d_pair(sB, &p.mapB0, bar, 0, kb * BK, tl.n0 / 64 + rank * 2, tl.e);
   } else if (KIND == GEMM_B2) {
-    tma_load_2d_pair(sA, &p.mapA0, bar, kb * BK, tl.write ? tl.row0 : p.oob_row);
-    tma_load_3d_pair(sB, &p.mapB0, bar, kb * BK, tl.n0 + rank * 128, tl.e);
+    if (A) tma_load_2d_pair(sA, &p.mapA0, bar, kb * BK, tl.write ? tl.row0 : p.oob_row);
+    if (B) tma_load_3d_pair(sB, &p.mapB0, bar, kb * BK, tl.n0 + rank * 128, tl.e);
   } else if (KIND == GEMM_B4) {
     const int seg = kb / p.k_blocks, kk = kb - seg * p.k_blocks;
-    tma_load_2d_pair(sA, seg ? &p.mapA1 : &p.mapA0, bar, kk * BK, tl.write ? tl.row0 : p.oob_row);
-    tma_load_3d_pair(sB, seg ? &p.mapB1 : &p.mapB0, bar, kk * BK, tl.n0 + rank * 128, tl.e);
+    if (A) tma_load_2d_pair(sA, seg ? &p.mapA1 : &p.mapA0, bar, kk * BK, tl.write ? tl.row0 : p.oob_row);
+    if (B) tma_load_3d_pair(sB, seg ? &p.mapB1 : &p.mapB0, bar, kk * BK, tl.n0 + rank * 128, tl.e);
   } else if (KIND == GEMM_B3) {
     const int row = tl.row0 + kb * BK;
     tma_load_3d_pair(sA, &p.mapA0, bar, 0, row, tl.m0 / 64);
@@ -125,8 +126,8 @@ __device__ __forceinline__ void issue_loads2(const GemmParams& p, const Tile2& t
   }
 }
 
-// The bound of 512 threads keeps the weight gradients at 128 registers: blocks of the bandwidth-bound kernels on the second
-// stream have to fit beside them.
+// The bound of 512 threads keeps the weight gradients at 128 registers: blocks of the bandwidth-bound kernels of the chain have to
+// fit beside them.
 template <int KIND>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Traits<KIND>::WGRAD ? 512 : GEMM2_THREADS, 1)
     grouped_gemm_pair_kernel(const __grid_constant__ GemmParams p) {
@@ -165,7 +166,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Traits<KIND>::WGRAD 
     tmem_alloc_pair(smem_u32(&tmem_base_slot), TMEM_COLS);
     tmem_relinquish_pair();
   }
-  chain_wait();  // everything above touches only this CTA's own state
+  constexpr bool PRELOAD = !TR::WGRAD;  // as in gemm.cu
+  if (!PRELOAD && !p.ready) chain_wait();  // everything above touches only this CTA's own state
   tc_fence_before();
   cluster_sync_all();  // barriers of both CTAs are initialised before anyone signals across the pair
   tc_fence_after();
@@ -180,11 +182,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Traits<KIND>::WGRAD 
       uint32_t it = 0;
       bool ok = true;
       RoleClock clk(leader ? p.timers : nullptr);
-      for (int rd = 0; rd * nclusters < ntiles && ok; ++rd) {
+      int kb = 0;  // the first K block of the first tile that is not on its way yet
+      if (PRELOAD) {
+        const Tile2 tl = cid < ntiles ? get_tile2<KIND>(p, cid, rank) : Tile2{};
+        const int pre = cid < ntiles ? min(STAGES2, p.k_blocks) : 0;
+        for (int i = 0; i < pre; ++i) {
+          if (leader) mbar_expect_tx(full_bar(i), 2 * STAGE2_BYTES);
+          issue_loads2<KIND, 2>(p, tl, i, rank, 0, smem_base + i * STAGE2_BYTES + A_BYTES, mapa_shared(full_bar(i), 0));
+        }
+        if (!p.ready) chain_wait();
+        for (; kb < pre; ++kb, ++it) {
+          issue_loads2<KIND, 1>(p, tl, kb, rank, smem_base + kb * STAGE2_BYTES, 0, mapa_shared(full_bar(kb), 0));
+          pos.next(STAGES2);
+        }
+      }
+      for (int rd = 0; rd * nclusters < ntiles && ok; ++rd, kb = 0) {
         const int t = tile_of_round<KIND>(rd, cid, nclusters);
         if (t >= ntiles) continue;
         const Tile2 tl = get_tile2<KIND>(p, t, rank);
-        for (int kb = 0; kb < tl.nkb; ++kb, ++it) {
+        for (; kb < tl.nkb; ++kb, ++it) {
           clk.start();
           if (!mbar_wait(empty_bar(pos.s), pos.phase ^ 1u)) {
             ok = false;
@@ -267,7 +283,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Traits<KIND>::WGRAD 
         mbar_wait(bar0 + 8u * (2 * STAGES2 + 4), 0u);
       }
     }
-  } else {
+  } else if (warp < 10) {
     // ------------------------------------------------------------------ epilogue (8 warps per CTA, own 128 rows:
     // two warps per TMEM lane quadrant, each draining half of the tile's columns, or every other tile: EpilogueTeams)
     const int ew = warp & 3;
@@ -275,6 +291,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Traits<KIND>::WGRAD 
     EpiStage es{smem_base + STAGES2 * STAGE2_BYTES + (warp - 2) * (EPI_UNITS * EPI_UNIT_BYTES), 0u};
     uint32_t tc = 0;
     bool ok = true;
+    if (PRELOAD && !p.ready) chain_wait();  // for what it reads itself
     const bool clocked = p.timers && leader && threadIdx.x == 64;
     if (clocked) sum_cycles(p.timers + 5, false);  // total
     for (int rd = 0; rd * nclusters < ntiles && ok; ++rd) {
@@ -318,6 +335,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Traits<KIND>::WGRAD 
     if (!ok && lane == 0) {
       record_status(p.status, DEV_TIMEOUT, 1300 + KIND);
     }
+  } else {
+    chain_warp(p.next_early);
   }
 
   tc_fence_before();

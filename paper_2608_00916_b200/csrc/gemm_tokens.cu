@@ -34,7 +34,7 @@ constexpr int TK_MAX_STAGES = 8;
 // held by its epilogue (3300 cycles a unit): 154 / 249 / 318 / 414 us at 256 / 512 / 768 / 1024 rows per expert against 146 / 229 /
 // 302 / 375.
 constexpr int TK_GROUPS = 3;
-constexpr int TK_THREADS = 64 + 128 * TK_GROUPS;  // warps: 0 TMA producer, 1 MMA issuer, 2.. epilogue
+constexpr int TK_THREADS = 96 + 128 * TK_GROUPS;  // warps: 0 TMA producer, 1 MMA issuer, 2.. epilogue, the last one chain (chain_warp)
 // Tiles hold up to 256 tokens, a stage 16 KB of weights and up to 16 KB of tokens, and the ring six of them; with few rows per
 // expert (p.small) up to 128 tokens, so that eight stages fit (and the host has half as many maps to encode, 0.65 us each).
 // Gate/up and dgrad-down, us, six stages -> eight: 154 / 93 -> 153 / 91 at 4 rows per expert, 158 / 101 -> 159 / 101 at 62, 160 / 106 ->
@@ -54,6 +54,7 @@ struct TokenGemmParams {
   int32_t* status;
   unsigned long long* timers;
   int n_tiles;             // weight tiles
+  int ready, next_early;   // as in GemmParams
   int row_group;
   int k_blocks, nseg, k_blocks1;
   int N_total;             // features of the output
@@ -82,31 +83,32 @@ struct TokenTile {
   int nt;       // weight tile
 };
 
-__device__ __forceinline__ int token_tiles(const TokenGemmParams& p) { return p.sched[p.small ? 0 : 2] * p.n_tiles; }
+__device__ __forceinline__ int token_tiles(const TokenGemmParams& p) { return __ldcg(p.sched + (p.small ? 0 : 2)) * p.n_tiles; }
 
 // An expert's rows are cut into as many tiles as it has pairs of 128-row blocks (small: blocks), all of one size but for the last.
 __device__ __forceinline__ TokenTile get_token_tile(const TokenGemmParams& p, int t) {
   TokenTile tl;
   int ri, b, first;
   if (p.row_group > 1) {
-    const int q = t / p.n_tiles, e = p.small ? p.tile_expert[q] : p.pair_tab[4 * q], most = p.small ? BM : 2 * BM;
-    first = p.pad_offsets[e];
-    b = p.small ? q - first / BM : (p.pair_tab[4 * q + 1] - first) / most;
-    expert_tile_order(t, p.n_tiles, p.row_group, q - b, (p.pad_offsets[e + 1] - first + most - 1) / most, ri, tl.nt);
+    const int q = t / p.n_tiles, e = __ldcg(p.small ? p.tile_expert + q : p.pair_tab + 4 * q), most = p.small ? BM : 2 * BM;
+    first = __ldcg(p.pad_offsets + e);
+    b = p.small ? q - first / BM : (__ldcg(p.pair_tab + 4 * q + 1) - first) / most;
+    expert_tile_order(t, p.n_tiles, p.row_group, q - b, (__ldcg(p.pad_offsets + e + 1) - first + most - 1) / most, ri, tl.nt);
   } else {
-    row_tile_order(t, p.n_tiles, p.row_group, p.sched[p.small ? 0 : 2], ri, tl.nt);
+    ri = t / p.n_tiles;
+    tl.nt = t - ri * p.n_tiles;
   }
   if (p.small) {
-    tl.e = p.tile_expert[ri];
-    first = p.pad_offsets[tl.e];
+    tl.e = __ldcg(p.tile_expert + ri);
+    first = __ldcg(p.pad_offsets + tl.e);
     b = ri - first / BM;
   } else {
-    const int4 info = *reinterpret_cast<const int4*>(p.pair_tab + 4 * ri);  // expert, first row of the pair
+    const int4 info = __ldcg(reinterpret_cast<const int4*>(p.pair_tab + 4 * ri));  // expert, first row of the pair
     tl.e = info.x;
-    first = p.pad_offsets[tl.e];
+    first = __ldcg(p.pad_offsets + tl.e);
     b = (info.y - first) / (2 * BM);
   }
-  const int count = p.counts[tl.e], most = p.small ? BM : 2 * BM, tiles = (count + most - 1) / most;
+  const int count = __ldcg(p.counts + tl.e), most = p.small ? BM : 2 * BM, tiles = (count + most - 1) / most;
   const int size = ((count + tiles - 1) / tiles + 15) & ~15, left = count - b * size;
   tl.n = min(size, (left + 15) & ~15);
   tl.row0 = first + b * size;
@@ -423,7 +425,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TK_THREADS, 1)
     tmem_alloc_pair(smem_u32(&tmem_base_slot), TMEM_COLS);
     tmem_relinquish_pair();
   }
-  chain_wait();  // everything above touches only this CTA's own state
   tc_fence_before();
   cluster_sync_all();  // barriers of both CTAs are initialised before anyone signals across the pair
   tc_fence_after();
@@ -445,14 +446,45 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TK_THREADS, 1)
       // took 343 us at 512 rows per expert (326 now) and 632 at 1024 (600), dgrad gate/up 664 at 1024 (638), scoring 241 tokens 230
       // (225).
       const uint32_t full0 = mapa_shared(full_bar(0), 0);
+      auto load_weights = [&](const CUtensorMap* a0, const CUtensorMap* a1, int kk, int wx, int e, uint32_t sA, uint32_t bar) {
+        if (KIND == GEMM_F3) {
+          tma_load_4d_pair(sA, a0, bar, 0, kk, wx, e);
+          tma_load_4d_pair(sA + CHUNK_BYTES, a1, bar, 0, kk, wx, e);
+        } else if (KIND == GEMM_F4) {
+          tma_load_4d_pair(sA, a0, bar, 0, kk, wx, e);
+        } else {  // B2, B4: K-major weights
+          tma_load_3d_pair(sA, a0, bar, kk, wx, e);
+        }
+      };
+      auto weight_coord = [&](const TokenTile& tl) {
+        return KIND == GEMM_F3 ? tl.nt * 2 + rank : KIND == GEMM_F4 ? tl.nt * 4 + rank * 2 : tl.nt * 256 + rank * 128;
+      };
+      auto token_box = [&](const TokenTile& tl) { return ((tl.n >> 1) + 15) / 16 - 1; };  // this CTA's tokens: 16 (box + 1) rows
+      // The weights are the caller's: those of the first stages are fetched before the kernel in front of this one has completed,
+      // the rows once it has (chain_warp).
+      int kk = 0;  // of the first tile: where the loop takes over
+      TokenTile tl = {};
+      if (cid < ntiles) tl = get_token_tile(p, cid);
+      {
+        const int pre = cid < ntiles ? min(static_cast<int>(stages), p.k_blocks) : 0, box = token_box(tl);
+        for (int i = 0; i < pre; ++i) {
+          if (leader) mbar_expect_tx(full_bar(i), 2 * (A_BYTES + (box + 1) * 16 * BK * 2));
+          load_weights(&p.a0, &p.a1, i * BK, weight_coord(tl), tl.e, smem_base + i * stage_bytes, full0 + 8u * i);
+        }
+        if (!p.ready) chain_wait();
+        for (; it < static_cast<uint32_t>(pre); ++it, kk += BK) {
+          tma_load_2d_pair(smem_base + it * stage_bytes + A_BYTES, &p.b[0][box], full0 + 8u * it, kk, tl.row0 + rank * (tl.n >> 1));
+          pos.next(stages);
+        }
+      }
       for (int t = cid; t < ntiles && ok; t += nclusters) {
-        const TokenTile tl = get_token_tile(p, t);
-        const int box = ((tl.n >> 1) + 15) / 16 - 1;  // the copy of this CTA's tokens: 16 (box + 1) rows, of the extra segment all
+        if (t != cid) tl = get_token_tile(p, t);
+        const int box = token_box(tl);  // (of the extra segment: all rows of the map's box)
         const int y = tl.row0 + rank * (tl.n >> 1);
-        const int wx = KIND == GEMM_F3 ? tl.nt * 2 + rank : KIND == GEMM_F4 ? tl.nt * 4 + rank * 2 : tl.nt * 256 + rank * 128;
+        const int wx = weight_coord(tl);
         const int segs = p.nseg + (p.k_blocks1 ? 1 : 0);
 #pragma unroll 1
-        for (int seg = 0; seg < segs && ok; ++seg) {
+        for (int seg = 0; seg < segs && ok; ++seg, kk = 0) {
           const bool extra = seg == p.nseg;
           const CUtensorMap* const a0 = extra ? &p.ax0 : KIND == GEMM_B4 && seg == 1 ? &p.a1 : &p.a0;
           const CUtensorMap* const a1 = extra ? &p.ax1 : &p.a1;  // F3: the up columns
@@ -460,7 +492,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TK_THREADS, 1)
           const uint32_t tx = 2 * (extra ? stage_bytes : A_BYTES + (box + 1) * 16 * BK * 2);  // of both CTAs
           const int k_end = (extra ? p.k_blocks1 : p.k_blocks) * BK;
 #pragma unroll 1
-          for (int kk = 0; kk < k_end; kk += BK, ++it) {
+          for (; kk < k_end; kk += BK, ++it) {
             clk.start();
             if (!mbar_wait(empty_bar(pos.s), pos.phase ^ 1u)) {
               ok = false;
@@ -469,14 +501,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TK_THREADS, 1)
             clk.add(0);
             if (leader) mbar_expect_tx(full_bar(pos.s), tx);
             const uint32_t sA = smem_base + pos.s * stage_bytes, bar = full0 + 8u * pos.s;
-            if (KIND == GEMM_F3) {
-              tma_load_4d_pair(sA, a0, bar, 0, kk, wx, tl.e);
-              tma_load_4d_pair(sA + CHUNK_BYTES, a1, bar, 0, kk, wx, tl.e);
-            } else if (KIND == GEMM_F4) {
-              tma_load_4d_pair(sA, a0, bar, 0, kk, wx, tl.e);
-            } else {  // B2, B4: K-major weights
-              tma_load_3d_pair(sA, a0, bar, kk, wx, tl.e);
-            }
+            load_weights(a0, a1, kk, wx, tl.e, sA, bar);
             tma_load_2d_pair(sA + A_BYTES, b, bar, kk, y);
             pos.next(stages);
           }
@@ -543,13 +568,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TK_THREADS, 1)
         mbar_wait(bar0 + 8u * (2 * TK_MAX_STAGES + 4), 0u);
       }
     }
-  } else {
+  } else if (warp < 2 + 4 * TK_GROUPS) {
     // ------------------------------------------------------------------ epilogue
     const int q = warp & 3;
     const int group = (warp - 2) >> 2;
     const uint32_t staging = smem_base + TK_RING_BYTES + group * TK_EPI_BYTES;
     uint32_t tc = 0;
     bool ok = true;
+    if (!p.ready) chain_wait();  // for what it reads itself
     const bool clocked = p.timers && leader && threadIdx.x == 64;
     if (clocked) sum_cycles(p.timers + 5, false);  // total
     for (int t = cid; t < ntiles; t += nclusters) {
@@ -590,6 +616,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TK_THREADS, 1)
       atomicAdd(p.timers + 7, 1ull);  // CTAs counted
     }
     if (!ok && lane == 0) record_status(p.status, DEV_TIMEOUT, 2300 + KIND);
+  } else {
+    chain_warp(p.next_early);
   }
 
   tc_fence_before();
@@ -635,6 +663,8 @@ moe_status launch_token_gemm(moe_ctx_impl* ctx, GemmKind kind, const WsLayout& L
   p.counts = reinterpret_cast<const int32_t*>(ws + L.counts);
   p.status = reinterpret_cast<int32_t*>(ws + L.status);
   p.timers = ctx->gemm_timers ? reinterpret_cast<unsigned long long*>(ws + L.timers) + 8 * (GEMM_KINDS + kind) : nullptr;
+  p.ready = io.ready ? 1 : 0;
+  p.next_early = io.next_early ? 1 : 0;
   p.nseg = 1;
   p.k_blocks1 = lo ? 1 : 0;
   bool ok = true;
