@@ -42,6 +42,7 @@ WsLayout make_layout(const Shape& s, int64_t T, bool row_buffers) {
   L.pair_tab = take(sizeof(int32_t) * 4 * L.max_m_tiles);
   L.fpair_tab = take(sizeof(int32_t) * 4 * L.max_m_tiles);
   L.single_tab = take(sizeof(int32_t) * s.E);
+  L.pace = take(sizeof(int32_t) * PACE_KINDS * PACE_SLOTS);
   L.tile_counts = take(sizeof(int32_t) * (L.tok_tiles + 1) * s.E);
   // rows: one per SIMT router block; the tensor-core router writes at most as many
   L.psum_part = take(sizeof(float) * (L.router_blocks + 1) * s.E);

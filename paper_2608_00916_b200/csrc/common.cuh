@@ -18,6 +18,7 @@ constexpr int ROUTER_TOK = 16;   // tokens per block in the router kernel
 constexpr int MAX_E = 256;
 constexpr int MAX_K = 32;
 constexpr int DWR_SPLIT = 8;     // token slices of the dW_r contraction
+constexpr int PACE_KINDS = 6, PACE_SLOTS = 64;  // progress counters of the expert GEMMs (Pace in gemm_common.cuh)
 
 // status word values written by kernels
 constexpr int DEV_OK = 0;
@@ -47,6 +48,7 @@ struct WsLayout {
   size_t pair_tab;     // int32[4 * max_m_tiles] pairs of 128-row blocks of one expert: {expert, first row, blocks, 0}
   size_t fpair_tab;    // int32[4 * max_m_tiles] full pairs only (both blocks exist)
   size_t single_tab;   // int32[E] tile index of the last block of every expert with an odd number of blocks
+  size_t pace;         // int32[PACE_KINDS][PACE_SLOTS] progress of the GEMMs that keep step (Pace in gemm_common.cuh)
   size_t tile_counts;  // int32[tok_tiles * E] per token-tile histogram, turned into a prefix along tiles
   size_t psum_part;    // float[router_blocks * E] per-block column sums of p
   size_t psum;         // float[E]

@@ -335,6 +335,13 @@ static int wgrad_group_for(int n_tiles, double rows_per_expert, int64_t columns,
   return n_tiles > 16 && rows_per_expert * static_cast<double>(columns) * 2.0 >= 24e6 ? 16 : 1;
 }
 
+// Whether the pairs of a GEMM keep step (Pace): where L2 does not hold what they share - the weights of wide experts, which row GEMMs
+// walk in groups, or the operands of one expert's weight gradient (24 MB as above) - and tiles are long, from 32 K blocks (about
+// 14 us) on: a round begins with a question that takes 1 us.
+static bool keeps_step(int row_group, bool wgrad, double k_blocks, double operand_bytes) {
+  return k_blocks >= 32.0 && (wgrad ? operand_bytes >= 24e6 : row_group > 1);
+}
+
 // Forward-only calls leave pad rows alone (nothing reads them afterwards), which at few rows per expert is most of what
 // the activations move: scoring 241 tokens (15 rows per expert) 296 -> 268 us, 2048 tokens 367 -> 356 us.  Below 192
 // rows per expert most tiles are partial as well, and A comes in groups of 32 rows of which the empty ones are not read:
@@ -396,6 +403,13 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
   p.nseg = (kind == GEMM_B4 || kind == GEMM_DX) ? 2 : 1;
   p.k_blocks1 = 0;
   p.out_scale = 1.f;
+  auto on_pairs = [&]() {
+    const bool wgrad = kind == GEMM_B3 || kind == GEMM_B5;
+    const double blocks = wgrad ? rows_per_expert / BK : p.k_blocks * p.nseg;
+    const double operands = rows_per_expert * 2.0 * (kind == GEMM_B5 ? d + 2.0 * f : d + static_cast<double>(f));
+    if (part == 0 && keeps_step(p.row_group, wgrad, blocks, operands)) p.pace = reinterpret_cast<int32_t*>(ws + L.pace) + kind * PACE_SLOTS;
+    return launch_pair_gemm(ctx, kind, p, st);
+  };
   bool ok = true;
   switch (kind) {
     case GEMM_F3:
@@ -412,7 +426,7 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
       p.save_pre = io.save_preactivations ? 1 : 0;
       if (!ok) return MOE_ERR_CUDA;
       p.row_group = row_group_for(p.n_tiles, ctx);
-      return pair ? launch_pair_gemm(ctx, kind, p, st) : launch_kind<GEMM_F3>(ctx, p, st);
+      return pair ? on_pairs() : launch_kind<GEMM_F3>(ctx, p, st);
     case GEMM_F4:
       ok = map_2d(fn, &p.mapA0, act, R, f, 128) && map_2d(fn, &p.mapS0, act, R, f, 32) &&
            map_mn(fn, &p.mapB0, W_down, E, f, d, pair ? 2 : 4);
@@ -425,7 +439,7 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
       p.ld_out = d;
       if (!ok) return MOE_ERR_CUDA;
       p.row_group = row_group_for(p.n_tiles, ctx);
-      return pair ? launch_pair_gemm(ctx, kind, p, st) : launch_kind<GEMM_F4>(ctx, p, st);
+      return pair ? on_pairs() : launch_kind<GEMM_F4>(ctx, p, st);
     case GEMM_B2:
       ok = map_2d(fn, &p.mapA0, o, R, d, 128) && map_3d(fn, &p.mapB0, W_down, E, f, d, pair ? 128 : 256);
       p.mapA1 = p.mapA0; p.mapB1 = p.mapB0;
@@ -440,7 +454,7 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
       p.rows_max = L.rows_max;
       if (!ok) return MOE_ERR_CUDA;
       p.row_group = row_group_for(p.n_tiles, ctx);
-      return pair ? launch_pair_gemm(ctx, kind, p, st) : launch_kind<GEMM_B2>(ctx, p, st);
+      return pair ? on_pairs() : launch_kind<GEMM_B2>(ctx, p, st);
     case GEMM_B4:
       ok = map_2d(fn, &p.mapA0, dhg, R, f, 128) && map_2d(fn, &p.mapA1, dhu, R, f, 128) &&
            map_3d(fn, &p.mapB0, W_gate, E, d, f, pair ? 128 : 256) &&
@@ -452,7 +466,7 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
       p.ld_out = d;
       if (!ok) return MOE_ERR_CUDA;
       p.row_group = row_group_for(p.n_tiles, ctx);
-      return pair ? launch_pair_gemm(ctx, kind, p, st) : launch_kind<GEMM_B4>(ctx, p, st);
+      return pair ? on_pairs() : launch_kind<GEMM_B4>(ctx, p, st);
     case GEMM_B3:
       ok = map_mn_rows(fn, &p.mapA0, act, R, f, 2) && map_mn_rows(fn, &p.mapB0, o, R, d, pair ? 2 : 4);
       p.mapA1 = p.mapA0; p.mapB1 = p.mapB0;
@@ -467,7 +481,7 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
       p.ld_out = d;
       p.expert_stride = static_cast<int64_t>(f) * d;
       if (!ok) return MOE_ERR_CUDA;
-      return pair         ? launch_pair_gemm(ctx, kind, p, st)
+      return pair         ? on_pairs()
              : p.acc_fp32 ? launch_kind<GEMM_B3, Accumulate::LOAD_ADD>(ctx, p, st)
                           : launch_kind<GEMM_B3>(ctx, p, st);
     case GEMM_B5:
@@ -485,7 +499,7 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
       p.ld_out = f;
       p.expert_stride = static_cast<int64_t>(d) * f;
       if (!ok) return MOE_ERR_CUDA;
-      return pair         ? launch_pair_gemm(ctx, kind, p, st)
+      return pair         ? on_pairs()
              : p.acc_fp32 ? launch_kind<GEMM_B5, Accumulate::LOAD_ADD>(ctx, p, st)
                           : launch_kind<GEMM_B5>(ctx, p, st);
     case GEMM_DX:

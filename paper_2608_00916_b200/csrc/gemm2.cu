@@ -183,6 +183,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Traits<KIND>::WGRAD 
       bool ok = true;
       RoleClock clk(leader ? p.timers : nullptr);
       int kb = 0;  // the first K block of the first tile that is not on its way yet
+      Pace pace(leader ? p.pace : nullptr, nclusters);
       if (PRELOAD) {
         const Tile2 tl = cid < ntiles ? get_tile2<KIND>(p, cid, rank) : Tile2{};
         const int pre = cid < ntiles ? min(STAGES2, p.k_blocks) : 0;
@@ -200,7 +201,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Traits<KIND>::WGRAD 
         const int t = tile_of_round<KIND>(rd, cid, nclusters);
         if (t >= ntiles) continue;
         const Tile2 tl = get_tile2<KIND>(p, t, rank);
+        pace.begin(rd);
+        const int mark = max(tl.nkb - PACE_MARGIN, kb);
+        if (tl.nkb <= kb) pace.near_end(rd);
         for (; kb < tl.nkb; ++kb, ++it) {
+          if (kb == mark) pace.near_end(rd);
           clk.start();
           if (!mbar_wait(empty_bar(pos.s), pos.phase ^ 1u)) {
             ok = false;

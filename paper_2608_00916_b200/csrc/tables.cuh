@@ -15,18 +15,19 @@ struct TableScratch {
 };
 
 struct TableOut {
-  int32_t *counts, *offsets, *pad_offsets, *sched, *tile_expert, *pair_tab, *fpair_tab, *single_tab, *expert_order;
+  int32_t *counts, *offsets, *pad_offsets, *sched, *tile_expert, *pair_tab, *fpair_tab, *single_tab, *expert_order, *pace;
 };
 
 inline TableOut table_pointers(const WsLayout& L, char* ws) {
   auto I = [&](size_t off) { return reinterpret_cast<int32_t*>(ws + off); };
   return TableOut{I(L.counts),   I(L.offsets),   I(L.pad_offsets), I(L.sched),       I(L.tile_expert),
-                  I(L.pair_tab), I(L.fpair_tab), I(L.single_tab),  I(L.expert_order)};
+                  I(L.pair_tab), I(L.fpair_tab), I(L.single_tab),  I(L.expert_order), I(L.pace)};
 }
 
 // Called by every thread of a block (at least 32 threads) after s_cnt[0..E) is complete and the block has synchronised.
 __device__ inline void build_expert_tables(int E, const int* s_cnt, TableScratch& sh, const TableOut& o) {
   const int tid = threadIdx.x, nthr = blockDim.x;
+  for (int i = tid; i < PACE_KINDS * PACE_SLOTS; i += nthr) o.pace[i] = 0;
   for (int e = tid; e < E; e += nthr) {
     const int run = s_cnt[e];
     o.counts[e] = run;

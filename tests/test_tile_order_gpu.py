@@ -34,6 +34,28 @@ def test_group_size_changes_no_bit(T, d, E, k, f, flags, monkeypatch):
         assert all(torch.equal(a, b) for a, b in zip(step(), plain)), group
 
 
+@pytest.mark.parametrize("T,d,E,k,f", [(1200, 2048, 4, 2, 1664), (4400, 2112, 2, 1, 2176)])
+def test_pairs_that_keep_step(T, d, E, k, f, monkeypatch):
+    """Tiles of 32 K blocks of wide experts, the second shape with weight gradients of 34 K blocks over 25 MB: the pairs wait for one
+    another.  The same bits without (a group of one row tile), and when the counters are those of an earlier backward pass."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(T)
+    n = lambda *s: torch.empty(*s, device="cuda").normal_(0, 0.05, generator=g).bfloat16()
+    x, W, dy = n(T, d), (n(d, E), n(E, d, f), n(E, d, f), n(E, f, d)), n(T, d)
+    steps = []
+    for group in (None, "1"):
+        if group:
+            monkeypatch.setenv("MOE_ROW_GROUP", group)
+        layer = MoELayer(d, E, f, k, 1)
+        for _ in range(2):
+            out = layer.forward(x, *W)
+            for _ in range(2):
+                grads = layer.backward(dy, 0.01)
+                steps.append([out["y"]] + [grads[m] for m in ("dx", "dW_gate", "dW_up", "dW_down")])
+        layer.poll()
+    assert all(torch.equal(a, b) for s in steps[1:] for a, b in zip(s, steps[0]))
+
+
 def test_weight_gradient_of_a_wide_expert():
     """2800 rows, 17 column tiles: by its own rule gate/up walks the three row tiles (the last one short) inside a column tile."""
     inp = synth.make_inputs(synth.MoEShape(22400, 576, 8, 1, 2176), 31, x_std=1.0)
