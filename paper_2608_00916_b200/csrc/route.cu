@@ -270,23 +270,24 @@ __device__ __forceinline__ void psum_columns(int E, int psum_rows, const float* 
   }
 }
 
-// counts, column sums of p, auxiliary loss and the scheduling tables, from complete sh.cnt and sh.ps (block synchronised)
-__device__ __forceinline__ void finish_tables(int64_t T, int E, int k, ScanScratch& sh, const TableOut& tabs,
+// counts, column sums of p, auxiliary loss and the scheduling tables, from complete sh.ps (block synchronised) and sh.cnt (of the
+// calling thread's experts at least: e = tid)
+__device__ __forceinline__ void finish_tables(int64_t T, int E, int k, int psum_rows, ScanScratch& sh, const TableOut& tabs,
                                               float* __restrict__ psum, int32_t* __restrict__ counts_out,
                                               float* __restrict__ aux_out) {
-  const int tid = threadIdx.x, G = SCAN_THREADS / E;
+  const int tid = threadIdx.x, groups = min(SCAN_THREADS / E, psum_rows);  // of psum_columns, that had a row
   for (int e = tid; e < E; e += SCAN_THREADS) {
     const int run = sh.cnt[e];
     counts_out[e] = run;
     float ps = 0.f;
-    for (int g = 0; g < G; ++g) ps += sh.ps[g * E + e];
+    for (int g = 0; g < groups; ++g) ps += sh.ps[g * E + e];
     psum[e] = ps;
     // aux term: (c_e / (T k)) * (Psum_e / T)
     sh.term[e] = (T > 0) ? (static_cast<float>(run) / static_cast<float>(T * k)) * (ps / static_cast<float>(T)) : 0.f;
   }
   __syncthreads();
-  if (tid >= 32 && tid < 64) {  // the second warp sums the aux terms in a fixed order while the first one scans
-    const int lane = tid - 32;
+  if (tid >= SCAN_THREADS - 32) {  // the last warp sums the aux terms in a fixed order while the first one scans
+    const int lane = tid & 31;
     float sterm = 0.f;
 #pragma unroll
     for (int u = 0; u < 8; ++u) sterm += (lane * 8 + u < E) ? sh.term[lane * 8 + u] : 0.f;
@@ -350,14 +351,16 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_kernel(int64_t T, int E, in
     }
   }
   __syncthreads();
-  finish_tables(T, E, k, sh, tabs, psum, counts_out, aux_out);
+  finish_tables(T, E, k, psum_rows, sh, tabs, psum, counts_out, aux_out);
 }
 
 // The permutation in one kernel, while every block can afford to look at all tile histograms (place_max_tiles): block 0
 // builds the counts, tables and the auxiliary loss; block b + 1 places the picks of token tile b.  Each block sums the
 // columns of tile_counts itself - over all tiles (expert totals, hence segment starts) and over the tiles before its own
 // (first rank) - so nothing waits for a scan by one block.  Bound by two rounds of L2 latency per wave of blocks.
-// Measured against scan_kernel followed by scatter_kernel at 128 experts: 241 tokens 13 -> 5 us, 16384 tokens 25 -> 14 us.
+// Measured against scan_kernel followed by scatter_kernel at 128 experts: 241 tokens 13 -> 5 us, 16384 tokens 25 -> 14 us.  Partial sums
+// of groups that had no tile, or no row of the router's, are not added up (8 experts: 128 groups; 256 tokens 6.3 -> 4.1 us from the wait
+// to the last block's end, and with the order of steps in build_expert_tables 5.4 -> 4.7 at 128 experts).
 //
 // The line.  The histograms are read once per block, so the traffic grows with the square of the token count, and with few
 // experts the 1024 / E partial sums per column, added up by one thread, weigh more than the tiles.  Permutation stage with rows
@@ -385,6 +388,8 @@ __global__ void __launch_bounds__(SCAN_THREADS) place_kernel(int64_t T, int E, i
   const int64_t n_picks = my_tile < 0 ? 0 : min(static_cast<int64_t>(TOK_TILE) * k, T * k - i0);
   if (my_tile >= 0)
     for (int i = tid; i < TOK_WARPS * E; i += SCAN_THREADS) pl_masks[i] = 0u;
+  else
+    psum_columns(E, psum_rows, psum_part, sh);
   {
     const int g = tid / E, e = tid - g * E;
     if (tid < G * E) {
@@ -412,20 +417,18 @@ __global__ void __launch_bounds__(SCAN_THREADS) place_kernel(int64_t T, int E, i
   }
   for (int e = tid; e < E; e += SCAN_THREADS) {
     int total = 0, before = 0;
-    for (int g = 0; g < G; ++g) {
+    for (int g = 0; g < min(G, tok_tiles); ++g) {  // the other groups had no tile
       total += sh.seg[g * E + e];
       if (my_tile >= 0) before += __float_as_int(sh.ps[g * E + e]);
     }
     sh.cnt[e] = total;
     s_before[e] = before;
   }
-  __syncthreads();
   if (my_tile < 0) {
-    psum_columns(E, psum_rows, psum_part, sh);
-    __syncthreads();
-    finish_tables(T, E, k, sh, tabs, psum, counts_out, aux_out);
+    finish_tables(T, E, k, psum_rows, sh, tabs, psum, counts_out, aux_out);
     return;
   }
+  __syncthreads();
   if (tid < 32) {  // segment starts: lane L owns experts 8L .. 8L+7
     int cn[8], pd[8], scn = 0, spd = 0;
 #pragma unroll

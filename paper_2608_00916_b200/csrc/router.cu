@@ -2,18 +2,21 @@
 // histogram, in one kernel.  x and W_r are bf16 (an fp32 W_r comes as three exact bf16 terms), so that a bf16 MMA with fp32
 // accumulation is an fp32 contraction up to summation order.
 //
-// CL CTAs share the 128 tokens of a tile, each contracts and routes 128 / CL of them: W_r^T is the M operand (128 experts, twice
-// above 128 of them), the CTA's tokens are N.  The K blocks are summed in four chains (fewer below four K blocks), each in an
-// accumulator of its own, and the chains in their order: the tensor core drops what lies below the last place of an accumulator,
-// so that the error grows with the length of a chain (rms 2.1e-6 with one chain, 0.5e-6 with four at d 2048 and unit-variance
-// logits).
+// CL CTAs share the 128 tokens of a tile.  W_r^T is the M operand (128 experts, twice above 128 of them), tokens are N.  The K blocks
+// are summed in four chains (fewer below four K blocks), each in an accumulator of its own, and the chains in their order: the
+// tensor core drops what lies below the last place of an accumulator, so that the error grows with the length of a chain (rms
+// 2.1e-6 with one chain, 0.5e-6 with four at d 2048 and unit-variance logits).
 // The order of the sums depends on d alone, so that a token's logits, and with them its experts, are the same bits whatever the
-// number of tokens of the call selects.  (Splitting the K blocks over the CTAs instead fetches a part of W_r per CTA, not all of
-// it, and took 17 us where this takes 19 up to 1000 tokens; but its sums change with the split, and a token near a tie got other
-// experts in another batch.)  The CTAs of a tile are a cluster only to add up the tile's histogram.  What bounds it: up to some ten
-// thousand tokens the latency of fetching W_r and the tokens through one SM each and of routing, hence the split; from there on the
-// stream of x from HBM.  With one CTA per tile the accumulators fill tensor memory, so that an SM holds one CTA: 42 -> 56 us at
-// 24576 tokens, 49 -> 60 at 32768 against one chain and two CTAs.
+// number of tokens of the call selects.  Two ways to share the work:
+//   by chains (SPLIT: four CTAs, four chains, up to 128 experts): each CTA sums one chain for all 128 tokens, fetching a quarter of
+//     W_r and of the tokens' columns, and sends the sums through the cluster to the CTA that routes the token
+//   by tokens: each CTA contracts the 128 / CL tokens that it routes, and fetches all of W_r
+// What bounds it: up to some ten thousand tokens the latency of fetching W_r and the tokens through one SM each and of routing,
+// hence the split; from there on the stream of x from HBM.  At d 2048 and 128 experts the sums of a tile are complete 3.8 us after
+// the kernel's first instruction by chains, and 2.9 us later where they are routed, 9.0 us by tokens; the kernel takes 11.6 and
+// 14.6 us at 241 tokens (scoring 221.8 -> 219.6 us with the tables' share, see place_kernel).  With one CTA per tile the
+// accumulators fill tensor memory, so that an SM holds one CTA: 42 -> 56 us at 24576 tokens, 49 -> 60 at 32768 against one chain and
+// two CTAs.
 //
 // Three steps between barriers.  (1) A warp per token: bias, softmax and its column sums; a lane holds NV / 4 groups of four
 // columns.  (2) A thread per token: top-k as a three-level tournament, groups of four columns, supers of four groups, the maxima
@@ -41,9 +44,10 @@ constexpr int RO_BK = 64;
 constexpr int RO_CHUNK_BYTES = 64 * RO_BK * 2;   // 8 KB per 64 columns of W_r and K block
 constexpr int RO_MAX_STAGES = 16;
 constexpr int RO_CHAINS = 4;  // partial sums of a logit
-// Bytes of the operand stages.  Every CTA fetches all of W_r, and waits for latency more than for bandwidth, so the copies in
+// Bytes of the operand stages by tokens.  Every CTA fetches all of W_r, and waits for latency more than for bandwidth, so the copies in
 // flight count: 100 -> 200 KB at d 2048 and 128 experts 20 -> 19 us at 128 tokens, 26 -> 23 at 8192, 35 -> 31 at 16384 (one chain).
-constexpr int RO_RING = 200 * 1024;
+// By chains the sums of all chains (67 KB) lie behind the stages: other CTAs send them while this one still contracts.
+constexpr int RO_RING = 200 * 1024, RO_SPLIT_RING = 128 * 1024;
 static_assert(RO_TOK == TOK_TILE, "the histogram written here is the permutation's");
 
 struct RouterParams {
@@ -66,6 +70,9 @@ struct RouterParams {
   uint32_t w_bytes, stage_bytes;  // of a stage: W_r, and with the tokens
 };
 
+__device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
 __device__ __forceinline__ void red_cluster_add(uint32_t addr, int v) {
   asm volatile("red.relaxed.cluster.shared::cluster.add.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
@@ -169,10 +176,12 @@ __device__ __forceinline__ float select_topk(int k, uint32_t row, uint32_t maxim
 
 __device__ __forceinline__ void routing_sync() { asm volatile("bar.sync 1, %0;" ::"n"(32 * RO_WARPS) : "memory"); }
 
-template <int CL, int NV>
+template <int CL, int NV, bool SPLIT>
 __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, 1)
     router_cluster_kernel(const __grid_constant__ RouterParams p) {
+  static_assert(!SPLIT || (CL == RO_CHAINS && NV == 4));
   constexpr int MINE = RO_TOK / CL;             // this CTA's tokens of the tile
+  constexpr int N = SPLIT ? RO_TOK : MINE;      // tokens it contracts
   constexpr uint32_t ACCS = NV / 4, TMEM_COLS = RO_CHAINS * ACCS * MINE;  // per chain an accumulator for each 128 experts, a column per token
   extern __shared__ unsigned char ro_smem_raw[];
   __shared__ __align__(8) uint64_t bars[2 * RO_MAX_STAGES + 1];  // full, empty, accumulator complete
@@ -185,7 +194,9 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, 1)
   const int tile = blockIdx.x / CL;
   const int64_t first = static_cast<int64_t>(tile) * RO_TOK + rank * MINE, left = p.T - first;
   const int tokens = left < MINE ? static_cast<int>(left) : MINE;  // of which are there (may be negative)
-  const int k_blocks = tokens > 0 ? p.k_total : 0;
+  // K blocks it contracts: its chain, or all of them
+  const int k_begin = SPLIT ? p.k_total * rank / RO_CHAINS : 0, k_end = SPLIT ? p.k_total * (rank + 1) / RO_CHAINS : tokens > 0 ? p.k_total : 0;
+  const int k_blocks = k_end - k_begin;
   const uint32_t smem_base = (smem_u32(ro_smem_raw) + 1023u) & ~1023u;
   const uint32_t bar0 = smem_u32(bars);
   const uint32_t acc_bar = bar0 + 8u * (2 * RO_MAX_STAGES);
@@ -221,11 +232,14 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, 1)
       uint32_t phase = 0, it = 0;
       bool ok = true;
       // (what this thread takes to refill a stage counts like latency: no divisions and no choice of maps in the loop)
-      const int k_end = tokens > 0 ? p.k_blocks * RO_BK : 0, segs = p.k_total / p.k_blocks;
-      for (int seg = 0; seg < segs && ok; ++seg) {
+      const int token0 = SPLIT ? tile * RO_TOK : static_cast<int>(first);
+      int seg = k_begin / p.k_blocks, kk = (k_begin - seg * p.k_blocks) * RO_BK;
+      for (int left_kb = k_blocks; left_kb > 0 && ok; ++seg, kk = 0) {
         const CUtensorMap* const mw = seg == 0 ? &p.map_w0 : (seg == 1 ? &p.map_w1 : &p.map_w2);
+        const int kk_end = min(p.k_blocks * RO_BK, kk + left_kb * RO_BK);
+        left_kb -= (kk_end - kk) / RO_BK;
 #pragma unroll 1
-        for (int kk = 0; kk < k_end; kk += RO_BK, ++it) {
+        for (; kk < kk_end; kk += RO_BK, ++it) {
           const uint32_t sW = smem_base + s * p.stage_bytes, bar = full_bar(s);
           if (!mbar_wait(empty_bar(s), phase ^ 1u)) {
             ok = false;
@@ -238,7 +252,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, 1)
 #pragma unroll 1
             for (int c = 0; c < p.w_chunks; ++c) tma_load_3d(sW + c * RO_CHUNK_BYTES, mw, bar, c * 64, kk, 0);
           }
-          tma_load_2d(sW + p.w_bytes, &p.map_x, bar, kk, static_cast<int>(first));
+          tma_load_2d(sW + p.w_bytes, &p.map_x, bar, kk, token0);
           if (++s == p.stages) {
             s = 0;
             phase ^= 1u;
@@ -255,13 +269,14 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, 1)
   } else if (warp == 1) {
     if (elect_one()) {  // MMA issuer
       // (experts beyond the chunks of W_r are whatever lies behind them; their accumulator lanes are not read)
-      constexpr uint32_t idesc = umma_idesc(128, MINE, 1, 0);
+      constexpr uint32_t idesc = umma_idesc(128, N, 1, 0);
       const uint64_t descW = smem_desc(smem_base, RO_CHUNK_BYTES, 1024);
       const uint64_t descX = smem_desc(smem_base + p.w_bytes, 0, 1024);
       int s = 0;
       uint32_t phase = 0;
       bool ok = true;
-      int chain = 0, first_kb = 0, next_kb = p.k_total / p.chains;  // chain c: K blocks c k_total / chains and on
+      // chain c: K blocks c k_total / chains and on
+      int chain = 0, first_kb = 0, next_kb = SPLIT ? k_blocks : p.k_total / p.chains;
       for (int kb = 0; kb < k_blocks; ++kb) {
         if (kb == next_kb) {
           ++chain;
@@ -278,7 +293,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, 1)
         for (int ks = 0; ks < RO_BK / 16; ++ks)
 #pragma unroll
           for (uint32_t h = 0; h < ACCS; ++h)
-            umma_bf16(tmem_base + (chain * ACCS + h) * MINE, descW + off + ((h * 2 * RO_CHUNK_BYTES + ks * 2048) >> 4), descX + off + (ks * 32 >> 4), idesc,
+            umma_bf16(tmem_base + (chain * ACCS + h) * N, descW + off + ((h * 2 * RO_CHUNK_BYTES + ks * 2048) >> 4), descX + off + (ks * 32 >> 4), idesc,
                       kb != first_kb || ks != 0 ? 1u : 0u);
         umma_commit(empty_bar(s));
         if (++s == p.stages) {
@@ -300,11 +315,13 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, 1)
       p.row_gate[i] = 0.f;
   }
 
-  const uint32_t part = smem_base;  // the logits of this CTA's tokens, over the operand stages
+  // the logits of this CTA's tokens, over the operand stages; SPLIT: behind them, a buffer for the sums of each chain
+  const uint32_t part = smem_base + (SPLIT ? p.stages * p.stage_bytes : 0u);
   constexpr uint32_t PITCH = 32 * NV * 4 + 16;  // rows 16 bytes apart in the banks
+  constexpr uint32_t CHAIN_BYTES = MINE * PITCH;
   if (warp >= 2) {
     constexpr uint32_t MAX_PITCH = 32 * (NV / 4) * 4 + 16;
-    const uint32_t maxima = part + MINE * PITCH;                // of the groups of four columns
+    const uint32_t maxima = part + (SPLIT ? RO_CHAINS : 1) * CHAIN_BYTES;  // of the groups of four columns
     const uint32_t picks = maxima + MINE * MAX_PITCH;           // {exponential, column}: k rows of MINE (and one, in other banks)
     const uint32_t pick_pitch = MINE * 8 + 8, recip = picks + p.k * pick_pitch;  // 1 / sum of the exponentials
     const int w = warp - 2, E = p.E, k = p.k;
@@ -325,6 +342,13 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, 1)
             const int col = 4 * (lane + 32 * q);
             const uint32_t a = part + i * PITCH + col * 4;
             float4 sum = lds_f4(a);
+            if (SPLIT) {
+#pragma unroll
+              for (int c = 1; c < RO_CHAINS; ++c) {
+                const float4 next = lds_f4(a + c * CHAIN_BYTES);
+                sum = make_float4(sum.x + next.x, sum.y + next.y, sum.z + next.z, sum.w + next.w);
+              }
+            }
             if (col < E) {  // E is a multiple of 8: the four columns exist or do not
               if (p.bias) {  // by words: it may lie anywhere in a buffer of parameters
                 const float* const b = p.bias + col;
@@ -390,7 +414,24 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, 1)
       if (!ok && lane == 0) record_status(p.status, DEV_TIMEOUT, 3300);
       tc_fence_after();
       const int ew = warp & 3;
-      if (ok && tokens > 0)
+      if constexpr (SPLIT) {
+        // the chain's sums of every token go to the CTA that routes it
+        cluster_wait();  // all four run
+        if (ok)
+#pragma unroll 1
+          for (int c = w >> 2; c < RO_TOK / 16; c += RO_WARPS / 4) {
+            const int e = ew * 32 + lane, tok0 = c * 16;
+            uint32_t r[16];
+            tmem_ld16(tmem_base + (static_cast<uint32_t>(ew * 32) << 16) + tok0, r);
+            tmem_ld_wait();
+            const uint32_t to = mapa_shared(part + rank * CHAIN_BYTES + (tok0 % MINE) * PITCH + e * 4, tok0 / MINE);
+            if (e < E)
+#pragma unroll
+              for (int i = 0; i < 16; ++i) st_cluster_f32(to + i * PITCH, __uint_as_float(r[i]));
+          }
+        tc_fence_before();
+        cluster_sync_diverged();  // the sums of all chains are there
+      } else if (ok && tokens > 0) {
 #pragma unroll 1
         for (int c = w >> 2; c < static_cast<int>(ACCS) * (MINE / 16); c += RO_WARPS / 4) {
           const int e = c / (MINE / 16) * 128 + ew * 32 + lane, tok0 = c % (MINE / 16) * 16;
@@ -411,15 +452,18 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, 1)
 #pragma unroll
             for (int i = 0; i < 16; ++i) asm volatile("st.shared.f32 [%0], %1;" ::"r"(part + (tok0 + i) * PITCH + e * 4), "f"(sum[i]) : "memory");
         }
-      tc_fence_before();
-      routing_sync();
+      }
+      if (!SPLIT) {
+        tc_fence_before();
+        routing_sync();
+      }
 #pragma unroll
       for (int q = 0; q < NV; ++q) acc[q] = 0.f;
     }
 #pragma unroll
     for (int q = 0; q < NV; ++q) s_psum[w][4 * (lane + 32 * (q / 4)) + q % 4] = acc[q];
     routing_sync();
-    if (CL > 1) cluster_wait();  // the tile's first CTA has cleared its counts
+    if (CL > 1 && !SPLIT) cluster_wait();  // the tile's first CTA has cleared its counts
     const int e = tid - 64;
     if (e < E) {
       float s = 0.f;
@@ -431,6 +475,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RO_THREADS, 1)
     }
   } else if (CL > 1) {
     cluster_wait();
+    if (SPLIT) cluster_sync_diverged();
   }
   if (CL > 1)
     cluster_sync_diverged();  // the counts of the tile are complete
@@ -458,21 +503,24 @@ int router_cluster(const Shape& s, int sm_count, int64_t T) {
   return s.E <= 128 && (s.E < 32 || tiles * 2 > sm_count) ? 1 : 2;
 }
 
-template <int CL, int NV>
+template <int CL, int NV, bool SPLIT = false>
 static moe_status launch_one(moe_ctx_impl* ctx, RouterParams& p, int tiles, cudaStream_t st) {
-  auto* const kernel = router_cluster_kernel<CL, NV>;
+  auto* const kernel = router_cluster_kernel<CL, NV, SPLIT>;
   // the stages (and what an MMA reads behind an odd number of chunks), and over them what the routing needs: the logits of the
   // CTA's tokens, the maxima of their groups, and {pick, column} and 1 / sum for k picks
   constexpr size_t mine = RO_TOK / CL;
-  auto routing = [](int k) { return mine * (128 * NV + 16) + mine * (32 * NV + 16) + k * (mine * 8 + 8) + mine * 4; };
-  auto smem_of = [](size_t ring, size_t over) { return (ring > over ? ring : over) + 1024; };
+  auto routing = [](int k) {
+    return (SPLIT ? RO_CHAINS : 1) * mine * (128 * NV + 16) + mine * (32 * NV + 16) + k * (mine * 8 + 8) + mine * 4;
+  };
+  auto smem_of = [](size_t ring, size_t over) { return (SPLIT ? ring + over : ring > over ? ring : over) + 1024; };
+  constexpr int ring = SPLIT ? RO_SPLIT_RING : RO_RING;
   p.w_bytes = p.w_chunks * RO_CHUNK_BYTES;
-  p.stage_bytes = p.w_bytes + mine * RO_BK * 2;
-  p.stages = std::min<int>(RO_RING / p.stage_bytes, RO_MAX_STAGES);
+  p.stage_bytes = p.w_bytes + (SPLIT ? RO_TOK : mine) * RO_BK * 2;
+  p.stages = std::min<int>(ring / p.stage_bytes, RO_MAX_STAGES);
   const size_t smem = smem_of(p.stages * p.stage_bytes + (p.w_chunks & 1) * RO_CHUNK_BYTES, routing(p.k));
-  constexpr int slot = (CL == 1 ? 0 : CL == 2 ? 1 : 2) + (NV == 4 ? 0 : 4);
+  constexpr int slot = SPLIT ? 3 : (CL == 1 ? 0 : CL == 2 ? 1 : 2) + (NV == 4 ? 0 : 4);
   if (!(ctx->router_attr & (1u << slot))) {  // per device (the context is bound to one), and for every context on it: the most of all
-    const size_t most = smem_of(RO_RING + RO_CHUNK_BYTES, routing(MAX_K));
+    const size_t most = smem_of(ring + RO_CHUNK_BYTES, routing(MAX_K));
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most)) != cudaSuccess)
       return MOE_ERR_CUDA;
     ctx->router_attr |= 1u << slot;
@@ -494,13 +542,14 @@ moe_status launch_router_tc(moe_ctx_impl* ctx, int64_t T, const WsLayout& L, cha
   auto map_w = [&](CUtensorMap* m, const uint16_t* w) {  // W_r as a one-slab tensor of weights
     return p.whole_chunks ? map_mn(fn, m, w, 1, s.d, s.E, p.w_chunks) : map_3d(fn, m, w, 1, s.d, s.E, 64);
   };
-  const int cl = router_cluster(s, ctx->sm_count, T);
-  bool ok = map_2d(fn, &p.map_x, io.x, T, s.d, RO_TOK / cl) && map_w(&p.map_w0, io.W_r);
-  if (io.W_r_mid) ok = ok && map_w(&p.map_w1, io.W_r_mid) && map_w(&p.map_w2, io.W_r_lo);
-  if (!ok) return MOE_ERR_CUDA;
   p.k_blocks = s.d / RO_BK;
   p.k_total = p.k_blocks * (io.W_r_mid ? 3 : 1);
   p.chains = p.k_total >= RO_CHAINS ? RO_CHAINS : p.k_total >= 2 ? 2 : 1;
+  const int cl = router_cluster(s, ctx->sm_count, T);
+  const bool split = cl == RO_CHAINS && s.E <= 128 && p.chains == RO_CHAINS;
+  bool ok = map_2d(fn, &p.map_x, io.x, T, s.d, split ? RO_TOK : RO_TOK / cl) && map_w(&p.map_w0, io.W_r);
+  if (io.W_r_mid) ok = ok && map_w(&p.map_w1, io.W_r_mid) && map_w(&p.map_w2, io.W_r_lo);
+  if (!ok) return MOE_ERR_CUDA;
   p.status = reinterpret_cast<int32_t*>(ws + L.status);
   p.row_gate = reinterpret_cast<float*>(ws + L.row_gate);
   p.rows = L.rows_alloc;
@@ -516,7 +565,7 @@ moe_status launch_router_tc(moe_ctx_impl* ctx, int64_t T, const WsLayout& L, cha
   const int tiles = static_cast<int>((T + RO_TOK - 1) / RO_TOK);
   if (s.E <= 128) {
     switch (cl) {
-      case 4: return launch_one<4, 4>(ctx, p, tiles, st);
+      case 4: return split ? launch_one<4, 4, true>(ctx, p, tiles, st) : launch_one<4, 4>(ctx, p, tiles, st);
       case 2: return launch_one<2, 4>(ctx, p, tiles, st);
       default: return launch_one<1, 4>(ctx, p, tiles, st);
     }
