@@ -144,7 +144,7 @@ MOE_API moe_status moe_selftest_timeout(moe_ctx* ctx, void* workspace, void* cud
  * of them if there were more), stores that number of pairs in *steps, and starts a new window.
  * Stage order: 0 router, 1 permute (histogram, scan, scatter, gather), 2 gate/up GEMM + SwiGLU,
  * 3 down GEMM, 4 combine, 5 combine-bwd (gather of dy rows), 6 dgrad-down + SwiGLU-bwd (+ dg), 7 wgrad-down, 8 dgrad gate/up,
- * 9 wgrad gate/up, 10 router-bwd (dl), 11 dW_r, 12 unpermute-bwd (dx), 13 router term of dx, 14..15 unused.
+ * 9 wgrad gate/up, 10 router-bwd (dl), 11 dW_r and the router term of dx, 12 unpermute-bwd (dx), 13..15 unused.
  * The events keep the kernels of a call apart; without them stages 10 and 12 run beside stages 7 and 9 and each GEMM begins
  * while the one before it drains, so the stage times add up to more than the step. */
 #define MOE_PROF_RING 64

@@ -524,17 +524,12 @@ static moe_status backward_impl(moe_ctx* ctx, int64_t T, const uint16_t* dy, flo
     if (!tc_router || T == 0) return MOE_OK;
     GemmIO rio = io;
     rio.ready = true;
-    {
-      StageTimer tm(c, st, 13);
-      const moe_status r2 = launch_grouped_gemm(c, GEMM_DX, T, L, ws, rio, st);
-      if (r2 != MOE_OK) return r2;
-    }
     StageTimer tm(c, st, 11);
     if (one_slice) {
       rio.dW_r = dW_r;
       rio.dW_r_accumulate = accumulate;
     }
-    return launch_grouped_gemm(c, GEMM_DWR, T, L, ws, rio, st);
+    return launch_router_gradient(c, T, L, ws, rio, st);
   };
   auto finish_dx = [&]() {
     StageTimer tm(c, st, 12);

@@ -218,6 +218,8 @@ struct GemmIO {
 };
 moe_status launch_grouped_gemm(moe_ctx_impl* ctx, GemmKind kind, int64_t T, const WsLayout& L, char* ws,
                                const GemmIO& io, cudaStream_t st);
+// DX and DWR in one launch
+moe_status launch_router_gradient(moe_ctx_impl* ctx, int64_t T, const WsLayout& L, char* ws, const GemmIO& io, cudaStream_t st);
 struct GemmParams;
 moe_status launch_pair_gemm(moe_ctx_impl* ctx, GemmKind kind, const GemmParams& p, cudaStream_t st);  // gemm2.cu
 // Low-rank adapters of an expert-LoRA call (all device pointers, bf16): A1 [E,d,r], B1g / B1u [E,r,f], A2 [E,f,r],
