@@ -65,9 +65,9 @@ def stage_work(shape: synth.MoEShape):
         "dgrad_gateup": ("tensor", 4 * R * f * d),
         "wgrad_gateup": ("tensor", 4 * R * d * f),
         "router_bwd": ("hbm", 8 * T * E + 12 * R),
-        "dW_r": ("hbm", 4 * T * d + 8 * T * E + 6 * d * E),  # with the router term of dx, in the same launch
+        "dW_r": ("hbm", 2 * T * d + 4 * T * E + 4 * d * E),  # its time is that of the launch, with the router term of dx
         "unpermute_bwd": ("hbm", 2 * R * d + 2 * T * d + 2 * T * d),
-        "dx_router_term": ("hbm", 0),  # in dW_r
+        "dx_router_term": ("hbm", 4 * T * E + 2 * T * d + 2 * d * E),
     }
 
 
