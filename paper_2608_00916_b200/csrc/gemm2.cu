@@ -39,7 +39,7 @@ struct Tile2 {
 template <int KIND>
 __device__ __forceinline__ int total_tiles2(const GemmParams& p) {
   if (Traits<KIND>::WGRAD) return p.E * p.m_tiles * p.n_tiles;  // m_tiles = 256-row pairs of the output
-  return __ldcg(p.sched + p.pair_count_slot) * p.n_tiles;       // number of row-block pairs in the table in use
+  return p.sched[p.pair_count_slot] * p.n_tiles;                // number of row-block pairs in the table in use
 }
 
 template <int KIND>
@@ -65,13 +65,13 @@ __device__ __forceinline__ Tile2 get_tile2(const GemmParams& p, int t, int rank)
     int pr, nt;
     if (p.row_group > 1 && p.pair_count_slot == 2) {
       const int q = t / p.n_tiles;
-      const int4 at = __ldcg(reinterpret_cast<const int4*>(p.pair_tab + 4 * q));
-      const int row0 = __ldcg(p.pad_offsets + at.x), rows = __ldcg(p.pad_offsets + at.x + 1) - row0;
+      const int4 at = *reinterpret_cast<const int4*>(p.pair_tab + 4 * q);
+      const int row0 = p.pad_offsets[at.x], rows = p.pad_offsets[at.x + 1] - row0;
       expert_tile_order(t, p.n_tiles, p.row_group, q - (at.y - row0) / (2 * BM), (rows + 2 * BM - 1) / (2 * BM), pr, nt);
     } else {
-      row_tile_order(t, p.n_tiles, p.row_group, __ldcg(p.sched + p.pair_count_slot), pr, nt);
+      row_tile_order(t, p.n_tiles, p.row_group, p.sched[p.pair_count_slot], pr, nt);
     }
-    const int4 info = __ldcg(reinterpret_cast<const int4*>(p.pair_tab + 4 * pr));  // expert, first row, blocks (1 or 2)
+    const int4 info = *reinterpret_cast<const int4*>(p.pair_tab + 4 * pr);  // expert, first row, blocks (1 or 2)
     tl.e = info.x;
     tl.row0 = info.y + rank * BM;
     tl.write = rank < info.z;

@@ -83,32 +83,32 @@ struct TokenTile {
   int nt;       // weight tile
 };
 
-__device__ __forceinline__ int token_tiles(const TokenGemmParams& p) { return __ldcg(p.sched + (p.small ? 0 : 2)) * p.n_tiles; }
+__device__ __forceinline__ int token_tiles(const TokenGemmParams& p) { return p.sched[p.small ? 0 : 2] * p.n_tiles; }
 
 // An expert's rows are cut into as many tiles as it has pairs of 128-row blocks (small: blocks), all of one size but for the last.
 __device__ __forceinline__ TokenTile get_token_tile(const TokenGemmParams& p, int t) {
   TokenTile tl;
   int ri, b, first;
   if (p.row_group > 1) {
-    const int q = t / p.n_tiles, e = __ldcg(p.small ? p.tile_expert + q : p.pair_tab + 4 * q), most = p.small ? BM : 2 * BM;
-    first = __ldcg(p.pad_offsets + e);
-    b = p.small ? q - first / BM : (__ldcg(p.pair_tab + 4 * q + 1) - first) / most;
-    expert_tile_order(t, p.n_tiles, p.row_group, q - b, (__ldcg(p.pad_offsets + e + 1) - first + most - 1) / most, ri, tl.nt);
+    const int q = t / p.n_tiles, e = p.small ? p.tile_expert[q] : p.pair_tab[4 * q], most = p.small ? BM : 2 * BM;
+    first = p.pad_offsets[e];
+    b = p.small ? q - first / BM : (p.pair_tab[4 * q + 1] - first) / most;
+    expert_tile_order(t, p.n_tiles, p.row_group, q - b, (p.pad_offsets[e + 1] - first + most - 1) / most, ri, tl.nt);
   } else {
     ri = t / p.n_tiles;
     tl.nt = t - ri * p.n_tiles;
   }
   if (p.small) {
-    tl.e = __ldcg(p.tile_expert + ri);
-    first = __ldcg(p.pad_offsets + tl.e);
+    tl.e = p.tile_expert[ri];
+    first = p.pad_offsets[tl.e];
     b = ri - first / BM;
   } else {
-    const int4 info = __ldcg(reinterpret_cast<const int4*>(p.pair_tab + 4 * ri));  // expert, first row of the pair
+    const int4 info = *reinterpret_cast<const int4*>(p.pair_tab + 4 * ri);  // expert, first row of the pair
     tl.e = info.x;
-    first = __ldcg(p.pad_offsets + tl.e);
+    first = p.pad_offsets[tl.e];
     b = (info.y - first) / (2 * BM);
   }
-  const int count = __ldcg(p.counts + tl.e), most = p.small ? BM : 2 * BM, tiles = (count + most - 1) / most;
+  const int count = p.counts[tl.e], most = p.small ? BM : 2 * BM, tiles = (count + most - 1) / most;
   const int size = ((count + tiles - 1) / tiles + 15) & ~15, left = count - b * size;
   tl.n = min(size, (left + 15) & ~15);
   tl.row0 = first + b * size;
@@ -396,6 +396,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TK_THREADS, 1)
   extern __shared__ unsigned char tk_smem_raw[];
   __shared__ __align__(8) uint64_t bars[2 * TK_MAX_STAGES + 5];  // full, empty, accumulator full / empty, drain (failure path)
   __shared__ uint32_t tmem_base_slot;
+  __shared__ int stage_n[TK_MAX_STAGES];  // tokens of the tile whose K block is in a stage (from the leader's producer to its issuer)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = static_cast<int>(cluster_ctarank());
@@ -468,7 +469,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TK_THREADS, 1)
       {
         const int pre = cid < ntiles ? min(static_cast<int>(stages), p.k_blocks) : 0, box = token_box(tl);
         for (int i = 0; i < pre; ++i) {
-          if (leader) mbar_expect_tx(full_bar(i), 2 * (A_BYTES + (box + 1) * 16 * BK * 2));
+          if (leader) {
+            stage_n[i] = tl.n;
+            mbar_expect_tx(full_bar(i), 2 * (A_BYTES + (box + 1) * 16 * BK * 2));
+          }
           load_weights(&p.a0, &p.a1, i * BK, weight_coord(tl), tl.e, smem_base + i * stage_bytes, full0 + 8u * i);
         }
         if (!p.ready) chain_wait();
@@ -499,7 +503,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TK_THREADS, 1)
               break;
             }
             clk.add(0);
-            if (leader) mbar_expect_tx(full_bar(pos.s), tx);
+            if (leader) {
+              stage_n[pos.s] = tl.n;
+              mbar_expect_tx(full_bar(pos.s), tx);
+            }
             const uint32_t sA = smem_base + pos.s * stage_bytes, bar = full0 + 8u * pos.s;
             load_weights(a0, a1, kk, wx, tl.e, sA, bar);
             tma_load_2d_pair(sA + A_BYTES, b, bar, kk, y);
@@ -528,7 +535,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TK_THREADS, 1)
       bool ok = true;
       RoleClock clk(p.timers);
       for (int t = cid; t < ntiles && ok; t += nclusters) {
-        const uint32_t idesc = umma_idesc(2 * BM, get_token_tile(p, t).n, A_MN, 0);
+        uint32_t idesc = 0;
         const int acc = tc & 1;
         const uint32_t aph = (tc >> 1) & 1u;
         ++tc;
@@ -549,6 +556,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TK_THREADS, 1)
           }
           clk.add(1);
           tc_fence_after();
+          // (looking the tile up in the tables here instead left the tensor cores without work for up to three L2 round trips a tile)
+          if (kb == 0) idesc = umma_idesc(2 * BM, stage_n[pos.s], A_MN, 0);
           const uint64_t off = (pos.s * stage_bytes) >> 4;
           const uint32_t done = empty_bar(pos.s);
           pos.next(stages);
