@@ -11,6 +11,14 @@ namespace moe {
 
 thread_local Chain* Chain::current_ = nullptr;
 
+// Whether the large GEMMs begin while the one before them drains (chain_warp in gemm_common.cuh).  With few rows per expert that fills
+// what the ends of the kernels leave idle.  With many, the power cap takes back in clocks what it saves in time, and pairs that begin
+// a GEMM at different times do not share operands as closely.  Steps at d 2048, f 768, 128 experts with against without, us:
+// 62 rows per expert 843 / 861, 512 rows 2306 / 2325, 1024 rows 4202 / 4136 (1024 on average, unequal: 4235 / 4293).  The small kernels
+// run beside the weight gradients, and the router's gradient fills the end of the GEMM before it, at every size: serial, it stood
+// alone for 25 us at 8191 tokens and 57 at 16384.
+static bool gemms_overlap(const Shape& s, int64_t T) { return T * s.k < static_cast<int64_t>(s.E) * 768; }
+
 static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 static std::atomic<long long> g_kernel_launches{0};
@@ -398,7 +406,7 @@ static moe_status forward_impl(bool training, moe_ctx* ctx, int64_t T, const uin
   if (T > 0) {
     {
       StageTimer tm(c, st, 2);
-      io.next_early = true;
+      io.next_early = gemms_overlap(s, T);
       if (lora) {
         rc = launch_lora_gemm(c, LORA_U, T, L, ws, io, *lora, st);
         if (rc == MOE_OK) rc = launch_lora_gemm(c, LORA_F3, T, L, ws, io, *lora, st);
@@ -519,9 +527,17 @@ static moe_status backward_impl(moe_ctx* ctx, int64_t T, const uint16_t* dy, flo
                       reinterpret_cast<float*>(ws + L.dg), reinterpret_cast<const int32_t*>(ws + L.counts), d_aux, dl,
                       reinterpret_cast<uint16_t*>(ws + L.dl_hi), reinterpret_cast<uint16_t*>(ws + L.dl_lo), st, dbg, /*ready=*/true);
   };
+  // what a GEMM may do: run before its predecessor has ended, if it needs nothing of it; let its successor in, if that is a small
+  // kernel that needs nothing of it (`beside`), or a GEMM
+  const bool overlap = gemms_overlap(s, T);
+  auto chained = [&](bool needs_last, bool beside = false) {
+    io.ready = overlap && !needs_last;
+    io.next_early = overlap || beside;
+  };
   // the router term of dx, and dW_r in slices of the tokens
   auto router_gemms = [&]() -> moe_status {
     if (!tc_router || T == 0) return MOE_OK;
+    chained(false, true);
     GemmIO rio = io;
     rio.ready = true;
     StageTimer tm(c, st, 11);
@@ -539,40 +555,40 @@ static moe_status backward_impl(moe_ctx* ctx, int64_t T, const uint16_t* dy, flo
       launch_unpermute_bwd(s, T, dxp, inv, dl, W_r, dx, st);
     }
   };
-  io.next_early = true;
   if (lora) {
     // base weights frozen: no dW_gate / dW_up / dW_down; the adapter gradients come from skinny GEMMs
-    auto run = [&](LoraOp op, bool ready) {
-      io.ready = ready;
+    auto run = [&](LoraOp op, bool needs_last, bool beside = false) {
+      chained(needs_last, beside);
       if (rc == MOE_OK) rc = launch_lora_gemm(c, op, T, L, ws, io, *lora, st);
     };
     if (T > 0) {  // row GEMMs have no tiles without tokens; weight gradients zero-fill
       StageTimer tm(c, st, 6);
-      run(LORA_W, false);
-      run(LORA_B2, false);
+      run(LORA_W, true);
+      run(LORA_B2, true);
     }
     {
       StageTimer tm(c, st, 7);
-      run(LORA_DB2, true);
-      run(LORA_DA2, true);
+      run(LORA_DB2, false);
+      run(LORA_DA2, false, true);
     }
     if (rc == MOE_OK) router_gradient();
     if (T > 0) {
       StageTimer tm(c, st, 8);
-      run(LORA_Z, true);
-      run(LORA_B4, false);
+      run(LORA_Z, false);
+      run(LORA_B4, true);
     }
     if (rc == MOE_OK) rc = router_gemms();
     {
       StageTimer tm(c, st, 9);  // dx included, which runs beside both
-      run(LORA_DB1, true);
+      run(LORA_DB1, false, true);
       if (rc == MOE_OK) finish_dx();
-      run(LORA_DA1, true);
+      run(LORA_DA1, false);
     }
     if (rc != MOE_OK) return rc;
   } else {
     if (T > 0) {
       StageTimer tm(c, st, 6);
+      chained(true);
       rc = launch_grouped_gemm(c, GEMM_B2, T, L, ws, io, st);
     }
     if (rc != MOE_OK) return rc;
@@ -592,21 +608,24 @@ static moe_status backward_impl(moe_ctx* ctx, int64_t T, const uint16_t* dy, flo
       }
       return MOE_OK;
     };
-    io.ready = true;  // from here on: only the dgrad-down GEMM's results are read, and the dy rows
     {
       StageTimer tm(c, st, 7);
+      chained(false, true);  // from here on only the dgrad-down GEMM's results are read, and here the dy rows
       rc = wgrad(GEMM_B3, 0);
     }
     if (rc != MOE_OK) return rc;
     router_gradient();
     if (T > 0) {
       StageTimer tm(c, st, 8);
+      chained(false, true);
       rc = launch_grouped_gemm(c, GEMM_B4, T, L, ws, io, st);
     }
     if (rc == MOE_OK) rc = router_gemms();
     if (rc != MOE_OK) return rc;
     {
       StageTimer tm(c, st, 9);
+      chained(false, true);
+      io.ready = true;
       rc = wgrad(GEMM_B5, n_groups);
     }
     if (rc != MOE_OK) return rc;

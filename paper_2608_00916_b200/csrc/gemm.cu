@@ -32,12 +32,12 @@ template <int KIND, Accumulate ACC>
 __device__ __forceinline__ void grouped_gemm(const GemmParams& p, const int worker, const int workers) {
   using TR = Traits<KIND>;
   constexpr int EPI_WARPS = 8;
-  extern __shared__ unsigned char gemm_smem_raw[];
-  __shared__ __align__(8) uint64_t bars[2 * STAGES + 5];  // full, empty, accumulator full / empty, drain (failure path)
-  __shared__ uint32_t tmem_base_slot;
+  extern __shared__ __align__(1024) unsigned char gemm_smem_raw[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t smem_base = (smem_u32(gemm_smem_raw) + 1023u) & ~1023u;
-  const uint32_t bar0 = smem_u32(bars);
+  const uint32_t smem_base = smem_u32(gemm_smem_raw);
+  // barriers: full, empty, accumulator full / empty, drain (failure path); behind them the base of the accumulators
+  constexpr int BARS = STAGES * STAGE_BYTES + EPI_BYTES, TMEM_SLOT = BARS + 8 * (2 * STAGES + 5);
+  const uint32_t bar0 = smem_base + BARS;
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
   auto empty_bar = [&](int s) { return bar0 + 8u * (STAGES + s); };
   auto tfull_bar = [&](int a) { return bar0 + 8u * (2 * STAGES + a); };
@@ -60,7 +60,7 @@ __device__ __forceinline__ void grouped_gemm(const GemmParams& p, const int work
     tma_prefetch_desc(&p.mapB0);
   }
   if (warp == 1) {
-    tmem_alloc(smem_u32(&tmem_base_slot), TMEM_COLS);
+    tmem_alloc(smem_base + TMEM_SLOT, TMEM_COLS);
     tmem_relinquish();
   }
   // Row GEMMs of the experts wait for the kernel before them in front of their rows (chain_warp).
@@ -69,7 +69,7 @@ __device__ __forceinline__ void grouped_gemm(const GemmParams& p, const int work
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = tmem_base_slot;
+  const uint32_t tmem_base = *reinterpret_cast<const volatile uint32_t*>(gemm_smem_raw + TMEM_SLOT);
   const int ntiles = total_tiles<KIND>(p);
 
   // The producer and the MMA issuer are one thread each.  What they do per K block (a wait, a few copies or four MMAs, a

@@ -26,7 +26,7 @@ constexpr int STAGES2 = 6;
 constexpr int GEMM2_THREADS = 352;  // warps: 0 TMA producer, 1 MMA issuer, 2..9 epilogue (two per TMEM lane quadrant), 10 chain
 constexpr int BH_BYTES = 128 * BK * 2;              // this CTA's half of B: 16 KB
 constexpr int STAGE2_BYTES = A_BYTES + BH_BYTES;    // 32 KB
-constexpr size_t GEMM2_SMEM = static_cast<size_t>(STAGES2) * STAGE2_BYTES + EPI_BYTES + 1024;
+constexpr size_t GEMM2_SMEM = static_cast<size_t>(STAGES2) * STAGE2_BYTES + EPI_BYTES + BARS_BYTES;
 
 struct Tile2 {
   int e, row0, m0, n0, nkb;
@@ -132,15 +132,15 @@ template <int KIND>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Traits<KIND>::WGRAD ? 512 : GEMM2_THREADS, 1)
     grouped_gemm_pair_kernel(const __grid_constant__ GemmParams p) {
   using TR = Traits<KIND>;
-  extern __shared__ unsigned char gemm2_smem_raw[];
-  __shared__ __align__(8) uint64_t bars[2 * STAGES2 + 5];  // full, empty, accumulator full / empty, drain (failure path)
-  __shared__ uint32_t tmem_base_slot;
+  extern __shared__ __align__(1024) unsigned char gemm2_smem_raw[];
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = static_cast<int>(cluster_ctarank());
   const bool leader = rank == 0;
-  const uint32_t smem_base = (smem_u32(gemm2_smem_raw) + 1023u) & ~1023u;
-  const uint32_t bar0 = smem_u32(bars);
+  const uint32_t smem_base = smem_u32(gemm2_smem_raw);
+  // barriers: full, empty, accumulator full / empty, drain (failure path); behind them the base of the accumulators
+  constexpr int BARS = STAGES2 * STAGE2_BYTES + EPI_BYTES, TMEM_SLOT = BARS + 8 * (2 * STAGES2 + 5);
+  const uint32_t bar0 = smem_base + BARS;
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
   auto empty_bar = [&](int s) { return bar0 + 8u * (STAGES2 + s); };
   auto tfull_bar = [&](int a) { return bar0 + 8u * (2 * STAGES2 + a); };
@@ -163,7 +163,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Traits<KIND>::WGRAD 
     tma_prefetch_desc(&p.mapB0);
   }
   if (warp == 1) {
-    tmem_alloc_pair(smem_u32(&tmem_base_slot), TMEM_COLS);
+    tmem_alloc_pair(smem_base + TMEM_SLOT, TMEM_COLS);
     tmem_relinquish_pair();
   }
   constexpr bool PRELOAD = !TR::WGRAD;  // as in gemm.cu
@@ -171,7 +171,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Traits<KIND>::WGRAD 
   tc_fence_before();
   cluster_sync_all();  // barriers of both CTAs are initialised before anyone signals across the pair
   tc_fence_after();
-  const uint32_t tmem_base = tmem_base_slot;
+  const uint32_t tmem_base = *reinterpret_cast<const volatile uint32_t*>(gemm2_smem_raw + TMEM_SLOT);
   const int ntiles = total_tiles2<KIND>(p);
   const int cid = blockIdx.x >> 1, nclusters = gridDim.x >> 1;
 
