@@ -14,10 +14,11 @@ thread_local Chain* Chain::current_ = nullptr;
 // Whether the large GEMMs begin while the one before them drains (chain_warp in gemm_common.cuh).  With few rows per expert that fills
 // what the ends of the kernels leave idle.  With many, the power cap takes back in clocks what it saves in time, and pairs that begin
 // a GEMM at different times do not share operands as closely.  Steps at d 2048, f 768, 128 experts with against without, us:
-// 62 rows per expert 843 / 861, 512 rows 2306 / 2325, 1024 rows 4202 / 4136 (1024 on average, unequal: 4235 / 4293).  The small kernels
-// run beside the weight gradients, and the router's gradient fills the end of the GEMM before it, at every size: serial, it stood
-// alone for 25 us at 8191 tokens and 57 at 16384.
-static bool gemms_overlap(const Shape& s, int64_t T) { return T * s.k < static_cast<int64_t>(s.E) * 768; }
+// 62 rows per expert 843 / 861, 128 rows 998 / 1018, 375 rows 1902 / 1916, 512 rows 2366 / 2359 (with adapters 2001 / 2070), 656 rows
+// 2896 / 2874, 1024 rows 4202 / 4136 (1024 on average, unequal: 4235 / 4293).  The small kernels run beside the weight
+// gradients, and the router's gradient fills the end of the GEMM before it, at every size: serial, it stood alone for 25 us at 8191
+// tokens and 57 at 16384.
+static bool gemms_overlap(const Shape& s, int64_t T) { return T * s.k < static_cast<int64_t>(s.E) * 576; }
 
 static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 

@@ -16,8 +16,8 @@ pytestmark = pytest.mark.gpu
     (1500, 512, 8, 2, 640, 16),            # pairs, then leftover blocks
     (3000, 2048, 8, 2, 768, FLAG_ROUTER_FP32),
     (40, 64, 64, 2, 64, 0),                # most experts without rows
-    (3071, 512, 8, 2, 640, 0),             # the last size at which the large GEMMs overlap
-    (3072, 512, 8, 2, 640, 0),             # the first at which only the small kernels run beside them
+    (2303, 512, 8, 2, 640, 0),             # the last size at which the large GEMMs overlap
+    (2304, 512, 8, 2, 640, 0),             # the first at which only the small kernels run beside them
 ])
 @pytest.mark.parametrize("mode", ["train", "accumulate", "lora"])
 def test_same_bits_with_and_without_events_between_the_kernels(T, d, E, k, f, flags, mode):
