@@ -517,7 +517,17 @@ static moe_status backward_impl(moe_ctx* ctx, int64_t T, const uint16_t* dy, flo
   }
   // One chain of kernels.  The small ones run beside the GEMM in front of them, whose blocks leave them registers enough: dl
   // (which needs the dgrad-down GEMM) beside the weight gradient of down, dx (dgrad gate/up and dl) beside that of gate and up.
-  // The two GEMMs over dl come in as the blocks of dgrad gate/up leave.
+  // The two GEMMs over dl come in as the blocks of dgrad gate/up leave.  What a `ready` kernel reads, and what orders it (chain_warp):
+  //   weight gradient of down   the dy rows                complete when dgrad-down, its predecessor, triggers
+  //   dl                        dg partials (dgrad-down)   complete when the weight gradient of down triggers
+  //   dgrad gate/up             dhg, dhu (dgrad-down)      its predecessor dl is let in no earlier (dl itself triggers without a wait)
+  //   both GEMMs over dl        dl                         complete when dgrad gate/up triggers
+  //   weight gradients of gate  xp (forward), dhg, dhu     complete when the GEMMs over dl trigger (E % 8 != 0: when dgrad gate/up does)
+  //     and up
+  //   dx                        dxr (the GEMMs over dl),   complete when the weight gradient in front of it triggers (dgrad gate/up ended
+  //                             dxp (dgrad gate/up)        before the GEMMs over dl did)
+  // and with adapters: dB2 the dy rows, dA2 the 64-wide buffer w, dl the dg partials (complete when dA2 triggers), z dhg and dhu, the two
+  // GEMMs over dl behind dgrad gate/up as above, dB1 dhg and dhu, dx beside dB1, dA1 the buffer z.
   int32_t* const dbg = c->debug_checks ? reinterpret_cast<int32_t*>(ws + L.status) : nullptr;
   const uint16_t* const dxp = reinterpret_cast<const uint16_t*>(ws + L.dxp);
   const bool one_slice = dwr_in_one_slice(T, dW_r);

@@ -346,7 +346,8 @@ __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait
 // Lets the next kernel of the chain be set up once every block of this one has got here or ended.
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // A small kernel whose inputs were complete before its predecessor in the chain began (ready) runs beside that one: chain_enter()
-// first, chain_leave() last, where one block waits for the predecessor, so that this kernel's end still stands for that one's.
+// first, chain_leave() last, where one block waits for the predecessor, so that this kernel's end still stands for that one's.  It lets
+// its successor in at once, whose start therefore says nothing about this kernel's predecessor (chain_warp in gemm_common.cuh).
 __device__ __forceinline__ void chain_enter(int ready) {
   if (!ready) chain_wait();
   chain_next();

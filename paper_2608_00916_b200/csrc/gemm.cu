@@ -116,8 +116,11 @@ __device__ __forceinline__ void grouped_gemm(const GemmParams& p, const int work
           pos.next(STAGES);
         }
       }
-      chain_next();  // not earlier without next_early: blocks of the next kernel that only wait would sit beside the main loop
       clk.report(0, 1);  // total; waiting for a free stage
+      // Not earlier without next_early: blocks of the next kernel that only wait would sit beside the main loop.  A trigger comes after
+      // a wait everywhere (chain_warp): a `ready` block without tiles, or whose K loop fits the ring, gets here while its predecessor runs.
+      if (p.ready) chain_wait();
+      chain_next();
       if (!ok) {
         // gave up: the copies already issued still land in this CTA's shared memory - wait for them (bounded again)
         // before the CTA may exit

@@ -514,8 +514,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TK_THREADS, 1)
           }
         }
       }
-      chain_next();
       clk.report(0, 1);
+      if (p.ready) chain_wait();  // as in gemm.cu
+      chain_next();
       if (!ok) {
         // gave up: the leader waits (bounded) for the copies of BOTH CTAs that were already issued, all credited to its full
         // barriers, so that neither CTA exits with copies in flight (the cluster barrier below holds the partner until then)

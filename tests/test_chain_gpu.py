@@ -19,7 +19,7 @@ pytestmark = pytest.mark.gpu
     (2303, 512, 8, 2, 640, 0),             # the last size at which the large GEMMs overlap
     (2304, 512, 8, 2, 640, 0),             # the first at which only the small kernels run beside them
 ])
-@pytest.mark.parametrize("mode", ["train", "accumulate", "lora"])
+@pytest.mark.parametrize("mode", ["train", "accumulate", "grouped", "lora"])
 def test_same_bits_with_and_without_events_between_the_kernels(T, d, E, k, f, flags, mode):
     if mode == "lora" and flags & FLAG_ROUTER_FP32:
         pytest.skip("adapters take a bf16 router weight")
@@ -41,10 +41,12 @@ def test_same_bits_with_and_without_events_between_the_kernels(T, d, E, k, f, fl
         else:
             out = layer.forward(x, *W)
             if mode == "train":
-                grads = layer.backward(dy, 0.01)
+                grads = layer.backward(dy, 0.01, want_db=True)
             else:
                 acc = {m: torch.ones(w.shape, device="cuda") for m, w in zip(("dW_r", "dW_gate", "dW_up", "dW_down"), W)}
-                grads = {"dx": layer.backward_accumulate(dy, 0.01, acc), **acc}
+                acc["db_r"] = torch.ones(E, device="cuda")
+                events = [torch.cuda.Event() for _ in range(6)] if mode == "grouped" else None  # three ranges of experts
+                grads = {"dx": layer.backward_accumulate(dy, 0.01, acc, group_events=events), **acc}
         return {"y": out["y"], **grads}
 
     layer.set_profiling(True)

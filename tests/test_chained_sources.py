@@ -30,6 +30,23 @@ def test_predecessor_outputs_are_not_declared_read_only():
     assert kernels >= 12
 
 
+def test_a_gemm_lets_its_successor_in_only_after_waiting():
+    """Small kernels beside a GEMM read what its predecessor has written without a wait of their own: the first trigger of a block
+    counts, so that each of its threads that triggers has waited.  (The other threads wait in front of the rows unless `ready`.)"""
+    for name in ("gemm.cu", "gemm2.cu", "gemm_tokens.cu"):
+        with open(os.path.join(CSRC, name)) as f:
+            lines = [line.split("//")[0].strip() for line in f]
+        triggers = [i for i, line in enumerate(lines) if "chain_next()" in line]
+        assert triggers, name
+        for i in triggers:
+            assert lines[i - 1 : i + 1] == ["if (p.ready) chain_wait();", "chain_next();"], f"{name}:{i + 1}"
+        assert any(line == "chain_warp(p.next_early);" for line in lines), name
+    with open(os.path.join(CSRC, "gemm_common.cuh")) as f:
+        text = f.read()
+    assert text.count("chain_next()") == 1
+    assert re.search(r"void chain_warp\(int next_early\) \{\s+chain_wait\(\);\s+if \(next_early\) chain_next\(\);\s+\}", text)
+
+
 def test_non_coherent_loads_are_of_inputs_only():
     loads = [(name, arg) for name, text in sources() for arg in re.findall(r"__ldg\(([^;]*)\);", text)]
     assert loads
