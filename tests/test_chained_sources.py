@@ -17,17 +17,35 @@ def sources():
             yield name, f.read()
 
 
+def chained_kernels(text):
+    """(name, parameter list, start, body) of every kernel whose body starts with the chain's wait, or with chain_enter."""
+    for m in re.finditer(r"__global__ [^;{]*?(\w+)\(([^{;]*?)\) \{\s+(chain_wait\(\)|chain_enter\(\w+\));", text):
+        yield m.group(1), m.group(2), m.group(3), text[m.end() : text.index("\n}\n", m.end()) + 1]
+
+
 def test_predecessor_outputs_are_not_declared_read_only():
-    kernels = 0
+    kernels = set()
     for name, text in sources():
-        for m in re.finditer(r"__global__ [^;{]*?(\w+)\(([^{;]*?)\) \{\s+chain_wait\(\);", text):
-            kernels += 1
-            for param in m.group(2).split(","):
+        for kernel, params, _, _ in chained_kernels(text):
+            kernels.add(kernel)
+            for param in params.split(","):
                 if "const" in param and "__restrict__" in param:
-                    assert param.split()[-1] in INPUTS, f"{name}: {m.group(1)}: {param.strip()}"
+                    assert param.split()[-1] in INPUTS, f"{name}: {kernel}: {param.strip()}"
         for helper, what in (("build_masks", "idx"), ("psum_columns", "psum_part"), ("scan_kernel", "tile_counts")):
             assert not re.search(helper + r"\([^{;]*__restrict__ " + what + r"\b", text), f"{name}: {helper}: {what}"
-    assert kernels >= 12
+    # those that may run beside their predecessor among them
+    assert {"router_bwd_kernel", "unpermute_sum_kernel", "dwr_partial_kernel", "unpermute_bwd_kernel"} <= kernels
+    assert len(kernels) == 15
+
+
+def test_a_kernel_beside_its_predecessor_ends_after_it():
+    for name, text in sources():
+        for kernel, _, start, body in chained_kernels(text):
+            if start.startswith("chain_enter"):
+                flag = start[len("chain_enter") :]
+                assert body.endswith(f"  chain_leave{flag};\n"), f"{name}: {kernel}"
+            else:
+                assert "chain_leave" not in body, f"{name}: {kernel}"
 
 
 def test_a_gemm_lets_its_successor_in_only_after_waiting():
