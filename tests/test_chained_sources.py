@@ -19,7 +19,7 @@ def sources():
 
 def chained_kernels(text):
     """(name, parameter list, start, body) of every kernel whose body starts with the chain's wait, or with chain_enter."""
-    for m in re.finditer(r"__global__ [^;{]*?(\w+)\(([^{;]*?)\) \{\s+(chain_wait\(\)|chain_enter\(\w+\));", text):
+    for m in re.finditer(r"__global__ [^;{(]*(?:__launch_bounds__\([^)]*\)\s+[^;{(]*)?\b(\w+)\(([^{;]*?)\) \{\s+(chain_wait\(\)|chain_enter\(\w+\));", text):
         yield m.group(1), m.group(2), m.group(3), text[m.end() : text.index("\n}\n", m.end()) + 1]
 
 
