@@ -526,6 +526,8 @@ static moe_status backward_impl(moe_ctx* ctx, int64_t T, const uint16_t* dy, flo
   //     and up
   //   dx                        dxr (the GEMMs over dl),   complete when the weight gradient in front of it triggers (dgrad gate/up ended
   //                             dxp (dgrad gate/up)        before the GEMMs over dl did)
+  //   E % 8 != 0: dW_r's        dl, and dx also dxp        complete when the weight gradient in front of both triggers: its predecessor is
+  //     partial sums, dx                                   dgrad gate/up, which ended after dl
   // and with adapters: dB2 the dy rows, dA2 the 64-wide buffer w, dl the dg partials (complete when dA2 triggers), z dhg and dhu, the two
   // GEMMs over dl behind dgrad gate/up as above, dB1 dhg and dhu, dx beside dB1, dA1 the buffer z.
   int32_t* const dbg = c->debug_checks ? reinterpret_cast<int32_t*>(ws + L.status) : nullptr;
@@ -558,13 +560,23 @@ static moe_status backward_impl(moe_ctx* ctx, int64_t T, const uint16_t* dy, flo
     }
     return launch_router_gradient(c, T, L, ws, rio, st);
   };
+  // Without tensor cores for the router dW_r's partial sums go in front of dx: both come in as the blocks of the weight gradient leave
+  // (their shared memory does not fit beside one) and run together, the one bound by arithmetic, the other by HBM.  Waiting for
+  // the weight gradient one after the other -> so, us a step: 60 experts of f 1408, 1000 / 4096 / 16384 tokens 963 / 1933 / 6000 -> 957 /
+  // 1851 / 5620, 100 of f 768 at 8192 tokens 4238 -> 4022, d 1024, 12 of f 768 at 2048 tokens 310 -> 280.  The partial sums behind dx: 943 /
+  // 1909 / 5856, 4138, 291; in front of the weight gradient: 968 / 1871 / 5833, 4153, 299.
   auto finish_dx = [&]() {
-    StageTimer tm(c, st, 12);
     if (tc_router && T > 0) {
+      StageTimer tm(c, st, 12);
       launch_unpermute_sum(s, T, dxp, inv, reinterpret_cast<const uint16_t*>(ws + L.dxr), dx, st, dbg, L.rows_max, /*ready=*/true);
-    } else {
-      launch_unpermute_bwd(s, T, dxp, inv, dl, W_r, dx, st);
+      return;
     }
+    {
+      StageTimer tm(c, st, 11);
+      launch_dwr_partial(s, T, x, dl, reinterpret_cast<float*>(ws + L.dwr_part), st, /*ready=*/true);
+    }
+    StageTimer tm(c, st, 12);
+    launch_unpermute_bwd(s, T, dxp, inv, dl, W_r, dx, st, /*ready=*/true);
   };
   if (lora) {
     // base weights frozen: no dW_gate / dW_up / dW_down; the adapter gradients come from skinny GEMMs
@@ -642,7 +654,7 @@ static moe_status backward_impl(moe_ctx* ctx, int64_t T, const uint16_t* dy, flo
     if (rc != MOE_OK) return rc;
   }
   if (!lora) finish_dx();
-  launch_dwr(s, T, x, dl, reinterpret_cast<float*>(ws + L.dwr_part), dW_r, db_r, tc_router && T > 0, st, accumulate, tc_router && one_slice);
+  launch_dwr(s, T, x, dl, reinterpret_cast<float*>(ws + L.dwr_part), dW_r, db_r, /*partials_ready=*/true, st, accumulate, tc_router && one_slice);
   if (c->profiling) c->prof_step++;
   return cudaGetLastError() == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
 }

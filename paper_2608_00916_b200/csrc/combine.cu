@@ -171,9 +171,8 @@ void launch_router_bwd(const Shape& s, int64_t T, const float* logits, const int
 constexpr int DW_BM = 64, DW_BK = 32;
 
 __global__ void __launch_bounds__(256) dwr_partial_kernel(int64_t T, int d, int E, const uint16_t* __restrict__ x,
-                                                          const float* dl, float* __restrict__ part) {
-  chain_wait();
-  chain_next();
+                                                          const float* dl, float* __restrict__ part, int ready) {
+  chain_enter(ready);
   // thread layout: 16 (row groups of 4) x 16 (column groups); columns handled: cg + 16*i for i < E/16 (<= 16)
   __shared__ float xs[DW_BK][DW_BM];        // x^T tile
   extern __shared__ float dls[];            // [DW_BK][E]
@@ -228,6 +227,7 @@ __global__ void __launch_bounds__(256) dwr_partial_kernel(int64_t T, int d, int 
       int e = cg + 16 * j;
       if (j < NC && e < E) dst[static_cast<int64_t>(c0 + rg * 4 + i) * E + e] = acc[i][j];
     }
+  chain_leave(ready);
 }
 
 __global__ void dwr_reduce_kernel(int64_t n, const float* part, float* __restrict__ dW_r,
@@ -263,13 +263,15 @@ __global__ void __launch_bounds__(256) dbr_kernel(int64_t T, int E, const float*
   }
 }
 
+void launch_dwr_partial(const Shape& s, int64_t T, const uint16_t* x, const float* dl, float* part, cudaStream_t st, bool ready) {
+  const dim3 grid(s.d / DW_BM, DWR_SPLIT);
+  launch_kernel(dwr_partial_kernel, grid, 256, sizeof(float) * DW_BK * s.E, st, T, s.d, s.E, x, dl, part, ready ? 1 : 0);
+}
+
 void launch_dwr(const Shape& s, int64_t T, const uint16_t* x, const float* dl, float* part, float* dW_r,
                 float* db_r, bool partials_ready, cudaStream_t st, bool accumulate, bool complete) {
   const int64_t n = static_cast<int64_t>(s.d) * s.E;
-  if (!partials_ready && !complete) {
-    dim3 grid(s.d / DW_BM, DWR_SPLIT);
-    launch_kernel(dwr_partial_kernel, grid, 256, sizeof(float) * DW_BK * s.E, st, T, s.d, s.E, x, dl, part);
-  }
+  if (!partials_ready && !complete) launch_dwr_partial(s, T, x, dl, part, st);
   if (!complete)
     launch_kernel(dwr_reduce_kernel, static_cast<unsigned>((n + 255) / 256), 256, 0, st, n, part, dW_r,
                   accumulate ? 1 : 0);
@@ -288,9 +290,8 @@ __global__ void __launch_bounds__(256) unpermute_bwd_kernel(int64_t T, int d, in
                                                             const int32_t* inv,
                                                             const float* dl,
                                                             const uint16_t* __restrict__ W_r,
-                                                            uint16_t* __restrict__ dx) {
-  chain_wait();
-  chain_next();
+                                                            uint16_t* __restrict__ dx, int ready) {
+  chain_enter(ready);
   extern __shared__ float ub_dl[];  // [UB_TOK][E]
   __shared__ int s_inv[UB_TOK][MAX_K];
   const int64_t t0 = static_cast<int64_t>(blockIdx.x) * UB_TOK;
@@ -370,6 +371,7 @@ __global__ void __launch_bounds__(256) unpermute_bwd_kernel(int64_t T, int d, in
       }
     }
   }
+  chain_leave(ready);
 }
 
 // dx[t,:] = dxr[t,:] + sum_j dxp[inv[t,j],:]; one block per token, 16-byte accesses, all row loads in flight at once.
@@ -426,10 +428,10 @@ void launch_unpermute_sum(const Shape& s, int64_t T, const uint16_t* dxp, const 
 }
 
 void launch_unpermute_bwd(const Shape& s, int64_t T, const uint16_t* dxp, const int32_t* inv, const float* dl,
-                          const uint16_t* W_r, uint16_t* dx, cudaStream_t st) {
+                          const uint16_t* W_r, uint16_t* dx, cudaStream_t st, bool ready) {
   if (T == 0) return;
   launch_kernel(unpermute_bwd_kernel, static_cast<unsigned>((T + UB_TOK - 1) / UB_TOK), 256,
-                sizeof(float) * UB_TOK * s.E, st, T, s.d, s.E, s.k, dxp, inv, dl, W_r, dx);
+                sizeof(float) * UB_TOK * s.E, st, T, s.d, s.E, s.k, dxp, inv, dl, W_r, dx, ready ? 1 : 0);
 }
 
 }  // namespace moe

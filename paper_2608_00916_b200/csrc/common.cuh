@@ -179,11 +179,13 @@ void launch_router_bwd(const Shape& s, int64_t T, const float* logits, const int
                        const int32_t* counts, float d_aux, float* dl, uint16_t* dl_hi, uint16_t* dl_lo,
                        cudaStream_t st, int32_t* dbg_status = nullptr, bool ready = false);
 // dg_tiles == 0: dg[t,j] has been filled by the caller (expert-parallel path) and is read instead of the partials
-// SIMT dW_r (any E) and the shared partial reduction / db_r; complete: dW_r needs neither
+// SIMT dW_r (any E): partial sums of token slices; launch_dwr: their sum and db_r (the partials too unless partials_ready; complete:
+// dW_r needs neither)
+void launch_dwr_partial(const Shape& s, int64_t T, const uint16_t* x, const float* dl, float* part, cudaStream_t st, bool ready = false);
 void launch_dwr(const Shape& s, int64_t T, const uint16_t* x, const float* dl, float* part, float* dW_r,
                 float* db_r, bool partials_ready, cudaStream_t st, bool accumulate = false, bool complete = false);
 void launch_unpermute_bwd(const Shape& s, int64_t T, const uint16_t* dxp, const int32_t* inv, const float* dl,
-                          const uint16_t* W_r, uint16_t* dx, cudaStream_t st);
+                          const uint16_t* W_r, uint16_t* dx, cudaStream_t st, bool ready = false);
 // dx[t,:] = dxr[t,:] + sum_j dxp[inv[t,j],:]  (router term already contracted on the tensor cores)
 void launch_unpermute_sum(const Shape& s, int64_t T, const uint16_t* dxp, const int32_t* inv, const uint16_t* dxr,
                           uint16_t* dx, cudaStream_t st, int32_t* dbg_status = nullptr, int64_t rows_max = 0, bool ready = false);

@@ -39,13 +39,18 @@ def test_predecessor_outputs_are_not_declared_read_only():
 
 
 def test_a_kernel_beside_its_predecessor_ends_after_it():
+    beside = set()
     for name, text in sources():
         for kernel, _, start, body in chained_kernels(text):
             if start.startswith("chain_enter"):
+                beside.add(kernel)
                 flag = start[len("chain_enter") :]
                 assert body.endswith(f"  chain_leave{flag};\n"), f"{name}: {kernel}"
             else:
                 assert "chain_leave" not in body, f"{name}: {kernel}"
+    # all small kernels of the backward pass that need nothing of the weight gradient in front of them, with the router on tensor
+    # cores and without
+    assert beside == {"router_bwd_kernel", "unpermute_sum_kernel", "dwr_partial_kernel", "unpermute_bwd_kernel"}
 
 
 def test_a_gemm_lets_its_successor_in_only_after_waiting():
