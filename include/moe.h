@@ -144,9 +144,11 @@ MOE_API moe_status moe_selftest_timeout(moe_ctx* ctx, void* workspace, void* cud
  * of them if there were more), stores that number of pairs in *steps, and starts a new window.
  * Stage order: 0 router, 1 permute (histogram, scan, scatter, gather), 2 gate/up GEMM + SwiGLU,
  * 3 down GEMM, 4 combine, 5 combine-bwd (gather of dy rows), 6 dgrad-down + SwiGLU-bwd (+ dg), 7 wgrad-down, 8 dgrad gate/up,
- * 9 wgrad gate/up, 10 router-bwd (dl), 11 dW_r and the router term of dx, 12 unpermute-bwd (dx), 13..15 unused.
+ * 9 wgrad gate/up, 10 router-bwd (dl), 11 dW_r and the router term of dx (one launch; with a number of experts that is no multiple
+ * of 8 dW_r's partial sums alone), 12 unpermute-bwd (dx), 13 sum of dW_r's partial sums and db_r, 14..15 unused.
  * The events keep the kernels of a call apart; without them stages 10 and 12 run beside stages 7 and 9 and each GEMM begins
- * while the one before it drains, so the stage times add up to more than the step. */
+ * while the one before it drains, so the stage times add up to more than the step.  In moe_lora_backward stage 9 is everything from
+ * the gradients of B1 to that of A1, stage 12 (and 11, where it stands in front of it) included. */
 #define MOE_PROF_RING 64
 MOE_API moe_status moe_set_profiling(moe_ctx* ctx, int enable);
 MOE_API moe_status moe_stage_times(moe_ctx* ctx, float* ms /* host */, int32_t* steps /* host */);

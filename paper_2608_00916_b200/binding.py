@@ -17,7 +17,7 @@ FLAG_ROUTER_FP32 = 32      # MOE_FLAG_ROUTER_FP32
 FLAG_DEBUG_CHECKS = 64     # MOE_FLAG_DEBUG_CHECKS
 STAGE_NAMES = ["router", "permute", "gemm_gateup_swiglu", "gemm_down", "combine", "combine_bwd",
                "dgrad_down_swiglu_bwd", "wgrad_down", "dgrad_gateup", "wgrad_gateup", "router_bwd", "dW_r",
-               "unpermute_bwd", "dx_router_term"]
+               "unpermute_bwd", "dW_r_sum"]
 EXPORTS = ["moe_create", "moe_destroy", "moe_workspace_bytes", "moe_workspace_find", "moe_status_string",
            "moe_poll_status", "moe_set_profiling", "moe_stage_times", "moe_forward", "moe_backward",
            "moe_e2e_device_bytes", "moe_step_host", "moe_router_wgrad_static", "moe_selftest_timeout",

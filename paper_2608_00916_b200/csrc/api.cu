@@ -654,7 +654,10 @@ static moe_status backward_impl(moe_ctx* ctx, int64_t T, const uint16_t* dy, flo
     if (rc != MOE_OK) return rc;
   }
   if (!lora) finish_dx();
-  launch_dwr(s, T, x, dl, reinterpret_cast<float*>(ws + L.dwr_part), dW_r, db_r, /*partials_ready=*/true, st, accumulate, tc_router && one_slice);
+  {
+    StageTimer tm(c, st, 13);
+    launch_dwr(s, T, x, dl, reinterpret_cast<float*>(ws + L.dwr_part), dW_r, db_r, /*partials_ready=*/true, st, accumulate, tc_router && one_slice);
+  }
   if (c->profiling) c->prof_step++;
   return cudaGetLastError() == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
 }

@@ -3,7 +3,7 @@ without a pause on one workspace and on alternating inputs (a read that came too
 import pytest
 import torch
 
-from paper_2608_00916_b200.binding import FLAG_ROUTER_FP32, MoELayer
+from paper_2608_00916_b200.binding import FLAG_ROUTER_FP32, STAGE_NAMES, MoELayer
 
 pytestmark = pytest.mark.gpu
 
@@ -59,3 +59,20 @@ def test_same_bits_with_and_without_events_between_the_kernels(T, d, E, k, f, fl
         for name, v in apart[i % 2].items():
             if v is not None:
                 assert torch.equal(got[name], v), (i, name)
+
+
+@pytest.mark.parametrize("E", [16, 12])  # the router's gradient on tensor cores, and without
+def test_every_stage_of_a_step_is_timed(E):
+    T, d, k, f = 700, 512, 2, 256
+    g = torch.Generator(device="cuda")
+    g.manual_seed(E)
+    n = lambda *s: torch.empty(*s, device="cuda").normal_(0, 0.05, generator=g).bfloat16()
+    x, W, dy = n(T, d), (n(d, E), n(E, d, f), n(E, d, f), n(E, f, d)), n(T, d)
+    layer = MoELayer(d, E, f, k)
+    layer.set_profiling(True)
+    for _ in range(2):
+        layer.forward(x, *W)
+        layer.backward(dy, 0.01)
+    stages, steps = layer.stage_times()
+    assert steps == 2 and len(STAGE_NAMES) == 14
+    assert all(ms > 0 for ms in stages[:14]) and not any(stages[14:]), stages
