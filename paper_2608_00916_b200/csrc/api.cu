@@ -224,6 +224,7 @@ moe_status moe_workspace_find(const moe_ctx* ctx, int64_t T, const char* name, s
              {"dg", L.dg, sizeof(float) * R},
              {"dl", L.dl, sizeof(float) * T * s.E},
              {"status", L.status, sizeof(int32_t) * 16},
+             {"pace", L.pace, sizeof(int32_t) * PACE_KINDS * PACE_SLOTS},
              {"timers", L.timers, sizeof(long long) * 16 * 8}};
   for (const Ent& e : tab)
     if (strcmp(e.n, name) == 0) {

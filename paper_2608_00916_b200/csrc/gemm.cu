@@ -357,9 +357,9 @@ static int wgrad_group_for(int n_tiles, double rows_per_expert, int64_t columns,
 
 // Whether the pairs of a GEMM keep step (Pace): where L2 does not hold what they share - the weights of wide experts, which row GEMMs
 // walk in groups, or the operands of one expert's weight gradient (24 MB as above) - and tiles are long, from 32 K blocks (about
-// 14 us) on: a round begins with a question that takes 1 us.
-static bool keeps_step(int row_group, bool wgrad, double k_blocks, double operand_bytes) {
-  return k_blocks >= 32.0 && (wgrad ? operand_bytes >= 24e6 : row_group > 1);
+// 14 us) on: a round begins with a question that takes 1 us.  MOE_ROW_GROUP=1 lets all pairs run freely (measurements).
+static bool keeps_step(int row_group, bool wgrad, double k_blocks, double operand_bytes, const moe_ctx_impl* ctx) {
+  return ctx->row_group_override != 1 && k_blocks >= 32.0 && (wgrad ? operand_bytes >= 24e6 : row_group > 1);
 }
 
 // Forward-only calls leave pad rows alone (nothing reads them afterwards), which at few rows per expert is most of what
@@ -428,7 +428,7 @@ static moe_status launch_gemm_variant(moe_ctx_impl* ctx, GemmKind kind, int64_t 
     const bool wgrad = kind == GEMM_B3 || kind == GEMM_B5;
     const double blocks = wgrad ? rows_per_expert / BK : p.k_blocks * p.nseg;
     const double operands = rows_per_expert * 2.0 * (kind == GEMM_B5 ? d + 2.0 * f : d + static_cast<double>(f));
-    if (part == 0 && keeps_step(p.row_group, wgrad, blocks, operands)) p.pace = reinterpret_cast<int32_t*>(ws + L.pace) + kind * PACE_SLOTS;
+    if (part == 0 && keeps_step(p.row_group, wgrad, blocks, operands, ctx)) p.pace = reinterpret_cast<int32_t*>(ws + L.pace) + kind * PACE_SLOTS;
     return launch_pair_gemm(ctx, kind, p, st);
   };
   bool ok = true;
