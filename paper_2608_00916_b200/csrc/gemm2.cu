@@ -26,6 +26,7 @@ constexpr int STAGES2 = 6;
 constexpr int GEMM2_THREADS = 352;  // warps: 0 TMA producer, 1 MMA issuer, 2..9 epilogue (two per TMEM lane quadrant), 10 chain
 constexpr int BH_BYTES = 128 * BK * 2;              // this CTA's half of B: 16 KB
 constexpr int STAGE2_BYTES = A_BYTES + BH_BYTES;    // 32 KB
+static_assert(ring_fits(STAGES2, STAGE2_BYTES));
 constexpr size_t GEMM2_SMEM = static_cast<size_t>(STAGES2) * STAGE2_BYTES + EPI_BYTES + BARS_BYTES;
 
 struct Tile2 {

@@ -96,6 +96,16 @@ def test_a_failed_launch_of_a_gemm_is_reported_once():
             assert re.search(r"  launch_kernel\([^;]*;\n  return cudaGetLastError\(\) == cudaSuccess \? MOE_OK : MOE_ERR_CUDA;", text), name
 
 
+def test_the_ring_of_a_gemm_starts_its_shared_memory():
+    """The operand tiles' swizzle needs stages at multiples of 1024 bytes: the ring is the dynamic memory itself, declared aligned, and
+    nothing static lies in front of it."""
+    for name, text in sources():
+        if name in ("gemm.cu", "gemm2.cu", "gemm_common.cuh"):
+            declared = re.findall(r"[^\n]*__shared__[^\n]*", text)
+            assert all(re.match(r"\s*extern __shared__ __align__\(1024\) unsigned char \w+\[\];", line) for line in declared), name
+            assert len(declared) == (name != "gemm_common.cuh"), name
+
+
 def compiles(tmp_path, argument):
     src = tmp_path / "launch.cu"
     src.write_text('#include "common.cuh"\n'
