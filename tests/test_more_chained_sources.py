@@ -33,3 +33,11 @@ def test_a_failed_launch_is_reported_once():
 def test_every_row_gemm_walks_its_tiles_in_groups_by_one_rule():
     text = dict(rules.sources())["gemm_tokens.cu"]
     assert "p.row_group = row_group_for(" in text
+
+
+def test_the_issuer_looks_a_tile_up_before_its_loop():
+    """Producer and issuer are one thread each, and what they do per K block sets the pace: nothing there but barriers, copies and MMAs."""
+    text = dict(rules.sources())["gemm_tokens.cu"]
+    loop = text[text.index("for (int kb = 0; kb < nkb; ++kb) {") : text.index("umma_commit_pair_both(done);")]
+    assert "idesc =" not in loop and not any(name in loop for name in ("__shared__", "get_token_tile", "stage_n"))
+    assert text.count("__shared__") == 3  # dynamic memory, the barriers, the base of the accumulators
