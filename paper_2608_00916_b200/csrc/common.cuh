@@ -101,8 +101,8 @@ struct moe_ctx_impl {
   int b4_pair_override;    // MOE_B4_PAIR = 0 / 1, if set (measurements: dgrad gate/up on one-CTA tiles / CTA pairs); else -1
   // cudaFuncSetAttribute (dynamic shared memory opt-in) is per device: remembered here, for the device the context is
   // bound to, per kernel family (0: one-CTA kernels, 1: CTA-pair kernels, 2: one-CTA
-  // weight gradients that load and add, 3: row GEMMs with the tokens as N) and GEMM kind
-  unsigned char attr_done[4][16];
+  // weight gradients that load and add, 3: row GEMMs with the tokens as N, 4: CTA pairs that keep step) and GEMM kind
+  unsigned char attr_done[5][16];
   unsigned router_attr;  // the same for the forms of the tensor-core router, one bit each
   int profiling;
   cudaEvent_t ev[MOE_PROF_RING][MOE_NUM_STAGES][2];

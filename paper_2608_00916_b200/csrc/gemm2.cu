@@ -129,7 +129,10 @@ __device__ __forceinline__ void issue_loads2(const GemmParams& p, const Tile2& t
 
 // The bound of 512 threads keeps the weight gradients at 128 registers: blocks of the bandwidth-bound kernels of the chain have to
 // fit beside them.
-template <int KIND>
+// PACED: the pairs keep step (Pace).  A kernel of its own: the question at every K block whether the end of a tile is near costs the copy
+// thread time where tiles are short, also when no counters are given - F4 of 12 K blocks at d 2048, f 768 2 % (388 -> 396 us at 1024 rows per
+// expert, 723 -> 739 at 2048), the weight gradients 1 %; as two loops with the question between them F4 takes 6 % longer.
+template <int KIND, bool PACED>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Traits<KIND>::WGRAD ? 512 : GEMM2_THREADS, 1)
     grouped_gemm_pair_kernel(const __grid_constant__ GemmParams p) {
   using TR = Traits<KIND>;
@@ -184,7 +187,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Traits<KIND>::WGRAD 
       bool ok = true;
       RoleClock clk(leader ? p.timers : nullptr);
       int kb = 0;  // the first K block of the first tile that is not on its way yet
-      Pace pace(leader ? p.pace : nullptr, nclusters);
+      Pace pace(PACED && leader ? p.pace : nullptr, nclusters);
       if (PRELOAD) {
         const Tile2 tl = cid < ntiles ? get_tile2<KIND>(p, cid, rank) : Tile2{};
         const int pre = cid < ntiles ? min(STAGES2, p.k_blocks) : 0;
@@ -202,11 +205,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Traits<KIND>::WGRAD 
         const int t = tile_of_round<KIND>(rd, cid, nclusters);
         if (t >= ntiles) continue;
         const Tile2 tl = get_tile2<KIND>(p, t, rank);
-        pace.begin(rd);
-        const int mark = max(tl.nkb - PACE_MARGIN, kb);
-        if (tl.nkb <= kb) pace.near_end(rd);
+        int mark = 0;
+        if (PACED) {
+          pace.begin(rd);
+          mark = max(tl.nkb - PACE_MARGIN, kb);
+          if (tl.nkb <= kb) pace.near_end(rd);
+        }
         for (; kb < tl.nkb; ++kb, ++it) {
-          if (kb == mark) pace.near_end(rd);
+          if (PACED && kb == mark) pace.near_end(rd);
           clk.start();
           if (!mbar_wait(empty_bar(pos.s), pos.phase ^ 1u)) {
             ok = false;
@@ -355,17 +361,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Traits<KIND>::WGRAD 
   }
 }
 
-template <int KIND>
-static moe_status launch_pair_kind(moe_ctx_impl* ctx, const GemmParams& p, cudaStream_t st) {
-  if (!ctx->attr_done[1][KIND]) {  // per device: the context is bound to one
-    if (cudaFuncSetAttribute(grouped_gemm_pair_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(GEMM2_SMEM)) != cudaSuccess)
+template <int KIND, bool PACED>
+static moe_status launch_pair_kernel(moe_ctx_impl* ctx, const GemmParams& p, cudaStream_t st) {
+  auto* const kernel = grouped_gemm_pair_kernel<KIND, PACED>;
+  unsigned char* const done = &ctx->attr_done[PACED ? 4 : 1][KIND];
+  if (!*done) {  // per device: the context is bound to one
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(GEMM2_SMEM)) != cudaSuccess)
       return MOE_ERR_CUDA;
-    ctx->attr_done[1][KIND] = 1;
+    *done = 1;
   }
   const int grid = ctx->sm_count & ~1;  // whole pairs
-  launch_kernel(grouped_gemm_pair_kernel<KIND>, grid, GEMM2_THREADS, GEMM2_SMEM, st, p);
+  launch_kernel(kernel, grid, GEMM2_THREADS, GEMM2_SMEM, st, p);
   return cudaGetLastError() == cudaSuccess ? MOE_OK : MOE_ERR_CUDA;
+}
+
+template <int KIND>
+static moe_status launch_pair_kind(moe_ctx_impl* ctx, const GemmParams& p, cudaStream_t st) {
+  return p.pace ? launch_pair_kernel<KIND, true>(ctx, p, st) : launch_pair_kernel<KIND, false>(ctx, p, st);
 }
 
 moe_status launch_pair_gemm(moe_ctx_impl* ctx, GemmKind kind, const GemmParams& p, cudaStream_t st) {

@@ -106,6 +106,15 @@ def test_the_ring_of_a_gemm_starts_its_shared_memory():
             assert len(declared) == (name != "gemm_common.cuh"), name
 
 
+def test_pairs_that_run_freely_ask_nothing_per_k_block():
+    """What the copy thread does per K block sets the pace of short tiles: only the kernels that keep step ask where a tile's end is."""
+    with open(os.path.join(CSRC, "gemm2.cu")) as f:
+        text = f.read()
+    loop = text[text.index("for (; kb < tl.nkb; ++kb, ++it) {") : text.index("issue_loads2<KIND>(p, tl, kb, rank, sA")]
+    asks = [line for line in loop.splitlines() if "pace" in line]
+    assert asks and all("if (PACED &&" in line for line in asks)
+
+
 def compiles(tmp_path, argument):
     src = tmp_path / "launch.cu"
     src.write_text('#include "common.cuh"\n'
