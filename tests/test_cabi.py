@@ -65,6 +65,19 @@ def test_workspace_arithmetic(lib):
         assert o1 + n1 <= o2
 
 
+@pytest.mark.parametrize("T", [1, 241, 1000, 8191, 16384, 32768])
+@pytest.mark.parametrize("d,E,f,k", [(2048, 128, 768, 8), (320, 12, 192, 3), (4096, 8, 14336, 2)])
+def test_row_buffers_start_at_whole_pages(lib, T, d, E, f, k):
+    """Wherever the tables in front of them end: row copies are slower at odd multiples of 512 bytes."""
+    layer = binding.MoELayer(d, E, f, k)
+    end = 0
+    for name in ("xp", "act", "o", "hg", "hu", "dhg", "dhu", "dxp", "dxr"):
+        off, n = layer.find(T, name)
+        assert off % 4096 == 0 and off >= end, name
+        end = off + n
+    assert end <= layer.workspace_bytes(T)
+
+
 def test_forward_rejects_bad_arguments_before_launch(lib):
     layer = binding.MoELayer(128, 8, 128, 2)
     vp = C.c_void_p
