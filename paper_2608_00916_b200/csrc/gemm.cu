@@ -63,8 +63,10 @@ __device__ __forceinline__ void grouped_gemm(const GemmParams& p, const int work
     tmem_alloc(smem_base + TMEM_SLOT, TMEM_COLS);
     tmem_relinquish();
   }
-  // Row GEMMs of the experts wait for the kernel before them in front of their rows (chain_warp).
-  constexpr bool PRELOAD = !TR::WGRAD && !TR::STATIC_M;
+  // Row GEMMs of the experts wait for the kernel before them in front of their rows (chain_warp).  Not dgrad-down, whose epilogue needs all
+  // registers (with it 8 bytes of them go to memory): alone 36.4 -> 35.4 us at d 768, f 2048 and 125 rows per expert, 64.4 -> 62.1 at 500 rows, where
+  // steps take 150.5 -> 150.2 and 355.5 -> 352.2.
+  constexpr bool PRELOAD = !TR::WGRAD && !TR::STATIC_M && KIND != GEMM_B2;
   if (!PRELOAD && !p.ready) chain_wait();  // everything above touches only this CTA's own state
   tc_fence_before();
   __syncthreads();

@@ -115,6 +115,20 @@ def test_pairs_that_run_freely_ask_nothing_per_k_block():
     assert asks and all("if (PACED &&" in line for line in asks)
 
 
+def test_no_gemm_keeps_registers_in_memory(tmp_path):
+    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+    runs = [subprocess.Popen([nvcc, *build.NVCC_FLAGS, "-Xptxas", "-v", "-c", os.path.join(CSRC, name), "-o", str(tmp_path / (name + ".o"))],
+                             stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True) for name in ("gemm.cu", "gemm2.cu", "gemm_tokens.cu")]
+    kernels = 0
+    for run in runs:
+        out, _ = run.communicate()
+        assert run.returncode == 0, out
+        for kernel, spilt in re.findall(r"Compiling entry function '(\w+)'.*?(\d+) bytes spill stores", out, flags=re.DOTALL):
+            kernels += 1
+            assert spilt == "0", kernel
+    assert kernels >= 20
+
+
 def compiles(tmp_path, argument):
     src = tmp_path / "launch.cu"
     src.write_text('#include "common.cuh"\n'
