@@ -13,11 +13,18 @@ thread_local Chain* Chain::current_ = nullptr;
 
 // Whether the large GEMMs begin while the one before them drains (chain_warp in gemm_common.cuh).  With few rows per expert that fills
 // what the ends of the kernels leave idle.  With many, the power cap takes back in clocks what it saves in time, and pairs that begin
-// a GEMM at different times do not share operands as closely.  Steps at d 2048, f 768, 128 experts with against without, us:
-// 62 rows per expert 843 / 861, 128 rows 998 / 1018, 375 rows 1902 / 1916, 512 rows 2366 / 2359 (with adapters 2001 / 2070), 656 rows
-// 2896 / 2874, 1024 rows 4202 / 4136 (1024 on average, unequal: 4235 / 4293).  The small kernels run beside the weight
-// gradients, and the router's gradient fills the end of the GEMM before it, at every size: serial, it stood alone for 25 us at 8191
-// tokens and 57 at 16384.
+// a GEMM at different times do not share operands as closely.  Without -> with, us a step, in one process (runs of one side differ by 0.3 %):
+//   rows per expert              256             375             512             656             1024
+//   d 2048, f 768, 128 experts   1441 -> 1437    1884 -> 1861    2309 -> 2287    2789 -> 2845    4149 -> 4200
+//     adapters                                                   2035 -> 1991    2530 -> 2486    3681 -> 3624
+//     scoring                                                    758 -> 760                      1392 -> 1387
+//   d 1024, f 768, 128 experts   835 -> 808                      1312 -> 1276                    2272 -> 2231
+//   d 4096, f 3072, 32 experts   2404 -> 2356                    3776 -> 3759    5218 -> 5216 (750)  6790 -> 6812
+//   d 4096, f 14336, 8 experts                                   4374 -> 4305    5789 -> 5752 (750)  7441 -> 7406
+// (62 rows, d 2048, an earlier build: 861 -> 843; adapters at 500 rows of d 4096, f 3072 2809 -> 2735, scoring 1209 -> 1214; at f 14336 and 512 rows
+// 3300 -> 3234 and 1384 -> 1375.)  The line lies where plain steps at d 2048 begin to lose; narrow experts and adapters would still gain
+// beyond it, by 1.5 - 2 %.  The small kernels run beside the weight gradients, and the router's gradient fills the end of the GEMM before
+// it, at every size: serial, it stood alone for 25 us at 8191 tokens and 57 at 16384.
 static bool gemms_overlap(const Shape& s, int64_t T) { return T * s.k < static_cast<int64_t>(s.E) * 576; }
 
 static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }

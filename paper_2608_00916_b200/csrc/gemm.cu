@@ -309,8 +309,10 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) grouped_gemm_kernel(const __g
 }
 
 // The two contractions over dl side by side: the first `dx_blocks` blocks DX, the others DWR.  Both are a launch and the latency of a
-// tile or two up to some thousand tokens, and equal in work beyond.  One after the other -> together, us a step: the smallest shape
-// (d 256, f 512, 8 experts, 256 tokens) 66.2 -> 64.7; 1000 tokens and more at d 2048 alike (0.998, 0.997).
+// tile or two up to some thousand tokens, and equal in work beyond (with an fp32 router weight DX has three segments to DWR's two).  One
+// after the other -> together, us a step: the smallest shape (d 256, f 512, 8 experts, 256 tokens) 66.2 -> 64.7; 1000 tokens and more at
+// d 2048 alike (0.998, 0.997).  The launches alone, between events, with dwr_reduce_kernel: 25 -> 26 at 1000 tokens, 34 -> 33 at 4096, 73 -> 69 at
+// 16384, with an fp32 weight 27 -> 26, 36 -> 33, 81 -> 86.
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
     router_gradient_kernel(const __grid_constant__ GemmParams dx, const __grid_constant__ GemmParams dwr, int dx_blocks) {
   const int block = blockIdx.x;
