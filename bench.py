@@ -30,8 +30,8 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # dram bytes per launch of the dominant kernel taken from the committed ncu capture (profiles/), by stage name;
 # None where no capture has been taken for the workload.
 NCU_TRAFFIC = {  # profiles/step_launch_list_and_dram_traffic_qwen.md, profiles/gemm_dram_traffic_skewed_and_coarse.md
-    ("qwen", "gemm_gateup_swiglu"): 1.965e9, ("qwen", "gemm_down"): 1.147e9, ("qwen", "dgrad_down_swiglu_bwd"): 1.839e9,
-    ("qwen", "wgrad_down"): 1.130e9, ("qwen", "dgrad_gateup"): 1.757e9, ("qwen", "wgrad_gateup"): 1.740e9,
+    ("qwen", "gemm_gateup_swiglu"): 2.001e9, ("qwen", "gemm_down"): 1.148e9, ("qwen", "dgrad_down_swiglu_bwd"): 1.872e9,
+    ("qwen", "wgrad_down"): 1.139e9, ("qwen", "dgrad_gateup"): 1.759e9, ("qwen", "wgrad_gateup"): 1.752e9,
     ("skewed", "gemm_gateup_swiglu"): 1.937e9, ("skewed", "gemm_down"): 1.134e9, ("skewed", "dgrad_down_swiglu_bwd"): 1.779e9,
     ("skewed", "wgrad_down"): 1.202e9, ("skewed", "dgrad_gateup"): 1.727e9, ("skewed", "wgrad_gateup"): 1.998e9,
 }
